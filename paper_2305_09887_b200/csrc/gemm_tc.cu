@@ -17,6 +17,8 @@
 //                 sums of dZ) is added up from the staged dZ tiles by the otherwise idle
 //                 epilogue warps.
 //
+// The rows kernel also runs on pairs of blocks (a cluster of two, one MMA of 256 rows: rows_use_pairs).
+//
 // Warp roles: warp 0 = loader (one lane), warp 1 = TMEM owner and MMA issuer (one lane), the
 // remaining warps = epilogue (each warp reads its quarter of the 128 TMEM lanes).  Every
 // mbarrier wait is bounded; a wait that runs out raises the context's device error word and
@@ -129,6 +131,7 @@ tc_weight_prep_kernel(const __grid_constant__ GroupDesc g, const __grid_constant
 struct RowsArgs {
     GroupDesc g;
     CUtensorMap mapA0h, mapA0l, mapA1h, mapA1l, mapBh, mapBl;
+    CUtensorMap mapOh, mapOl;  // plane output: boxes of 64 columns x 32 rows
     int kb0, kb1;          // 64-wide k blocks taken from source 0 / source 1
     int BN, Npad, N;       // column tile, B rows per part, valid output columns
     int tmem_cols, stages; // columns of one accumulator buffer (two are allocated); pipeline depth
@@ -149,25 +152,29 @@ struct RowsArgs {
 // column tile, column tiles of one row tile adjacent).  Two accumulator buffers in tensor
 // memory let the epilogue of one tile overlap the main loop of the next; the shared-memory
 // ring keeps running across tiles.  Warps: 0 = loader, 1 = MMA issuer / TMEM owner,
-// 2..9 = epilogue (two warps per TMEM lane quarter, alternating 32-column chunks).
-constexpr int ROWS_THREADS = 320;
-constexpr int ROWS_EPI_THREADS = 256;
-constexpr int ROWS_STAGING_BYTES = 4096;          // per epilogue warp: a 32 x 32 fp32 block (or two 32 x 32 bf16)
+// 2..5 = epilogue (a warp per TMEM lane quarter, 64 columns at a time).
+constexpr int ROWS_THREADS = 192;
+constexpr int ROWS_EPI_WARPS = 4;
+constexpr int ROWS_MAX_STAGES = 6;
+enum RowsOut { OUT_F32, OUT_PLANES, OUT_GATED };  // fp32; split planes; split planes gated by the sign of `gate_hi`
+constexpr int ROWS_SLAB_BYTES = 2 * 32 * 128;     // per epilogue warp: 32 rows x 64 columns of both planes
 constexpr int ROWS_RING_BUDGET = 192 * 1024;      // shared memory for the operand ring
-constexpr int ROWS_SMEM_MAX = ROWS_RING_BUDGET + 1024 + 8 * ROWS_STAGING_BYTES;
+constexpr int ROWS_SMEM_MAX = ROWS_RING_BUDGET + 1024 + ROWS_EPI_WARPS * ROWS_SLAB_BYTES;
 
 struct RowsBarriers {
-    uint64_t full[MAX_STAGES];
-    uint64_t empty[MAX_STAGES];
+    uint64_t full[ROWS_MAX_STAGES];
+    uint64_t empty[ROWS_MAX_STAGES];
     uint64_t acc_full[2];   // all MMAs of the tile in this buffer finished
     uint64_t acc_empty[2];  // the epilogue has drained this buffer
     uint32_t tmem_base;
     int abort;
 };
 
+// PAIR: the barrier may be signalled from the pair's other block
+template <bool PAIR>
 __device__ __forceinline__ bool rows_wait(uint64_t* bar, uint32_t parity, RowsBarriers* pb, int* error_word) {
     for (uint32_t i = 0; i < tc::WAIT_POLLS; ++i) {
-        if (tc::mbar_try_wait(bar, parity)) return true;
+        if (PAIR ? tc::mbar_try_wait_cluster(bar, parity) : tc::mbar_try_wait(bar, parity)) return true;
         if ((i & 1023u) == 1023u && *reinterpret_cast<volatile int*>(&pb->abort)) break;
     }
     *reinterpret_cast<volatile int*>(&pb->abort) = 1;
@@ -175,16 +182,23 @@ __device__ __forceinline__ bool rows_wait(uint64_t* bar, uint32_t parity, RowsBa
     return false;
 }
 
-template <bool PLANES_OUT>
-__global__ void __launch_bounds__(ROWS_THREADS, 1) tc_rows_kernel(const __grid_constant__ RowsArgs a) {
+// PAIR = false: a block works on tiles of 128 rows by itself.  PAIR = true: two blocks of a cluster work on tiles of
+// 256 rows; `rank` 0 issues the MMAs of both (see tc_common.cuh).
+template <int OUT, bool PAIR>
+__device__ __forceinline__ void rows_body(const RowsArgs& a) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ RowsBarriers pb;
+    __shared__ __align__(16) float bias_slab[ROWS_EPI_WARPS][64];
     uint8_t* smem = align_1024(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int TILE_ROWS = PAIR ? 2 * TC_BM : TC_BM;
+    const int rank = PAIR ? (int)tc::cluster_rank() : 0;
+    const int64_t first_tile = PAIR ? blockIdx.x >> 1 : blockIdx.x, tile_step = PAIR ? gridDim.x >> 1 : gridDim.x;
     const int BN = a.BN, stages = a.stages, KB = a.kb0 + a.kb1;
+    const int b_rows = PAIR ? BN / 2 : BN;  // rows of the right operand this block stages
     const int n_tiles = a.Npad / BN;
     const int64_t total_tiles = a.row_tiles * n_tiles;
-    const uint32_t b_tile_bytes = (uint32_t)BN * 128u;
+    const uint32_t b_tile_bytes = (uint32_t)b_rows * 128u;
     const bool single = a.single != 0;
     const uint32_t np = single ? 1u : 2u;  // planes staged per operand
     const uint32_t stage_bytes = np * (PLANE_TILE_BYTES + b_tile_bytes);
@@ -200,7 +214,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, 1) tc_rows_kernel(const __grid_c
         }
         for (int b = 0; b < 2; ++b) {
             tc::mbar_init(&pb.acc_full[b], 1);
-            tc::mbar_init(&pb.acc_empty[b], ROWS_EPI_THREADS);
+            tc::mbar_init(&pb.acc_empty[b], (PAIR ? 2 : 1) * ROWS_EPI_WARPS);  // the first block's counts the warps of both
         }
         pb.abort = 0;
         tc::fence_barrier_init();
@@ -212,55 +226,101 @@ __global__ void __launch_bounds__(ROWS_THREADS, 1) tc_rows_kernel(const __grid_c
         tc::prefetch_tensormap(&a.mapBl);
     }
     if (warp == 1) {
-        tc::tmem_alloc(&pb.tmem_base, 2u * (uint32_t)a.tmem_cols);
-        tc::tmem_relinquish();
+        if constexpr (PAIR) {
+            tc::tmem_alloc_pair(&pb.tmem_base, 2u * (uint32_t)a.tmem_cols);
+            tc::tmem_relinquish_pair();
+        } else {
+            tc::tmem_alloc(&pb.tmem_base, 2u * (uint32_t)a.tmem_cols);
+            tc::tmem_relinquish();
+        }
     }
     tc::tc_fence_before_sync();
     __syncthreads();
+    if constexpr (PAIR) tc::cluster_sync();  // both blocks' barriers and tensor memory exist before either is signalled
     tc::tc_fence_after_sync();
     const uint32_t tmem_base = pb.tmem_base;
 
     if (warp == 0) {
         if (lane == 0) {
-            int64_t it = 0;  // k blocks issued so far by this block
+            int s = 0;
+            uint32_t phase = 0;   // of the stage about to be filled: flips when the ring wraps
+            int64_t filled = 0;
             bool ok = true;
-            for (int64_t tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+            for (int64_t tile = first_tile; tile < total_tiles && ok; tile += tile_step) {
                 int k, r0;
-                if (!locate_tile(a.g, TC_BM, tile / n_tiles, &k, &r0)) break;
+                if (!locate_tile(a.g, TILE_ROWS, tile / n_tiles, &k, &r0)) break;
                 const int n0 = (int)(tile % n_tiles) * BN;
-                const int arow = (int)(a.g.row_ws[k] + r0);
-                const int brow = k * a.Npad + n0;
-                for (int kb = 0; kb < KB; ++kb, ++it) {
-                    const int s = (int)(it % stages);
-                    ok = rows_wait(&pb.empty[s], (uint32_t)((it / stages) & 1) ^ 1u, &pb, a.error_word);
+                const int arow = (int)(a.g.row_ws[k] + r0) + rank * TC_BM;
+                const int brow = k * a.Npad + n0 + rank * b_rows;
+                for (int kb = 0; kb < KB; ++kb) {
+                    ok = rows_wait<PAIR>(&pb.empty[s], phase ^ 1u, &pb, a.error_word);
                     if (!ok) break;
-                    tc::mbar_arrive_expect_tx(&pb.full[s], stage_bytes);
-                    if (kb < a.kb0) {
-                        tc::tma_load_2d(a_hi(s), &a.mapA0h, &pb.full[s], kb * TC_BK, arow);
-                        if (!single) tc::tma_load_2d(a_lo(s), &a.mapA0l, &pb.full[s], kb * TC_BK, arow);
+                    const CUtensorMap* mh = kb < a.kb0 ? &a.mapA0h : &a.mapA1h;
+                    const CUtensorMap* ml = kb < a.kb0 ? &a.mapA0l : &a.mapA1l;
+                    const int ax = (kb < a.kb0 ? kb : kb - a.kb0) * TC_BK;
+                    if constexpr (PAIR) {
+                        // both blocks' bytes are counted on the first block's barrier, whose loader announces them; the
+                        // other's bytes may land before that (the phase still lacks the announcing arrival)
+                        if (rank == 0) tc::mbar_arrive_expect_tx(&pb.full[s], 2u * stage_bytes);
+                        const uint32_t bar = tc::leader_addr(&pb.full[s]);
+                        tc::tma_load_2d_pair(a_hi(s), mh, bar, ax, arow);
+                        tc::tma_load_2d_pair(b_hi(s), &a.mapBh, bar, kb * TC_BK, brow);
+                        if (!single) {
+                            tc::tma_load_2d_pair(a_lo(s), ml, bar, ax, arow);
+                            tc::tma_load_2d_pair(b_lo(s), &a.mapBl, bar, kb * TC_BK, brow);
+                        }
                     } else {
-                        tc::tma_load_2d(a_hi(s), &a.mapA1h, &pb.full[s], (kb - a.kb0) * TC_BK, arow);
-                        if (!single) tc::tma_load_2d(a_lo(s), &a.mapA1l, &pb.full[s], (kb - a.kb0) * TC_BK, arow);
+                        tc::mbar_arrive_expect_tx(&pb.full[s], stage_bytes);
+                        tc::tma_load_2d(a_hi(s), mh, &pb.full[s], ax, arow);
+                        if (!single) tc::tma_load_2d(a_lo(s), ml, &pb.full[s], ax, arow);
+                        tc::tma_load_2d(b_hi(s), &a.mapBh, &pb.full[s], kb * TC_BK, brow);
+                        if (!single) tc::tma_load_2d(b_lo(s), &a.mapBl, &pb.full[s], kb * TC_BK, brow);
                     }
-                    tc::tma_load_2d(b_hi(s), &a.mapBh, &pb.full[s], kb * TC_BK, brow);
-                    if (!single) tc::tma_load_2d(b_lo(s), &a.mapBl, &pb.full[s], kb * TC_BK, brow);
+                    ++filled;
+                    if (++s == stages) {
+                        s = 0;
+                        phase ^= 1u;
+                    }
+                }
+            }
+            if constexpr (PAIR) {
+                // Leave no signal under way: every stage filled is waited for until it has been released (both blocks
+                // get that signal) or, after a give-up, until its loads have landed (the first block, for both).
+                const int64_t tail = filled < stages ? filled : stages;
+                for (int64_t n = filled - tail; n < filled; ++n) {
+                    const int ts = (int)(n % stages);
+                    const uint32_t tp = (uint32_t)((n / stages) & 1);
+                    if (!ok || !rows_wait<PAIR>(&pb.empty[ts], tp, &pb, a.error_word)) {
+                        ok = false;
+                        if (rank == 0)
+                            for (uint32_t i = 0; i < (1u << 14) && !tc::mbar_try_wait_cluster(&pb.full[ts], tp); ++i) {}
+                    }
                 }
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t idesc = tc::idesc_bf16(TC_BM, BN, false, false);
-            int64_t it = 0, t = 0;  // k blocks consumed, tiles started
+        if (lane == 0 && rank == 0) {
+            const uint32_t idesc = tc::idesc_bf16(TILE_ROWS, BN, false, false);
+            auto mma = [&](uint32_t d, uint64_t da, uint64_t db, uint32_t acc) {
+                if constexpr (PAIR) tc::mma_bf16_pair(d, da, db, idesc, acc);
+                else tc::mma_bf16(d, da, db, idesc, acc);
+            };
+            auto commit = [&](uint64_t* bar) {
+                if constexpr (PAIR) tc::mma_commit_pair(bar);
+                else tc::mma_commit(bar);
+            };
+            int s = 0;
+            uint32_t phase = 0;
+            int64_t t = 0;  // tiles started
             bool ok = true;
-            for (int64_t tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++t) {
+            for (int64_t tile = first_tile; tile < total_tiles && ok; tile += tile_step, ++t) {
                 const int buf = (int)(t & 1);
-                ok = rows_wait(&pb.acc_empty[buf], (uint32_t)((t >> 1) & 1) ^ 1u, &pb, a.error_word);
+                ok = rows_wait<PAIR>(&pb.acc_empty[buf], (uint32_t)((t >> 1) & 1) ^ 1u, &pb, a.error_word);
                 if (!ok) break;
                 tc::tc_fence_after_sync();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * a.tmem_cols);
-                for (int kb = 0; kb < KB; ++kb, ++it) {
-                    const int s = (int)(it % stages);
-                    ok = rows_wait(&pb.full[s], (uint32_t)((it / stages) & 1), &pb, a.error_word);
+                for (int kb = 0; kb < KB; ++kb) {
+                    ok = rows_wait<PAIR>(&pb.full[s], phase, &pb, a.error_word);
                     if (!ok) break;
                     tc::tc_fence_after_sync();
                     const uint32_t ah = tc::smem_u32(a_hi(s)), al = tc::smem_u32(a_lo(s));
@@ -270,149 +330,198 @@ __global__ void __launch_bounds__(ROWS_THREADS, 1) tc_rows_kernel(const __grid_c
                         const uint32_t off = ks * 32;  // 16 bf16 = 32 bytes along K inside the swizzle row
                         const uint64_t dah = tc::smem_desc_sw128(ah + off, 16, 1024), dbh = tc::smem_desc_sw128(bh + off, 16, 1024);
                         if (single) {
-                            tc::mma_bf16(d_tmem, dah, dbh, idesc, (kb | ks) ? 1u : 0u);
+                            mma(d_tmem, dah, dbh, (kb | ks) ? 1u : 0u);
                         } else {
                             const uint64_t dal = tc::smem_desc_sw128(al + off, 16, 1024), dbl = tc::smem_desc_sw128(bl + off, 16, 1024);
-                            tc::mma_bf16(d_tmem, dal, dbh, idesc, (kb | ks) ? 1u : 0u);
-                            tc::mma_bf16(d_tmem, dah, dbl, idesc, 1u);
-                            tc::mma_bf16(d_tmem, dah, dbh, idesc, 1u);
+                            mma(d_tmem, dal, dbh, (kb | ks) ? 1u : 0u);
+                            mma(d_tmem, dah, dbl, 1u);
+                            mma(d_tmem, dah, dbh, 1u);
                         }
                     }
-                    tc::mma_commit(&pb.empty[s]);
+                    commit(&pb.empty[s]);
+                    if (++s == stages) {
+                        s = 0;
+                        phase ^= 1u;
+                    }
                 }
-                if (ok) tc::mma_commit(&pb.acc_full[buf]);
+                if (ok) commit(&pb.acc_full[buf]);
             }
         }
     } else {
-        const int ew = warp - 2;          // 0..7
-        const int q = warp & 3;           // the TMEM lane quarter this warp may read
-        const int col_phase = ew >> 2;    // which of the two warps of the quarter: even or odd chunks
-        uint8_t* stg = smem + (size_t)stages * stage_bytes + (size_t)ew * ROWS_STAGING_BYTES;  // 4 KB per warp
+        const int q = warp & 3;           // the TMEM lane quarter this warp may read: rows 32 q .. 32 q + 31 of the tile
+        uint8_t* slab_hi = smem + (size_t)stages * stage_bytes + (size_t)q * ROWS_SLAB_BYTES;  // [32 rows][64 columns] of either plane
+        uint8_t* slab_lo = slab_hi + ROWS_SLAB_BYTES / 2;
+        const uint32_t swz = (uint32_t)(lane & 7);
         int64_t t = 0;
         bool ok = true;
-        for (int64_t tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++t) {
+        for (int64_t tile = first_tile; tile < total_tiles && ok; tile += tile_step, ++t) {
             int k, r0;
-            if (!locate_tile(a.g, TC_BM, tile / n_tiles, &k, &r0)) break;
+            if (!locate_tile(a.g, TILE_ROWS, tile / n_tiles, &k, &r0)) break;
+            r0 += rank * TC_BM + q * 32;  // the warp's first row (of a pair's tile: in this block's half)
             const int n0 = (int)(tile % n_tiles) * BN;
             const int buf = (int)(t & 1);
-            ok = rows_wait(&pb.acc_full[buf], (uint32_t)((t >> 1) & 1), &pb, a.error_word);
+            const int rows_here = min(32, a.g.rows[k] - r0);  // live rows of the warp; not positive past the part's end
+            const bool live = lane < rows_here;
+            const int64_t orow0 = a.g.row_ws[k] + r0;
+            // a chunk's bias (lane l: columns l and l + 32) and the lane's row of its gate, requested a chunk ahead
+            const float* bias = a.bias_offset >= 0 ? a.params + (int64_t)a.g.part[k] * a.P + a.bias_offset : nullptr;
+            float nb0 = 0.f, nb1 = 0.f;
+            uint4 gw[8];
+            auto request = [&](int c0) {
+                const int n = n0 + c0;
+                if (bias) {
+                    nb0 = n + lane < a.N ? __ldg(bias + n + lane) : 0.f;
+                    nb1 = n + 32 + lane < a.N ? __ldg(bias + n + 32 + lane) : 0.f;
+                }
+                if constexpr (OUT == OUT_GATED) {
+                    const uint4* gp = reinterpret_cast<const uint4*>(a.gate_hi + (orow0 + lane) * a.out_planes.ld + n);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) gw[j] = live && n + 8 * j < a.out_planes.ld ? gp[j] : make_uint4(0u, 0u, 0u, 0u);
+                }
+            };
+            request(0);
+            ok = rows_wait<PAIR>(&pb.acc_full[buf], (uint32_t)((t >> 1) & 1), &pb, a.error_word);
             if (!ok) break;
             tc::tc_fence_after_sync();
-            const uint32_t d_tmem = tmem_base + (uint32_t)(buf * a.tmem_cols);
-            const int i = r0 + q * 32 + lane;
-            const bool live = i < a.g.rows[k];
-            const float* bias = a.bias_offset >= 0 ? a.params + (int64_t)a.g.part[k] * a.P + a.bias_offset : nullptr;
-            const int rows_here = min(32, a.g.rows[k] - (r0 + q * 32));  // live rows of this warp's quarter
-            const int64_t orow0 = a.g.row_ws[k] + r0 + q * 32;
-            for (int c0 = col_phase * 32; c0 < BN; c0 += 64) {
-                // the gate words this thread will need after the transpose, requested before the
-                // accumulator is read so that their latency hides behind it
-                uint4 gq[4];
-                if constexpr (PLANES_OUT) {
-                    if (a.gate_hi) {
-                        const int gn = n0 + c0 + 8 * (lane & 3);
-                        const bool g_ok = gn < a.out_planes.ld && c0 + 8 * (lane & 3) < BN;
+            const uint32_t acc = tmem_base + (uint32_t)(buf * a.tmem_cols) + ((uint32_t)(q * 32) << 16);
+            // Longest chain of the products with K <= 256, and bound by what its stores can move (8 warps with half the work
+            // each took as long).  Stores of 64-byte pieces by the warps, or of own rows 32 bytes at a time, were slower
+            // (gated 99 and 126 us against 90); unrolled chunks did not fit the instruction cache (11 us a tile against 7).
+#pragma unroll 1
+            for (int c0 = 0; c0 < BN && rows_here > 0; c0 += 64) {
+                uint32_t raw[2][32];
+                tc::tmem_load_issue(acc + (uint32_t)c0, raw[0]);
+                if (c0 + 32 < BN) tc::tmem_load_issue(acc + (uint32_t)(c0 + 32), raw[1]);
+                if (bias) {
+                    __syncwarp();
+                    bias_slab[q][lane] = nb0;
+                    bias_slab[q][32 + lane] = nb1;
+                    __syncwarp();
+                }
+                uint32_t mask[32];  // 0xFFFF in the halves that the gate lets pass
+                if constexpr (OUT == OUT_GATED) {
 #pragma unroll
-                        for (int it = 0; it < 4; ++it) {
-                            const int row = it * 8 + (lane >> 2);
-                            gq[it] = (g_ok && row < rows_here)
-                                         ? *reinterpret_cast<const uint4*>(a.gate_hi + (orow0 + row) * a.out_planes.ld + gn)
-                                         : make_uint4(0u, 0u, 0u, 0u);
-                        }
+                    for (int j = 0; j < 8; ++j) {
+                        mask[4 * j] = positive_halves(gw[j].x);
+                        mask[4 * j + 1] = positive_halves(gw[j].y);
+                        mask[4 * j + 2] = positive_halves(gw[j].z);
+                        mask[4 * j + 3] = positive_halves(gw[j].w);
                     }
                 }
-                float v[32];
-                tc::tmem_load_32x32(d_tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);
-                if (rows_here <= 0) continue;
+                if (c0 + 64 < BN) request(c0 + 64);
+                tc::tmem_load_wait(raw[0]);
+                tc::tmem_load_wait(raw[1]);
                 const int nbase = n0 + c0;
-                if constexpr (!PLANES_OUT) {
-                    // fp32 output (logits): each thread stores its own row, pack by pack
-                    if (!live) continue;
+                if constexpr (OUT == OUT_F32) {
+                    // fp32 output (logits): every lane stores its own row
                     float* o = a.out + (orow0 + lane) * a.ld_out;
+                    if (live) {
 #pragma unroll
-                    for (int j = 0; j < 32; j += 8) {
-                        const int n = nbase + j;
-                        if (n >= a.N || c0 + j >= BN) break;  // BN is a multiple of 16, not always of 32
-                        float x[8];
+                        for (int j = 0; j < 64; j += 4) {
+                            const int n = nbase + j;
+                            float x[4];
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            float tv = v[j + e];
-                            if (n + e < a.N) {
-                                if (bias) tv += __ldg(bias + n + e);
-                                if (a.relu) tv = fmaxf(tv, 0.f);
+                            for (int e = 0; e < 4; ++e) {
+                                x[e] = __uint_as_float(raw[j >> 5][(j & 31) + e]);
+                                if (bias) x[e] += bias_slab[q][j + e];
+                                if (a.relu) x[e] = fmaxf(x[e], 0.f);
                             }
-                            x[e] = tv;
-                        }
-                        if (n + 7 < a.N) {
-                            *reinterpret_cast<float4*>(o + n) = make_float4(x[0], x[1], x[2], x[3]);
-                            *reinterpret_cast<float4*>(o + n + 4) = make_float4(x[4], x[5], x[6], x[7]);
-                        } else {
-                            for (int e = 0; e < 8 && n + e < a.N; ++e) o[n + e] = x[e];
+                            if (n + 3 < a.N) {
+                                *reinterpret_cast<float4*>(o + n) = make_float4(x[0], x[1], x[2], x[3]);
+                            } else {
+#pragma unroll
+                                for (int e = 0; e < 4; ++e)
+                                    if (n + e < a.N) o[n + e] = x[e];
+                            }
                         }
                     }
+                    __syncwarp();
                 } else {
-                    // Plane output.  The warp's 32 x 32 block goes through its staging slab as fp32
-                    // (16-byte chunk j of row r stored at chunk j ^ (r & 7): conflict free both ways),
-                    // so that afterwards a thread owns 8 consecutive columns of a row: bias is two
-                    // vector loads per chunk, and every store instruction writes whole 64-byte row
-                    // segments of a plane.
-                    float4* st = reinterpret_cast<float4*>(stg);  // [32 rows][8 chunks of 4 floats]
-                    __syncwarp();
+                    // Columns past the layer's width need no masking: the repacked weights are zero there and so is the
+                    // bias, hence the accumulator, the sum and its ReLU are zero and the padding columns stay zero.
+                    // (What lies past the accumulator's BN columns is past the planes' too and is not stored.)
+                    uint32_t h[32], l[32];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        st[lane * 8 + (j ^ (lane & 7))] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-                    __syncwarp();
-                    const int p = lane & 3;
-                    const int n = nbase + 8 * p;
-                    const bool col_ok = n < a.out_planes.ld && c0 + 8 * p < BN;
-                    float bv[8];
+                    for (int j = 0; j < 32; j += 2) {
+                        float x[4];
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) bv[e] = (bias && col_ok && n + e < a.N) ? __ldg(bias + n + e) : 0.f;
-                    // the thread's 16 bytes of row (lane >> 2) of the block, in either plane; the four
-                    // rows it finishes are 8 rows apart
-                    const uint32_t out_row_bytes = (uint32_t)a.out_planes.ld * 2u;
-                    char* oh = reinterpret_cast<char*>(a.out_planes.hi + (orow0 + (lane >> 2)) * a.out_planes.ld + n);
-                    char* ol = reinterpret_cast<char*>(a.out_planes.lo + (orow0 + (lane >> 2)) * a.out_planes.ld + n);
-#pragma unroll
-                    for (int it = 0; it < 4; ++it) {
-                        const int row = it * 8 + (lane >> 2);
-                        const float4 x0 = st[row * 8 + ((2 * p) ^ (row & 7))];
-                        const float4 x1 = st[row * 8 + ((2 * p + 1) ^ (row & 7))];
-                        if (row < rows_here && col_ok) {
-                            Pack8 x;
-                            x.v[0] = x0.x; x.v[1] = x0.y; x.v[2] = x0.z; x.v[3] = x0.w;
-                            x.v[4] = x1.x; x.v[5] = x1.y; x.v[6] = x1.z; x.v[7] = x1.w;
-                            // Columns past the layer's width need no masking: the repacked weights are zero
-                            // there and so is bv, hence the accumulator, the sum and its ReLU are zero
-                            // and the padding columns of the planes stay zero.
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) {
-                                const float tv = x.v[e] + bv[e];
-                                x.v[e] = a.relu ? fmaxf(tv, 0.f) : tv;
-                            }
-                            if (a.gate_hi) {
-                                const uint32_t gw[4] = {gq[it].x, gq[it].y, gq[it].z, gq[it].w};
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) {
-                                    const float gate = __uint_as_float((e & 1) ? (gw[e >> 1] & 0xFFFF0000u) : (gw[e >> 1] << 16));
-                                    if (!(gate > 0.f)) x.v[e] = 0.f;
-                                }
-                            }
-                            uint4 h, l;
-                            x.to_planes_lean(h, l);
-                            *reinterpret_cast<uint4*>(oh + (size_t)(it * 8) * out_row_bytes) = h;
-                            *reinterpret_cast<uint4*>(ol + (size_t)(it * 8) * out_row_bytes) = l;
+                        for (int e = 0; e < 4; ++e) x[e] = __uint_as_float(raw[j >> 4][2 * (j & 15) + e]);
+                        if (bias) {
+                            const float4 b4 = *reinterpret_cast<const float4*>(&bias_slab[q][2 * j]);
+                            add_pair(x[0], x[1], b4.x, b4.y);
+                            add_pair(x[2], x[3], b4.z, b4.w);
                         }
+                        if (a.relu) {
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) x[e] = fmaxf(x[e], 0.f);
+                        }
+                        split_pair(x[0], x[1], h[j], l[j]);
+                        split_pair(x[2], x[3], h[j + 1], l[j + 1]);
+                        if constexpr (OUT == OUT_GATED) {
+                            h[j] &= mask[j];
+                            l[j] &= mask[j];
+                            h[j + 1] &= mask[j + 1];
+                            l[j + 1] &= mask[j + 1];
+                        }
+                    }
+                    // Out through shared memory (row r's 16-byte piece j at piece j ^ (r % 8)), one bulk-tensor store per plane.
+                    if (lane == 0) tc::tma_store_wait_read();  // the chunk before has left the slab
+                    __syncwarp();
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const uint32_t at = (uint32_t)lane * 128u + (((uint32_t)j ^ swz) << 4);
+                        *reinterpret_cast<uint4*>(slab_hi + at) = make_uint4(h[4 * j], h[4 * j + 1], h[4 * j + 2], h[4 * j + 3]);
+                        *reinterpret_cast<uint4*>(slab_lo + at) = make_uint4(l[4 * j], l[4 * j + 1], l[4 * j + 2], l[4 * j + 3]);
+                    }
+                    if (rows_here == 32) {
+                        tc::fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0 && nbase < a.out_planes.ld) {
+                            tc::tma_store_2d(&a.mapOh, slab_hi, nbase, (int)orow0);
+                            tc::tma_store_2d(&a.mapOl, slab_lo, nbase, (int)orow0);
+                            tc::tma_store_commit();
+                        }
+                    } else {  // the part's last rows: the rows behind them are not this part's
+                        __syncwarp();
+                        const int n = nbase + 8 * (lane & 7);
+                        for (int row = lane >> 3; row < rows_here; row += 4) {
+                            const uint32_t at = (uint32_t)row * 128u + ((uint32_t)((lane ^ row) & 7) << 4);
+                            if (n < a.out_planes.ld) {
+                                const int64_t o = (orow0 + row) * a.out_planes.ld + n;
+                                *reinterpret_cast<uint4*>(a.out_planes.hi + o) = *reinterpret_cast<const uint4*>(slab_hi + at);
+                                *reinterpret_cast<uint4*>(a.out_planes.lo + o) = *reinterpret_cast<const uint4*>(slab_lo + at);
+                            }
+                        }
+                        __syncwarp();
                     }
                 }
             }
             tc::tc_fence_before_sync();
-            tc::mbar_arrive(&pb.acc_empty[buf]);  // all 256 epilogue threads arrive: the buffer may be overwritten
+            __syncwarp();
+            if (lane == 0) {  // every epilogue warp (of both blocks) arrives: the buffer may be overwritten
+                if constexpr (PAIR) tc::mbar_arrive_cluster(tc::leader_addr(&pb.acc_empty[buf]));
+                else tc::mbar_arrive(&pb.acc_empty[buf]);
+            }
         }
+        if (OUT != OUT_F32 && lane == 0) tc::tma_store_wait_all();
     }
     tc::tc_fence_before_sync();
     __syncthreads();
-    if (warp == 1) tc::tmem_dealloc(tmem_base, 2u * (uint32_t)a.tmem_cols);
+    if constexpr (PAIR) {
+        tc::cluster_sync();  // neither block leaves while the other may still signal it or read its operands
+        if (warp == 1) tc::tmem_dealloc_pair(tmem_base, 2u * (uint32_t)a.tmem_cols);
+    } else {
+        if (warp == 1) tc::tmem_dealloc(tmem_base, 2u * (uint32_t)a.tmem_cols);
+    }
+}
+
+template <int OUT>
+__global__ void __launch_bounds__(ROWS_THREADS, 1) tc_rows_kernel(const __grid_constant__ RowsArgs a) {
+    rows_body<OUT, false>(a);
+}
+template <int OUT>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(ROWS_THREADS, 1) tc_rows_pair_kernel(const __grid_constant__ RowsArgs a) {
+    rows_body<OUT, true>(a);
 }
 
 // ------------------------------------------------------------------------------------
@@ -736,23 +845,28 @@ bool make_tensor_map_bf16(CUtensorMap* out, const void* base, uint64_t rows, uin
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Column tile of the rows kernel for `d` columns: at most 256 wide, equal tiles, a multiple of 16; from 64 columns on a
+// multiple of 32, the step of an MMA of a pair of blocks; more than one tile: of 64, what the epilogue stores at a time.
+static int column_tile(int d) {
+    const int tiles = (int)ceil_div(d, 256), step = tiles > 1 ? 64 : d >= 64 ? 32 : 16;
+    return (int)ceil_div(ceil_div(d, tiles), step) * step;
+}
+
 TcLayerPlan tc_plan_layer(LayerShape ls) {
     TcLayerPlan p{};
     p.Kf = ls.nsrc * TC_BK * (int)ceil_div(ls.d_in, TC_BK);
-    int tiles = (int)ceil_div(ls.d_out, 256);
-    p.BN_f = (int)ceil_div(ceil_div(ls.d_out, tiles), 16) * 16;
-    p.Npad_f = p.BN_f * tiles;
+    p.BN_f = column_tile(ls.d_out);
+    p.Npad_f = p.BN_f * (int)ceil_div(ls.d_out, 256);
     p.Kd = ls.nsrc * TC_BK * (int)ceil_div(ls.d_out, TC_BK);
-    tiles = (int)ceil_div(ls.d_in, 256);
-    p.BN_d = (int)ceil_div(ceil_div(ls.d_in, tiles), 16) * 16;
-    p.Npad_d = p.BN_d * tiles;
+    p.BN_d = column_tile(ls.d_in);
+    p.Npad_d = p.BN_d * (int)ceil_div(ls.d_in, 256);
     return p;
 }
 
 TcLayerPlan tc_plan_head(LayerShape ls, int head_cp) {
     TcLayerPlan p = tc_plan_layer(ls);  // the dgrad operand is the usual one
     p.Kf = TC_BK * (int)ceil_div(ls.d_in, TC_BK);
-    p.BN_f = p.Npad_f = (int)ceil_div(ls.nsrc * head_cp, 16) * 16;
+    p.BN_f = p.Npad_f = column_tile(ls.nsrc * head_cp);  // at most 128 columns
     return p;
 }
 
@@ -779,28 +893,53 @@ int32_t launch_tc_weight_prep(rtma_ctx* ctx, const GroupDesc& g, const TcPrepJob
     return RTMA_OK;
 }
 
-static int32_t launch_rows(rtma_ctx* ctx, RowsArgs& a, int kclass, cudaStream_t s) {
+// Do a product's tiles go to pairs of blocks (256 rows, each block staging half of the weight tile)?  A block by itself
+// moves 96 KB through shared memory per 64 of K and 128 x 256 outputs, a third of it activations, next to what the MMAs
+// read there; a pair 64 KB each.  That pays where the main loop is the longest chain: medium graph (200 k rows, 8 parts),
+// us alone / in pairs: K = 512, 256 columns 151 / 115, gated 154 / 130; operands rounded to bf16, K = 1024, 500 k rows
+// 500 / 442.  With K <= 256 the output is the longer chain and the pair's blocks wait for each other: 84 / 90, gated 90 / 95,
+// 96 columns 53 / 60.  And only where a launch has tiles for every SM: 10 k rows a part, 3 parts 12.5 / 13.2.
+static bool rows_use_pairs(const rtma_ctx* ctx, const GroupDesc& g, int K, int BN) {
+    return BN % 32 == 0 && BN >= 128 && K >= 384 && group_tiles(g, TC_BM) >= ctx->sm_count;
+}
+
+static int32_t launch_rows(rtma_ctx* ctx, RowsArgs& a, int64_t rows_total, bool pairs, int kclass, cudaStream_t s) {
     if (!ctx->rows_configured) {  // per device: the context is bound to one
-        RTMA_CUDA(ctx, cudaFuncSetAttribute(reinterpret_cast<const void*>(tc_rows_kernel<true>),
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize, ROWS_SMEM_MAX));
-        RTMA_CUDA(ctx, cudaFuncSetAttribute(reinterpret_cast<const void*>(tc_rows_kernel<false>),
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize, ROWS_SMEM_MAX));
+        const void* kernels[] = {reinterpret_cast<const void*>(tc_rows_kernel<OUT_F32>), reinterpret_cast<const void*>(tc_rows_kernel<OUT_PLANES>),
+                                 reinterpret_cast<const void*>(tc_rows_kernel<OUT_GATED>),
+                                 reinterpret_cast<const void*>(tc_rows_pair_kernel<OUT_F32>),
+                                 reinterpret_cast<const void*>(tc_rows_pair_kernel<OUT_PLANES>),
+                                 reinterpret_cast<const void*>(tc_rows_pair_kernel<OUT_GATED>)};
+        for (const void* kernel : kernels)
+            RTMA_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ROWS_SMEM_MAX));
         ctx->rows_configured = true;
     }
-    const size_t stage_bytes = (a.single ? 1 : 2) * ((size_t)PLANE_TILE_BYTES + (size_t)a.BN * 128);
-    a.stages = std::max(1, std::min<int>(MAX_STAGES, (int)(ROWS_RING_BUDGET / stage_bytes)));
+    const size_t stage_bytes = (a.single ? 1 : 2) * ((size_t)PLANE_TILE_BYTES + (size_t)(pairs ? a.BN / 2 : a.BN) * 128);
+    a.stages = std::max(1, std::min<int>(ROWS_MAX_STAGES, (int)(ROWS_RING_BUDGET / stage_bytes)));
     a.tmem_cols = (int)tmem_columns_for(a.BN);
     a.error_word = ctx->error_word;
-    a.row_tiles = group_tiles(a.g, TC_BM);
+    a.row_tiles = group_tiles(a.g, pairs ? 2 * TC_BM : TC_BM);
     if (a.row_tiles == 0) return RTMA_OK;
     const int64_t total_tiles = a.row_tiles * (a.Npad / a.BN);
-    const unsigned grid = (unsigned)std::min<int64_t>(total_tiles, ctx->sm_count);
-    // the epilogue staging slabs are only allocated for plane output: shared memory comes out of L1
+    const unsigned grid = pairs ? 2u * (unsigned)std::min<int64_t>(total_tiles, ctx->sm_count / 2)
+                                : (unsigned)std::min<int64_t>(total_tiles, ctx->sm_count);
+    if (a.out_planes.hi && !plane_maps(&a.mapOh, &a.mapOl, a.out_planes, rows_total, (uint64_t)a.out_planes.ld, 64, 32))
+        return rtma_fail(ctx, RTMA_ERR_CUDA, "cuTensorMapEncodeTiled refused the output planes");
+    // the epilogue's slabs are only allocated for plane output: shared memory comes out of L1
+    const size_t ring = a.stages * stage_bytes + 1024;
+    const size_t smem = a.out_planes.hi ? ring + ROWS_EPI_WARPS * ROWS_SLAB_BYTES : ring;
     {
         KernelScope ks(ctx, kclass, s);
-        const size_t ring = a.stages * stage_bytes + 1024;
-        if (a.out_planes.hi) tc_rows_kernel<true><<<grid, ROWS_THREADS, ring + 8 * ROWS_STAGING_BYTES, s>>>(a);
-        else tc_rows_kernel<false><<<grid, ROWS_THREADS, ring, s>>>(a);
+        const int out = !a.out_planes.hi ? OUT_F32 : a.gate_hi ? OUT_GATED : OUT_PLANES;
+#define RTMA_ROWS(KERNEL)                                                                            \
+    do {                                                                                             \
+        if (out == OUT_F32) KERNEL<OUT_F32><<<grid, ROWS_THREADS, smem, s>>>(a);                     \
+        else if (out == OUT_PLANES) KERNEL<OUT_PLANES><<<grid, ROWS_THREADS, smem, s>>>(a);          \
+        else KERNEL<OUT_GATED><<<grid, ROWS_THREADS, smem, s>>>(a);                                  \
+    } while (0)
+        if (pairs) RTMA_ROWS(tc_rows_pair_kernel);
+        else RTMA_ROWS(tc_rows_kernel);
+#undef RTMA_ROWS
     }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
@@ -813,10 +952,12 @@ int32_t launch_tc_forward(rtma_ctx* ctx, const GroupDesc& g, LayerShape ls, cons
     RowsArgs a{};
     a.g = g;
     a.single = single ? 1 : 0;
+    const bool pairs = rows_use_pairs(ctx, g, p.Kf, p.BN_f);
+    const uint32_t b_rows = (uint32_t)(pairs ? p.BN_f / 2 : p.BN_f);
     if (!plane_maps(&a.mapA0h, &a.mapA0l, H, rows_total, ls.d_in, TC_BK, TC_BM) ||
         !plane_maps(&a.mapA1h, &a.mapA1l, N, rows_total, ls.d_in, TC_BK, TC_BM) ||
-        !make_tensor_map_bf16(&a.mapBh, Bf_hi, (uint64_t)g.num * p.Npad_f, p.Kf, p.Kf, TC_BK, p.BN_f) ||
-        !make_tensor_map_bf16(&a.mapBl, Bf_lo, (uint64_t)g.num * p.Npad_f, p.Kf, p.Kf, TC_BK, p.BN_f))
+        !make_tensor_map_bf16(&a.mapBh, Bf_hi, (uint64_t)g.num * p.Npad_f, p.Kf, p.Kf, TC_BK, b_rows) ||
+        !make_tensor_map_bf16(&a.mapBl, Bf_lo, (uint64_t)g.num * p.Npad_f, p.Kf, p.Kf, TC_BK, b_rows))
         return rtma_fail(ctx, RTMA_ERR_CUDA, "cuTensorMapEncodeTiled refused the forward operands");
     if (ls.nsrc == 2) {
         a.kb0 = a.kb1 = p.Kf / (2 * TC_BK);
@@ -837,7 +978,7 @@ int32_t launch_tc_forward(rtma_ctx* ctx, const GroupDesc& g, LayerShape ls, cons
     a.bias_offset = ls.has_bias ? ls.param_offset + (int64_t)ls.nsrc * ls.d_in * ls.d_out : -1;
     a.relu = relu ? 1 : 0;
     a.gate_hi = nullptr;
-    return launch_rows(ctx, a, KC_GEMM_FWD, s);
+    return launch_rows(ctx, a, rows_total, pairs, KC_GEMM_FWD, s);
 }
 
 int32_t launch_tc_dgrad(rtma_ctx* ctx, const GroupDesc& g, LayerShape ls, const TcLayerPlan& p, int64_t rows_total,
@@ -846,10 +987,12 @@ int32_t launch_tc_dgrad(rtma_ctx* ctx, const GroupDesc& g, LayerShape ls, const 
     RowsArgs a{};
     a.g = g;
     a.single = single ? 1 : 0;
+    const bool pairs = rows_use_pairs(ctx, g, p.Kd, p.BN_d);
+    const uint32_t b_rows = (uint32_t)(pairs ? p.BN_d / 2 : p.BN_d);
     if (!plane_maps(&a.mapA0h, &a.mapA0l, dZ, rows_total, ls.d_out, TC_BK, TC_BM) ||
         !plane_maps(&a.mapA1h, &a.mapA1l, Q, rows_total, ls.d_out, TC_BK, TC_BM) ||
-        !make_tensor_map_bf16(&a.mapBh, Bd_hi, (uint64_t)g.num * p.Npad_d, p.Kd, p.Kd, TC_BK, p.BN_d) ||
-        !make_tensor_map_bf16(&a.mapBl, Bd_lo, (uint64_t)g.num * p.Npad_d, p.Kd, p.Kd, TC_BK, p.BN_d))
+        !make_tensor_map_bf16(&a.mapBh, Bd_hi, (uint64_t)g.num * p.Npad_d, p.Kd, p.Kd, TC_BK, b_rows) ||
+        !make_tensor_map_bf16(&a.mapBl, Bd_lo, (uint64_t)g.num * p.Npad_d, p.Kd, p.Kd, TC_BK, b_rows))
         return rtma_fail(ctx, RTMA_ERR_CUDA, "cuTensorMapEncodeTiled refused the dgrad operands");
     if (ls.nsrc == 2) {
         a.kb0 = a.kb1 = p.Kd / (2 * TC_BK);
@@ -870,7 +1013,7 @@ int32_t launch_tc_dgrad(rtma_ctx* ctx, const GroupDesc& g, LayerShape ls, const 
     a.bias_offset = -1;
     a.relu = 0;
     a.gate_hi = gate ? H.hi : nullptr;
-    return launch_rows(ctx, a, KC_GEMM_DGRAD, s);
+    return launch_rows(ctx, a, rows_total, pairs, KC_GEMM_DGRAD, s);
 }
 
 int tc_wgrad_blocks_per_slot(const LayerShape& ls) {

@@ -48,6 +48,30 @@ __device__ __forceinline__ float add_f32_bf16(float acc, unsigned short x_bits) 
     asm("add.rn.f32.bf16 %0, %1, %2;" : "=f"(d) : "h"(x_bits), "f"(acc));
     return d;
 }
+// Two fp32 additions as one instruction: (a0, a1) + (b0, b1), each rounded to nearest
+__device__ __forceinline__ void add_pair(float& a0, float& a1, float b0, float b1) {
+    asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tadd.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}"
+        : "+f"(a0), "+f"(a1)
+        : "f"(b0), "f"(b1));
+}
+// (x0, x1) -> packed hi and lo words, bit for bit as in Pack8::to_planes_cvt: both remainders by one fused pair
+// operation (hi * -1 + x is exact)
+__device__ __forceinline__ void split_pair(float x0, float x1, uint32_t& h, uint32_t& l) {
+    const __nv_bfloat162 hh = __floats2bfloat162_rn(x0, x1);
+    h = *reinterpret_cast<const uint32_t*>(&hh);
+    float f0 = __uint_as_float(h << 16), f1 = __uint_as_float(h & 0xFFFF0000u);
+    asm("{\n\t.reg .b64 f, x, m;\n\tmov.b64 f, {%0, %1};\n\tmov.b64 x, {%2, %3};\n\tmov.b64 m, {%4, %4};\n\t"
+        "fma.rn.f32x2 f, f, m, x;\n\tmov.b64 {%0, %1}, f;\n\t}"
+        : "+f"(f0), "+f"(f1)
+        : "f"(x0), "f"(x1), "f"(-1.f));
+    const __nv_bfloat162 ll = __floats2bfloat162_rn(f0, f1);
+    l = *reinterpret_cast<const uint32_t*>(&ll);
+}
+// 0xFFFF in each half whose bf16 number is > 0
+__device__ __forceinline__ uint32_t positive_halves(uint32_t w) {
+    const __nv_bfloat162 z = __floats2bfloat162_rn(0.f, 0.f);
+    return __hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&w), z);
+}
 // Eight consecutive elements (16 bytes per plane); a 32-bit word holds elements 2i (low half) and 2i+1.
 struct Pack8 {
     float v[8];
