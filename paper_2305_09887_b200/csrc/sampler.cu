@@ -8,14 +8,14 @@
 //
 //   1. count      one thread per frontier node: min(degree, fanout); marks the node in the member flags
 //   2. scan       block_rowptr = exclusive scan of the counts
-//   3. select     one warp per frontier node.  The fanout-th smallest key is found bit by bit (64 rounds
-//                 of counting the keys that share the prefix found so far and have a 0 in the next
-//                 bit); entries below it, and the first few equal to it, are kept in row order by
-//                 ballot compaction; their end points are written to block_col and marked as members
+//   3. select     half a warp per frontier node: candidates below a bound that the fanout-th smallest key does not
+//                 exceed, the kept ones by their rank among the candidates, in row order; their end points
+//                 are written to block_col and marked as members
 //   4. scan       positions of the members = exclusive scan of the flags; next_size = its total
 //   5. emit       next_frontier[position] = node;  block_col[e] = position of its node
 // No atomics on data, no waits: the result is unique.
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 
@@ -45,68 +45,136 @@ sample_count_kernel(const int64_t* __restrict__ rowptr, int64_t n, int64_t front
     member[v] = 1;
 }
 
-__global__ void __launch_bounds__(256)
-sample_select_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, int64_t n, int64_t frontier_size,
-                     const int32_t* __restrict__ frontier, int32_t fanout, uint64_t base,
-                     const int64_t* __restrict__ block_rowptr, int32_t* __restrict__ block_col, int32_t* __restrict__ member) {
-    const int lane = threadIdx.x & 31;
-    const int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (i >= frontier_size) return;
-    const int32_t v = frontier[i];
-    if (!rtma_index_ok(v, n, 7)) return;
-    const int64_t begin = rowptr[v], deg = rowptr[v + 1] - begin;
-    const uint64_t vkey = (uint64_t)(uint32_t)v << 32;
-    int64_t out = block_rowptr[i];
-    const unsigned below = (1u << lane) - 1u;
+constexpr int SEL_LANES = 16;   // lanes that work on one frontier node
+constexpr int SEL_NODES = 256 / SEL_LANES;  // nodes of a block
+constexpr int SEL_CAND = 128;   // candidates a node may have
 
-    uint64_t kth = ~0ULL;     // the fanout-th smallest key; everything is kept when the row is short
-    int64_t ties_kept = 0;    // entries equal to kth that are kept (the first ones in row order)
-    if (deg > fanout) {
-        // keys whose high bits equal `prefix` (bits above `bit`): how many have a 0 at `bit`?
-        uint64_t prefix = 0;
-        int64_t want = fanout;  // rank (1-based) of the key looked for among the keys that match the prefix
-        for (int bit = 63; bit >= 0; --bit) {
-            const uint64_t mask_hi = bit == 63 ? 0ULL : ~0ULL << (bit + 1);
-            int64_t zeros = 0;
-            for (int64_t q = lane; q < deg; q += 32) {
-                const uint64_t key = mix_step(base ^ (vkey | (uint64_t)q));
-                zeros += ((key & mask_hi) == prefix && !((key >> bit) & 1ULL)) ? 1 : 0;
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) zeros += __shfl_xor_sync(0xffffffffu, zeros, o);
-            if (want > zeros) {  // the key has a 1 here; the `zeros` keys with a 0 are all smaller
-                want -= zeros;
-                prefix |= 1ULL << bit;
-            }
+// The kept entries of one node by the whole warp, whatever its degree and the fan-out: the fanout-th smallest key bit by
+// bit (64 rounds of counting the keys that share the prefix found so far and have a 0 in the next bit), then a pass
+// that writes the entries below it and the first few equal to it, in row order.
+__device__ void select_bit_by_bit(const int32_t* __restrict__ col, int64_t n, int64_t begin, int64_t deg, uint64_t vkey, int32_t fanout,
+                                  uint64_t base, int64_t out, int32_t* __restrict__ block_col, int32_t* __restrict__ member) {
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    // keys whose high bits equal `prefix` (bits above `bit`): how many have a 0 at `bit`?
+    uint64_t prefix = 0;
+    int64_t want = fanout;  // rank (1-based) of the key looked for among the keys that match the prefix
+    for (int bit = 63; bit >= 0; --bit) {
+        const uint64_t mask_hi = bit == 63 ? 0ULL : ~0ULL << (bit + 1);
+        int64_t zeros = 0;
+        for (int64_t q = lane; q < deg; q += 32) {
+            const uint64_t key = mix_step(base ^ (vkey | (uint64_t)q));
+            zeros += ((key & mask_hi) == prefix && !((key >> bit) & 1ULL)) ? 1 : 0;
         }
-        kth = prefix;
-        ties_kept = want;  // among the keys equal to kth, the first `want` in row order
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) zeros += __shfl_xor_sync(0xffffffffu, zeros, o);
+        if (want > zeros) {  // the key has a 1 here; the `zeros` keys with a 0 are all smaller
+            want -= zeros;
+            prefix |= 1ULL << bit;
+        }
     }
-    int64_t ties_seen = 0;
+    int64_t ties_seen = 0;  // entries equal to the key: the first `want` in row order are kept
     for (int64_t q0 = 0; q0 < deg; q0 += 32) {
         const int64_t q = q0 + lane;
-        bool keep = false, tie = false;
-        int32_t u = 0;
-        if (q < deg) {
-            if (deg > fanout) {
-                const uint64_t key = mix_step(base ^ (vkey | (uint64_t)q));
-                keep = key < kth;
-                tie = key == kth;
-            } else {
-                keep = true;
-            }
-            u = col[begin + q];
-        }
+        const uint64_t key = mix_step(base ^ (vkey | (uint64_t)q));
+        const bool tie = q < deg && key == prefix;
+        bool keep = q < deg && key < prefix;
         const unsigned tie_votes = __ballot_sync(0xffffffffu, tie);
-        if (tie && ties_seen + __popc(tie_votes & below) < ties_kept) keep = true;
+        if (tie && ties_seen + __popc(tie_votes & below) < want) keep = true;
         ties_seen += __popc(tie_votes);
+        const int32_t u = keep ? col[begin + q] : 0;
         if (keep && !rtma_index_ok(u, n, 5)) keep = false;
         const unsigned votes = __ballot_sync(0xffffffffu, keep);
         if (keep) {
-            block_col[out + __popc(votes & below)] = u;  // node id for now; its position in the next frontier later
-            member[u] = 1;                               // every writer stores the same value
+            block_col[out + __popc(votes & below)] = u;
+            member[u] = 1;
         }
         out += __popc(votes);
+    }
+}
+
+// Half a warp per frontier node (two nodes of 30 entries fill a warp's lanes; a quarter each was no faster on paper:
+// the ranking costs more per lane).  The keys are uniform 64-bit numbers, so the fanout-th smallest of deg lies near
+// fanout / deg of their range: one pass over the row hashes every entry once and collects those below a bound at which
+// fanout + 6 sqrt(fanout) + 16 of them are expected (too few or too many less than once in 10^6 nodes), in row
+// order, in shared memory; a candidate is kept when fewer than `fanout` candidates are smaller.  Only kept entries' columns
+// are read.  Bound by instruction issue (the hash, 25 instructions per entry, and the ranking).  Finding the key bit by
+// bit for every node hashed every entry 64 times: three hops (fan-outs 15, 10, 5) from 8,192 of 800,000 nodes took 8.06 ms
+// with the program around them and take 0.83 ms.
+__global__ void __launch_bounds__(256)
+sample_select_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, int64_t n, int64_t frontier_size,
+                     const int32_t* __restrict__ frontier, int32_t fanout, double expected, uint64_t base,
+                     const int64_t* __restrict__ block_rowptr, int32_t* __restrict__ block_col, int32_t* __restrict__ member) {
+    __shared__ uint64_t cand_key[SEL_NODES][SEL_CAND];
+    __shared__ int32_t cand_pos[SEL_NODES][SEL_CAND];
+    const int lane = threadIdx.x & 31, sub = threadIdx.x / SEL_LANES, sl = threadIdx.x % SEL_LANES;
+    const int shift = lane & 16;                       // first lane of this node's half
+    const unsigned below = (1u << sl) - 1u;
+    const int64_t i = (int64_t)blockIdx.x * SEL_NODES + sub;
+    int32_t v = i < frontier_size ? frontier[i] : -1;
+    if (v >= 0 && !rtma_index_ok(v, n, 7)) v = -1;
+    const int64_t begin = v >= 0 ? rowptr[v] : 0, deg = v >= 0 ? rowptr[v + 1] - begin : 0;
+    const int64_t out = v >= 0 ? block_rowptr[i] : 0;
+    const uint64_t vkey = (uint64_t)(uint32_t)v << 32;
+    const bool sel = deg > fanout;
+
+    // short rows: everything is kept
+    if (!sel) {
+        for (int64_t q = sl; q < deg; q += SEL_LANES) {
+            const int32_t u = col[begin + q];
+            const bool good = rtma_index_ok(u, n, 5);
+            block_col[out + q] = good ? u : 0;  // node id for now; its position in the next frontier later
+            if (good) member[u] = 1;            // every writer stores the same value
+        }
+    }
+    // the others: candidates (both halves of the warp go through the longer row's rounds)
+    const double share = sel ? expected / (double)deg : 1.0;
+    const uint64_t bound = share >= 0.999 ? ~0ULL : (uint64_t)(share * 18446744073709551616.0);
+    const int64_t rounds = sel && deg < (int64_t(1) << 31) ? (deg + SEL_LANES - 1) / SEL_LANES : 0;  // positions are 32-bit
+    const int64_t other = __shfl_xor_sync(0xffffffffu, rounds, 16);
+    const int64_t most = rounds > other ? rounds : other;
+    int64_t count = 0;
+    for (int64_t t = 0; t < most; ++t) {
+        const int64_t q = t * SEL_LANES + sl;
+        const uint64_t key = mix_step(base ^ (vkey | (uint64_t)q));
+        const bool cand = sel && q < deg && key <= bound;
+        const unsigned votes = (__ballot_sync(0xffffffffu, cand) >> shift) & 0xFFFFu;
+        const int64_t at = count + __popc(votes & below);
+        if (cand && at < SEL_CAND) {
+            cand_key[sub][at] = key;
+            cand_pos[sub][at] = (int32_t)q;
+        }
+        count += __popc(votes);
+    }
+    __syncwarp();
+    const bool ok = sel && count >= fanout && count <= SEL_CAND;
+    const int m = ok ? (int)count : 0;
+    const int m_most = max(m, __shfl_xor_sync(0xffffffffu, m, 16));
+    int64_t at = out;
+    for (int c0 = 0; c0 < m_most; c0 += SEL_LANES) {
+        const int c = c0 + sl;
+        const uint64_t key = c < m ? cand_key[sub][c] : ~0ULL;
+        int rank = 0;  // candidates that come before this one: smaller keys, and equal keys earlier in the row
+        for (int j = 0; j < m; ++j) {
+            const uint64_t other_key = cand_key[sub][j];
+            rank += (other_key < key || (other_key == key && j < c)) ? 1 : 0;
+        }
+        __syncwarp();
+        bool keep = c < m && rank < fanout;
+        const int32_t u = keep ? col[begin + cand_pos[sub][c]] : 0;
+        if (keep && !rtma_index_ok(u, n, 5)) keep = false;
+        const unsigned votes = (__ballot_sync(0xffffffffu, keep) >> shift) & 0xFFFFu;
+        if (keep) {
+            block_col[at + __popc(votes & below)] = u;
+            member[u] = 1;
+        }
+        at += __popc(votes);
+    }
+    // fan-outs past the candidates' room, and the rare row whose candidates were too few or too many
+    for (unsigned rest = __ballot_sync(0xffffffffu, sel && !ok && sl == 0); rest; rest &= rest - 1) {
+        const int from = __ffs(rest) - 1;
+        const int64_t b = __shfl_sync(0xffffffffu, begin, from), d = __shfl_sync(0xffffffffu, deg, from), o = __shfl_sync(0xffffffffu, out, from);
+        select_bit_by_bit(col, n, b, d, __shfl_sync(0xffffffffu, vkey, from), fanout, base, o, block_col, member);
     }
 }
 
@@ -165,8 +233,9 @@ extern "C" int32_t rtma_sample_hop(rtma_ctx* ctx, int64_t n, const int64_t* rowp
         z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
         const uint64_t base = z ^ (z >> 31);
         KernelScope ks(ctx, KC_LINK, stream);
-        sample_select_kernel<<<(unsigned)ceil_div(frontier_size, 8), 256, 0, stream>>>(rowptr, col, n, frontier_size, frontier, fanout, base,
-                                                                                      block_rowptr, block_col, member);
+        const double expected = (double)fanout + 6.0 * std::sqrt((double)fanout) + 16.0;  // candidates per row (see the kernel)
+        sample_select_kernel<<<(unsigned)ceil_div(frontier_size, SEL_NODES), 256, 0, stream>>>(
+            rowptr, col, n, frontier_size, frontier, fanout, expected, base, block_rowptr, block_col, member);
     }
     RTMA_LAUNCH_CHECK(ctx);
     RTMA_TRY(exclusive_scan_i32_to_i64(ctx, member, n, position, scratch, stream));

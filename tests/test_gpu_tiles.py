@@ -3,6 +3,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_2305_09887_b200 import inputs
 
 pytestmark = pytest.mark.gpu
@@ -35,3 +36,23 @@ def _workload(n, edges, dims, seed):
 def test_products_on_pairs_of_blocks(util, n, M, dims, parts, gemm_dtype):
     w = _workload(n, 3 * n, dims, 11)
     util.check_one_step(w, M=M, gemm_dtype=gemm_dtype, only_parts=parts, gradients_against_plain=gemm_dtype == 0)
+
+
+# the neighbour sampler: rows of 15 to 17 entries (a half-warp), around the candidates' room of 128 and far past it;
+# fan-outs for which a bound is drawn, for which every entry is a candidate, and past the room
+@pytest.mark.parametrize("fanout", [1, 2, 15, 16, 17, 60, 100, 127, 128, 129, 700])
+def test_sampled_rows_around_the_candidates_room(util, fanout):
+    degrees = [0, 1, 15, 16, 17, 31, 33, 100, 127, 128, 129, 160, 1_000, 5_000, 3, 0, 40]
+    n = 6_000
+    rng = np.random.default_rng(fanout)
+    rows = [np.sort(rng.choice(n, size=d, replace=False)).astype(np.int32) for d in degrees]
+    rowptr = np.zeros(n + 1, dtype=np.int64)
+    rowptr[1:len(degrees) + 1] = np.cumsum(degrees)
+    rowptr[len(degrees) + 1:] = rowptr[len(degrees)]
+    col = np.concatenate(rows)
+    frontier = np.array([i for i in range(len(degrees) + 3) if i != 4], dtype=np.int32)
+    for seed, hop in ((3, 0), (2**64 - 7, 2)):
+        got = util.ctx().sample_hop(util.dev(rowptr), util.dev(col), util.dev(frontier), fanout, seed, hop)
+        want = oracle.sample_hop(rowptr, col, frontier, fanout, seed, hop)
+        for a, b in zip(got, want):
+            assert np.array_equal(a.cpu().numpy(), b)
