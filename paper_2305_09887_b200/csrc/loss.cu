@@ -302,9 +302,9 @@ softmax_xent_wide_kernel(const __grid_constant__ GroupDesc g, const Mat logits, 
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         const float lse = zmax + logf(sum);
         if (lane == 0) loss += lse - z[label];
-        for (int c = lane; c < C; c += 32) {
+        for (int c = lane; c < (int)dZ.ld; c += 32) {  // the padding columns are written as zeros
             __nv_bfloat16 h, l;
-            split_bf16((expf(z[c] - lse) - (c == label ? 1.f : 0.f)) * inv_n, h, l);
+            split_bf16(c < C ? (expf(z[c] - lse) - (c == label ? 1.f : 0.f)) * inv_n : 0.f, h, l);
             dZ.hi[r * dZ.ld + c] = h;
             dZ.lo[r * dZ.ld + c] = l;
         }

@@ -437,11 +437,12 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
             __nv_bfloat16* q_lo = plan.q_width ? cur.take<__nv_bfloat16>((size_t)rows * planes_ld(plan.q_width) + 8) : nullptr;
             float* partial = cur.take<float>((size_t)slots * plan.max_layer_params + 4);
             float* tile_loss = cur.take<float>((size_t)loss_tiles(g) + 4);
+            const size_t counters_at = cur.used;  // from here to counters_end: zero on entry
             int* ticket = cur.take<int>(64);  // work counter of the aggregation kernels (zero between launches)
             unsigned long long* dense_counts = cur.take<unsigned long long>(3 * RTMA_MAX_PARTS);
             int* dense_flags = cur.take<int>(RTMA_MAX_PARTS);  // per trainer: aggregated on the tensor cores
             unsigned long long* sym_sums = cur.take<unsigned long long>(4);
-            const size_t zero_bytes = cur.used;  // everything above starts from zero: rows between parts stay zero
+            const size_t counters_end = cur.used;
             int* heavy_list = cur.take<int>((size_t)spmm_order_entries(g) + 4);
             // entries outside the window of a row's tile, for the parts aggregated on the tensor cores
             unsigned long long* win_bits = cur.take<unsigned long long>((size_t)rows * (DENSE_WINDOW / 64) + 2);
@@ -475,7 +476,33 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                 return rtma_fail(ctx, RTMA_ERR_WORKSPACE, "internal: wave needs %zu bytes, share is %zu", cur.used, share);
             if (rows == 0) continue;
 
-            RTMA_CUDA(ctx, cudaMemsetAsync(ctx->arena + gi * share, 0, zero_bytes, s));
+            // the rows between the parts of every matrix that a tile may read past a part's end
+            {
+                Planes mats[CLEAR_MAX];
+                int count = 0;
+                for (int l = 0; l < m.L; ++l) {
+                    mats[count++] = Hl[l];
+                    if (Nl[l].hi) mats[count++] = Nl[l];
+                    if (l < m.L - 1 && m.post) mats[count++] = Zl[l];
+                }
+                if (link) mats[count++] = R;
+                if (head) {
+                    mats[count++] = T;
+                    mats[count++] = NT;
+                    mats[count++] = DQ;
+                } else {
+                    mats[count++] = dZlast;
+                }
+                RTMA_TRY(launch_clear_gaps(ctx, g, mats, count, ticket, (int)((counters_end - counters_at) / sizeof(int)), s));
+                if (link && prows > 0) {
+                    count = 0;
+                    for (int k = 0; k < m.Kd; ++k) {
+                        mats[count++] = El[k];
+                        mats[count++] = ZDl[k];
+                    }
+                    RTMA_TRY(launch_clear_gaps(ctx, gd, mats, count, nullptr, 0, s));
+                }
+            }
             if (m.gcn) RTMA_TRY(launch_gcn_scale(ctx, g, rowptr_out, inv_deg, s));  // (deg + 1)^-1/2 in the same array
             else RTMA_TRY(launch_inv_degree(ctx, g, rowptr_out, inv_deg, s));
             RTMA_TRY(launch_symmetry_check(ctx, g, rowptr_out, col_out, sym_sums, s));

@@ -77,6 +77,11 @@ int32_t launch_to_planes(rtma_ctx* ctx, const GroupDesc& g, const float* X, cons
                          Planes out, cudaStream_t s);
 // Split planes -> dense fp32 [rows x d] (verification taps).
 int32_t launch_from_planes(rtma_ctx* ctx, Planes src, int64_t first_row, int64_t rows, int d, float* dst, cudaStream_t s);
+// Zeros the rows between the parts of every listed matrix (addressed by g's scratch rows), and `words` 32-bit words at
+// `counters` (NULL: none).  What the kernels write covers a part's rows and their padding columns; the rows between the
+// parts are read as zeros by the tiles that run past a part's end.
+constexpr int CLEAR_MAX = 40;
+int32_t launch_clear_gaps(rtma_ctx* ctx, const GroupDesc& g, const Planes* mats, int count, int* counters, int words, cudaStream_t s);
 // inv_deg[row_ws + i] = 1 / local degree (0 for an isolated node).
 int32_t launch_inv_degree(rtma_ctx* ctx, const GroupDesc& g, const int64_t* rowptr_out, float* inv_deg, cudaStream_t s);
 // Raises the context's "not symmetric" flag (reported by rtma_check) unless every entry (u, v) of every

@@ -56,3 +56,31 @@ def test_sampled_rows_around_the_candidates_room(util, fanout):
         want = oracle.sample_hop(rowptr, col, frontier, fanout, seed, hop)
         for a, b in zip(got, want):
             assert np.array_equal(a.cpu().numpy(), b)
+
+
+# the scratch a call finds holds whatever the calls before it left there: here the NaNs of a wider model on other parts
+@pytest.mark.parametrize("dims, variant", [((20, 40, 131), (0, 0, 0)), ((33, 90, 70, 3), (0, 0, 0)), ((20, 36, 36, 5), (1, 1, 1)),
+                                           ((24, 33), (0, 0, 0))])
+def test_scratch_left_by_another_call_does_not_matter(util, dims, variant):
+    from paper_2305_09887_b200 import binding
+    w = _workload(2_000, 9_000, dims, 21)
+    params0 = inputs.variant_params(variant, dims, 4)
+    pre = util.gpu_preprocess(w, M=7)
+    other = _workload(2_000, 9_000, (64, 300, 300, 9), 22)
+    pre_other = util.gpu_preprocess(other, M=3)
+
+    def steps(c):
+        params = util.dev(np.tile(params0, (7, 1)))
+        loss = torch.zeros(7, 3, device="cuda")
+        c.local_steps(dims, 0.05, 7, pre["part_host"], pre["edge_host"], pre["rowptr_out"], pre["col_out"], pre["Xp"], pre["yp"],
+                      params, 3, loss_out=loss, variant=variant)
+        torch.cuda.synchronize()
+        return params, loss
+
+    clean = steps(binding.Context(0))
+    c = binding.Context(0)
+    nan = torch.full_like(pre_other["Xp"], float("nan"))
+    c.local_steps(other.dims, 0.05, 3, pre_other["part_host"], pre_other["edge_host"], pre_other["rowptr_out"], pre_other["col_out"],
+                  nan, pre_other["yp"], util.dev(np.tile(other.params0, (3, 1))), 2)
+    after = steps(c)
+    assert torch.isfinite(clean[0]).all() and torch.equal(clean[0], after[0]) and torch.equal(clean[1], after[1])
