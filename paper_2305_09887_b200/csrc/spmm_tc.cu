@@ -41,6 +41,7 @@ constexpr int DT_BM = DENSE_TILE_ROWS;           // rows of a tile
 constexpr int DT_BK = 64;                        // window rows per pipeline stage
 constexpr int DT_HALO = DENSE_HALO;              // window rows before the tile, and after it
 constexpr int DT_KB = DENSE_WINDOW / DT_BK;
+static_assert(DT_KB <= 8 && GROUP_ROW_ALIGN % 32 == 0, "a byte holds the blocks of a window, 32 rows lie in one part");
 constexpr int DT_A_BYTES = DT_BM * 128;          // one plane of A for one stage: 16 KB
 constexpr int DT_ATOM_BYTES = DT_BK * 128;       // 64 source rows x 64 columns of one plane: 8 KB
 constexpr int DT_STAGING_BYTES = 4096;           // per epilogue warp
@@ -67,6 +68,7 @@ struct DenseArgs {
     const float* inv_deg;
     const int* dense;              // per trainer: 1 = this part is aggregated here
     const unsigned long long* win_bits;  // [scratch row][DT_KB]: bit c of word b = the row has window column 64 b + c
+    const unsigned char* block_mask;  // per 32 scratch rows: the window blocks in which one of them has an entry
     const unsigned char* left_cnt; // per scratch row: entries outside the window (DT_OVERFLOW: more than DT_LCAP);
                                    // where it is not 0 the output row holds their sum when the kernel starts
     CUtensorMap mapSh, mapSl;      // source planes, boxes of 64 columns x DT_BK rows
@@ -119,11 +121,15 @@ __device__ __forceinline__ void tmem_load_32x16(uint32_t taddr, float (&v)[16]) 
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// the stages of a tile: window blocks that overlap the part's rows
-__device__ __forceinline__ void tile_blocks(int r0, int n_p, int* kb_first, int* kb_end) {
-    const int w0 = r0 - DT_HALO;
-    *kb_first = w0 < 0 ? (-w0) / DT_BK : 0;
-    *kb_end = min(DT_KB, (n_p - w0 + DT_BK - 1) / DT_BK);
+// The stages of a tile: bit b = some row of the tile has an entry in window block b (of 100-member super-nodes kept
+// together, 4.7 of 6 on average; the blocks left out cost 64 source rows through shared memory and an MMA of zeros each).
+// A tile without any takes the block of its own first rows, so that its accumulator is written.
+__device__ __forceinline__ uint32_t tile_blocks(const unsigned char* block_mask, int64_t ws, int r0, int n_p) {
+    uint32_t m = 0;
+#pragma unroll
+    for (int j = 0; j < DT_BM / 32; ++j)
+        if (r0 + 32 * j < n_p) m |= __ldg(block_mask + (ws + r0) / 32 + j);
+    return m ? m : 1u << (DT_HALO / DT_BK);
 }
 
 // TRANSPOSED = false: A counts, out = (1 / deg v) * A src;  true: A = counts x 1 / deg u, out = A src
@@ -192,14 +198,13 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
                 const bool joined = NA <= 2;
                 const uint32_t idesc_both = tc::idesc_bf16(DT_BM, 128 * NA, false, true);
                 const uint32_t idesc_hi = tc::idesc_bf16(DT_BM, 64 * NA, false, true);
-                int kb_first, kb_end;
-                tile_blocks(r0, a.g.rows[k], &kb_first, &kb_end);
+                const uint32_t blocks = tile_blocks(a.block_mask, a.g.row_ws[k], r0, a.g.rows[k]);
                 const int buf = (int)(t & 1);
                 ok = dense_wait(&pb.acc_empty[buf], (uint32_t)((t >> 1) & 1) ^ 1u, &pb, a.error_word);
                 if (!ok) break;
                 tc::tc_fence_after_sync();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * a.tmem_cols);
-                for (int kb = kb_first; kb < kb_end; ++kb, ++it) {
+                for (uint32_t rest = blocks; rest; rest &= rest - 1, ++it) {
                     const int s = (int)(it % stages);
                     ok = dense_wait(&pb.full[s], (uint32_t)((it / stages) & 1), &pb, a.error_word);
                     if (!ok) break;
@@ -212,7 +217,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
                         const uint64_t dah = tc::smem_desc_sw128(ah + ks * 32, 16, 1024);
                         const uint64_t db = tc::smem_desc_sw128(bh + ks * 2048, DT_ATOM_BYTES, 1024);
                         const uint64_t dbl = tc::smem_desc_sw128(bh + NA * DT_ATOM_BYTES + ks * 2048, DT_ATOM_BYTES, 1024);
-                        const uint32_t first = (kb > kb_first || ks > 0) ? 1u : 0u;
+                        const uint32_t first = (rest != blocks || ks > 0) ? 1u : 0u;
                         if (joined) {
                             tc::mma_bf16(d_tmem, dah, db, idesc_both, first);
                         } else {
@@ -251,9 +256,8 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
             const int n_p = a.g.rows[k];
             const int ct = (int)(tile % n_ct);
             const int NA = min(DT_TILE_ATOMS, a.n_atoms - DT_TILE_ATOMS * ct);
-            int kb_first, kb_end;
-            tile_blocks(r0, n_p, &kb_first, &kb_end);
             const int64_t ws = a.g.row_ws[k];
+            const uint32_t blocks = tile_blocks(a.block_mask, ws, r0, n_p);
             unsigned long long bits[DT_KB];
             if (r0 + r < n_p) {
                 const ulonglong2* wb = reinterpret_cast<const ulonglong2*>(a.win_bits + (ws + r0 + r) * DT_KB);
@@ -282,7 +286,8 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
                 ok = meet();
                 if (!ok) break;
             }
-            for (int kb = kb_first; kb < kb_end; ++kb, ++it) {
+            for (uint32_t rest = blocks; rest; rest &= rest - 1, ++it) {
+                const int kb = __ffs(rest) - 1;
                 const int s = (int)(it % stages);
                 ok = dense_wait(&pb.empty[s], (uint32_t)((it / stages) & 1) ^ 1u, &pb, a.error_word);
                 if (!ok) break;
@@ -651,12 +656,13 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
 __global__ void __launch_bounds__(256)
 dense_lists_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict__ rowptr_out,
                    const int32_t* __restrict__ col_out, int* __restrict__ dense,
-                   unsigned long long* __restrict__ win_bits, unsigned char* __restrict__ left_cnt,
-                   int32_t* __restrict__ left_col) {
+                   unsigned long long* __restrict__ win_bits, unsigned char* __restrict__ block_mask,
+                   unsigned char* __restrict__ left_cnt, int32_t* __restrict__ left_col) {
     int k, r0;
     if (!locate_tile(g, 256, blockIdx.x, &k, &r0)) return;
     const int i = r0 + threadIdx.x;
-    if (i >= g.rows[k] || !*reinterpret_cast<volatile int*>(dense + g.part[k])) return;
+    if (!__any_sync(0xffffffffu, i < g.rows[k] && *reinterpret_cast<volatile int*>(dense + g.part[k]))) return;
+    const bool live = i < g.rows[k];
     const int64_t* rp = rowptr_out + g.row_abs[k] + g.part[k];
     const int32_t* cols = col_out + g.edge_abs[k];
     const int64_t row = g.row_ws[k] + i;
@@ -666,7 +672,8 @@ dense_lists_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restric
     for (int q = 0; q < DT_KB; ++q) bits[q] = 0ULL;
     bool repeated = false;
     int cnt = 0;
-    for (int64_t e = rp[i]; e < rp[i + 1]; ++e) {
+    const int64_t e_end = live ? rp[i + 1] : 0;
+    for (int64_t e = live ? rp[i] : 0; e < e_end; ++e) {
         const int c = cols[e];
         if (!rtma_index_ok(c, g.rows[k], 5)) continue;
         if (c >= w_begin && c < w_end) {
@@ -684,6 +691,13 @@ dense_lists_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restric
             ++cnt;
         }
     }
+    __syncwarp();
+    uint32_t blocks = 0;
+#pragma unroll
+    for (int q = 0; q < DT_KB; ++q) blocks |= bits[q] ? 1u << q : 0u;
+    blocks = __reduce_or_sync(0xffffffffu, blocks);
+    if (!live) return;
+    if ((threadIdx.x & 31) == 0) block_mask[row / 32] = (unsigned char)blocks;  // parts start at multiples of 64 scratch rows
 #pragma unroll
     for (int q = 0; q < DT_KB; ++q) win_bits[row * DT_KB + q] = bits[q];
     left_cnt[row] = cnt <= DT_LCAP ? (unsigned char)cnt : DT_OVERFLOW;
@@ -755,11 +769,11 @@ int32_t launch_dense_probe(rtma_ctx* ctx, const GroupDesc& g, const int64_t* row
 }
 
 int32_t launch_dense_lists(rtma_ctx* ctx, const GroupDesc& g, const int64_t* rowptr_out, const int32_t* col_out,
-                           int* dense, unsigned long long* win_bits, unsigned char* left_cnt, int32_t* left_col,
-                           cudaStream_t s) {
+                           int* dense, unsigned long long* win_bits, unsigned char* block_mask, unsigned char* left_cnt,
+                           int32_t* left_col, cudaStream_t s) {
     const int64_t tiles = group_tiles(g, 256);
     if (tiles == 0) return RTMA_OK;
-    { KernelScope ks(ctx, KC_INV_DEGREE, s); dense_lists_kernel<<<(unsigned)tiles, 256, 0, s>>>(g, rowptr_out, col_out, dense, win_bits, left_cnt, left_col); }
+    { KernelScope ks(ctx, KC_INV_DEGREE, s); dense_lists_kernel<<<(unsigned)tiles, 256, 0, s>>>(g, rowptr_out, col_out, dense, win_bits, block_mask, left_cnt, left_col); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }
@@ -785,6 +799,7 @@ int32_t launch_spmm_dense(rtma_ctx* ctx, int kclass, const GroupDesc& g, const i
     a.inv_deg = inv_deg;
     a.dense = dense;
     a.win_bits = order.win_bits;
+    a.block_mask = order.block_mask;
     a.left_cnt = order.left_cnt;
     a.out = out;
     a.width = (int)planes_ld(d);

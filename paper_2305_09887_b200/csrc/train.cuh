@@ -103,6 +103,8 @@ struct SpmmOrder {
                                     // (255: more than DENSE_LEFT_CAP), and their columns [row][DENSE_LEFT_CAP]
     const int32_t* left_col;
     const unsigned long long* win_bits;  // device, per scratch row of such a part: its window as DENSE_WINDOW bits
+    const unsigned char* block_mask;     // device, per 32 scratch rows of such a part: bit b = one of them has an entry in
+                                         // its window's 64-row block b
     bool all_dense;          // host: every part of the wave is flagged, the gather kernels have nothing to do
 };
 // list: spmm_order_entries(g) ints; count: 8 ints (16-byte aligned), zero on entry: the number of listed
@@ -136,11 +138,12 @@ int32_t launch_dense_probe(rtma_ctx* ctx, const GroupDesc& g, const int64_t* row
                            int mode, unsigned long long* counts, int* dense, cudaStream_t s);
 // Once per call, after launch_dense_probe, for every row of the flagged parts: the window as a bit mask and the
 // entries outside it.  win_bits: DENSE_WINDOW / 64 words per scratch row (16-byte aligned); left_cnt: one byte
-// per scratch row; left_col: DENSE_LEFT_CAP ints per scratch row (16-byte aligned).  Clears the flag of a
+// per scratch row; left_col: DENSE_LEFT_CAP ints per scratch row (16-byte aligned); block_mask: one byte per 32
+// scratch rows.  Clears the flag of a
 // part in which a row repeats an entry inside its window.
 int32_t launch_dense_lists(rtma_ctx* ctx, const GroupDesc& g, const int64_t* rowptr_out, const int32_t* col_out,
-                           int* dense, unsigned long long* win_bits, unsigned char* left_cnt, int32_t* left_col,
-                           cudaStream_t s);
+                           int* dense, unsigned long long* win_bits, unsigned char* block_mask, unsigned char* left_cnt,
+                           int32_t* left_col, cudaStream_t s);
 // The parts of g flagged in order.dense: out = Abar src (transposed: Abar^T src on a symmetric part), window
 // entries by tensor-core tiles, the others summed into the output rows beforehand by a gather pass.  Other
 // parts are left alone.

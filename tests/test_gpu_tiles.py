@@ -84,3 +84,16 @@ def test_scratch_left_by_another_call_does_not_matter(util, dims, variant):
                   nan, pre_other["yp"], util.dev(np.tile(other.params0, (3, 1))), 2)
     after = steps(c)
     assert torch.isfinite(clean[0]).all() and torch.equal(clean[0], after[0]) and torch.equal(clean[1], after[1])
+
+
+# tensor-core aggregation forced: tiles without any entry, with entries outside the window only, and part ends inside a
+# tile's 32-row groups
+@pytest.mark.parametrize("n, edges, M", [(500, 60, 5), (700, 1_500, 4), (2_600, 4_000, 3)])
+def test_tiles_with_empty_window_blocks(util, n, edges, M):
+    w = _workload(n, edges, (20, 70, 48, 40), 31)
+    util.ctx().set_dense_aggregation(2)
+    try:
+        got, want = util.check_one_step(w, M=M)
+        util.check_k_steps_and_average(w, got, want, 2)
+    finally:
+        util.ctx().set_dense_aggregation(1)
