@@ -594,7 +594,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
     const bool single = a.single != 0;
     const uint32_t np = single ? 1u : 2u;  // planes staged per operand
     const uint32_t stage_bytes = np * (a_plane_bytes + b_plane_bytes);
-    const uint32_t tx_bytes = np * ((uint32_t)na_tiles * a_tile_bytes + b_plane_bytes);
+    // 64-column halves of the left-operand tiles that hold columns of the matrix; the others are not loaded (what their part
+    // of shared memory holds only reaches accumulator rows that are not stored)
+    int halves[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) halves[t] = t < na_tiles ? (j0_of[t] + 64 < d_in ? 2 : 1) : 0;
+    const uint32_t tx_bytes = np * ((uint32_t)(halves[0] + halves[1]) * ATOM_BYTES + b_plane_bytes);
     auto a_hi = [&](int s) { return smem + (size_t)s * stage_bytes; };
     auto a_lo = [&](int s) { return smem + (size_t)s * stage_bytes + a_plane_bytes; };
     auto b_hi = [&](int s) { return smem + (size_t)s * stage_bytes + np * a_plane_bytes; };
@@ -632,7 +637,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
                 for (int t = 0; t < na_tiles; ++t) {
                     const CUtensorMap* mapAh = src_of[t] == 0 ? &a.mapHh : &a.mapNh;
                     const CUtensorMap* mapAl = src_of[t] == 0 ? &a.mapHl : &a.mapNl;
-                    for (int h = 0; h < 2; ++h) {
+                    for (int h = 0; h < halves[t]; ++h) {
                         tc::tma_load_2d(a_hi(s) + t * a_tile_bytes + h * ATOM_BYTES, mapAh, &pb.full[s], j0_of[t] + 64 * h, row + kb * BK);
                         if (!single)
                             tc::tma_load_2d(a_lo(s) + t * a_tile_bytes + h * ATOM_BYTES, mapAl, &pb.full[s], j0_of[t] + 64 * h, row + kb * BK);
@@ -1016,8 +1021,13 @@ int32_t launch_tc_dgrad(rtma_ctx* ctx, const GroupDesc& g, LayerShape ls, const 
     return launch_rows(ctx, a, rows_total, pairs, KC_GEMM_DGRAD, s);
 }
 
-int tc_wgrad_blocks_per_slot(const LayerShape& ls) {
-    return (int)(ceil_div(ls.nsrc * ceil_div(ls.d_in, TC_BM), 2) * ceil_div(ceil_div(ls.d_out, 64), 4));
+WgradCost tc_wgrad_cost(const LayerShape& ls, bool single) {
+    const int64_t a_tiles = ls.nsrc * ceil_div(ls.d_in, TC_BM), atoms = ceil_div(ls.d_out, 64);
+    WgradCost c;
+    c.blocks_per_slot = ceil_div(a_tiles, 2) * ceil_div(atoms, 4);
+    c.bytes_per_row = (single ? 1 : 2) * 128 * (std::min<int64_t>(a_tiles, 2) * (ls.d_in > 64 ? 2 : 1) + std::min<int64_t>(atoms, 4));
+    c.params = (int64_t)(ls.nsrc * ls.d_in + 1) * ls.d_out;
+    return c;
 }
 
 int32_t launch_tc_wgrad(rtma_ctx* ctx, const GroupDesc& g, const SplitPlan& sp, LayerShape ls, int64_t rows_total,

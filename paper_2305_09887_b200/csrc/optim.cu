@@ -18,7 +18,9 @@ reduce_sgd_kernel(const __grid_constant__ GroupDesc g, const __grid_constant__ S
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= count) return;
     float gsum = 0.f;
-    for (int s = sp.split_begin[k]; s < sp.split_begin[k + 1]; ++s) gsum += partial[(int64_t)s * stride + i];
+    const int s_end = sp.split_begin[k + 1];
+#pragma unroll 8
+    for (int s = sp.split_begin[k]; s < s_end; ++s) gsum += __ldcs(partial + (int64_t)s * stride + i);  // eight loads in flight
     const int64_t at = (int64_t)g.part[k] * ls.P + ls.param_offset + i;
     if (grads_record) grads_record[at] = gsum;
     params[at] -= lr * gsum;
@@ -40,7 +42,9 @@ reduce_sgd_head_kernel(const __grid_constant__ GroupDesc g, const __grid_constan
     else if (ls.nsrc == 2 && row < ls.d_in) at_partial = (int64_t)row * 2 * cp + c;   // Ws: H^T dZ
     else at_partial = (int64_t)(row - (ls.nsrc - 1) * ls.d_in) * 2 * cp + cp + c;     // Wn (or W): H^T Q
     float gsum = 0.f;
-    for (int s = sp.split_begin[k]; s < sp.split_begin[k + 1]; ++s) gsum += partial[(int64_t)s * stride + at_partial];
+    const int s_end = sp.split_begin[k + 1];
+#pragma unroll 8
+    for (int s = sp.split_begin[k]; s < s_end; ++s) gsum += __ldcs(partial + (int64_t)s * stride + at_partial);
     const int64_t at = (int64_t)g.part[k] * ls.P + ls.param_offset + i;
     if (grads_record) grads_record[at] = gsum;
     params[at] -= lr * gsum;

@@ -147,34 +147,45 @@ ScratchPlan plan_scratch(const Model& m, bool head, bool record) {
     return sp;
 }
 
-// Row chunks of the weight gradient: enough of them to give the GPU a few blocks per SM,
-// each a multiple of the row alignment.
-int splits_for(int64_t n_p, int parts_in_flight, int blocks_per_slot) {
-    // The kernel runs one block per SM at a time, so its time goes as (waves of blocks) x (rows per
-    // chunk).  Taking every part for as large as this one, pick the chunk count with the smallest such
-    // product, or the fewest chunks within 3 % of it (fewer partial sums to add up afterwards).
+// Row chunks of the weight gradient, every part taken for as large as this one.
+// At least `fewest`, the chunks (of 1024 rows or more) at which (waves of blocks) x (rows per chunk) is within 3 % of its
+// least: the tensor cores truncate when they accumulate, and with chunks 2.5 times as long the parameters of 5 M rows
+// moved by 1.3e-5 in five steps.  More than that where it is faster: a block (one per SM at a time) takes a fixed 4 us and then
+// stages its rows at about 41 bytes per ns, and every chunk adds a set of partial sums that is written and read back
+// (about 4,000 bytes per ns).  Small parts gain: 3 parts of 10,000 rows ran 30 blocks, 37 us a launch, now 120 of 256 rows.
+int splits_for(int64_t n_p, int parts_in_flight, const WgradCost& c) {
     constexpr int64_t SMS = 148;
     if (n_p <= 0) return 1;
-    const int64_t most = std::min<int64_t>(64, std::max<int64_t>(1, ceil_div(n_p, 1024)));
-    auto cost_of = [&](int64_t ns) {
-        const int64_t rows = aligned_rows(ceil_div(n_p, ns));
-        const int64_t blocks = (int64_t)parts_in_flight * ceil_div(n_p, rows) * blocks_per_slot;
-        return ceil_div(blocks, SMS) * rows;
+    auto waves_of = [&](int64_t ns, int64_t* rows, int64_t* slots) {
+        *rows = aligned_rows(ceil_div(n_p, ns));
+        *slots = (int64_t)parts_in_flight * ceil_div(n_p, *rows);
+        return ceil_div(*slots * c.blocks_per_slot, SMS);
     };
-    int64_t best_cost = INT64_MAX;
-    for (int64_t ns = 1; ns <= most; ++ns) best_cost = std::min(best_cost, cost_of(ns));
-    for (int64_t ns = 1; ns <= most; ++ns)
-        if (cost_of(ns) * 100 <= best_cost * 103) return (int)ns;
-    return (int)most;
+    auto least_within = [&](int64_t from, int64_t to, auto cost) {
+        double best = cost(from);
+        for (int64_t ns = from + 1; ns <= to; ++ns) best = std::min(best, cost(ns));
+        for (int64_t ns = from; ns < to; ++ns)
+            if (cost(ns) <= best * 1.03) return ns;
+        return to;
+    };
+    const int64_t fewest = least_within(1, std::min<int64_t>(64, std::max<int64_t>(1, ceil_div(n_p, 1024))), [&](int64_t ns) {
+        int64_t rows, slots;
+        const int64_t waves = waves_of(ns, &rows, &slots);
+        return (double)waves * (double)rows;
+    });
+    const int64_t most = std::max(fewest, std::min<int64_t>(64, ceil_div(n_p, 128)));
+    return (int)least_within(fewest, most, [&](int64_t ns) {
+        int64_t rows, slots;
+        const int64_t waves = waves_of(ns, &rows, &slots);
+        return (double)waves * (4000.0 + (double)rows * c.bytes_per_row / 41.0) + (double)slots * (double)c.params * 2.0 * sizeof(float) / 4000.0;
+    });
 }
 
-// blocks_per_slot: blocks the weight-gradient kernel launches per chunk for the layer in hand (the
-// chunks of all running parts together should come to about two blocks per SM)
-int plan_splits(const GroupDesc& g, int parts_in_flight, int blocks_per_slot, SplitPlan* sp) {
+int plan_splits(const GroupDesc& g, int parts_in_flight, const WgradCost& cost, SplitPlan* sp) {
     int slots = 0;
     for (int k = 0; k < g.num; ++k) {
         sp->split_begin[k] = slots;
-        const int nsplit = splits_for(g.rows[k], parts_in_flight, blocks_per_slot);
+        const int nsplit = splits_for(g.rows[k], parts_in_flight, cost);
         sp->rows_per_split[k] = (int32_t)std::max<int64_t>(GROUP_ROW_ALIGN, aligned_rows(ceil_div(g.rows[k], nsplit)));
         slots += (int)std::max<int64_t>(1, ceil_div(g.rows[k], sp->rows_per_split[k]));
     }
@@ -360,7 +371,7 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                     shape.nsrc = 1;
                     shape.d_out = 2 * m.Cp;
                 }
-                slots = std::max(slots, plan_splits(g, running, tc_wgrad_blocks_per_slot(shape), &wave_spl[l]));
+                slots = std::max(slots, plan_splits(g, running, tc_wgrad_cost(shape, single_pass), &wave_spl[l]));
             }
             int wave_steps = 0;
             for (int k = 0; k < g.num; ++k) wave_steps = std::max(wave_steps, steps[g.part[k]]);
@@ -426,10 +437,12 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                     El[k] = take_pair_planes(m.ddims[k]);
                     ZDl[k] = take_pair_planes(m.ddims[k + 1]);
                 }
-                int dslots = 0;  // one chunking for all decoder layers: that of the layer with the most blocks per chunk
-                int dec_bps = 1;
-                for (int k = 0; k < m.Kd; ++k) dec_bps = std::max(dec_bps, tc_wgrad_blocks_per_slot(m.dec[k]));
-                dslots = plan_splits(gd, running, dec_bps, &spd);
+                WgradCost widest{};  // one chunking for all decoder layers: that of the costliest
+                for (int k = 0; k < m.Kd; ++k) {
+                    const WgradCost c = tc_wgrad_cost(m.dec[k], single_pass);
+                    if (c.blocks_per_slot * c.bytes_per_row > widest.blocks_per_slot * widest.bytes_per_row) widest = c;
+                }
+                const int dslots = plan_splits(gd, running, widest, &spd);
                 dec_partial = cur.take<float>((size_t)dslots * plan.max_layer_params + 4);
                 dec_tile_loss = cur.take<float>((size_t)loss_tiles(gd) + 4);
             }

@@ -251,8 +251,13 @@ int32_t launch_tc_forward(rtma_ctx* ctx, const GroupDesc& g, LayerShape ls, cons
 int32_t launch_tc_dgrad(rtma_ctx* ctx, const GroupDesc& g, LayerShape ls, const TcLayerPlan& p, int64_t rows_total,
                         Planes dZ, Planes Q, const __nv_bfloat16* Bd_hi, const __nv_bfloat16* Bd_lo, Planes H, bool gate,
                         bool single, cudaStream_t s);
-// Blocks launch_tc_wgrad starts per chunk of rows for a layer of this shape.
-int tc_wgrad_blocks_per_slot(const LayerShape& ls);
+// What a chunk of rows costs launch_tc_wgrad for a layer of this shape.
+struct WgradCost {
+    int64_t blocks_per_slot;  // blocks started per chunk
+    int64_t bytes_per_row;    // that one of them stages
+    int64_t params;           // partial sums a chunk leaves
+};
+WgradCost tc_wgrad_cost(const LayerShape& ls, bool single);
 // partial[slot][(nsrc d_in + 1) x d_out] = [H | N | 1]^T dZ ([N | 1]^T dZ for a one-matrix layer)
 // over one chunk of rows.
 int32_t launch_tc_wgrad(rtma_ctx* ctx, const GroupDesc& g, const SplitPlan& sp, LayerShape ls, int64_t rows_total,

@@ -97,3 +97,12 @@ def test_tiles_with_empty_window_blocks(util, n, edges, M):
         util.check_k_steps_and_average(w, got, want, 2)
     finally:
         util.ctx().set_dense_aggregation(1)
+
+
+# weight gradient: part sizes around the 64-row steps and 128-row chunks, widths around the 64-column halves of a
+# left-operand tile (33, 64: the second half is not loaded; 65, 130: it is) and odd output widths
+@pytest.mark.parametrize("dims, n, M", [((33, 64, 65, 3), 600, 5), ((64, 130, 33, 20), 1_300, 10), ((130, 66, 5), 129, 1), ((8, 8, 8, 8), 2_111, 8)])
+def test_weight_gradient_chunks(util, dims, n, M):
+    w = _workload(n, 3 * n, dims, 41)
+    got, want = util.check_one_step(w, M=M)
+    util.check_k_steps_and_average(w, got, want, 3)
