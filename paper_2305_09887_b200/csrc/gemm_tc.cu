@@ -87,41 +87,74 @@ struct PrepBatch {
     PrepArgs job[PREP_MAX_JOBS];
 };
 
-// blockIdx.z = layer (all layers of a step are repacked by one launch), blockIdx.y = part
+// blockIdx.z = layer (all layers of a step are repacked by one launch), blockIdx.y = part, blockIdx.x = tile of 32 rows
+// (n or j) x 64 of K.  The forward operand is the transpose: its tile goes through shared memory, so that both the
+// weights and the planes move in whole lines (read down their columns, one 32-byte sector per value, the weights took
+// 17 us a step for 8 parts of 128-256-256-47).
+constexpr int PREP_ROWS = 32, PREP_K = 64;
+__host__ __device__ inline int prep_tiles(int npad, int k) { return (npad + PREP_ROWS - 1) / PREP_ROWS * (k / PREP_K); }
+
 __global__ void __launch_bounds__(256)
 tc_weight_prep_kernel(const __grid_constant__ GroupDesc g, const __grid_constant__ PrepBatch batch,
                       const float* __restrict__ params) {
+    __shared__ float tile[PREP_K][PREP_ROWS + 1];
     const PrepArgs& a = batch.job[blockIdx.z];
-    const int k = blockIdx.y;
+    const int k = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float* W = params + (int64_t)g.part[k] * a.ls.P + a.ls.param_offset;
-    const int d_in = a.ls.d_in, d_out = a.ls.d_out;
-    const int64_t nf = (int64_t)a.Npad_f * a.Kf;
-    const int64_t nd = a.Bd_hi ? (int64_t)a.Npad_d * a.Kd : 0;
-    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < nf + nd; i += (int64_t)gridDim.x * 256) {
-        float x = 0.f;
-        __nv_bfloat16 *hi, *lo;
-        if (i < nf) {
-            const int n = (int)(i / a.Kf), kk = (int)(i % a.Kf);
-            if (a.head_cp > 0) {
-                const int blk = n / a.head_cp, c = n % a.head_cp;  // which weight matrix, which of its columns
-                if (blk < a.ls.nsrc && c < d_out && kk < d_in) x = W[(int64_t)(blk * d_in + kk) * d_out + c];
-            } else {
-                const int half = a.Kf / a.ls.nsrc;  // one block of K per weight matrix
-                const int src = kk < half ? kk : kk - half;
-                if (n < d_out && src < d_in) x = W[(int64_t)(kk < half ? src : d_in + src) * d_out + n];
-            }
-            hi = a.Bf_hi + (int64_t)k * nf + i;
-            lo = a.Bf_lo + (int64_t)k * nf + i;
-        } else {
-            const int64_t ii = i - nf;
-            const int j = (int)(ii / a.Kd), kk = (int)(ii % a.Kd);
-            const int half = a.Kd / a.ls.nsrc;
-            const int c = kk < half ? kk : kk - half;
-            if (j < d_in && c < d_out) x = W[(int64_t)(kk < half ? j : d_in + j) * d_out + c];
-            hi = a.Bd_hi + (int64_t)k * nd + ii;
-            lo = a.Bd_lo + (int64_t)k * nd + ii;
+    const int d_in = a.ls.d_in, d_out = a.ls.d_out, nsrc = a.ls.nsrc;
+    const int fwd_tiles = prep_tiles(a.Npad_f, a.Kf);
+    int at = blockIdx.x;
+    if (at < fwd_tiles) {
+        const int kt = a.Kf / PREP_K, n0 = at / kt * PREP_ROWS, kk0 = at % kt * PREP_K;
+        const int n = n0 + lane;
+        // head form: which weight matrix, which of its columns (at most two matrices); else one block of K per matrix
+        const int blk = a.head_cp > 0 && n >= a.head_cp ? 1 : 0, c = n - blk * a.head_cp;
+        const int half = a.head_cp > 0 || nsrc == 1 ? a.Kf : a.Kf / 2;
+        const bool n_ok = blk < nsrc && c < d_out;
+        float x[PREP_K / 8];
+#pragma unroll
+        for (int j = 0; j < PREP_K / 8; ++j) {
+            const int kk = kk0 + warp + 8 * j;
+            const int second = kk >= half ? 1 : 0, src = kk - second * half;
+            x[j] = n_ok && src < d_in ? __ldg(W + (int64_t)((blk + second) * d_in + src) * d_out + c) : 0.f;
         }
-        split_bf16(x, *hi, *lo);
+#pragma unroll
+        for (int j = 0; j < PREP_K / 8; ++j) tile[warp + 8 * j][lane] = x[j];
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < PREP_ROWS / 8; ++j) {
+            const int r = warp + 8 * j;
+            if (n0 + r >= a.Npad_f) break;
+            uint32_t h, l;
+            split_pair(tile[2 * lane][r], tile[2 * lane + 1][r], h, l);
+            const int64_t o = ((int64_t)k * a.Npad_f + n0 + r) * a.Kf + kk0 + 2 * lane;
+            *reinterpret_cast<uint32_t*>(a.Bf_hi + o) = h;
+            *reinterpret_cast<uint32_t*>(a.Bf_lo + o) = l;
+        }
+        return;
+    }
+    at -= fwd_tiles;
+    if (!a.Bd_hi || at >= prep_tiles(a.Npad_d, a.Kd)) return;
+    const int kt = a.Kd / PREP_K, j0 = at / kt * PREP_ROWS, kk = at % kt * PREP_K + 2 * lane;
+    const int half = nsrc == 1 ? a.Kd : a.Kd / 2;  // a multiple of 64: both of the lane's values lie in one block
+    const int m = kk >= half ? 1 : 0, c = kk - m * half;
+    float x[PREP_ROWS / 8][2];
+#pragma unroll
+    for (int j = 0; j < PREP_ROWS / 8; ++j) {
+        const int row = j0 + warp + 8 * j;
+        const float* w = W + (int64_t)(m * d_in + row) * d_out + c;
+        x[j][0] = row < d_in && c < d_out ? __ldg(w) : 0.f;
+        x[j][1] = row < d_in && c + 1 < d_out ? __ldg(w + 1) : 0.f;
+    }
+#pragma unroll
+    for (int j = 0; j < PREP_ROWS / 8; ++j) {
+        const int row = j0 + warp + 8 * j;
+        if (row >= a.Npad_d) break;
+        uint32_t h, l;
+        split_pair(x[j][0], x[j][1], h, l);
+        const int64_t o = ((int64_t)k * a.Npad_d + row) * a.Kd + kk;
+        *reinterpret_cast<uint32_t*>(a.Bd_hi + o) = h;
+        *reinterpret_cast<uint32_t*>(a.Bd_lo + o) = l;
     }
 }
 
@@ -735,24 +768,38 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
         }
         if (ok) {
             const int q = warp & 3;
+            // Every thread stores its own row, four floats at a time; where rows do not start on 16-byte boundaries (90 columns,
+            // or an odd number of parameters) that would be single floats, 32 rows apart (23 us a launch on chunks of 256 rows, 18
+            // this way): then 32 x 32 blocks go through shared memory (the ring is free: behind the column sums' 16 KB, 33 floats
+            // a row) and a store writes 128 bytes of a row.  With aligned rows the detour costs more: 48.6 -> 52.3 us.
             const bool vec_ok = (d_out % 4 == 0) && (reinterpret_cast<uintptr_t>(P) % 16 == 0);
+            float* slab = reinterpret_cast<float*>(a_hi(0) + 16384) + q * 32 * 33;
             for (int t = 0; t < na_tiles; ++t) {
-                const int j = j0_of[t] + q * 32 + lane;
-                const bool live = j < d_in;
-                float* o = P + (int64_t)(src_of[t] * d_in + j) * d_out + cbase;
+                const int j0 = j0_of[t] + q * 32;
+                const int rows_here = min(32, d_in - j0);
+                if (rows_here <= 0) continue;
+                float* o = P + (int64_t)(src_of[t] * d_in + j0) * d_out + cbase + lane;
                 for (int c0 = 0; c0 < 64 * NA; c0 += 32) {
                     float v[32];
                     tc::tmem_load_32x32(tmem_base + (uint32_t)(t * a.acc_cols) + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);
-                    if (!live) continue;
+                    if (vec_ok) {
+                        if (lane < rows_here) {
+                            float* own = P + (int64_t)(src_of[t] * d_in + j0 + lane) * d_out + cbase + c0;
 #pragma unroll
-                    for (int jj = 0; jj < 32; jj += 4) {
-                        const int c = c0 + jj;
-                        if (c >= ccount) break;
-                        if (vec_ok && c + 3 < ccount) {
-                            *reinterpret_cast<float4*>(o + c) = make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]);
-                        } else {
-                            for (int e = 0; e < 4 && c + e < ccount; ++e) o[c + e] = v[jj + e];
+                            for (int jj = 0; jj < 32; jj += 4)
+                                if (c0 + jj < ccount) *reinterpret_cast<float4*>(own + jj) = make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]);
                         }
+                        __syncwarp();
+                        continue;
+                    }
+                    if (c0 >= ccount) break;
+                    __syncwarp();
+#pragma unroll
+                    for (int jj = 0; jj < 32; ++jj) slab[lane * 33 + jj] = v[jj];
+                    __syncwarp();
+                    if (c0 + lane < ccount) {
+#pragma unroll 8
+                        for (int r = 0; r < rows_here; ++r) o[(int64_t)r * d_out + c0] = slab[r * 33 + lane];
                     }
                 }
             }
@@ -886,13 +933,13 @@ int32_t launch_tc_weight_prep(rtma_ctx* ctx, const GroupDesc& g, const TcPrepJob
     if (g.num == 0 || njobs == 0) return RTMA_OK;
     if (njobs > PREP_MAX_JOBS) return rtma_fail(ctx, RTMA_ERR_INVALID_ARG, "internal: %d weight repack jobs", njobs);
     PrepBatch b{};
-    int64_t most = 0;
+    int most = 0;
     for (int j = 0; j < njobs; ++j) {
         const TcLayerPlan& p = jobs[j].plan;
         b.job[j] = PrepArgs{jobs[j].ls, jobs[j].head_cp, p.Npad_f, p.Kf, p.Npad_d, p.Kd, jobs[j].Bf_hi, jobs[j].Bf_lo, jobs[j].Bd_hi, jobs[j].Bd_lo};
-        most = std::max(most, (int64_t)p.Npad_f * p.Kf + (jobs[j].Bd_hi ? (int64_t)p.Npad_d * p.Kd : 0));
+        most = std::max(most, prep_tiles(p.Npad_f, p.Kf) + (jobs[j].Bd_hi ? prep_tiles(p.Npad_d, p.Kd) : 0));
     }
-    dim3 grid((unsigned)std::min<int64_t>(ceil_div(most, 256), 64), (unsigned)g.num, (unsigned)njobs);
+    dim3 grid((unsigned)most, (unsigned)g.num, (unsigned)njobs);
     { KernelScope ks(ctx, KC_WEIGHT_PREP, s); tc_weight_prep_kernel<<<grid, 256, 0, s>>>(g, b, params); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
