@@ -334,7 +334,8 @@ post_reduce_sgd_kernel(const __grid_constant__ GroupDesc g, const LayerShape ls,
     const int64_t count = (g.rows[k] + POST_TILE_ROWS - 1) / POST_TILE_ROWS;
     float s = 0.f;
     if (j < 2 * d + 1)
-        for (int64_t t = lane_t; t < count; t += 8) s += partial[(first + t) * (2 * d + 1) + j];
+#pragma unroll 8
+        for (int64_t t = lane_t; t < count; t += 8) s += __ldcs(partial + (first + t) * (2 * d + 1) + j);  // eight loads in flight
     red[lane_t][col] = s;
     __syncthreads();
     if (lane_t != 0 || j >= 2 * d + 1) return;
