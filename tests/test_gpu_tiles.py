@@ -106,3 +106,11 @@ def test_weight_gradient_chunks(util, dims, n, M):
     w = _workload(n, 3 * n, dims, 41)
     got, want = util.check_one_step(w, M=M)
     util.check_k_steps_and_average(w, got, want, 3)
+
+
+# the loss of the head form: 1, 2, 4 and 8 lanes a row, around their limits of 8, 16, 32 and 64 classes
+@pytest.mark.parametrize("classes", [8, 9, 15, 16, 17, 32, 33, 47, 63, 64])
+def test_head_loss_lanes(util, classes):
+    w = _workload(700, 2_500, (20, 130 if classes <= 32 else 260, classes), 61)
+    got, want = util.check_one_step(w, M=4)
+    util.check_k_steps_and_average(w, got, want, 2)
