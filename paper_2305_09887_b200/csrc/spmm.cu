@@ -652,35 +652,36 @@ spmm_narrow_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restric
 // Rows of at most 8 values (one 16-byte piece per plane; two-class heads): one THREAD per row.  With a
 // handful of neighbours per row and 32 bytes to fetch from each, handing rows out to warps costs more
 // than the work; here the offsets, the weights and the results are coalesced over the warp's 32 rows and
-// every thread walks its own entries, four neighbours in flight.  A hub row keeps its warp busy for as
-// many rounds as it has entries, which a launch of hundreds of thousands of warps absorbs.
+// every thread walks its own entries, two neighbours in flight.  A row of more than TINY_LONG entries would keep the
+// 31 others waiting (local degrees follow a power law: on average the longest of 32 rows decided, 530 and 690 us forward and
+// backward for 5 M rows and 8 M entries); such rows are done afterwards by the whole warp, 64 entries at a time, and
+// summed by a fixed shuffle tree: 311 and 325 us.  (A limit of 6 makes no difference there and costs uniform graphs 40 %.)
 constexpr int TINY_TILE_ROWS = 256;
+constexpr int TINY_LONG = 12;
 constexpr int TINY_INFLIGHT = 2;  // neighbours in flight per thread: few registers, so that five blocks fit an SM
 template <int MODE>
 __global__ void __launch_bounds__(TINY_TILE_ROWS, 5)
 spmm_tiny_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict__ rowptr_out,
-                 const int32_t* __restrict__ col_out, const float* __restrict__ inv_deg, const Planes src, const Planes out) {
+                 const int32_t* __restrict__ col_out, const float* __restrict__ inv_deg, const Planes src, const Planes out, const int d) {
     int k, r0;
     if (!locate_tile(g, TINY_TILE_ROWS, blockIdx.x, &k, &r0)) return;
-    const int i = r0 + threadIdx.x;
-    if (i >= g.rows[k]) return;
+    const int n_p = g.rows[k], i = r0 + threadIdx.x, lane = threadIdx.x & 31;
     const int64_t* rp = rowptr_out + g.row_abs[k] + g.part[k];
     const int64_t ws = g.row_ws[k];
     const int32_t* cols = col_out + g.edge_abs[k];
-    const int64_t b = rp[i], e = rp[i + 1];
+    const int b = i < n_p ? (int)rp[i] : 0, e = i < n_p ? (int)rp[i + 1] : 0;  // a part has fewer than 2^31 entries
     const __nv_bfloat16* sh = src.hi + ws * src.ld;
     const __nv_bfloat16* sl = src.lo + ws * src.ld;
     const float* wv = inv_deg + ws;
-    Pack8 acc;
-    acc.zero();
-    for (int64_t t = b; t < e; t += TINY_INFLIGHT) {
+    // acc += entries t, t + step of the row that ends at `to`
+    auto add_two = [&](Pack8& acc, const int64_t t, const int64_t step, const int to) {
         int32_t nb[TINY_INFLIGHT];
         float wt[TINY_INFLIGHT];
         uint4 xh[TINY_INFLIGHT], xl[TINY_INFLIGHT];
 #pragma unroll
         for (int j = 0; j < TINY_INFLIGHT; ++j) {
-            nb[j] = t + j < e ? __ldg(cols + t + j) : -1;
-            if (nb[j] >= 0 && !rtma_index_ok(nb[j], g.rows[k], 5)) nb[j] = -1;
+            nb[j] = t + j * step < to ? __ldg(cols + t + j * step) : -1;
+            if (nb[j] >= 0 && !rtma_index_ok(nb[j], n_p, 5)) nb[j] = -1;
         }
 #pragma unroll
         for (int j = 0; j < TINY_INFLIGHT; ++j) {
@@ -697,7 +698,29 @@ spmm_tiny_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict_
                 else acc.add_planes_mixed(xh[j], xl[j]);
             }
         }
+    };
+    Pack8 acc;
+    acc.zero();
+    const bool is_long = e - b > TINY_LONG;
+    if (!is_long)
+        for (int64_t t = b; t < e; t += TINY_INFLIGHT) add_two(acc, t, 1, e);
+    for (unsigned rest = __ballot_sync(0xffffffffu, is_long); rest; rest &= rest - 1) {
+        const int from = __ffs(rest) - 1;
+        const int rb = __shfl_sync(0xffffffffu, b, from), re = __shfl_sync(0xffffffffu, e, from);
+        Pack8 sum;
+        sum.zero();
+        for (int64_t t = (int64_t)rb + lane; t < re; t += 32 * TINY_INFLIGHT) add_two(sum, t, 32, re);
+        __syncwarp();
+#pragma unroll
+        for (int v = 0; v < 8; ++v) {
+            if (v < d) {  // the columns past the width hold zeros
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) sum.v[v] += __shfl_xor_sync(0xffffffffu, sum.v[v], o);
+            }
+            if (lane == from) acc.v[v] = v < d ? sum.v[v] : 0.f;
+        }
     }
+    if (i >= n_p) return;
     const float w = MODE == 1 ? 1.f : wv[i];
     if (MODE == 2)  // the self loop
         acc.fma_planes_mixed(w, *reinterpret_cast<const uint4*>(sh + (int64_t)i * src.ld), *reinterpret_cast<const uint4*>(sl + (int64_t)i * src.ld));
@@ -724,7 +747,7 @@ int32_t dispatch_spmm(rtma_ctx* ctx, int kclass, const GroupDesc& g, const int64
         return launch_spmm_dense(ctx, kclass, g, rowptr_out, col_out, inv_deg, order, src, out, d, MODE == 1, s);
     if (d <= 8) {
         const int64_t tiles = group_tiles(g, TINY_TILE_ROWS);
-        { KernelScope ks(ctx, kclass, s); spmm_tiny_kernel<MODE><<<(unsigned)tiles, TINY_TILE_ROWS, 0, s>>>(g, rowptr_out, col_out, inv_deg, src, out); }
+        { KernelScope ks(ctx, kclass, s); spmm_tiny_kernel<MODE><<<(unsigned)tiles, TINY_TILE_ROWS, 0, s>>>(g, rowptr_out, col_out, inv_deg, src, out, d); }
         RTMA_LAUNCH_CHECK(ctx);
         return RTMA_OK;
     }

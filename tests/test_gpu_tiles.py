@@ -114,3 +114,25 @@ def test_head_loss_lanes(util, classes):
     w = _workload(700, 2_500, (20, 130 if classes <= 32 else 260, classes), 61)
     got, want = util.check_one_step(w, M=4)
     util.check_k_steps_and_average(w, got, want, 2)
+
+
+# aggregation of rows of at most 8 values: rows around the 12 entries that a thread takes by itself, hubs of 60 to 66 entries
+# (a round of the warp) and of 1500, in every mode
+@pytest.mark.parametrize("classes, variant", [(2, (0, 0, 0)), (7, (0, 0, 0)), (8, (0, 0, 0)), (2, (1, 0, 0))])
+def test_tiny_rows_with_hubs(util, classes, variant):
+    n = 3_000
+    rng = np.random.default_rng(71)
+    u, v = [], []
+    for hub, degree in enumerate([5, 8, 11, 12, 13, 31, 32, 33, 60, 63, 64, 65, 66, 128, 129, 1_500]):
+        others = 100 + rng.choice(n - 100, size=degree, replace=False)
+        u += [hub] * degree
+        v += list(others)
+    keys = np.unique(np.concatenate([np.array(u) * n + v, np.array(v) * n + u]))
+    w = _workload(n, 10, (20, 40, classes), 72)
+    g = w.graph
+    g.rowptr = np.searchsorted(keys, np.arange(n + 1) * n).astype(g.rowptr.dtype)
+    g.col = (keys % n).astype(np.int32)
+    params0 = inputs.variant_params(variant, w.dims, 73)
+    for M in (1, 2):
+        got, want = util.check_one_step(w, M=M, variant=variant, params0=params0)
+        util.check_k_steps_and_average(w, got, want, 2, variant=variant, params0=params0)
