@@ -477,6 +477,20 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
     if (warp == 0) tc::tmem_dealloc(tmem_base, 2u * (uint32_t)a.tmem_cols);
 }
 
+// The n-th set bit of m (n from 0), or 32: halving by popcounts.  (__fns walks the bits.)
+__device__ __forceinline__ unsigned nth_bit(unsigned m, int n) {
+    unsigned pos = 0;
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) {
+        const int c = __popc((m >> pos) & ((1u << w) - 1u));
+        if (n >= c) {
+            n -= c;
+            pos += w;
+        }
+    }
+    return n == 0 && (m >> pos & 1u) ? pos : 32u;
+}
+
 // The entries outside the window of their row's tile, before the tiles run: for every row that has any,
 // out[row] = their sum (transposed pass: weighted by 1 / deg of the column), unscaled; the tile's epilogue adds
 // its product and the scale.  A warp takes 32 consecutive rows: their counts and listed columns with one load
@@ -521,7 +535,7 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
 #pragma unroll
                 for (int t = 0; t < NR; ++t) {
                     // the (t * S + sub)-th row still to do
-                    const unsigned owner = __fns(rest, 0, t * S + sub + 1);
+                    const unsigned owner = S == 1 ? (unsigned)(__ffs(rest) - 1) : nth_bit(rest, t * S + sub);
                     const bool have = owner < 32u;
                     const int from = have ? (int)owner : 0;
                     row[t] = i0 + from;
@@ -531,9 +545,12 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
                     cols[t].z = __shfl_sync(0xffffffffu, my_cols.z, from);
                     cols[t].w = __shfl_sync(0xffffffffu, my_cols.w, from);
                     if (!have) cnt[t] = 0;
+                    if (S == 1) rest &= rest - 1;
                 }
+                if (S > 1) {
 #pragma unroll
-                for (int t = 0; t < S * NR; ++t) rest &= rest - 1;
+                    for (int t = 0; t < S * NR; ++t) rest &= rest - 1;
+                }
                 Pack8 acc[NR];
 #pragma unroll
                 for (int t = 0; t < NR; ++t) acc[t].zero();
@@ -609,7 +626,7 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
 #pragma unroll
                             for (int b = 0; b < 4; ++b) {
                                 // quarter `sub` takes the entries sub, sub + S, ... of those still to do
-                                const unsigned from = __fns(votes, 0, b * S + sub + 1);
+                                const unsigned from = nth_bit(votes, b * S + sub);
                                 u[b] = __shfl_sync(0xffffffffu, c, from < 32u ? (int)from : 0);
                                 if (from >= 32u) u[b] = -1;
                             }
