@@ -103,6 +103,7 @@ int32_t parse_model(rtma_ctx* ctx, const rtma_model_desc* md, Model* m) {
 struct ScratchPlan {
     size_t per_row_bytes;     // planes, logits, 1/deg
     size_t max_layer_params;  // largest (2 d_in + 1) d_out
+    size_t max_decoder_params;  // the same of the decoder's layers (link prediction)
     size_t prep_bytes;        // repacked weights, per part
     int q_width;              // widest Abar^T dZ (widths of the layers above the first)
     size_t post_width;        // widest normalised / PReLU layer output (0: none)
@@ -139,7 +140,7 @@ ScratchPlan plan_scratch(const Model& m, bool head, bool record) {
     sp.per_pair_bytes = 0;
     for (int k = 0; k < m.Kd; ++k) {
         sp.per_pair_bytes += 4 * planes_ld(m.ddims[k]) + 4 * planes_ld(m.ddims[k + 1]);
-        sp.max_layer_params = std::max(sp.max_layer_params, (size_t)(m.ddims[k] + 1) * m.ddims[k + 1]);
+        sp.max_decoder_params = std::max(sp.max_decoder_params, (size_t)(m.ddims[k] + 1) * m.ddims[k + 1]);
         sp.prep_bytes += sizeof(__nv_bfloat16) * tc_prep_elems(tc_plan_layer(m.dec[k]), true) + 4 * 256;
         if (k < m.Kd - 1) sp.post_width = std::max(sp.post_width, (size_t)m.ddims[k + 1]);
     }
@@ -197,7 +198,7 @@ size_t part_scratch_bytes(const Model& m, const ScratchPlan& sp, int64_t n_p, in
     const size_t rows = (size_t)aligned_rows(n_p);
     const size_t prows = (size_t)aligned_rows(pairs);
     const size_t matrices = 8 * m.L + 8 * m.Kd + 24;  // every matrix start is rounded up to 256 bytes
-    const size_t decoder = sp.per_pair_bytes * prows + sizeof(float) * (64 * sp.max_layer_params + (size_t)ceil_div(pairs, 32) + 256) +
+    const size_t decoder = sp.per_pair_bytes * prows + sizeof(float) * (64 * sp.max_decoder_params + (size_t)ceil_div(pairs, 32) + 256) +
                            sizeof(float) * ((size_t)ceil_div(pairs, 64) + 1) * (2 * sp.post_width + 1);
     return sp.per_row_bytes * rows + sizeof(float) * (64 * sp.max_layer_params + (size_t)ceil_div(n_p, 32) + 256) +
            (m.Kd ? decoder : 0) + rows / 32 +
@@ -443,7 +444,7 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                     if (c.blocks_per_slot * c.bytes_per_row > widest.blocks_per_slot * widest.bytes_per_row) widest = c;
                 }
                 const int dslots = plan_splits(gd, running, widest, &spd);
-                dec_partial = cur.take<float>((size_t)dslots * plan.max_layer_params + 4);
+                dec_partial = cur.take<float>((size_t)dslots * plan.max_decoder_params + 4);
                 dec_tile_loss = cur.take<float>((size_t)loss_tiles(gd) + 4);
             }
             // Abar^T dZ of the layer in hand; carved at the widest layer, addressed at each layer's own width
