@@ -27,9 +27,14 @@ pair_product_kernel(const __grid_constant__ GroupDesc gd, const __grid_constant_
     if (!locate_tile(gd, PAIR_WARPS, blockIdx.x, &k, &r0)) return;
     const int lane = threadIdx.x & 31, i = r0 + (threadIdx.x >> 5);
     if (i >= gd.rows[k]) return;
-    if (!rtma_index_ok(pu[gd.row_abs[k] + i], g.rows[k], 7) || !rtma_index_ok(pv[gd.row_abs[k] + i], g.rows[k], 7)) return;
-    const int64_t ru = g.row_ws[k] + pu[gd.row_abs[k] + i], rv = g.row_ws[k] + pv[gd.row_abs[k] + i];
     const int64_t out = gd.row_ws[k] + i;
+    if (!rtma_index_ok(pu[gd.row_abs[k] + i], g.rows[k], 7) || !rtma_index_ok(pv[gd.row_abs[k] + i], g.rows[k], 7)) {
+        // checked build: the pair counts as zeros (the scratch may hold anything)
+        for (int col = lane * 8; col < d; col += 256)
+            *reinterpret_cast<uint4*>(E.hi + out * E.ld + col) = *reinterpret_cast<uint4*>(E.lo + out * E.ld + col) = make_uint4(0u, 0u, 0u, 0u);
+        return;
+    }
+    const int64_t ru = g.row_ws[k] + pu[gd.row_abs[k] + i], rv = g.row_ws[k] + pv[gd.row_abs[k] + i];
     for (int col = lane * 8; col < d; col += 256) {
         Pack8 a, b;
         load_pack(R, ru, col, a);

@@ -40,6 +40,18 @@ def rel_err(a, b):
     return float(np.abs(a - b).max() / max(np.abs(b).max(), 1e-30)) if b.size else 0.0
 
 
+def fill_scratch_with_nan(c, g):
+    """Leaves NaNs all over the scratch of context c: a step of a wide normalised model (Layer Normalization and PReLU
+    pass NaNs on, ReLU would not) whose features and parameters are NaN."""
+    dims, variant = (64, 300, 300, 100), (0, 1, 1)
+    part_id, part_offsets, perm, local_id = c.partition(g.n, None, 1, 1)
+    rowptr_out, col_out, _, _, edge_host = c.build_induced_csr(dev(g.rowptr), dev(g.col), 1, part_id, part_offsets, perm, local_id)
+    params = torch.full((1, binding.param_count(dims, variant)), float("nan"), device="cuda")
+    c.local_steps(dims, 0.1, 1, [0, g.n], edge_host, rowptr_out, col_out, torch.full((g.n, 64), float("nan"), device="cuda"),
+                  torch.zeros(g.n, dtype=torch.int32, device="cuda"), params, 1, variant=variant)
+    torch.cuda.synchronize()
+
+
 def gpu_preprocess(w, M=None, seed=None, use_groups=None, grouped=None):
     """partition + induced CSR + row gather on the GPU for workload w."""
     c = ctx()

@@ -8,6 +8,7 @@ import numpy as np
 import pytest
 import torch
 
+import gpu_util
 from paper_2305_09887_b200 import binding, inputs
 
 pytestmark = pytest.mark.gpu
@@ -73,3 +74,23 @@ def test_checked_build_reports_a_label_out_of_range(tiny_workload):
                   perm=perm)
     with pytest.raises(binding.RtmaError, match="label 8 outside"):
         c.check()
+
+
+def test_a_bad_pair_counts_as_zeros(tiny_workload):
+    w = tiny_workload
+    g = w.graph
+    c = binding.Context(0, checked=True)
+    gpu_util.fill_scratch_with_nan(c, g)
+    part_id, part_offsets, perm, local_id = c.partition(g.n, None, w.partition_seed, 2)
+    rowptr_out, col_out, _, _, edge_host = c.build_induced_csr(_dev(g.rowptr), _dev(g.col), 2, part_id, part_offsets, perm, local_id)
+    part_host = part_offsets.cpu().tolist()
+    dims, ddims = (64, 40, 24), (24, 16, 1)
+    rng = np.random.default_rng(5)
+    pu, pv = (rng.integers(0, min(part_host[1], g.n - part_host[1]), size=180).astype(np.int32) for _ in range(2))
+    pu[77] = 1 << 20
+    params = _dev(np.tile(rng.normal(size=binding.link_param_count(dims, ddims)).astype(np.float32) * 0.1, (2, 1)))
+    c.link_steps(dims, ddims, 0.05, 2, part_host, edge_host, rowptr_out, col_out, c.gather_rows(_dev(w.X), perm), [0, 101, 180],
+                 _dev(pu), _dev(pv), _dev((rng.random(180) < 0.5).astype(np.int32)), params, 2)
+    with pytest.raises(binding.RtmaError, match=f"{1 << 20} outside"):
+        c.check()
+    assert torch.isfinite(params).all()
