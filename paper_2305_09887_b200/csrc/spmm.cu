@@ -65,19 +65,19 @@ to_planes_kernel(const __grid_constant__ GroupDesc g, const float* __restrict__ 
         if (i >= g.rows[k]) return;
         // perm: the features are still in the graph's node order; row i of the partition order is node perm[i]
         const int64_t node = perm ? (int64_t)perm[g.row_abs[k] + i] : g.row_abs[k] + i;
-        if (!rtma_index_ok(node, n_total, 4)) continue;
-        const float* x = X + node * (int64_t)d;
+        const bool node_ok = rtma_index_ok(node, n_total, 4);  // checked build: a row without a node counts as zeros
+        const float* x = X + (node_ok ? node : 0) * (int64_t)d;
         const int64_t o = (g.row_ws[k] + i) * out.ld;
         for (int c0 = lane * 8; c0 < out.ld; c0 += 256) {
             Pack8 p;
-            if (vec && c0 + 8 <= d) {  // rows start on 16-byte boundaries: two vector loads
+            if (vec && node_ok && c0 + 8 <= d) {  // rows start on 16-byte boundaries: two vector loads
                 const float4 a = __ldg(reinterpret_cast<const float4*>(x + c0));
                 const float4 b = __ldg(reinterpret_cast<const float4*>(x + c0 + 4));
                 p.v[0] = a.x; p.v[1] = a.y; p.v[2] = a.z; p.v[3] = a.w;
                 p.v[4] = b.x; p.v[5] = b.y; p.v[6] = b.z; p.v[7] = b.w;
             } else {
 #pragma unroll
-                for (int e = 0; e < 8; ++e) p.v[e] = c0 + e < d ? __ldg(x + c0 + e) : 0.f;
+                for (int e = 0; e < 8; ++e) p.v[e] = node_ok && c0 + e < d ? __ldg(x + c0 + e) : 0.f;
             }
             uint4 h, l;
             p.to_planes_cvt(h, l);

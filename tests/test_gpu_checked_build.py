@@ -76,6 +76,33 @@ def test_checked_build_reports_a_label_out_of_range(tiny_workload):
         c.check()
 
 
+def test_a_row_with_a_bad_permutation_entry_counts_as_zeros(tiny_workload):
+    w = tiny_workload
+    g = w.graph
+    c = binding.Context(0, checked=True)
+    gpu_util.fill_scratch_with_nan(c, g)
+    part_id, part_offsets, perm, local_id = c.partition(g.n, None, w.partition_seed, w.M)
+    rowptr_out, col_out, _, _, edge_host = c.build_induced_csr(_dev(g.rowptr), _dev(g.col), w.M, part_id, part_offsets, perm, local_id)
+    yp = c.gather_rows(_dev(w.y), perm)
+    part_host = part_offsets.cpu().tolist()
+
+    def steps(X, order):
+        params = _dev(np.tile(w.params0, (w.M, 1)))
+        c.local_steps(w.dims, w.lr, w.M, part_host, edge_host, rowptr_out, col_out, X, yp, params, 2, perm=order)
+        return params
+
+    bad = perm.clone()
+    bad[900] = g.n + 3
+    got = steps(_dev(w.X), bad)
+    with pytest.raises(binding.RtmaError, match=f"permutation entry {g.n + 3} outside"):
+        c.check()
+    X = _dev(w.X)
+    X[int(perm[900])] = 0.0
+    want = steps(X, perm)
+    c.check()
+    assert torch.equal(got, want)
+
+
 def test_a_bad_pair_counts_as_zeros(tiny_workload):
     w = tiny_workload
     g = w.graph
