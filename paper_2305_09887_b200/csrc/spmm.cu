@@ -652,12 +652,15 @@ spmm_narrow_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restric
 // Rows of at most 8 values (one 16-byte piece per plane; two-class heads): one THREAD per row.  With a
 // handful of neighbours per row and 32 bytes to fetch from each, handing rows out to warps costs more
 // than the work; here the offsets, the weights and the results are coalesced over the warp's 32 rows and
-// every thread walks its own entries, two neighbours in flight.  A row of more than TINY_LONG entries would keep the
-// 31 others waiting (local degrees follow a power law: on average the longest of 32 rows decided, 530 and 690 us forward and
-// backward for 5 M rows and 8 M entries); such rows are done afterwards by the whole warp, 64 entries at a time, and
-// summed by a fixed shuffle tree: 311 and 325 us.  (A limit of 6 makes no difference there and costs uniform graphs 40 %.)
+// every thread walks its own entries, two neighbours in flight and the columns of the next two.  A row much longer than the 31
+// others would keep them waiting (local degrees follow a power law: the longest of 32 rows decided, 658 us backward for 5 M
+// rows and 8 M entries); such rows are done afterwards by the whole warp, 64 entries at a time, and summed by a fixed
+// shuffle tree: 273 us.  From how many entries on is each warp's own choice, by the rounds of two entries that it costs;
+// a row by the whole warp counts three (its two loads one after the other, and the tree).  With a fixed limit of 12 rows
+// of similar length went one by one through the whole warp: 1,800 rows of 25 entries took 53 us, by threads 15; 500,000 of
+// them 258 and 170; with the count at one and a quarter 300,000 rows of 60 entries took 300, now 231.
 constexpr int TINY_TILE_ROWS = 256;
-constexpr int TINY_LONG = 12;
+constexpr int TINY_LONG = 12;  // the lowest limit; the others are its doublings
 constexpr int TINY_INFLIGHT = 2;  // neighbours in flight per thread: few registers, so that five blocks fit an SM
 template <int MODE>
 __global__ void __launch_bounds__(TINY_TILE_ROWS, 5)
@@ -673,65 +676,93 @@ spmm_tiny_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict_
     const __nv_bfloat16* sh = src.hi + ws * src.ld;
     const __nv_bfloat16* sl = src.lo + ws * src.ld;
     const float* wv = inv_deg + ws;
-    // acc += entries t, t + step of the row that ends at `to`
-    auto add_two = [&](Pack8& acc, const int64_t t, const int64_t step, const int to) {
-        int32_t nb[TINY_INFLIGHT];
-        float wt[TINY_INFLIGHT];
-        uint4 xh[TINY_INFLIGHT], xl[TINY_INFLIGHT];
+    // acc += entries t, t + step, t + 2 step, ... of the row that ends at `to`, two a round; a round's columns are requested
+    // while the round before is summed
+    auto add_all = [&](Pack8& acc, int64_t t, const int64_t step, const int to) {
+        int32_t next[TINY_INFLIGHT];
+        auto columns = [&]() {
 #pragma unroll
-        for (int j = 0; j < TINY_INFLIGHT; ++j) {
-            nb[j] = t + j * step < to ? __ldg(cols + t + j * step) : -1;
-            if (nb[j] >= 0 && !rtma_index_ok(nb[j], n_p, 5)) nb[j] = -1;
-        }
-#pragma unroll
-        for (int j = 0; j < TINY_INFLIGHT; ++j) {
-            if (nb[j] >= 0) {
-                if (MODE != 0) wt[j] = __ldg(wv + nb[j]);
-                xh[j] = __ldg(reinterpret_cast<const uint4*>(sh + (int64_t)nb[j] * src.ld));
-                xl[j] = __ldg(reinterpret_cast<const uint4*>(sl + (int64_t)nb[j] * src.ld));
+            for (int j = 0; j < TINY_INFLIGHT; ++j) {
+                next[j] = t + j * step < to ? __ldg(cols + t + j * step) : -1;
+                if (next[j] >= 0 && !rtma_index_ok(next[j], n_p, 5)) next[j] = -1;
             }
-        }
+        };
+        columns();
+#pragma unroll 1
+        while (t < to) {
+            int32_t nb[TINY_INFLIGHT];
+            float wt[TINY_INFLIGHT];
+            uint4 xh[TINY_INFLIGHT], xl[TINY_INFLIGHT];
 #pragma unroll
-        for (int j = 0; j < TINY_INFLIGHT; ++j) {
-            if (nb[j] >= 0) {
-                if (MODE != 0) acc.fma_planes_mixed(wt[j], xh[j], xl[j]);
-                else acc.add_planes_mixed(xh[j], xl[j]);
+            for (int j = 0; j < TINY_INFLIGHT; ++j) {
+                nb[j] = next[j];
+                if (nb[j] >= 0) {
+                    if (MODE != 0) wt[j] = __ldg(wv + nb[j]);
+                    xh[j] = __ldg(reinterpret_cast<const uint4*>(sh + (int64_t)nb[j] * src.ld));
+                    xl[j] = __ldg(reinterpret_cast<const uint4*>(sl + (int64_t)nb[j] * src.ld));
+                }
+            }
+            t += TINY_INFLIGHT * step;
+            columns();
+#pragma unroll
+            for (int j = 0; j < TINY_INFLIGHT; ++j) {
+                if (nb[j] >= 0) {
+                    if (MODE != 0) acc.fma_planes_mixed(wt[j], xh[j], xl[j]);
+                    else acc.add_planes_mixed(xh[j], xl[j]);
+                }
             }
         }
     };
-    Pack8 acc;
-    acc.zero();
-    const bool is_long = e - b > TINY_LONG;
-    if (!is_long)
-        for (int64_t t = b; t < e; t += TINY_INFLIGHT) add_two(acc, t, 1, e);
+    // scale and store the lane's own row
+    auto finish = [&](Pack8& acc) {
+        const float w = MODE == 1 ? 1.f : wv[i];
+        if (MODE == 2)  // the self loop
+            acc.fma_planes_mixed(w, *reinterpret_cast<const uint4*>(sh + (int64_t)i * src.ld), *reinterpret_cast<const uint4*>(sl + (int64_t)i * src.ld));
+        if (MODE != 1) {
+#pragma unroll
+            for (int v = 0; v < 8; ++v) acc.v[v] *= w;
+        }
+        uint4 h, l;
+        acc.to_planes_lean(h, l);
+        *reinterpret_cast<uint4*>(out.hi + (ws + i) * out.ld) = h;
+        *reinterpret_cast<uint4*>(out.lo + (ws + i) * out.ld) = l;
+    };
+    const int entries = e - b, longest = __reduce_max_sync(0xffffffffu, entries);
+    int limit = longest, rounds = longest / 2;
+    for (int64_t l = TINY_LONG; l < longest; l *= 2) {
+        const int n_long = __popc(__ballot_sync(0xffffffffu, entries > l));
+        const int r = __reduce_max_sync(0xffffffffu, entries > l ? 0 : entries) / 2 + 3 * n_long;
+        if (r < rounds) {
+            limit = (int)l;
+            rounds = r;
+        }
+    }
+    const bool is_long = entries > limit;
+    if (!is_long && i < n_p) {
+        Pack8 acc;
+        acc.zero();
+        add_all(acc, b, 1, e);
+        finish(acc);
+    }
     for (unsigned rest = __ballot_sync(0xffffffffu, is_long); rest; rest &= rest - 1) {
         const int from = __ffs(rest) - 1;
         const int rb = __shfl_sync(0xffffffffu, b, from), re = __shfl_sync(0xffffffffu, e, from);
         Pack8 sum;
         sum.zero();
-        for (int64_t t = (int64_t)rb + lane; t < re; t += 32 * TINY_INFLIGHT) add_two(sum, t, 32, re);
+        add_all(sum, (int64_t)rb + lane, 32, re);
         __syncwarp();
 #pragma unroll
         for (int v = 0; v < 8; ++v) {
             if (v < d) {  // the columns past the width hold zeros
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) sum.v[v] += __shfl_xor_sync(0xffffffffu, sum.v[v], o);
+            } else {
+                sum.v[v] = 0.f;
             }
-            if (lane == from) acc.v[v] = v < d ? sum.v[v] : 0.f;
         }
+        if (lane == from) finish(sum);
+        __syncwarp();
     }
-    if (i >= n_p) return;
-    const float w = MODE == 1 ? 1.f : wv[i];
-    if (MODE == 2)  // the self loop
-        acc.fma_planes_mixed(w, *reinterpret_cast<const uint4*>(sh + (int64_t)i * src.ld), *reinterpret_cast<const uint4*>(sl + (int64_t)i * src.ld));
-    if (MODE != 1) {
-#pragma unroll
-        for (int v = 0; v < 8; ++v) acc.v[v] *= w;
-    }
-    uint4 h, l;
-    acc.to_planes_lean(h, l);
-    *reinterpret_cast<uint4*>(out.hi + (ws + i) * out.ld) = h;
-    *reinterpret_cast<uint4*>(out.lo + (ws + i) * out.ld) = l;
 }
 
 template <int MODE>

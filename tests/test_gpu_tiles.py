@@ -136,3 +136,44 @@ def test_tiny_rows_with_hubs(util, classes, variant):
     for M in (1, 2):
         got, want = util.check_one_step(w, M=M, variant=variant, params0=params0)
         util.check_k_steps_and_average(w, got, want, 2, variant=variant, params0=params0)
+
+
+# the same in warps of 32 rows of every kind: all about as long (the threads take them), a few long ones among short ones
+# (the whole warp does), limits of 12, 24 and 48 entries
+@pytest.mark.parametrize("classes, variant", [(2, (0, 0, 0)), (7, (1, 0, 0))])
+def test_tiny_rows_of_similar_and_of_mixed_lengths(util, classes, variant):
+    rng = np.random.default_rng(81)
+    kinds = [[25], [13], [12, 13], [60], [3, 3, 3, 40], [1] * 31 + [13], [1] * 31 + [14], [2] * 15 + [30], [11, 23], [23] * 15 + [90], [47] * 10 + [400], [0, 200]]
+    degrees = [k[i % len(k)] for k in kinds for i in range(32)]
+    rows, n = len(degrees), 4_000
+    u = np.repeat(np.arange(rows), degrees)
+    v = np.concatenate([rows + rng.choice(n - rows, size=d, replace=False) for d in degrees])
+    keys = np.unique(np.concatenate([u * n + v, v * n + u]))
+    w = _workload(n, 10, (20, 40, classes), 82)
+    w.graph.rowptr = np.searchsorted(keys, np.arange(n + 1) * n).astype(w.graph.rowptr.dtype)
+    w.graph.col = (keys % n).astype(np.int32)
+    params0 = inputs.variant_params(variant, w.dims, 83)
+    got, want = util.check_one_step(w, M=1, variant=variant, params0=params0)
+    util.check_k_steps_and_average(w, got, want, 2, variant=variant, params0=params0)
+
+
+# Rows of 32 entries cost the threads of a warp three times as many rounds as rows of 10.  (Were they taken one by one by the
+# whole warp, as hubs are, the launch would take five times as long or more; times of the two-class aggregation, backward.)
+def test_tiny_rows_of_similar_length_are_not_taken_for_hubs(util):
+    from paper_2305_09887_b200 import binding
+    n, c, times = 1 << 17, binding.Context(0), []
+    i = torch.arange(n, device="cuda")
+    for degree in (10, 32):
+        step = torch.cat([torch.arange(1, degree // 2 + 1), -torch.arange(1, degree // 2 + 1)]).cuda() * 997   # a circulant graph
+        col = torch.sort((i[:, None] + step) % n, dim=1)[0].to(torch.int32).flatten().contiguous()
+        rowptr = torch.arange(n + 1, device="cuda", dtype=torch.int64) * degree
+        X, y = torch.randn(n, 8, device="cuda"), torch.zeros(n, dtype=torch.int32, device="cuda")
+        params = util.dev(inputs.xavier_params((8, 16, 2), 1)[None])
+        c.profile(True)
+        best = 1e9
+        for _ in range(6):
+            c.local_steps((8, 16, 2), 0.0, 1, [0, n], [0, n * degree], rowptr, col, X, y, params, 3)
+            best = min(best, c.profile_read()["spmm_backward"][0])
+        c.profile(False)
+        times.append(best)
+    assert times[1] <= 4.2 * times[0], times
