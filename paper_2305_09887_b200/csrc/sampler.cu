@@ -50,33 +50,36 @@ constexpr int SEL_NODES = 256 / SEL_LANES;  // nodes of a block
 constexpr int SEL_CAND = 128;   // candidates a node may have
 
 // The kept entries of one node by the whole warp, whatever its degree and the fan-out: the fanout-th smallest key bit by
-// bit (64 rounds of counting the keys that share the prefix found so far and have a 0 in the next bit), then a pass
-// that writes the entries below it and the first few equal to it, in row order.
+// bit (rounds of counting the keys that share the prefix found so far and have a 0 in the next bit, until no more keys
+// share it than are still to be kept: about log2 of the degree of them), then a pass that writes the entries below the
+// prefix and the first few that share it, in row order.
 __device__ void select_bit_by_bit(const int32_t* __restrict__ col, int64_t n, int64_t begin, int64_t deg, uint64_t vkey, int32_t fanout,
                                   uint64_t base, int64_t out, int32_t* __restrict__ block_col, int32_t* __restrict__ member) {
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
-    // keys whose high bits equal `prefix` (bits above `bit`): how many have a 0 at `bit`?
-    uint64_t prefix = 0;
-    int64_t want = fanout;  // rank (1-based) of the key looked for among the keys that match the prefix
-    for (int bit = 63; bit >= 0; --bit) {
-        const uint64_t mask_hi = bit == 63 ? 0ULL : ~0ULL << (bit + 1);
+    uint64_t prefix = 0, mask = 0;    // bits found so far, and which they are
+    int64_t want = fanout, left = deg;  // keys to be kept among those that share the prefix, and how many share it
+    for (int bit = 63; bit >= 0 && left > want; --bit) {
         int64_t zeros = 0;
         for (int64_t q = lane; q < deg; q += 32) {
             const uint64_t key = mix_step(base ^ (vkey | (uint64_t)q));
-            zeros += ((key & mask_hi) == prefix && !((key >> bit) & 1ULL)) ? 1 : 0;
+            zeros += ((key & mask) == prefix && !((key >> bit) & 1ULL)) ? 1 : 0;
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) zeros += __shfl_xor_sync(0xffffffffu, zeros, o);
+        mask |= 1ULL << bit;
         if (want > zeros) {  // the key has a 1 here; the `zeros` keys with a 0 are all smaller
             want -= zeros;
+            left -= zeros;
             prefix |= 1ULL << bit;
+        } else {
+            left = zeros;
         }
     }
-    int64_t ties_seen = 0;  // entries equal to the key: the first `want` in row order are kept
+    int64_t ties_seen = 0;  // entries that share the prefix: the first `want` in row order are kept (all, or those with equal keys)
     for (int64_t q0 = 0; q0 < deg; q0 += 32) {
         const int64_t q = q0 + lane;
-        const uint64_t key = mix_step(base ^ (vkey | (uint64_t)q));
+        const uint64_t key = mix_step(base ^ (vkey | (uint64_t)q)) & mask;
         const bool tie = q < deg && key == prefix;
         bool keep = q < deg && key < prefix;
         const unsigned tie_votes = __ballot_sync(0xffffffffu, tie);
@@ -93,14 +96,16 @@ __device__ void select_bit_by_bit(const int32_t* __restrict__ col, int64_t n, in
     }
 }
 
-// Half a warp per frontier node (two nodes of 30 entries fill a warp's lanes; a quarter each was no faster on paper:
-// the ranking costs more per lane).  The keys are uniform 64-bit numbers, so the fanout-th smallest of deg lies near
-// fanout / deg of their range: one pass over the row hashes every entry once and collects those below a bound at which
-// fanout + 6 sqrt(fanout) + 16 of them are expected (too few or too many less than once in 10^6 nodes), in row
-// order, in shared memory; a candidate is kept when fewer than `fanout` candidates are smaller.  Only kept entries' columns
-// are read.  Bound by instruction issue (the hash, 25 instructions per entry, and the ranking).  Finding the key bit by
-// bit for every node hashed every entry 64 times: three hops (fan-outs 15, 10, 5) from 8,192 of 800,000 nodes took 8.06 ms
-// with the program around them and take 0.83 ms.
+// Half a warp per frontier node (two nodes of 30 entries fill a warp's lanes).  The keys are uniform 64-bit numbers, so the
+// fanout-th smallest of deg lies near fanout / deg of their range: one pass over the row hashes every entry once and collects
+// those below a bound at which `expected` of them are expected, in row order, in shared memory; a candidate is kept when
+// fewer than `fanout` candidates are smaller.  Only kept entries' columns are read.  Bound by instruction issue (the hash,
+// 25 instructions per entry, and the ranking).  Finding the key bit by bit for every node hashed every entry 64 times:
+// three hops (fan-outs 15, 10, 5) from 8,192 of 800,000 nodes took 8.06 ms with the program around them and take 0.83 ms.
+// expected = fanout + 6 sqrt(fanout) + 16, but no more than half way between the fan-out and the candidates' room: too few
+// or too many candidates come once in 10^6 rows up to a fan-out of 35, in 20,000 at 50, in 1,000 at 64, in 60 at 80 and in 8 at
+// SEL_FANOUT; such rows, and all that are cut to larger fan-outs, are done bit by bit.
+constexpr int SEL_FANOUT = 96;  // largest fan-out for which candidates are collected
 __global__ void __launch_bounds__(256)
 sample_select_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, int64_t n, int64_t frontier_size,
                      const int32_t* __restrict__ frontier, int32_t fanout, double expected, uint64_t base,
@@ -130,7 +135,7 @@ sample_select_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restri
     // the others: candidates (both halves of the warp go through the longer row's rounds)
     const double share = sel ? expected / (double)deg : 1.0;
     const uint64_t bound = share >= 0.999 ? ~0ULL : (uint64_t)(share * 18446744073709551616.0);
-    const int64_t rounds = sel && deg < (int64_t(1) << 31) ? (deg + SEL_LANES - 1) / SEL_LANES : 0;  // positions are 32-bit
+    const int64_t rounds = sel && fanout <= SEL_FANOUT && deg < (int64_t(1) << 31) ? (deg + SEL_LANES - 1) / SEL_LANES : 0;  // positions are 32-bit
     const int64_t other = __shfl_xor_sync(0xffffffffu, rounds, 16);
     const int64_t most = rounds > other ? rounds : other;
     int64_t count = 0;
@@ -233,7 +238,8 @@ extern "C" int32_t rtma_sample_hop(rtma_ctx* ctx, int64_t n, const int64_t* rowp
         z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
         const uint64_t base = z ^ (z >> 31);
         KernelScope ks(ctx, KC_LINK, stream);
-        const double expected = (double)fanout + 6.0 * std::sqrt((double)fanout) + 16.0;  // candidates per row (see the kernel)
+        // candidates per row (see the kernel)
+        const double expected = std::min((double)fanout + 6.0 * std::sqrt((double)fanout) + 16.0, 0.5 * ((double)fanout + SEL_CAND));
         sample_select_kernel<<<(unsigned)ceil_div(frontier_size, SEL_NODES), 256, 0, stream>>>(
             rowptr, col, n, frontier_size, frontier, fanout, expected, base, block_rowptr, block_col, member);
     }

@@ -177,3 +177,39 @@ def test_tiny_rows_of_similar_length_are_not_taken_for_hubs(util):
         c.profile(False)
         times.append(best)
     assert times[1] <= 4.2 * times[0], times
+
+
+# 300 rows of 97 to 700 entries around the largest fan-out with candidates (96: one row in eight has too few or too many of
+# them) and past it, where the search over the row's keys ends as soon as all that share the prefix are kept
+@pytest.mark.parametrize("fanout", [64, 80, 95, 96, 97, 98, 200, 699])
+def test_sampled_rows_around_the_largest_fanout_with_candidates(util, fanout):
+    rng = np.random.default_rng(100 + fanout)
+    degrees = np.concatenate([[97, 98, 99, 200, 201, 700], rng.integers(97, 700, size=294)])
+    n = 5_000
+    rowptr = np.zeros(n + 1, dtype=np.int64)
+    rowptr[1:] = np.cumsum(np.concatenate([degrees, np.zeros(n - degrees.size, dtype=np.int64)]))
+    col = np.concatenate([np.sort(rng.choice(n, size=d, replace=False)) for d in degrees]).astype(np.int32)
+    frontier = np.arange(degrees.size, dtype=np.int32)
+    got = util.ctx().sample_hop(util.dev(rowptr), util.dev(col), util.dev(frontier), fanout, 17, 1)
+    for a, b in zip(got, oracle.sample_hop(rowptr, col, frontier, fanout, 17, 1)):
+        assert np.array_equal(a.cpu().numpy(), b)
+
+
+# A large fan-out costs a few times what a small one does on the same rows of 600 entries (12 times while every key was searched
+# for through all of its 64 bits).
+def test_large_fanouts_do_not_search_bit_by_bit_to_the_end(util):
+    from paper_2305_09887_b200 import binding
+    n, degree, c = 20_000, 600, binding.Context(0)
+    rowptr = torch.arange(n + 1, device="cuda", dtype=torch.int64) * degree
+    col = torch.randint(n, (n * degree,), device="cuda", dtype=torch.int32)
+    frontier = torch.arange(0, n, 2, device="cuda", dtype=torch.int32)
+    times = []
+    c.profile(True)
+    for fanout in (25, 128):
+        best = 1e9
+        for _ in range(6):
+            c.sample_hop(rowptr, col, frontier, fanout, 5, 1)
+            best = min(best, c.profile_read()["link_pairs"][0])
+        times.append(best)
+    c.profile(False)
+    assert times[1] <= 7.0 * times[0], times
