@@ -946,13 +946,18 @@ int32_t launch_tc_weight_prep(rtma_ctx* ctx, const GroupDesc& g, const TcPrepJob
 }
 
 // Do a product's tiles go to pairs of blocks (256 rows, each block staging half of the weight tile)?  A block by itself
-// moves 96 KB through shared memory per 64 of K and 128 x 256 outputs, a third of it activations, next to what the MMAs
-// read there; a pair 64 KB each.  That pays where the main loop is the longest chain: medium graph (200 k rows, 8 parts),
-// us alone / in pairs: K = 512, 256 columns 151 / 115, gated 154 / 130; operands rounded to bf16, K = 1024, 500 k rows
-// 500 / 442.  With K <= 256 the output is the longer chain and the pair's blocks wait for each other: 84 / 90, gated 90 / 95,
-// 96 columns 53 / 60.  And only where a launch has tiles for every SM: 10 k rows a part, 3 parts 12.5 / 13.2.
-static bool rows_use_pairs(const rtma_ctx* ctx, const GroupDesc& g, int K, int BN) {
-    return BN % 32 == 0 && BN >= 128 && K >= 384 && group_tiles(g, TC_BM) >= ctx->sm_count;
+// moves 96 KB through shared memory per 64 of K, two planes and 128 x 256 outputs, a third of it activations, next to what
+// the MMAs read there; a pair 64 KB each.  That pays where this main loop is the longest chain, hence from a depth K times
+// planes on.  Where the output is the longer chain the pair's blocks only wait for each other.  us alone / in pairs:
+//   two planes, 200 k rows: K = 512, 256 columns 151 / 115, gated 154 / 130; all products of a step with K = 384, 160 columns
+//   205 / 194, gated 162 / 155; but K = 256 84 / 90, gated 90 / 95;
+//   one plane (operands rounded to bf16): K = 512, 256 columns and the layers around it 167 / 179, gated 185 / 192; K = 768, 384
+//   columns 273 / 264; K = 1024, 512 columns 359 / 335.  Gated it starts to pay later, the gate words are read with one plane
+//   as with two: K = 768 294 / 306, K = 896 367 / 380, K = 1024 394 / 390.
+// And only where a launch has tiles for every SM: 10 k rows a part, 3 parts 12.5 / 13.2.
+static bool rows_use_pairs(const rtma_ctx* ctx, const GroupDesc& g, int K, int BN, bool single, bool gated) {
+    const int deep = single ? (gated ? 1024 : 768) : 384;
+    return BN % 32 == 0 && BN >= 128 && K >= deep && group_tiles(g, TC_BM) >= ctx->sm_count;
 }
 
 static int32_t launch_rows(rtma_ctx* ctx, RowsArgs& a, int64_t rows_total, bool pairs, int kclass, cudaStream_t s) {
@@ -1004,7 +1009,7 @@ int32_t launch_tc_forward(rtma_ctx* ctx, const GroupDesc& g, LayerShape ls, cons
     RowsArgs a{};
     a.g = g;
     a.single = single ? 1 : 0;
-    const bool pairs = rows_use_pairs(ctx, g, p.Kf, p.BN_f);
+    const bool pairs = rows_use_pairs(ctx, g, p.Kf, p.BN_f, single, false);
     const uint32_t b_rows = (uint32_t)(pairs ? p.BN_f / 2 : p.BN_f);
     if (!plane_maps(&a.mapA0h, &a.mapA0l, H, rows_total, ls.d_in, TC_BK, TC_BM) ||
         !plane_maps(&a.mapA1h, &a.mapA1l, N, rows_total, ls.d_in, TC_BK, TC_BM) ||
@@ -1039,7 +1044,7 @@ int32_t launch_tc_dgrad(rtma_ctx* ctx, const GroupDesc& g, LayerShape ls, const 
     RowsArgs a{};
     a.g = g;
     a.single = single ? 1 : 0;
-    const bool pairs = rows_use_pairs(ctx, g, p.Kd, p.BN_d);
+    const bool pairs = rows_use_pairs(ctx, g, p.Kd, p.BN_d, single, gate);
     const uint32_t b_rows = (uint32_t)(pairs ? p.BN_d / 2 : p.BN_d);
     if (!plane_maps(&a.mapA0h, &a.mapA0l, dZ, rows_total, ls.d_out, TC_BK, TC_BM) ||
         !plane_maps(&a.mapA1h, &a.mapA1l, Q, rows_total, ls.d_out, TC_BK, TC_BM) ||

@@ -25,6 +25,28 @@ def _workload(n, edges, dims, seed):
     return w
 
 
+def kernels_of(call):
+    """Names of the kernels that `call` launches; empty where the profiler cannot trace them."""
+    try:
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+            call()
+            torch.cuda.synchronize()
+        return {e.key for e in prof.key_averages()}
+    except RuntimeError:
+        return set()
+
+
+def _steps(c, util, w, got, params0, K, **options):
+    """Parameters and losses of all trainers after K steps (an int or one count per trainer)."""
+    params = util.dev(np.tile(params0, (got["M"], 1)))
+    loss = torch.zeros(got["M"], K if isinstance(K, int) else max(K), device="cuda")
+    torch.cuda.synchronize()
+    c.local_steps(w.dims, w.lr, got["M"], got["part_host"], got["edge_host"], got["rowptr_out"], got["col_out"], got["Xp"], got["yp"],
+                  params, K, loss_out=loss, **options)
+    torch.cuda.synchronize()
+    return params, loss
+
+
 # enough 128-row tiles for every SM and K >= 384: the products of the second layer go to pairs of blocks.  Parts of
 # about 850 and 300 rows: the last 256-row tile of a part lies half, wholly or not at all past its end.
 @pytest.mark.parametrize("n, M, dims, parts, gemm_dtype", [
@@ -36,6 +58,25 @@ def _workload(n, edges, dims, seed):
 def test_products_on_pairs_of_blocks(util, n, M, dims, parts, gemm_dtype):
     w = _workload(n, 3 * n, dims, 11)
     util.check_one_step(w, M=M, gemm_dtype=gemm_dtype, only_parts=parts, gradients_against_plain=gemm_dtype == 0)
+
+
+# pairs of blocks where the main loop is deep enough for them, by K and the operands' planes, later where the output reads a gate
+@pytest.mark.parametrize("dims, gemm_dtype, variant, pairs", [
+    ((70, 200, 200, 5), 0, (0, 0, 0), True), ((70, 200, 200, 5), 1, (0, 0, 0), False),
+    ((20, 392, 172), 1, (0, 0, 0), True), ((20, 232, 264, 5), 1, (0, 0, 0), False),   # K = 896; 512, gated 640
+    ((20, 70, 392, 5), 1, (0, 1, 1), False), ((20, 200, 392, 5), 1, (0, 1, 1), True),   # K = 896: 70 columns; 200, not gated
+    ((20, 200, 392, 5), 1, (0, 0, 0), False), ((20, 200, 520, 5), 1, (0, 0, 0), True),  # gated: K = 896; 1152
+])
+def test_pairs_of_blocks_are_taken_by_depth(util, dims, gemm_dtype, variant, pairs):
+    n, M = 19_600, 4
+    w = _workload(n, 3 * n, dims, 15)
+    got = util.gpu_preprocess(w, M=M)
+    assert sum(-(-r // 128) for r in np.diff(got["part_host"])) >= torch.cuda.get_device_properties(0).multi_processor_count
+    params0 = inputs.variant_params(variant, dims, 16)
+    names = kernels_of(lambda: _steps(util.ctx(), util, w, got, params0, 1, gemm_dtype=gemm_dtype, variant=variant))
+    if names:
+        assert any("tc_rows_kernel" in k for k in names)
+        assert any("tc_rows_pair_kernel" in k for k in names) == pairs, sorted(names)
 
 
 # the neighbour sampler: rows of 15 to 17 entries (a half-warp), around the candidates' room of 128 and far past it;
