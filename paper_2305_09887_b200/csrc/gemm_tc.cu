@@ -164,7 +164,8 @@ tc_weight_prep_kernel(const __grid_constant__ GroupDesc g, const __grid_constant
 struct RowsArgs {
     GroupDesc g;
     CUtensorMap mapA0h, mapA0l, mapA1h, mapA1l, mapBh, mapBl;
-    CUtensorMap mapOh, mapOl;  // plane output: boxes of 64 columns x 32 rows
+    CUtensorMap mapOh, mapOl;    // plane output: boxes of 64 columns x 32 rows
+    CUtensorMap mapOh32, mapOl32;  // and of 32 x 32, for the last columns of a tile whose width is an odd multiple of 32
     int kb0, kb1;          // 64-wide k blocks taken from source 0 / source 1
     int BN, Npad, N;       // column tile, B rows per part, valid output columns
     int tmem_cols, stages; // columns of one accumulator buffer (two are allocated); pipeline depth
@@ -384,7 +385,6 @@ __device__ __forceinline__ void rows_body(const RowsArgs& a) {
         const int q = warp & 3;           // the TMEM lane quarter this warp may read: rows 32 q .. 32 q + 31 of the tile
         uint8_t* slab_hi = smem + (size_t)stages * stage_bytes + (size_t)q * ROWS_SLAB_BYTES;  // [32 rows][64 columns] of either plane
         uint8_t* slab_lo = slab_hi + ROWS_SLAB_BYTES / 2;
-        const uint32_t swz = (uint32_t)(lane & 7);
         int64_t t = 0;
         bool ok = true;
         for (int64_t tile = first_tile; tile < total_tiles && ok; tile += tile_step, ++t) {
@@ -398,6 +398,7 @@ __device__ __forceinline__ void rows_body(const RowsArgs& a) {
             const int64_t orow0 = a.g.row_ws[k] + r0;
             // a chunk's bias (lane l: columns l and l + 32) and the lane's row of its gate, requested a chunk ahead
             const float* bias = a.bias_offset >= 0 ? a.params + (int64_t)a.g.part[k] * a.P + a.bias_offset : nullptr;
+            const int gate_end = min((int)a.out_planes.ld, n0 + BN);
             float nb0 = 0.f, nb1 = 0.f;
             uint4 gw[8];
             auto request = [&](int c0) {
@@ -409,7 +410,7 @@ __device__ __forceinline__ void rows_body(const RowsArgs& a) {
                 if constexpr (OUT == OUT_GATED) {
                     const uint4* gp = reinterpret_cast<const uint4*>(a.gate_hi + (orow0 + lane) * a.out_planes.ld + n);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) gw[j] = live && n + 8 * j < a.out_planes.ld ? gp[j] : make_uint4(0u, 0u, 0u, 0u);
+                    for (int j = 0; j < 8; ++j) gw[j] = live && n + 8 * j < gate_end ? gp[j] : make_uint4(0u, 0u, 0u, 0u);
                 }
             };
             request(0);
@@ -422,9 +423,10 @@ __device__ __forceinline__ void rows_body(const RowsArgs& a) {
             // (gated 99 and 126 us against 90); unrolled chunks did not fit the instruction cache (11 us a tile against 7).
 #pragma unroll 1
             for (int c0 = 0; c0 < BN && rows_here > 0; c0 += 64) {
+                const bool half = c0 + 32 >= BN;  // 32 columns or fewer are left
                 uint32_t raw[2][32];
                 tc::tmem_load_issue(acc + (uint32_t)c0, raw[0]);
-                if (c0 + 32 < BN) tc::tmem_load_issue(acc + (uint32_t)(c0 + 32), raw[1]);
+                if (!half) tc::tmem_load_issue(acc + (uint32_t)(c0 + 32), raw[1]);
                 if (bias) {
                     __syncwarp();
                     bias_slab[q][lane] = nb0;
@@ -451,6 +453,7 @@ __device__ __forceinline__ void rows_body(const RowsArgs& a) {
                     if (live) {
 #pragma unroll
                         for (int j = 0; j < 64; j += 4) {
+                            if (j >= 32 && half) break;
                             const int n = nbase + j;
                             float x[4];
 #pragma unroll
@@ -475,34 +478,43 @@ __device__ __forceinline__ void rows_body(const RowsArgs& a) {
                     // (What lies past the accumulator's BN columns is past the planes' too and is not stored.)
                     uint32_t h[32], l[32];
 #pragma unroll
-                    for (int j = 0; j < 32; j += 2) {
-                        float x[4];
+                    for (int q0 = 0; q0 < 32; q0 += 16) {
+                        if (q0 > 0 && half) break;
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) x[e] = __uint_as_float(raw[j >> 4][2 * (j & 15) + e]);
-                        if (bias) {
-                            const float4 b4 = *reinterpret_cast<const float4*>(&bias_slab[q][2 * j]);
-                            add_pair(x[0], x[1], b4.x, b4.y);
-                            add_pair(x[2], x[3], b4.z, b4.w);
-                        }
-                        if (a.relu) {
+                        for (int j = q0; j < q0 + 16; j += 2) {
+                            float x[4];
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) x[e] = fmaxf(x[e], 0.f);
-                        }
-                        split_pair(x[0], x[1], h[j], l[j]);
-                        split_pair(x[2], x[3], h[j + 1], l[j + 1]);
-                        if constexpr (OUT == OUT_GATED) {
-                            h[j] &= mask[j];
-                            l[j] &= mask[j];
-                            h[j + 1] &= mask[j + 1];
-                            l[j + 1] &= mask[j + 1];
+                            for (int e = 0; e < 4; ++e) x[e] = __uint_as_float(raw[j >> 4][2 * (j & 15) + e]);
+                            if (bias) {
+                                const float4 b4 = *reinterpret_cast<const float4*>(&bias_slab[q][2 * j]);
+                                add_pair(x[0], x[1], b4.x, b4.y);
+                                add_pair(x[2], x[3], b4.z, b4.w);
+                            }
+                            if (a.relu) {
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) x[e] = fmaxf(x[e], 0.f);
+                            }
+                            split_pair(x[0], x[1], h[j], l[j]);
+                            split_pair(x[2], x[3], h[j + 1], l[j + 1]);
+                            if constexpr (OUT == OUT_GATED) {
+                                h[j] &= mask[j];
+                                l[j] &= mask[j];
+                                h[j + 1] &= mask[j + 1];
+                                l[j + 1] &= mask[j + 1];
+                            }
                         }
                     }
-                    // Out through shared memory (row r's 16-byte piece j at piece j ^ (r % 8)), one bulk-tensor store per plane.
+                    // Out through shared memory, one bulk-tensor store per plane: row r's 16-byte piece j at piece j ^ (r % 8), of
+                    // rows of 32 columns at piece j ^ (r / 2 % 4), as the maps' swizzles have it.
+                    const uint32_t pitch = half ? 64u : 128u;
+                    auto swizzle = [&](uint32_t row) { return half ? row >> 1 & 3u : row & 7u; };
+                    const uint32_t own = (uint32_t)lane * pitch, swz = swizzle(lane);
                     if (lane == 0) tc::tma_store_wait_read();  // the chunk before has left the slab
                     __syncwarp();
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
-                        const uint32_t at = (uint32_t)lane * 128u + (((uint32_t)j ^ swz) << 4);
+                        if (j >= 4 && half) break;
+                        const uint32_t at = own + (((uint32_t)j ^ swz) << 4);
                         *reinterpret_cast<uint4*>(slab_hi + at) = make_uint4(h[4 * j], h[4 * j + 1], h[4 * j + 2], h[4 * j + 3]);
                         *reinterpret_cast<uint4*>(slab_lo + at) = make_uint4(l[4 * j], l[4 * j + 1], l[4 * j + 2], l[4 * j + 3]);
                     }
@@ -510,16 +522,16 @@ __device__ __forceinline__ void rows_body(const RowsArgs& a) {
                         tc::fence_proxy_async_smem();
                         __syncwarp();
                         if (lane == 0 && nbase < a.out_planes.ld) {
-                            tc::tma_store_2d(&a.mapOh, slab_hi, nbase, (int)orow0);
-                            tc::tma_store_2d(&a.mapOl, slab_lo, nbase, (int)orow0);
+                            tc::tma_store_2d(half ? &a.mapOh32 : &a.mapOh, slab_hi, nbase, (int)orow0);
+                            tc::tma_store_2d(half ? &a.mapOl32 : &a.mapOl, slab_lo, nbase, (int)orow0);
                             tc::tma_store_commit();
                         }
                     } else {  // the part's last rows: the rows behind them are not this part's
                         __syncwarp();
                         const int n = nbase + 8 * (lane & 7);
                         for (int row = lane >> 3; row < rows_here; row += 4) {
-                            const uint32_t at = (uint32_t)row * 128u + ((uint32_t)((lane ^ row) & 7) << 4);
-                            if (n < a.out_planes.ld) {
+                            if (n < a.out_planes.ld && !(half && (lane & 7) >= 4)) {
+                                const uint32_t at = (uint32_t)row * pitch + ((((uint32_t)lane & 7u) ^ swizzle(row)) << 4);
                                 const int64_t o = (orow0 + row) * a.out_planes.ld + n;
                                 *reinterpret_cast<uint4*>(a.out_planes.hi + o) = *reinterpret_cast<const uint4*>(slab_hi + at);
                                 *reinterpret_cast<uint4*>(a.out_planes.lo + o) = *reinterpret_cast<const uint4*>(slab_lo + at);
@@ -893,14 +905,16 @@ bool make_tensor_map_bf16(CUtensorMap* out, const void* base, uint64_t rows, uin
     const cuuint32_t box[2] = {box_cols, box_rows};
     const cuuint32_t estride[2] = {1, 1};
     return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), gdim, gstride, box, estride,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, box_cols <= 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // Column tile of the rows kernel for `d` columns: at most 256 wide, equal tiles, a multiple of 16; from 64 columns on a
-// multiple of 32, the step of an MMA of a pair of blocks; more than one tile: of 64, what the epilogue stores at a time.
+// multiple of 32, the step of an MMA of a pair of blocks.  Not coarser: with tiles in multiples of 64, what the epilogue stores
+// at a time, 300 columns paid for 384 instead of 320 (a step of 200 k rows, 128 -> 300 -> 300: forward 395 / 386 us, input
+// gradients 352 / 334; one plane 244 / 231 and 256 / 250); in multiples of 16 it gains nothing.
 static int column_tile(int d) {
-    const int tiles = (int)ceil_div(d, 256), step = tiles > 1 ? 64 : d >= 64 ? 32 : 16;
+    const int tiles = (int)ceil_div(d, 256), step = d >= 64 ? 32 : 16;
     return (int)ceil_div(ceil_div(d, tiles), step) * step;
 }
 
@@ -980,7 +994,8 @@ static int32_t launch_rows(rtma_ctx* ctx, RowsArgs& a, int64_t rows_total, bool 
     const int64_t total_tiles = a.row_tiles * (a.Npad / a.BN);
     const unsigned grid = pairs ? 2u * (unsigned)std::min<int64_t>(total_tiles, ctx->sm_count / 2)
                                 : (unsigned)std::min<int64_t>(total_tiles, ctx->sm_count);
-    if (a.out_planes.hi && !plane_maps(&a.mapOh, &a.mapOl, a.out_planes, rows_total, (uint64_t)a.out_planes.ld, 64, 32))
+    if (a.out_planes.hi && (!plane_maps(&a.mapOh, &a.mapOl, a.out_planes, rows_total, (uint64_t)a.out_planes.ld, 64, 32) ||
+                            !plane_maps(&a.mapOh32, &a.mapOl32, a.out_planes, rows_total, (uint64_t)a.out_planes.ld, 32, 32)))
         return rtma_fail(ctx, RTMA_ERR_CUDA, "cuTensorMapEncodeTiled refused the output planes");
     // the epilogue's slabs are only allocated for plane output: shared memory comes out of L1
     const size_t ring = a.stages * stage_bytes + 1024;

@@ -233,7 +233,7 @@ __device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
 
 // ---- host side: tensor-map encoding through the driver entry point ------------------------
 // 2-D row-major bf16 matrix [rows x cols], `ld` elements between rows, box = box_cols x box_rows
-// (box_cols <= 64), 128-byte swizzle of 16-byte chunks in shared memory, out-of-range elements
+// (box_cols <= 64), 128-byte swizzle of 16-byte chunks in shared memory (64-byte up to 32 columns), out-of-range elements
 // read as zero.  Returns false if the driver refuses.
 bool make_tensor_map_bf16(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, uint64_t ld,
                           uint32_t box_cols, uint32_t box_rows);
