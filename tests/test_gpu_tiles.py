@@ -47,17 +47,73 @@ def _steps(c, util, w, got, params0, K, **options):
     return params, loss
 
 
-# enough 128-row tiles for every SM and K >= 384: the products of the second layer go to pairs of blocks.  Parts of
+# enough 128-row tiles for every SM and a deep enough K: the products of the second layer go to pairs of blocks.  Parts of
 # about 850 and 300 rows: the last 256-row tile of a part lies half, wholly or not at all past its end.
-@pytest.mark.parametrize("n, M, dims, parts, gemm_dtype", [
-    (19_600, 23, (70, 200, 200, 5), (0, 7, 22), 0),     # 224-column tiles over 200 columns
-    (19_600, 23, (70, 200, 200, 5), (3,), 1),
-    (19_000, 60, (20, 200, 136, 7), (0, 31, 59), 0),    # two or three 128-row tiles a part
-    (19_600, 23, (40, 520, 520, 3), (5,), 0),           # three column tiles of 192
+@pytest.mark.parametrize("n, M, dims, parts, gemm_dtype, variant, pairs", [
+    (19_600, 23, (70, 200, 200, 5), (0, 7, 22), 0, (0, 0, 0), True),     # 224-column tiles over 200 columns
+    (19_600, 23, (70, 200, 200, 5), (3,), 1, (0, 0, 0), False),          # bf16 operands: too shallow for pairs
+    (19_600, 23, (70, 520, 264, 5), (3,), 1, (0, 0, 0), True),           # K = 1152
+    (19_000, 60, (20, 200, 136, 7), (0, 31, 59), 0, (0, 0, 0), True),    # two or three 128-row tiles a part
+    (19_600, 23, (40, 520, 520, 3), (5,), 0, (0, 0, 0), True),           # three column tiles
+    (19_600, 23, (70, 260, 172), (0, 22), 0, (0, 0, 0), True),           # fp32 scores, 172 columns
+    (19_600, 23, (40, 456, 280, 5), (5,), 0, (1, 1, 1), True),           # one weight matrix; pre-activations, plain input gradient
+    (19_600, 23, (40, 264, 200, 5), (5,), 0, (0, 1, 1), True),
 ])
-def test_products_on_pairs_of_blocks(util, n, M, dims, parts, gemm_dtype):
+def test_products_on_pairs_of_blocks(util, n, M, dims, parts, gemm_dtype, variant, pairs):
     w = _workload(n, 3 * n, dims, 11)
-    util.check_one_step(w, M=M, gemm_dtype=gemm_dtype, only_parts=parts, gradients_against_plain=gemm_dtype == 0)
+    params0 = inputs.variant_params(variant, dims, 12)
+    got, _ = util.check_one_step(w, M=M, gemm_dtype=gemm_dtype, only_parts=parts, variant=variant, params0=params0,
+                                 gradients_against_plain=gemm_dtype == 0)
+    assert sum(-(-r // 128) for r in np.diff(got["part_host"])) >= torch.cuda.get_device_properties(0).multi_processor_count
+    names = kernels_of(lambda: _steps(util.ctx(), util, w, got, params0, 1, gemm_dtype=gemm_dtype, variant=variant))
+    assert not names or any("tc_rows_pair_kernel" in k for k in names) == pairs, sorted(names)
+
+
+# decoder layers with pairs of nodes as their rows: 19,000 and more of them
+def test_decoder_products_on_pairs_of_blocks(util):
+    from test_gpu_link import _check_link
+    w = inputs.tiny()
+    w.graph = inputs.uniform_graph(3_000, 12_000, 5)
+    w.dims = (20, 400)
+    w.X, w.y = inputs.normal_features(3_000, 20, 6), inputs.uniform_labels(3_000, 8, 7)
+    _check_link(util, w, (0, 0, 0), (400, 130, 1), per_part=10_000, K=1, M=1)
+
+
+# Which kernel a launch takes depends on how many tiles it has, hence on the trainers that share it; their results do not: all
+# trainers of a call on one stream (pairs of blocks, M of 256), each on its own (single blocks, M of 128), in waves, and with
+# step counts that thin the launches out.
+@pytest.mark.parametrize("dims, gemm_dtype, variant", [
+    ((40, 520, 264, 172), 0, (0, 0, 0)),
+    ((40, 520, 264, 172), 1, (0, 0, 0)),
+    ((40, 520, 264, 5), 0, (1, 1, 1)),
+    ((40, 520, 264, 5), 1, (0, 1, 1)),
+])
+def test_pairs_of_blocks_do_not_change_a_bit(util, dims, gemm_dtype, variant):
+    from paper_2305_09887_b200 import binding
+    M, n = 4, 25_600
+    w = _workload(n, 2 * n, dims, 13)
+    params0 = inputs.variant_params(variant, dims, 14)
+    got = util.gpu_preprocess(w, M=M)
+    options = dict(gemm_dtype=gemm_dtype, variant=variant)
+    whole = binding.Context(0)
+    names = kernels_of(lambda: _steps(whole, util, w, got, params0, 2, **options))
+    one = _steps(whole, util, w, got, params0, 2, **options)
+    streams = [torch.cuda.Stream() for _ in range(M)]
+    alone_names = kernels_of(lambda: _steps(whole, util, w, got, params0, 2, streams=streams, **options))
+    if names and alone_names:
+        assert any("tc_rows_pair_kernel" in k for k in names) and not any("tc_rows_pair_kernel" in k for k in alone_names)
+    for a, b in zip(one, _steps(whole, util, w, got, params0, 2, streams=streams, **options)):
+        assert torch.equal(a, b)
+    single = binding.Context(0)
+    _steps(single, util, w, got, params0, 1, **options)
+    capped = binding.Context(0)
+    capped.set_workspace_limit(int(single.workspace_bytes * 0.55))
+    for a, b in zip(one, _steps(capped, util, w, got, params0, 2, **options)):
+        assert torch.equal(a, b)
+    uneven = _steps(whole, util, w, got, params0, [2, 1, 2, 1], **options)
+    assert torch.equal(uneven[0][::2], one[0][::2]) and torch.equal(uneven[1][::2], one[1][::2])
+    short = _steps(whole, util, w, got, params0, 1, **options)
+    assert torch.equal(uneven[0][1::2], short[0][1::2])
 
 
 # pairs of blocks where the main loop is deep enough for them, by K and the operands' planes, later where the output reads a gate
@@ -99,32 +155,51 @@ def test_sampled_rows_around_the_candidates_room(util, fanout):
             assert np.array_equal(a.cpu().numpy(), b)
 
 
-# the scratch a call finds holds whatever the calls before it left there: here the NaNs of a wider model on other parts
-@pytest.mark.parametrize("dims, variant", [((20, 40, 131), (0, 0, 0)), ((33, 90, 70, 3), (0, 0, 0)), ((20, 36, 36, 5), (1, 1, 1)),
-                                           ((24, 33), (0, 0, 0))])
-def test_scratch_left_by_another_call_does_not_matter(util, dims, variant):
+# the scratch a call finds holds whatever the calls before it left there: here NaNs
+@pytest.mark.parametrize("dims, variant, dense", [((20, 40, 131), (0, 0, 0), 1), ((33, 90, 70, 3), (0, 0, 0), 1), ((20, 36, 36, 5), (1, 1, 1), 1),
+                                                  ((24, 33), (0, 0, 0), 1), ((33, 90, 70, 40), (0, 0, 0), 2), ((20, 36, 136, 5), (0, 1, 1), 2)])
+def test_scratch_left_by_another_call_does_not_matter(util, dims, variant, dense):
     from paper_2305_09887_b200 import binding
     w = _workload(2_000, 9_000, dims, 21)
     params0 = inputs.variant_params(variant, dims, 4)
     pre = util.gpu_preprocess(w, M=7)
-    other = _workload(2_000, 9_000, (64, 300, 300, 9), 22)
-    pre_other = util.gpu_preprocess(other, M=3)
-
-    def steps(c):
-        params = util.dev(np.tile(params0, (7, 1)))
-        loss = torch.zeros(7, 3, device="cuda")
-        c.local_steps(dims, 0.05, 7, pre["part_host"], pre["edge_host"], pre["rowptr_out"], pre["col_out"], pre["Xp"], pre["yp"],
-                      params, 3, loss_out=loss, variant=variant)
-        torch.cuda.synchronize()
-        return params, loss
-
-    clean = steps(binding.Context(0))
     c = binding.Context(0)
-    nan = torch.full_like(pre_other["Xp"], float("nan"))
-    c.local_steps(other.dims, 0.05, 3, pre_other["part_host"], pre_other["edge_host"], pre_other["rowptr_out"], pre_other["col_out"],
-                  nan, pre_other["yp"], util.dev(np.tile(other.params0, (3, 1))), 2)
-    after = steps(c)
+    c.set_dense_aggregation(dense)
+    util.fill_scratch_with_nan(c, w.graph)
+    after = _steps(c, util, w, pre, params0, 3, variant=variant)
+    fresh = binding.Context(0)
+    fresh.set_dense_aggregation(dense)
+    clean = _steps(fresh, util, w, pre, params0, 3, variant=variant)
     assert torch.isfinite(clean[0]).all() and torch.equal(clean[0], after[0]) and torch.equal(clean[1], after[1])
+
+
+# the same for link prediction, whose decoder has matrices with the pairs as rows: 37 to 300 of them a part, none in one part
+# (the embeddings' gradient is summed by atomics: two runs differ by the order of fp32 additions, measured 3e-7)
+@pytest.mark.parametrize("dense", [1, 2])
+def test_scratch_left_by_another_call_does_not_matter_to_link_prediction(util, dense):
+    from paper_2305_09887_b200 import binding
+    w = _workload(2_000, 9_000, (33, 90, 40), 23)
+    ddims, variant, M, counts = (40, 70, 20, 1), (0, 1, 1), 5, [37, 0, 300, 64, 129]
+    pre = util.gpu_preprocess(w, M=M)
+    rng = np.random.default_rng(24)
+    rows = np.diff(pre["part_host"])
+    pairs = [rng.integers(0, r, size=(2, k)).astype(np.int32) for r, k in zip(rows, counts)]
+    pu, pv = (util.dev(np.concatenate([p[j] for p in pairs])) for j in (0, 1))
+    label = util.dev((rng.random(sum(counts)) < 0.5).astype(np.int32))
+    p0 = oracle.link_init_params(variant, w.dims, ddims, 25).astype(np.float32)
+    out = []
+    for poisoned in (False, True):
+        c = binding.Context(0)
+        c.set_dense_aggregation(dense)
+        if poisoned:
+            util.fill_scratch_with_nan(c, w.graph)
+        params, loss = util.dev(np.tile(p0, (M, 1))), torch.zeros(M, 2, device="cuda")
+        c.link_steps(w.dims, ddims, w.lr, M, pre["part_host"], pre["edge_host"], pre["rowptr_out"], pre["col_out"], pre["Xp"],
+                     [0] + list(np.cumsum(counts)), pu, pv, label, params, 2, loss_out=loss, variant=variant)
+        torch.cuda.synchronize()
+        out.append((params.cpu().numpy(), loss.cpu().numpy()))
+    for a, b in zip(*out):
+        assert np.isfinite(a).all() and util.rel_err(a, b) <= 1e-5
 
 
 # tensor-core aggregation forced: tiles without any entry, with entries outside the window only, and part ends inside a
