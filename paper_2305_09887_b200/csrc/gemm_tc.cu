@@ -217,8 +217,9 @@ __device__ __forceinline__ bool rows_wait(uint64_t* bar, uint32_t parity, RowsBa
 }
 
 // PAIR = false: a block works on tiles of 128 rows by itself.  PAIR = true: two blocks of a cluster work on tiles of
-// 256 rows; `rank` 0 issues the MMAs of both (see tc_common.cuh).
-template <int OUT, bool PAIR>
+// 256 rows; `rank` 0 issues the MMAs of both (see tc_common.cuh).  HALF: the last 64 columns of a tile are 32 at most, which
+// the epilogue finishes by themselves (compiled apart: the test costs gated tiles of 64 columns a twentieth).
+template <int OUT, bool PAIR, bool HALF>
 __device__ __forceinline__ void rows_body(const RowsArgs& a) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ RowsBarriers pb;
@@ -423,7 +424,7 @@ __device__ __forceinline__ void rows_body(const RowsArgs& a) {
             // (gated 99 and 126 us against 90); unrolled chunks did not fit the instruction cache (11 us a tile against 7).
 #pragma unroll 1
             for (int c0 = 0; c0 < BN && rows_here > 0; c0 += 64) {
-                const bool half = c0 + 32 >= BN;  // 32 columns or fewer are left
+                const bool half = HALF && c0 + 32 >= BN;  // 32 columns or fewer are left
                 uint32_t raw[2][32];
                 tc::tmem_load_issue(acc + (uint32_t)c0, raw[0]);
                 if (!half) tc::tmem_load_issue(acc + (uint32_t)(c0 + 32), raw[1]);
@@ -560,13 +561,13 @@ __device__ __forceinline__ void rows_body(const RowsArgs& a) {
     }
 }
 
-template <int OUT>
+template <int OUT, bool HALF>
 __global__ void __launch_bounds__(ROWS_THREADS, 1) tc_rows_kernel(const __grid_constant__ RowsArgs a) {
-    rows_body<OUT, false>(a);
+    rows_body<OUT, false, HALF>(a);
 }
-template <int OUT>
+template <int OUT, bool HALF>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(ROWS_THREADS, 1) tc_rows_pair_kernel(const __grid_constant__ RowsArgs a) {
-    rows_body<OUT, true>(a);
+    rows_body<OUT, true, HALF>(a);
 }
 
 // ------------------------------------------------------------------------------------
@@ -974,15 +975,19 @@ static bool rows_use_pairs(const rtma_ctx* ctx, const GroupDesc& g, int K, int B
     return BN % 32 == 0 && BN >= 128 && K >= deep && group_tiles(g, TC_BM) >= ctx->sm_count;
 }
 
+using RowsKernel = void (*)(RowsArgs);
+static const RowsKernel rows_kernels[2][2][3] = {  // [pairs][last 64 columns of a tile are 32 at most][output]
+    {{tc_rows_kernel<OUT_F32, false>, tc_rows_kernel<OUT_PLANES, false>, tc_rows_kernel<OUT_GATED, false>},
+     {tc_rows_kernel<OUT_F32, true>, tc_rows_kernel<OUT_PLANES, true>, tc_rows_kernel<OUT_GATED, true>}},
+    {{tc_rows_pair_kernel<OUT_F32, false>, tc_rows_pair_kernel<OUT_PLANES, false>, tc_rows_pair_kernel<OUT_GATED, false>},
+     {tc_rows_pair_kernel<OUT_F32, true>, tc_rows_pair_kernel<OUT_PLANES, true>, tc_rows_pair_kernel<OUT_GATED, true>}}};
+
 static int32_t launch_rows(rtma_ctx* ctx, RowsArgs& a, int64_t rows_total, bool pairs, int kclass, cudaStream_t s) {
     if (!ctx->rows_configured) {  // per device: the context is bound to one
-        const void* kernels[] = {reinterpret_cast<const void*>(tc_rows_kernel<OUT_F32>), reinterpret_cast<const void*>(tc_rows_kernel<OUT_PLANES>),
-                                 reinterpret_cast<const void*>(tc_rows_kernel<OUT_GATED>),
-                                 reinterpret_cast<const void*>(tc_rows_pair_kernel<OUT_F32>),
-                                 reinterpret_cast<const void*>(tc_rows_pair_kernel<OUT_PLANES>),
-                                 reinterpret_cast<const void*>(tc_rows_pair_kernel<OUT_GATED>)};
-        for (const void* kernel : kernels)
-            RTMA_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ROWS_SMEM_MAX));
+        for (const auto& by_width : rows_kernels)
+            for (const auto& by_output : by_width)
+                for (const RowsKernel kernel : by_output)
+                    RTMA_CUDA(ctx, cudaFuncSetAttribute(reinterpret_cast<const void*>(kernel), cudaFuncAttributeMaxDynamicSharedMemorySize, ROWS_SMEM_MAX));
         ctx->rows_configured = true;
     }
     const size_t stage_bytes = (a.single ? 1 : 2) * ((size_t)PLANE_TILE_BYTES + (size_t)(pairs ? a.BN / 2 : a.BN) * 128);
@@ -994,8 +999,9 @@ static int32_t launch_rows(rtma_ctx* ctx, RowsArgs& a, int64_t rows_total, bool 
     const int64_t total_tiles = a.row_tiles * (a.Npad / a.BN);
     const unsigned grid = pairs ? 2u * (unsigned)std::min<int64_t>(total_tiles, ctx->sm_count / 2)
                                 : (unsigned)std::min<int64_t>(total_tiles, ctx->sm_count);
+    const bool half = a.BN % 64 != 0 && a.BN % 64 <= 32;
     if (a.out_planes.hi && (!plane_maps(&a.mapOh, &a.mapOl, a.out_planes, rows_total, (uint64_t)a.out_planes.ld, 64, 32) ||
-                            !plane_maps(&a.mapOh32, &a.mapOl32, a.out_planes, rows_total, (uint64_t)a.out_planes.ld, 32, 32)))
+                            (half && !plane_maps(&a.mapOh32, &a.mapOl32, a.out_planes, rows_total, (uint64_t)a.out_planes.ld, 32, 32))))
         return rtma_fail(ctx, RTMA_ERR_CUDA, "cuTensorMapEncodeTiled refused the output planes");
     // the epilogue's slabs are only allocated for plane output: shared memory comes out of L1
     const size_t ring = a.stages * stage_bytes + 1024;
@@ -1003,15 +1009,7 @@ static int32_t launch_rows(rtma_ctx* ctx, RowsArgs& a, int64_t rows_total, bool 
     {
         KernelScope ks(ctx, kclass, s);
         const int out = !a.out_planes.hi ? OUT_F32 : a.gate_hi ? OUT_GATED : OUT_PLANES;
-#define RTMA_ROWS(KERNEL)                                                                            \
-    do {                                                                                             \
-        if (out == OUT_F32) KERNEL<OUT_F32><<<grid, ROWS_THREADS, smem, s>>>(a);                     \
-        else if (out == OUT_PLANES) KERNEL<OUT_PLANES><<<grid, ROWS_THREADS, smem, s>>>(a);          \
-        else KERNEL<OUT_GATED><<<grid, ROWS_THREADS, smem, s>>>(a);                                  \
-    } while (0)
-        if (pairs) RTMA_ROWS(tc_rows_pair_kernel);
-        else RTMA_ROWS(tc_rows_kernel);
-#undef RTMA_ROWS
+        rows_kernels[pairs ? 1 : 0][half ? 1 : 0][out]<<<grid, ROWS_THREADS, smem, s>>>(a);
     }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
