@@ -2,10 +2,10 @@
 // gradient (softmax - onehot) / n_p is written as split bf16 planes (it feeds the tensor-core
 // products of the backward pass).
 //
-// Up to 64 classes: one thread per row (the kernel is bound by instruction issue, and a row in one
-// thread needs no cross-lane reductions).  Up to 128 classes: one warp per row, eight rows per warp,
-// a lane keeping four consecutive logits in registers.  Wider rows are swept three times (max, sum
-// of exponentials, gradient).
+// Up to 64 classes: one thread per row, in the head form with more than 8 classes 2, 4 or 8 lanes (the kernel is bound by
+// instruction issue, and a row in one thread needs no cross-lane reductions).  Up to 128 classes: one warp per row, eight
+// rows per warp, a lane keeping four consecutive logits in registers.  Wider rows are swept three times (max, sum of
+// exponentials, gradient).
 // Loss sums are reduced in a fixed order (warp -> block -> part): results do not change from
 // run to run.
 #include "train.cuh"
@@ -195,8 +195,7 @@ softmax_xent_row_kernel(const __grid_constant__ GroupDesc g, const Mat logits, c
 // classes): the row's scores are z = [T_self +] NT + b, with T_self the row's own product H Ws (absent
 // for one-matrix layers) and NT the aggregated product Abar (H Wn), both split planes; they are formed
 // in the thread's registers and never stored (`scores` != NULL records them, for verification).  The
-// rest is softmax_xent_row_kernel.  A thread per row: used for up to 8 classes.
-template <int NV4>
+// rest is softmax_xent_row_kernel.  Up to 8 classes, one 16-byte piece per plane: a thread per row.
 __global__ void __launch_bounds__(LOSS_TILE_ROWS)
 softmax_xent_head_kernel(const __grid_constant__ GroupDesc g, const Planes Tself, const Planes NT,
                          const float* __restrict__ params, const int64_t P, const int64_t bias_offset, const int C,
@@ -211,58 +210,34 @@ softmax_xent_head_kernel(const __grid_constant__ GroupDesc g, const Planes Tself
         const int64_t r = g.row_ws[k] + i;
         const float* bias = params + (int64_t)g.part[k] * P + bias_offset;
         const int label = checked_label(yp[g.row_abs[k] + i], C);
-        const int n8 = (int)(NT.ld >> 3) < NV4 / 2 ? (int)(NT.ld >> 3) : NV4 / 2;
-        float v[4 * NV4];
-#pragma unroll
-        for (int q = 0; q < NV4 / 2; ++q) {
-            Pack8 x;
-            x.zero();
-            if (q < n8) {
-                x.add_planes(*reinterpret_cast<const uint4*>(NT.hi + r * NT.ld + 8 * q), *reinterpret_cast<const uint4*>(NT.lo + r * NT.ld + 8 * q));
-                if (Tself.hi)
-                    x.add_planes(*reinterpret_cast<const uint4*>(Tself.hi + r * Tself.ld + 8 * q),
-                                 *reinterpret_cast<const uint4*>(Tself.lo + r * Tself.ld + 8 * q));
-            }
-#pragma unroll
-            for (int e = 0; e < 8; ++e) v[8 * q + e] = x.v[e] + (8 * q + e < C ? __ldg(bias + 8 * q + e) : 0.f);
-        }
-        if (scores.ptr) {
-#pragma unroll
-            for (int c = 0; c < 4 * NV4; ++c)
-                if (c < C) scores.ptr[r * scores.ld + c] = v[c];
-        }
+        Pack8 x;
+        x.zero();
+        x.add_planes(*reinterpret_cast<const uint4*>(NT.hi + r * NT.ld), *reinterpret_cast<const uint4*>(NT.lo + r * NT.ld));
+        if (Tself.hi)
+            x.add_planes(*reinterpret_cast<const uint4*>(Tself.hi + r * Tself.ld), *reinterpret_cast<const uint4*>(Tself.lo + r * Tself.ld));
         float zmax = -INFINITY;
 #pragma unroll
-        for (int c = 0; c < 4 * NV4; ++c) {
-            if (c >= C) v[c] = -INFINITY;
-            zmax = fmaxf(zmax, v[c]);
+        for (int c = 0; c < 8; ++c) {
+            x.v[c] = c < C ? x.v[c] + __ldg(bias + c) : -INFINITY;
+            zmax = fmaxf(zmax, x.v[c]);
+            if (scores.ptr && c < C) scores.ptr[r * scores.ld + c] = x.v[c];
         }
         float sum = 0.f, zl = 0.f;
 #pragma unroll
-        for (int c = 0; c < 4 * NV4; ++c) {
-            if (c == label) zl = v[c];
-            v[c] = c < C ? expf(v[c] - zmax) : 0.f;
-            sum += v[c];
+        for (int c = 0; c < 8; ++c) {
+            if (c == label) zl = x.v[c];
+            x.v[c] = c < C ? expf(x.v[c] - zmax) : 0.f;
+            sum += x.v[c];
         }
         loss = zmax + logf(sum) - zl;
         const float scale = 1.0f / (sum * (float)n_p);  // softmax / n_p = e * scale
         const float hot = 1.0f / (float)n_p;
-        uint4* ph = reinterpret_cast<uint4*>(dZ.hi + r * dZ.ld);
-        uint4* pl = reinterpret_cast<uint4*>(dZ.lo + r * dZ.ld);
 #pragma unroll
-        for (int q = 0; q < NV4 / 2; ++q) {
-            if (q >= n8) break;
-            Pack8 x;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int c = 8 * q + e;
-                x.v[e] = c < C ? v[c] * scale - (c == label ? hot : 0.f) : 0.f;  // padding columns stay zero
-            }
-            uint4 h, l;
-            x.to_planes_cvt(h, l);
-            ph[q] = h;
-            pl[q] = l;
-        }
+        for (int c = 0; c < 8; ++c) x.v[c] = c < C ? x.v[c] * scale - (c == label ? hot : 0.f) : 0.f;  // padding columns stay zero
+        uint4 h, l;
+        x.to_planes_cvt(h, l);
+        *reinterpret_cast<uint4*>(dZ.hi + r * dZ.ld) = h;
+        *reinterpret_cast<uint4*>(dZ.lo + r * dZ.ld) = l;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
@@ -438,8 +413,8 @@ int32_t launch_softmax_xent_head(rtma_ctx* ctx, const GroupDesc& g, Planes Tself
     if (tiles > 0) {
         KernelScope ks(ctx, KC_LOSS, s);
 #define RTMA_HEAD(LPR) softmax_xent_head_lanes_kernel<LPR><<<(unsigned)tiles, LOSS_TILE_ROWS * LPR, 0, s>>>(g, Tself, NT, params, P, bias_offset, C, yp, dZ, scores, tile_loss)
-        if (C <= 8)  // one 16-byte piece per plane: a thread per row
-            softmax_xent_head_kernel<2><<<(unsigned)tiles, LOSS_TILE_ROWS, 0, s>>>(g, Tself, NT, params, P, bias_offset, C, yp, dZ, scores, tile_loss);
+        if (C <= 8)
+            softmax_xent_head_kernel<<<(unsigned)tiles, LOSS_TILE_ROWS, 0, s>>>(g, Tself, NT, params, P, bias_offset, C, yp, dZ, scores, tile_loss);
         else if (C <= 16) RTMA_HEAD(2);
         else if (C <= 32) RTMA_HEAD(4);
         else RTMA_HEAD(8);
