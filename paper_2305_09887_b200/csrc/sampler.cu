@@ -53,7 +53,8 @@ constexpr int SEL_CAND = 128;   // candidates a node may have
 // bit (rounds of counting the keys that share the prefix found so far and have a 0 in the next bit, until no more keys
 // share it than are still to be kept: about log2 of the degree of them), then a pass that writes the entries below the
 // prefix and the first few that share it, in row order.
-__device__ void select_bit_by_bit(const int32_t* __restrict__ col, int64_t n, int64_t begin, int64_t deg, uint64_t vkey, int32_t fanout,
+// (A function of its own: as part of the kernel it cost the common path 15 us of the three hops.)
+__device__ __noinline__ void select_bit_by_bit(const int32_t* __restrict__ col, int64_t n, int64_t begin, int64_t deg, uint64_t vkey, int32_t fanout,
                                   uint64_t base, int64_t out, int32_t* __restrict__ block_col, int32_t* __restrict__ member) {
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
@@ -106,7 +107,7 @@ __device__ void select_bit_by_bit(const int32_t* __restrict__ col, int64_t n, in
 // or too many candidates come once in 10^6 rows up to a fan-out of 35, in 20,000 at 50, in 1,000 at 64, in 60 at 80 and in 8 at
 // SEL_FANOUT; such rows, and all that are cut to larger fan-outs, are done bit by bit.
 constexpr int SEL_FANOUT = 96;  // largest fan-out for which candidates are collected
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 5)  // with the call 54 registers otherwise, four blocks an SM: three hops 838 us, so 833
 sample_select_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, int64_t n, int64_t frontier_size,
                      const int32_t* __restrict__ frontier, int32_t fanout, double expected, uint64_t base,
                      const int64_t* __restrict__ block_rowptr, int32_t* __restrict__ block_col, int32_t* __restrict__ member) {
