@@ -964,7 +964,7 @@ int32_t launch_tc_weight_prep(rtma_ctx* ctx, const GroupDesc& g, const TcPrepJob
 // moves 96 KB through shared memory per 64 of K, two planes and 128 x 256 outputs, a third of it activations, next to what
 // the MMAs read there; a pair 64 KB each.  That pays where this main loop is the longest chain, hence from a depth K times
 // planes on.  Where the output is the longer chain the pair's blocks only wait for each other.  us alone / in pairs:
-//   two planes, 200 k rows: K = 512, 256 columns 151 / 115, gated 154 / 130; all products of a step with K = 384, 160 columns
+//   two planes, 200 k rows: K = 512, 256 columns 145 / 115, gated 150 / 127; all products of a step with K = 384, 160 columns
 //   205 / 194, gated 162 / 155; but K = 256 84 / 90, gated 90 / 95;
 //   one plane (operands rounded to bf16): K = 512, 256 columns and the layers around it 167 / 179, gated 185 / 192; K = 768, 384
 //   columns 273 / 264; K = 1024, 512 columns 359 / 335.  Gated it starts to pay later, the gate words are read with one plane

@@ -252,7 +252,7 @@ softmax_xent_head_kernel(const __grid_constant__ GroupDesc g, const Planes Tself
 
 // The head form with 9 to 64 classes: LPR lanes own a row, eight columns each, so that the loads and stores of a warp cover
 // whole pieces of rows; the maximum and the sum go over the row's lanes.  With a thread per row every load touched 32
-// lines and every store half a sector: 53 us for 200,000 rows of 47 classes (115 MB), 44 us this way; bound by the
+// lines and every store half a sector: 52 us for 200,000 rows of 47 classes (115 MB), 41 us this way; bound by the
 // instructions of 47 exponentials a row.
 template <int LPR>
 __global__ void __launch_bounds__(LOSS_TILE_ROWS * LPR)
