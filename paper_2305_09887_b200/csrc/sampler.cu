@@ -50,25 +50,27 @@ constexpr int SEL_NODES = 256 / SEL_LANES;  // nodes of a block
 constexpr int SEL_CAND = 128;   // candidates a node may have
 
 // The kept entries of one node by the whole warp, whatever its degree and the fan-out: the fanout-th smallest key bit by
-// bit (rounds of counting the keys that share the prefix found so far and have a 0 in the next bit, until no more keys
-// share it than are still to be kept: about log2 of the degree of them), then a pass that writes the entries below the
-// prefix and the first few that share it, in row order.
-// (A function of its own: as part of the kernel it cost the common path 15 us of the three hops.)
-__device__ __noinline__ void select_bit_by_bit(const int32_t* __restrict__ col, int64_t n, int64_t begin, int64_t deg, uint64_t vkey, int32_t fanout,
+// bit (rounds of counting the keys that share the prefix found so far and have a 0 in the next bit), then a pass that
+// writes the entries below the prefix and the first few that share it, in row order.  OFTEN: the rounds end as soon as no
+// more keys share the prefix than are still to be kept, after about log2 of the degree of them; where one row in a million comes
+// here the count is left out, it costs the kernel four registers and 2 % of the time of small fan-outs.
+template <bool OFTEN>
+__device__ void select_bit_by_bit(const int32_t* __restrict__ col, int64_t n, int64_t begin, int64_t deg, uint64_t vkey, int32_t fanout,
                                   uint64_t base, int64_t out, int32_t* __restrict__ block_col, int32_t* __restrict__ member) {
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
-    uint64_t prefix = 0, mask = 0;    // bits found so far, and which they are
+    uint64_t prefix = 0;
     int64_t want = fanout, left = deg;  // keys to be kept among those that share the prefix, and how many share it
-    for (int bit = 63; bit >= 0 && left > want; --bit) {
+    int bit = 63;
+    for (; bit >= 0 && (!OFTEN || left > want); --bit) {
+        const uint64_t above = bit == 63 ? 0ULL : ~0ULL << (bit + 1);
         int64_t zeros = 0;
         for (int64_t q = lane; q < deg; q += 32) {
             const uint64_t key = mix_step(base ^ (vkey | (uint64_t)q));
-            zeros += ((key & mask) == prefix && !((key >> bit) & 1ULL)) ? 1 : 0;
+            zeros += ((key & above) == prefix && !((key >> bit) & 1ULL)) ? 1 : 0;
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) zeros += __shfl_xor_sync(0xffffffffu, zeros, o);
-        mask |= 1ULL << bit;
         if (want > zeros) {  // the key has a 1 here; the `zeros` keys with a 0 are all smaller
             want -= zeros;
             left -= zeros;
@@ -77,6 +79,7 @@ __device__ __noinline__ void select_bit_by_bit(const int32_t* __restrict__ col, 
             left = zeros;
         }
     }
+    const uint64_t mask = OFTEN && bit >= 0 ? ~0ULL << (bit + 1) : ~0ULL;  // the bits that were found (at least one: left > want at first)
     int64_t ties_seen = 0;  // entries that share the prefix: the first `want` in row order are kept (all, or those with equal keys)
     for (int64_t q0 = 0; q0 < deg; q0 += 32) {
         const int64_t q = q0 + lane;
@@ -107,7 +110,9 @@ __device__ __noinline__ void select_bit_by_bit(const int32_t* __restrict__ col, 
 // or too many candidates come once in 10^6 rows up to a fan-out of 35, in 20,000 at 50, in 1,000 at 64, in 60 at 80 and in 8 at
 // SEL_FANOUT; such rows, and all that are cut to larger fan-outs, are done bit by bit.
 constexpr int SEL_FANOUT = 96;  // largest fan-out for which candidates are collected
-__global__ void __launch_bounds__(256, 5)  // with the call 54 registers otherwise, four blocks an SM: three hops 838 us, so 833
+constexpr int SEL_RARE = 35;    // largest fan-out at which a row without the right number of them is one in a million
+template <bool OFTEN>
+__global__ void __launch_bounds__(256)
 sample_select_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, int64_t n, int64_t frontier_size,
                      const int32_t* __restrict__ frontier, int32_t fanout, double expected, uint64_t base,
                      const int64_t* __restrict__ block_rowptr, int32_t* __restrict__ block_col, int32_t* __restrict__ member) {
@@ -180,7 +185,7 @@ sample_select_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restri
     for (unsigned rest = __ballot_sync(0xffffffffu, sel && !ok && sl == 0); rest; rest &= rest - 1) {
         const int from = __ffs(rest) - 1;
         const int64_t b = __shfl_sync(0xffffffffu, begin, from), d = __shfl_sync(0xffffffffu, deg, from), o = __shfl_sync(0xffffffffu, out, from);
-        select_bit_by_bit(col, n, b, d, __shfl_sync(0xffffffffu, vkey, from), fanout, base, o, block_col, member);
+        select_bit_by_bit<OFTEN>(col, n, b, d, __shfl_sync(0xffffffffu, vkey, from), fanout, base, o, block_col, member);
     }
 }
 
@@ -241,7 +246,7 @@ extern "C" int32_t rtma_sample_hop(rtma_ctx* ctx, int64_t n, const int64_t* rowp
         KernelScope ks(ctx, KC_LINK, stream);
         // candidates per row (see the kernel)
         const double expected = std::min((double)fanout + 6.0 * std::sqrt((double)fanout) + 16.0, 0.5 * ((double)fanout + SEL_CAND));
-        sample_select_kernel<<<(unsigned)ceil_div(frontier_size, SEL_NODES), 256, 0, stream>>>(
+        (fanout > SEL_RARE ? sample_select_kernel<true> : sample_select_kernel<false>)<<<(unsigned)ceil_div(frontier_size, SEL_NODES), 256, 0, stream>>>(
             rowptr, col, n, frontier_size, frontier, fanout, expected, base, block_rowptr, block_col, member);
     }
     RTMA_LAUNCH_CHECK(ctx);
