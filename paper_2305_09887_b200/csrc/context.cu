@@ -238,6 +238,7 @@ __device__ __forceinline__ int64_t block_exclusive_scan(int64_t v, int64_t* tota
 
 __global__ void __launch_bounds__(SCAN_THREADS) scan_reduce_kernel(const int32_t* __restrict__ in, int64_t n,
                                                                     int64_t* __restrict__ block_sums) {
+    wait_for_kernel_before();
     __shared__ int64_t total;
     const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
     int64_t s = 0;
@@ -251,6 +252,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_reduce_kernel(const int32_t
 }
 
 __global__ void __launch_bounds__(1024) scan_spine_kernel(int64_t* __restrict__ block_sums, int64_t nb) {
+    wait_for_kernel_before();
     __shared__ int64_t total;
     int64_t carry = 0;
     for (int64_t start = 0; start < nb; start += blockDim.x) {
@@ -266,6 +268,7 @@ __global__ void __launch_bounds__(1024) scan_spine_kernel(int64_t* __restrict__ 
 __global__ void __launch_bounds__(SCAN_THREADS) scan_apply_kernel(const int32_t* __restrict__ in, int64_t n,
                                                                    const int64_t* __restrict__ block_sums,
                                                                    int64_t* __restrict__ out) {
+    wait_for_kernel_before();
     __shared__ int64_t total;
     const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
     int32_t v[SCAN_ITEMS];
@@ -292,11 +295,11 @@ size_t scan_scratch_elems(int64_t n) { return (size_t)ceil_div(n + 1, SCAN_TILE)
 int32_t exclusive_scan_i32_to_i64(rtma_ctx* ctx, const int32_t* in, int64_t n, int64_t* out,
                                   int64_t* scratch, cudaStream_t stream) {
     const int64_t nb = ceil_div(n + 1, SCAN_TILE);
-    { KernelScope ks(ctx, KC_SCAN, stream); scan_reduce_kernel<<<(unsigned)nb, SCAN_THREADS, 0, stream>>>(in, n, scratch); }
+    { KernelScope ks(ctx, KC_SCAN, stream); launch_kernel(scan_reduce_kernel, (unsigned)nb, SCAN_THREADS, 0, stream, in, n, scratch); }
     RTMA_LAUNCH_CHECK(ctx);
-    { KernelScope ks(ctx, KC_SCAN, stream); scan_spine_kernel<<<1, 1024, 0, stream>>>(scratch, nb); }
+    { KernelScope ks(ctx, KC_SCAN, stream); launch_kernel(scan_spine_kernel, 1, 1024, 0, stream, scratch, nb); }
     RTMA_LAUNCH_CHECK(ctx);
-    { KernelScope ks(ctx, KC_SCAN, stream); scan_apply_kernel<<<(unsigned)nb, SCAN_THREADS, 0, stream>>>(in, n, scratch, out); }
+    { KernelScope ks(ctx, KC_SCAN, stream); launch_kernel(scan_apply_kernel, (unsigned)nb, SCAN_THREADS, 0, stream, in, n, scratch, out); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }

@@ -17,6 +17,7 @@ template <int NSRC, int C>
 __global__ void __launch_bounds__(DN_THREADS)
 dgrad_narrow_kernel(const __grid_constant__ GroupDesc g, const LayerShape ls, const float* __restrict__ params,
                     const Planes dZ, const Planes Q, const Planes H, const int gate) {
+    wait_for_kernel_before();
     int k, r0;
     if (!locate_tile(g, DN_TILE_ROWS, blockIdx.x, &k, &r0)) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -97,7 +98,7 @@ int32_t launch_dgrad_narrow(rtma_ctx* ctx, const GroupDesc& g, LayerShape ls, co
     const int gt = gate ? 1 : 0;
     {
         KernelScope ks(ctx, KC_GEMM_DGRAD, s);
-#define RTMA_DN(NS, CC) dgrad_narrow_kernel<NS, CC><<<(unsigned)tiles, DN_THREADS, 0, s>>>(g, ls, params, dZ, Q, H, gt)
+#define RTMA_DN(NS, CC) launch_kernel(dgrad_narrow_kernel<NS, CC>, (unsigned)tiles, DN_THREADS, 0, s, g, ls, params, dZ, Q, H, gt)
         const int key = ls.nsrc * 10 + ls.d_out;
         switch (key) {
             case 11: RTMA_DN(1, 1); break;

@@ -97,6 +97,7 @@ __host__ __device__ inline int prep_tiles(int npad, int k) { return (npad + PREP
 __global__ void __launch_bounds__(256)
 tc_weight_prep_kernel(const __grid_constant__ GroupDesc g, const __grid_constant__ PrepBatch batch,
                       const float* __restrict__ params) {
+    wait_for_kernel_before();
     __shared__ float tile[PREP_K][PREP_ROWS + 1];
     const PrepArgs& a = batch.job[blockIdx.z];
     const int k = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -273,6 +274,7 @@ __device__ __forceinline__ void rows_body(const RowsArgs& a) {
     __syncthreads();
     if constexpr (PAIR) tc::cluster_sync();  // both blocks' barriers and tensor memory exist before either is signalled
     tc::tc_fence_after_sync();
+    wait_for_kernel_before();
     const uint32_t tmem_base = pb.tmem_base;
 
     if (warp == 0) {
@@ -621,6 +623,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
     const bool bias_tile = blockIdx.x == 0;  // these blocks also produce the bias gradient of their columns
 
     if (KB == 0) {  // empty chunk: the gradient contribution is zero
+        wait_for_kernel_before();
         for (int t = 0; t < na_tiles; ++t)
             for (int idx = threadIdx.x; idx < TC_BM * ccount; idx += TC_THREADS) {
                 const int j = j0_of[t] + idx / ccount;
@@ -671,6 +674,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
     tc::tc_fence_before_sync();
     __syncthreads();
     tc::tc_fence_after_sync();
+    wait_for_kernel_before();
     const uint32_t tmem_base = pb.tmem_base;
 
     if (warp == 0) {
@@ -827,6 +831,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
 // self-test of the bounded wait: a barrier nothing ever arrives at
 // ------------------------------------------------------------------------------------
 __global__ void wait_selftest_kernel(int* error_word, int polls) {
+    wait_for_kernel_before();
     __shared__ uint64_t bar;
     if (threadIdx.x == 0) {
         tc::mbar_init(&bar, 1);
@@ -842,7 +847,7 @@ __global__ void wait_selftest_kernel(int* error_word, int polls) {
 extern "C" int32_t rtma_selftest_wait_timeout(rtma_ctx* ctx, void* stream) {
     if (!ctx) return RTMA_ERR_INVALID_ARG;
     RTMA_CUDA(ctx, cudaSetDevice(ctx->device));
-    wait_selftest_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(ctx->error_word, 1 << 10);
+    launch_kernel(wait_selftest_kernel, 1, 32, 0, static_cast<cudaStream_t>(stream), ctx->error_word, 1 << 10);
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }
@@ -955,7 +960,7 @@ int32_t launch_tc_weight_prep(rtma_ctx* ctx, const GroupDesc& g, const TcPrepJob
         most = std::max(most, prep_tiles(p.Npad_f, p.Kf) + (jobs[j].Bd_hi ? prep_tiles(p.Npad_d, p.Kd) : 0));
     }
     dim3 grid((unsigned)most, (unsigned)g.num, (unsigned)njobs);
-    { KernelScope ks(ctx, KC_WEIGHT_PREP, s); tc_weight_prep_kernel<<<grid, 256, 0, s>>>(g, b, params); }
+    { KernelScope ks(ctx, KC_WEIGHT_PREP, s); launch_kernel(tc_weight_prep_kernel, grid, 256, 0, s, g, b, params); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }
@@ -1009,7 +1014,7 @@ static int32_t launch_rows(rtma_ctx* ctx, RowsArgs& a, int64_t rows_total, bool 
     {
         KernelScope ks(ctx, kclass, s);
         const int out = !a.out_planes.hi ? OUT_F32 : a.gate_hi ? OUT_GATED : OUT_PLANES;
-        rows_kernels[pairs ? 1 : 0][half ? 1 : 0][out]<<<grid, ROWS_THREADS, smem, s>>>(a);
+        launch_kernel(rows_kernels[pairs ? 1 : 0][half ? 1 : 0][out], grid, ROWS_THREADS, smem, s, a);
     }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
@@ -1134,7 +1139,7 @@ int32_t launch_tc_wgrad(rtma_ctx* ctx, const GroupDesc& g, const SplitPlan& sp, 
         a.mapHl = a.mapNl;
     }
     dim3 grid((unsigned)ceil_div(ls.nsrc * a.jt_per_src, 2), (unsigned)slots, (unsigned)ceil_div(a.n_atoms, 4));
-    { KernelScope ks(ctx, KC_GEMM_WGRAD, s); tc_wgrad_kernel<<<grid, TC_THREADS, a.stages * stage_bytes + 1024, s>>>(a); }
+    { KernelScope ks(ctx, KC_GEMM_WGRAD, s); launch_kernel(tc_wgrad_kernel, grid, TC_THREADS, a.stages * stage_bytes + 1024, s, a); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }

@@ -27,6 +27,7 @@ constexpr int CSR_WARPS = CSR_THREADS / 32;
 // part8[v] = part_id[v] as one byte (at most 64 parts), four nodes per thread
 __global__ void __launch_bounds__(256)
 pack_parts_kernel(int64_t n, const int32_t* __restrict__ part_id, uint8_t* __restrict__ part8, const bool aligned) {
+    wait_for_kernel_before();
     const int64_t i = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4;
     if (aligned && i + 3 < n) {
         const int4 p = *reinterpret_cast<const int4*>(part_id + i);
@@ -42,6 +43,7 @@ induced_count_kernel(int64_t n, int M, const RowT* __restrict__ rowptr, const in
                      const uint8_t* __restrict__ part8, const int64_t* __restrict__ part_offsets,
                      const int32_t* __restrict__ local_id, int32_t* __restrict__ counts,
                      uint32_t* __restrict__ keep_bits) {
+    wait_for_kernel_before();
     const int lane = threadIdx.x & 31;
     const int64_t u = (int64_t)blockIdx.x * CSR_WARPS + (threadIdx.x >> 5);
     if (u >= n) return;
@@ -82,6 +84,7 @@ induced_offsets_kernel(int64_t n, int M, const int64_t* __restrict__ part_offset
                        const int64_t* __restrict__ slots, const RowT* __restrict__ rowptr,
                        int64_t* __restrict__ rowptr_out, int64_t* __restrict__ edge_offsets,
                        int64_t* __restrict__ kept_cut) {
+    wait_for_kernel_before();
     __shared__ int64_t offs[RTMA_MAX_PARTS + 1];
     for (int b = threadIdx.x; b <= M; b += CSR_THREADS) offs[b] = part_offsets[b];
     __syncthreads();
@@ -113,6 +116,7 @@ induced_fill_kernel(int64_t n, int M, const RowT* __restrict__ rowptr, const int
                     const int32_t* __restrict__ local_id,
                     const int64_t* __restrict__ rowptr_out, const int64_t* __restrict__ edge_offsets,
                     int32_t* __restrict__ col_out) {
+    wait_for_kernel_before();
     const int lane = threadIdx.x & 31;
     const int64_t u = (int64_t)blockIdx.x * CSR_WARPS + (threadIdx.x >> 5);
     if (u >= n) return;
@@ -148,6 +152,7 @@ induced_fill_bits_kernel(int64_t n, int M, const RowT* __restrict__ rowptr, cons
                          const int32_t* __restrict__ local_id, const int64_t* __restrict__ rowptr_out,
                          const int64_t* __restrict__ edge_offsets, const uint32_t* __restrict__ keep_bits,
                          int32_t* __restrict__ col_out) {
+    wait_for_kernel_before();
     const int lane = threadIdx.x & 31;
     const int64_t u = (int64_t)blockIdx.x * CSR_THREADS + threadIdx.x;
     int64_t begin = 0, end = 0, out = 0;
@@ -203,6 +208,7 @@ template <int VEC_BYTES>
 __global__ void __launch_bounds__(256)
 gather_rows_kernel(int64_t n, int64_t row_bytes, const char* __restrict__ src, const int32_t* __restrict__ perm,
                    char* __restrict__ dst) {
+    wait_for_kernel_before();
     const int lane = threadIdx.x & 31;
     const int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (i >= n) return;
@@ -223,6 +229,7 @@ gather_rows_kernel(int64_t n, int64_t row_bytes, const char* __restrict__ src, c
 // rows of 4 bytes (labels, ids): one thread per row
 __global__ void __launch_bounds__(256)
 gather_words_kernel(int64_t n, const int32_t* __restrict__ src, const int32_t* __restrict__ perm, int32_t* __restrict__ dst) {
+    wait_for_kernel_before();
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (i < n && rtma_index_ok(perm[i], n, 4)) dst[i] = __ldg(src + perm[i]);
 }
@@ -249,7 +256,7 @@ extern "C" int32_t rtma_build_induced_csr(rtma_ctx* ctx, int64_t n, int32_t rowp
         if (n == 0) return RTMA_OK;
         RTMA_TRY(rtma_reserve(ctx, ArenaCursor::granule((size_t)n + 16)));
         uint8_t* part8 = reinterpret_cast<uint8_t*>(ctx->arena);
-        { KernelScope ks(ctx, KC_CSR_FILL, stream); pack_parts_kernel<<<pack_blocks, 256, 0, stream>>>(n, part_id, part8, reinterpret_cast<uintptr_t>(part_id) % 16 == 0); }
+        { KernelScope ks(ctx, KC_CSR_FILL, stream); launch_kernel(pack_parts_kernel, pack_blocks, 256, 0, stream, n, part_id, part8, reinterpret_cast<uintptr_t>(part_id) % 16 == 0); }
         RTMA_LAUNCH_CHECK(ctx);
         // the bits of the COUNT phase, if that was the last one and ran on these very arrays
         const bool from_bits = ctx->keep_bits && ctx->keep_n == n && ctx->keep_M == M && ctx->keep_rowptr == rowptr &&
@@ -258,19 +265,19 @@ extern "C" int32_t rtma_build_induced_csr(rtma_ctx* ctx, int64_t n, int32_t rowp
         if (from_bits) {
             const unsigned thread_blocks = (unsigned)ceil_div(n, CSR_THREADS);
             if (rowptr_is_64)
-                induced_fill_bits_kernel<int64_t><<<thread_blocks, CSR_THREADS, 0, stream>>>(
+                launch_kernel(induced_fill_bits_kernel<int64_t>, thread_blocks, CSR_THREADS, 0, stream,
                     n, M, static_cast<const int64_t*>(rowptr), col, part8, part_offsets, local_id, rowptr_out, edge_offsets,
                     ctx->keep_bits, col_out);
             else
-                induced_fill_bits_kernel<int32_t><<<thread_blocks, CSR_THREADS, 0, stream>>>(
+                launch_kernel(induced_fill_bits_kernel<int32_t>, thread_blocks, CSR_THREADS, 0, stream,
                     n, M, static_cast<const int32_t*>(rowptr), col, part8, part_offsets, local_id, rowptr_out, edge_offsets,
                     ctx->keep_bits, col_out);
         } else if (rowptr_is_64) {
-            induced_fill_kernel<int64_t><<<row_blocks, CSR_THREADS, 0, stream>>>(
+            launch_kernel(induced_fill_kernel<int64_t>, row_blocks, CSR_THREADS, 0, stream,
                 n, M, static_cast<const int64_t*>(rowptr), col, part8, part_offsets, local_id, rowptr_out,
                 edge_offsets, col_out);
         } else {
-            induced_fill_kernel<int32_t><<<row_blocks, CSR_THREADS, 0, stream>>>(
+            launch_kernel(induced_fill_kernel<int32_t>, row_blocks, CSR_THREADS, 0, stream,
                 n, M, static_cast<const int32_t*>(rowptr), col, part8, part_offsets, local_id, rowptr_out,
                 edge_offsets, col_out);
         }
@@ -314,13 +321,13 @@ extern "C" int32_t rtma_build_induced_csr(rtma_ctx* ctx, int64_t n, int32_t rowp
             }
             if (ctx->keep_bits && ctx->keep_words >= words) keep_bits = ctx->keep_bits;
         }
-        { KernelScope ks(ctx, KC_CSR_COUNT, stream); pack_parts_kernel<<<pack_blocks, 256, 0, stream>>>(n, part_id, part8, reinterpret_cast<uintptr_t>(part_id) % 16 == 0); }
+        { KernelScope ks(ctx, KC_CSR_COUNT, stream); launch_kernel(pack_parts_kernel, pack_blocks, 256, 0, stream, n, part_id, part8, reinterpret_cast<uintptr_t>(part_id) % 16 == 0); }
         RTMA_LAUNCH_CHECK(ctx);
         if (rowptr_is_64)
-            { KernelScope ks(ctx, KC_CSR_COUNT, stream); induced_count_kernel<int64_t><<<row_blocks, CSR_THREADS, 0, stream>>>(
+            { KernelScope ks(ctx, KC_CSR_COUNT, stream); launch_kernel(induced_count_kernel<int64_t>, row_blocks, CSR_THREADS, 0, stream,
                 n, M, static_cast<const int64_t*>(rowptr), col, part8, part_offsets, local_id, counts, keep_bits); }
         else
-            { KernelScope ks(ctx, KC_CSR_COUNT, stream); induced_count_kernel<int32_t><<<row_blocks, CSR_THREADS, 0, stream>>>(
+            { KernelScope ks(ctx, KC_CSR_COUNT, stream); launch_kernel(induced_count_kernel<int32_t>, row_blocks, CSR_THREADS, 0, stream,
                 n, M, static_cast<const int32_t*>(rowptr), col, part8, part_offsets, local_id, counts, keep_bits); }
         RTMA_LAUNCH_CHECK(ctx);
         if (keep_bits) {
@@ -334,10 +341,10 @@ extern "C" int32_t rtma_build_induced_csr(rtma_ctx* ctx, int64_t n, int32_t rowp
     RTMA_TRY(exclusive_scan_i32_to_i64(ctx, counts, n, slots, scratch, stream));
     const unsigned off_blocks = (unsigned)ceil_div(n + M, CSR_THREADS);
     if (rowptr_is_64)
-        { KernelScope ks(ctx, KC_CSR_OFFSETS, stream); induced_offsets_kernel<int64_t><<<off_blocks, CSR_THREADS, 0, stream>>>(
+        { KernelScope ks(ctx, KC_CSR_OFFSETS, stream); launch_kernel(induced_offsets_kernel<int64_t>, off_blocks, CSR_THREADS, 0, stream,
             n, M, part_offsets, slots, static_cast<const int64_t*>(rowptr), rowptr_out, edge_offsets, kept_cut); }
     else
-        { KernelScope ks(ctx, KC_CSR_OFFSETS, stream); induced_offsets_kernel<int32_t><<<off_blocks, CSR_THREADS, 0, stream>>>(
+        { KernelScope ks(ctx, KC_CSR_OFFSETS, stream); launch_kernel(induced_offsets_kernel<int32_t>, off_blocks, CSR_THREADS, 0, stream,
             n, M, part_offsets, slots, static_cast<const int32_t*>(rowptr), rowptr_out, edge_offsets, kept_cut); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
@@ -355,13 +362,13 @@ extern "C" int32_t rtma_gather_rows(rtma_ctx* ctx, int64_t n, int64_t row_bytes,
     const unsigned blocks = (unsigned)ceil_div(n, 8);
     const uintptr_t align = reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst) | (uintptr_t)row_bytes;
     if (row_bytes == 4 && align % 4 == 0)
-        { KernelScope ks(ctx, KC_GATHER_ROWS, stream); gather_words_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, stream>>>(n, static_cast<const int32_t*>(src), perm, static_cast<int32_t*>(dst)); }
+        { KernelScope ks(ctx, KC_GATHER_ROWS, stream); launch_kernel(gather_words_kernel, (unsigned)ceil_div(n, 256), 256, 0, stream, n, static_cast<const int32_t*>(src), perm, static_cast<int32_t*>(dst)); }
     else if (align % 16 == 0)
-        { KernelScope ks(ctx, KC_GATHER_ROWS, stream); gather_rows_kernel<16><<<blocks, 256, 0, stream>>>(n, row_bytes, static_cast<const char*>(src), perm, static_cast<char*>(dst)); }
+        { KernelScope ks(ctx, KC_GATHER_ROWS, stream); launch_kernel(gather_rows_kernel<16>, blocks, 256, 0, stream, n, row_bytes, static_cast<const char*>(src), perm, static_cast<char*>(dst)); }
     else if (align % 4 == 0)
-        { KernelScope ks(ctx, KC_GATHER_ROWS, stream); gather_rows_kernel<4><<<blocks, 256, 0, stream>>>(n, row_bytes, static_cast<const char*>(src), perm, static_cast<char*>(dst)); }
+        { KernelScope ks(ctx, KC_GATHER_ROWS, stream); launch_kernel(gather_rows_kernel<4>, blocks, 256, 0, stream, n, row_bytes, static_cast<const char*>(src), perm, static_cast<char*>(dst)); }
     else
-        { KernelScope ks(ctx, KC_GATHER_ROWS, stream); gather_rows_kernel<1><<<blocks, 256, 0, stream>>>(n, row_bytes, static_cast<const char*>(src), perm, static_cast<char*>(dst)); }
+        { KernelScope ks(ctx, KC_GATHER_ROWS, stream); launch_kernel(gather_rows_kernel<1>, blocks, 256, 0, stream, n, row_bytes, static_cast<const char*>(src), perm, static_cast<char*>(dst)); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }

@@ -23,6 +23,7 @@ __device__ __forceinline__ void load_pack(const Planes m, int64_t r, int col, Pa
 __global__ void __launch_bounds__(32 * PAIR_WARPS)
 pair_product_kernel(const __grid_constant__ GroupDesc gd, const __grid_constant__ GroupDesc g, const Planes R,
                     const int32_t* __restrict__ pu, const int32_t* __restrict__ pv, const Planes E, const int d) {
+    wait_for_kernel_before();
     int k, r0;
     if (!locate_tile(gd, PAIR_WARPS, blockIdx.x, &k, &r0)) return;
     const int lane = threadIdx.x & 31, i = r0 + (threadIdx.x >> 5);
@@ -54,6 +55,7 @@ __global__ void __launch_bounds__(32 * PAIR_WARPS)
 pair_scatter_kernel(const __grid_constant__ GroupDesc gd, const __grid_constant__ GroupDesc g, const Planes R,
                     const int32_t* __restrict__ pu, const int32_t* __restrict__ pv, const Planes dE,
                     float* __restrict__ dR, const int64_t ld, const int d) {
+    wait_for_kernel_before();
     int k, r0;
     if (!locate_tile(gd, PAIR_WARPS, blockIdx.x, &k, &r0)) return;
     const int lane = threadIdx.x & 31, i = r0 + (threadIdx.x >> 5);
@@ -80,6 +82,7 @@ pair_scatter_kernel(const __grid_constant__ GroupDesc gd, const __grid_constant_
 __global__ void __launch_bounds__(256)
 scratch_to_planes_kernel(const __grid_constant__ GroupDesc g, const float* __restrict__ src, const int64_t ld, const int d,
                          const Planes out) {
+    wait_for_kernel_before();
     int k, r0;
     if (!locate_tile(g, 32, blockIdx.x, &k, &r0)) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -103,6 +106,7 @@ scratch_to_planes_kernel(const __grid_constant__ GroupDesc g, const float* __res
 __global__ void __launch_bounds__(BCE_TILE)
 bce_kernel(const __grid_constant__ GroupDesc gd, const Planes S, const int32_t* __restrict__ label,
            float* __restrict__ tile_loss, float* __restrict__ score_out) {
+    wait_for_kernel_before();
     __shared__ float part[BCE_TILE];
     int k, r0;
     if (!locate_tile(gd, BCE_TILE, blockIdx.x, &k, &r0)) return;
@@ -135,7 +139,7 @@ int32_t launch_pair_product(rtma_ctx* ctx, const GroupDesc& gd, const GroupDesc&
                             const int32_t* pv, Planes E, int d, cudaStream_t s) {
     const int64_t tiles = group_tiles(gd, PAIR_WARPS);
     if (tiles == 0) return RTMA_OK;
-    { KernelScope ks(ctx, KC_LINK, s); pair_product_kernel<<<(unsigned)tiles, 32 * PAIR_WARPS, 0, s>>>(gd, g, R, pu, pv, E, d); }
+    { KernelScope ks(ctx, KC_LINK, s); launch_kernel(pair_product_kernel, (unsigned)tiles, 32 * PAIR_WARPS, 0, s, gd, g, R, pu, pv, E, d); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }
@@ -145,13 +149,13 @@ int32_t launch_pair_scatter(rtma_ctx* ctx, const GroupDesc& gd, const GroupDesc&
     const int64_t tiles = group_tiles(gd, PAIR_WARPS);
     if (tiles > 0) {
         KernelScope ks(ctx, KC_LINK, s);
-        pair_scatter_kernel<<<(unsigned)tiles, 32 * PAIR_WARPS, 0, s>>>(gd, g, R, pu, pv, dE, dR, ld, d);
+        launch_kernel(pair_scatter_kernel, (unsigned)tiles, 32 * PAIR_WARPS, 0, s, gd, g, R, pu, pv, dE, dR, ld, d);
     }
     RTMA_LAUNCH_CHECK(ctx);
     const int64_t node_tiles = group_tiles(g, 32);
     if (node_tiles > 0) {
         KernelScope ks(ctx, KC_LINK, s);
-        scratch_to_planes_kernel<<<(unsigned)node_tiles, 256, 0, s>>>(g, dR, ld, d, dR_planes);
+        launch_kernel(scratch_to_planes_kernel, (unsigned)node_tiles, 256, 0, s, g, dR, ld, d, dR_planes);
     }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
@@ -161,7 +165,7 @@ int32_t launch_bce(rtma_ctx* ctx, const GroupDesc& gd, Planes S, const int32_t* 
                    float* score_out, cudaStream_t s) {
     const int64_t tiles = group_tiles(gd, BCE_TILE);
     if (tiles == 0) return RTMA_OK;
-    { KernelScope ks(ctx, KC_LINK, s); bce_kernel<<<(unsigned)tiles, BCE_TILE, 0, s>>>(gd, S, label, tile_loss, score_out); }
+    { KernelScope ks(ctx, KC_LINK, s); launch_kernel(bce_kernel, (unsigned)tiles, BCE_TILE, 0, s, gd, S, label, tile_loss, score_out); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }

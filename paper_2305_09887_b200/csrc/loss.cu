@@ -28,6 +28,7 @@ template <int J>
 __global__ void __launch_bounds__(LOSS_THREADS)
 softmax_xent_kernel(const __grid_constant__ GroupDesc g, const Mat logits, const int C, const int32_t* __restrict__ yp,
                     const Planes dZ, float* __restrict__ tile_loss) {
+    wait_for_kernel_before();
     __shared__ float warp_loss[LOSS_THREADS / 32];
     int k, r0;
     if (!locate_tile(g, LOSS_TILE_ROWS, blockIdx.x, &k, &r0)) return;
@@ -129,6 +130,7 @@ template <int NV4>
 __global__ void __launch_bounds__(LOSS_TILE_ROWS)
 softmax_xent_row_kernel(const __grid_constant__ GroupDesc g, const Mat logits, const int C, const int32_t* __restrict__ yp,
                         const Planes dZ, float* __restrict__ tile_loss) {
+    wait_for_kernel_before();
     __shared__ float warp_loss[LOSS_TILE_ROWS / 32];
     int k, r0;
     if (!locate_tile(g, LOSS_TILE_ROWS, blockIdx.x, &k, &r0)) return;
@@ -200,6 +202,7 @@ __global__ void __launch_bounds__(LOSS_TILE_ROWS)
 softmax_xent_head_kernel(const __grid_constant__ GroupDesc g, const Planes Tself, const Planes NT,
                          const float* __restrict__ params, const int64_t P, const int64_t bias_offset, const int C,
                          const int32_t* __restrict__ yp, const Planes dZ, const Mat scores, float* __restrict__ tile_loss) {
+    wait_for_kernel_before();
     __shared__ float warp_loss[LOSS_TILE_ROWS / 32];
     int k, r0;
     if (!locate_tile(g, LOSS_TILE_ROWS, blockIdx.x, &k, &r0)) return;
@@ -259,6 +262,7 @@ __global__ void __launch_bounds__(LOSS_TILE_ROWS * LPR)
 softmax_xent_head_lanes_kernel(const __grid_constant__ GroupDesc g, const Planes Tself, const Planes NT,
                                const float* __restrict__ params, const int64_t P, const int64_t bias_offset, const int C,
                                const int32_t* __restrict__ yp, const Planes dZ, const Mat scores, float* __restrict__ tile_loss) {
+    wait_for_kernel_before();
     constexpr int WARPS = LOSS_TILE_ROWS * LPR / 32;
     __shared__ float warp_loss[WARPS];
     int k, r0;
@@ -326,6 +330,7 @@ softmax_xent_head_lanes_kernel(const __grid_constant__ GroupDesc g, const Planes
 __global__ void __launch_bounds__(LOSS_THREADS)
 softmax_xent_wide_kernel(const __grid_constant__ GroupDesc g, const Mat logits, const int C, const int32_t* __restrict__ yp,
                          const Planes dZ, float* __restrict__ tile_loss) {
+    wait_for_kernel_before();
     __shared__ float warp_loss[LOSS_THREADS / 32];
     int k, r0;
     if (!locate_tile(g, LOSS_TILE_ROWS, blockIdx.x, &k, &r0)) return;
@@ -368,6 +373,7 @@ softmax_xent_wide_kernel(const __grid_constant__ GroupDesc g, const Mat logits, 
 __global__ void __launch_bounds__(256)
 loss_finalize_kernel(const __grid_constant__ GroupDesc g, const float* __restrict__ tile_loss,
                      float* __restrict__ loss_out, const int64_t loss_stride, const int64_t loss_col) {
+    wait_for_kernel_before();
     __shared__ float red[256];
     const int k = blockIdx.x;
     int64_t first = 0;
@@ -394,12 +400,12 @@ int32_t launch_softmax_xent(rtma_ctx* ctx, const GroupDesc& g, Mat logits, int C
     const int64_t tiles = group_tiles(g, LOSS_TILE_ROWS);
     if (tiles > 0) {
         KernelScope ks(ctx, KC_LOSS, s);
-        if (C <= 16) softmax_xent_row_kernel<4><<<(unsigned)tiles, LOSS_TILE_ROWS, 0, s>>>(g, logits, C, yp, dZ, tile_loss);
-        else if (C <= 32) softmax_xent_row_kernel<8><<<(unsigned)tiles, LOSS_TILE_ROWS, 0, s>>>(g, logits, C, yp, dZ, tile_loss);
-        else if (C <= 48) softmax_xent_row_kernel<12><<<(unsigned)tiles, LOSS_TILE_ROWS, 0, s>>>(g, logits, C, yp, dZ, tile_loss);
-        else if (C <= 64) softmax_xent_row_kernel<16><<<(unsigned)tiles, LOSS_TILE_ROWS, 0, s>>>(g, logits, C, yp, dZ, tile_loss);
-        else if (C <= LOSS_REG_CLASSES) softmax_xent_kernel<4><<<(unsigned)tiles, LOSS_THREADS, 0, s>>>(g, logits, C, yp, dZ, tile_loss);
-        else softmax_xent_wide_kernel<<<(unsigned)tiles, LOSS_THREADS, 0, s>>>(g, logits, C, yp, dZ, tile_loss);
+        if (C <= 16) launch_kernel(softmax_xent_row_kernel<4>, (unsigned)tiles, LOSS_TILE_ROWS, 0, s, g, logits, C, yp, dZ, tile_loss);
+        else if (C <= 32) launch_kernel(softmax_xent_row_kernel<8>, (unsigned)tiles, LOSS_TILE_ROWS, 0, s, g, logits, C, yp, dZ, tile_loss);
+        else if (C <= 48) launch_kernel(softmax_xent_row_kernel<12>, (unsigned)tiles, LOSS_TILE_ROWS, 0, s, g, logits, C, yp, dZ, tile_loss);
+        else if (C <= 64) launch_kernel(softmax_xent_row_kernel<16>, (unsigned)tiles, LOSS_TILE_ROWS, 0, s, g, logits, C, yp, dZ, tile_loss);
+        else if (C <= LOSS_REG_CLASSES) launch_kernel(softmax_xent_kernel<4>, (unsigned)tiles, LOSS_THREADS, 0, s, g, logits, C, yp, dZ, tile_loss);
+        else launch_kernel(softmax_xent_wide_kernel, (unsigned)tiles, LOSS_THREADS, 0, s, g, logits, C, yp, dZ, tile_loss);
         RTMA_LAUNCH_CHECK(ctx);
     }
     return launch_loss_finalize(ctx, g, tile_loss, loss_out, loss_stride, loss_col, s);
@@ -412,9 +418,9 @@ int32_t launch_softmax_xent_head(rtma_ctx* ctx, const GroupDesc& g, Planes Tself
     const int64_t tiles = group_tiles(g, LOSS_TILE_ROWS);
     if (tiles > 0) {
         KernelScope ks(ctx, KC_LOSS, s);
-#define RTMA_HEAD(LPR) softmax_xent_head_lanes_kernel<LPR><<<(unsigned)tiles, LOSS_TILE_ROWS * LPR, 0, s>>>(g, Tself, NT, params, P, bias_offset, C, yp, dZ, scores, tile_loss)
+#define RTMA_HEAD(LPR) launch_kernel(softmax_xent_head_lanes_kernel<LPR>, (unsigned)tiles, LOSS_TILE_ROWS * LPR, 0, s, g, Tself, NT, params, P, bias_offset, C, yp, dZ, scores, tile_loss)
         if (C <= 8)
-            softmax_xent_head_kernel<<<(unsigned)tiles, LOSS_TILE_ROWS, 0, s>>>(g, Tself, NT, params, P, bias_offset, C, yp, dZ, scores, tile_loss);
+            launch_kernel(softmax_xent_head_kernel, (unsigned)tiles, LOSS_TILE_ROWS, 0, s, g, Tself, NT, params, P, bias_offset, C, yp, dZ, scores, tile_loss);
         else if (C <= 16) RTMA_HEAD(2);
         else if (C <= 32) RTMA_HEAD(4);
         else RTMA_HEAD(8);
@@ -427,7 +433,7 @@ int32_t launch_softmax_xent_head(rtma_ctx* ctx, const GroupDesc& g, Planes Tself
 int32_t launch_loss_finalize(rtma_ctx* ctx, const GroupDesc& g, const float* tile_loss, float* loss_out,
                              int64_t loss_stride, int64_t loss_col, cudaStream_t s) {
     if (loss_out && g.num > 0) {
-        { KernelScope ks(ctx, KC_LOSS, s); loss_finalize_kernel<<<g.num, 256, 0, s>>>(g, tile_loss, loss_out, loss_stride, loss_col); }
+        { KernelScope ks(ctx, KC_LOSS, s); launch_kernel(loss_finalize_kernel, g.num, 256, 0, s, g, tile_loss, loss_out, loss_stride, loss_col); }
         RTMA_LAUNCH_CHECK(ctx);
     }
     return RTMA_OK;

@@ -12,6 +12,7 @@ __global__ void __launch_bounds__(256)
 reduce_sgd_kernel(const __grid_constant__ GroupDesc g, const __grid_constant__ SplitPlan sp, const LayerShape ls,
                   const float* __restrict__ partial, const float lr, float* __restrict__ params,
                   float* __restrict__ grads_record) {
+    wait_for_kernel_before();
     const int k = blockIdx.y;
     const int64_t stride = (int64_t)(ls.nsrc * ls.d_in + 1) * ls.d_out;  // the weight matrices and the bias row
     const int64_t count = ls.has_bias ? stride : stride - ls.d_out;       // the bias row is last
@@ -31,6 +32,7 @@ __global__ void __launch_bounds__(256)
 reduce_sgd_head_kernel(const __grid_constant__ GroupDesc g, const __grid_constant__ SplitPlan sp, const LayerShape ls,
                        const int cp, const float* __restrict__ partial, const float lr, float* __restrict__ params,
                        float* __restrict__ grads_record) {
+    wait_for_kernel_before();
     const int k = blockIdx.y;
     const int64_t count = (int64_t)(ls.nsrc * ls.d_in + 1) * ls.d_out;  // the layer's parameters: weight matrices, bias
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
@@ -53,6 +55,7 @@ reduce_sgd_head_kernel(const __grid_constant__ GroupDesc g, const __grid_constan
 __global__ void __launch_bounds__(256)
 copy_rows_kernel(const float* __restrict__ src, const int64_t ld_src, float* __restrict__ dst, const int64_t ld_dst,
                  const int64_t rows, const int width) {
+    wait_for_kernel_before();
     const int64_t total = rows * width;
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < total; i += (int64_t)gridDim.x * 256) {
         const int64_t r = i / width;
@@ -67,6 +70,7 @@ template <int VEC, bool WITH_GRADS>
 __global__ void __launch_bounds__(256)
 aggregate_kernel(float* __restrict__ params, const float* __restrict__ grads, const float lr, const int64_t P,
                  const int M, const uint64_t active, float* __restrict__ global_out) {
+    wait_for_kernel_before();
     const float inv_m = 1.0f / (float)__popcll(active);
     const int64_t packs = P / VEC;
     for (int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x; j < packs; j += (int64_t)gridDim.x * 256) {
@@ -130,11 +134,11 @@ int32_t aggregate_impl(rtma_ctx* ctx, float* params, const float* grads, float l
     const int64_t packs = vec ? P / 4 : P;
     const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(packs, 256), (int64_t)sm_count(ctx->device) * 8);
     if (vec) {
-        if (grads) { KernelScope ks(ctx, KC_AGGREGATE, stream); aggregate_kernel<4, true><<<grid, 256, 0, stream>>>(params, grads, lr, P, M, active, global_out); }
-        else { KernelScope ks(ctx, KC_AGGREGATE, stream); aggregate_kernel<4, false><<<grid, 256, 0, stream>>>(params, nullptr, 0.f, P, M, active, global_out); }
+        if (grads) { KernelScope ks(ctx, KC_AGGREGATE, stream); launch_kernel(aggregate_kernel<4, true>, grid, 256, 0, stream, params, grads, lr, P, M, active, global_out); }
+        else { KernelScope ks(ctx, KC_AGGREGATE, stream); launch_kernel(aggregate_kernel<4, false>, grid, 256, 0, stream, params, nullptr, 0.f, P, M, active, global_out); }
     } else {
-        if (grads) { KernelScope ks(ctx, KC_AGGREGATE, stream); aggregate_kernel<1, true><<<grid, 256, 0, stream>>>(params, grads, lr, P, M, active, global_out); }
-        else { KernelScope ks(ctx, KC_AGGREGATE, stream); aggregate_kernel<1, false><<<grid, 256, 0, stream>>>(params, nullptr, 0.f, P, M, active, global_out); }
+        if (grads) { KernelScope ks(ctx, KC_AGGREGATE, stream); launch_kernel(aggregate_kernel<1, true>, grid, 256, 0, stream, params, grads, lr, P, M, active, global_out); }
+        else { KernelScope ks(ctx, KC_AGGREGATE, stream); launch_kernel(aggregate_kernel<1, false>, grid, 256, 0, stream, params, nullptr, 0.f, P, M, active, global_out); }
     }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
@@ -147,7 +151,7 @@ int32_t launch_reduce_sgd(rtma_ctx* ctx, const GroupDesc& g, const SplitPlan& sp
     if (g.num == 0) return RTMA_OK;
     const int64_t count = (int64_t)(ls.nsrc * ls.d_in + 1) * ls.d_out;
     dim3 grid((unsigned)ceil_div(count, 256), (unsigned)g.num);
-    { KernelScope ks(ctx, KC_REDUCE_SGD, s); reduce_sgd_kernel<<<grid, 256, 0, s>>>(g, sp, ls, partial, lr, params, grads_record); }
+    { KernelScope ks(ctx, KC_REDUCE_SGD, s); launch_kernel(reduce_sgd_kernel, grid, 256, 0, s, g, sp, ls, partial, lr, params, grads_record); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }
@@ -157,7 +161,7 @@ int32_t launch_reduce_sgd_head(rtma_ctx* ctx, const GroupDesc& g, const SplitPla
     if (g.num == 0) return RTMA_OK;
     const int64_t count = (int64_t)(ls.nsrc * ls.d_in + 1) * ls.d_out;
     dim3 grid((unsigned)ceil_div(count, 256), (unsigned)g.num);
-    { KernelScope ks(ctx, KC_REDUCE_SGD, s); reduce_sgd_head_kernel<<<grid, 256, 0, s>>>(g, sp, ls, head_cp, partial, lr, params, grads_record); }
+    { KernelScope ks(ctx, KC_REDUCE_SGD, s); launch_kernel(reduce_sgd_head_kernel, grid, 256, 0, s, g, sp, ls, head_cp, partial, lr, params, grads_record); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }
@@ -166,7 +170,7 @@ int32_t launch_copy_rows(rtma_ctx* ctx, const float* src, int64_t ld_src, float*
                          int width, cudaStream_t s) {
     if (rows <= 0 || width <= 0) return RTMA_OK;
     const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(rows * width, 256), 148 * 16);
-    { KernelScope ks(ctx, KC_COPY, s); copy_rows_kernel<<<grid, 256, 0, s>>>(src, ld_src, dst, ld_dst, rows, width); }
+    { KernelScope ks(ctx, KC_COPY, s); launch_kernel(copy_rows_kernel, grid, 256, 0, s, src, ld_src, dst, ld_dst, rows, width); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }

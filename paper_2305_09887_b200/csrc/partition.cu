@@ -46,6 +46,7 @@ __device__ __forceinline__ int part_of(int64_t v, const int32_t* __restrict__ gr
 __global__ void __launch_bounds__(PART_THREADS)
 part_count_kernel(int64_t n, const int32_t* __restrict__ group_id, uint64_t seed, int M, int64_t num_chunks,
                   int32_t* __restrict__ counts, const int32_t* __restrict__ order_in) {
+    wait_for_kernel_before();
     __shared__ int32_t hist[PART_WARPS][RTMA_MAX_PARTS + 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t chunk = (int64_t)blockIdx.x * PART_WARPS + warp;
@@ -68,6 +69,7 @@ part_scatter_kernel(int64_t n, const int32_t* __restrict__ group_id, uint64_t se
                     const int64_t* __restrict__ scanned, int32_t* __restrict__ part_id,
                     int64_t* __restrict__ part_offsets, int32_t* __restrict__ perm,
                     int32_t* __restrict__ local_id, const int32_t* __restrict__ order_in) {
+    wait_for_kernel_before();
     __shared__ int32_t cursor[PART_WARPS][RTMA_MAX_PARTS + 1];
     __shared__ int32_t first_slot[RTMA_MAX_PARTS + 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -127,10 +129,10 @@ extern "C" int32_t rtma_partition(rtma_ctx* ctx, int64_t n, const int32_t* group
     int64_t* scanned = cur.take<int64_t>(cells + 1);
     int64_t* scratch = cur.take<int64_t>(scan_scratch_elems(cells));
     const unsigned blocks = (unsigned)ceil_div(num_chunks, PART_WARPS);
-    { KernelScope ks(ctx, KC_PART_COUNT, stream); part_count_kernel<<<blocks, PART_THREADS, 0, stream>>>(n, group_id, seed, M, num_chunks, counts, nullptr); }
+    { KernelScope ks(ctx, KC_PART_COUNT, stream); launch_kernel(part_count_kernel, blocks, PART_THREADS, 0, stream, n, group_id, seed, M, num_chunks, counts, nullptr); }
     RTMA_LAUNCH_CHECK(ctx);
     RTMA_TRY(exclusive_scan_i32_to_i64(ctx, counts, cells, scanned, scratch, stream));
-    { KernelScope ks(ctx, KC_PART_SCATTER, stream); part_scatter_kernel<<<blocks, PART_THREADS, 0, stream>>>(n, group_id, seed, M, num_chunks, scanned, part_id,
+    { KernelScope ks(ctx, KC_PART_SCATTER, stream); launch_kernel(part_scatter_kernel, blocks, PART_THREADS, 0, stream, n, group_id, seed, M, num_chunks, scanned, part_id,
                                                              part_offsets, perm, local_id, nullptr); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
@@ -155,6 +157,7 @@ __device__ __forceinline__ int radix_digit(int32_t group, int shift) {
 __global__ void __launch_bounds__(PART_THREADS)
 radix_count_kernel(int64_t n, const int32_t* __restrict__ order_in, const int32_t* __restrict__ group_id, int shift,
                    int64_t num_chunks, int32_t* __restrict__ counts) {
+    wait_for_kernel_before();
     __shared__ int32_t hist[PART_WARPS][RADIX_BUCKETS + 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t chunk = (int64_t)blockIdx.x * PART_WARPS + warp;
@@ -174,6 +177,7 @@ radix_count_kernel(int64_t n, const int32_t* __restrict__ order_in, const int32_
 __global__ void __launch_bounds__(PART_THREADS)
 radix_scatter_kernel(int64_t n, const int32_t* __restrict__ order_in, const int32_t* __restrict__ group_id, int shift,
                      int64_t num_chunks, const int64_t* __restrict__ scanned, int32_t* __restrict__ order_out) {
+    wait_for_kernel_before();
     __shared__ int32_t cursor[PART_WARPS][RADIX_BUCKETS + 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t chunk = (int64_t)blockIdx.x * PART_WARPS + warp;
@@ -228,17 +232,17 @@ extern "C" int32_t rtma_partition_grouped(rtma_ctx* ctx, int64_t n, const int32_
     const int32_t* in = nullptr;  // NULL: node id order
     for (int pass = 0; pass < 4; ++pass) {
         int32_t* out = order[pass & 1];
-        { KernelScope ks(ctx, KC_PART_COUNT, stream); radix_count_kernel<<<blocks, PART_THREADS, 0, stream>>>(n, in, group_id, 8 * pass, num_chunks, counts); }
+        { KernelScope ks(ctx, KC_PART_COUNT, stream); launch_kernel(radix_count_kernel, blocks, PART_THREADS, 0, stream, n, in, group_id, 8 * pass, num_chunks, counts); }
         RTMA_LAUNCH_CHECK(ctx);
         RTMA_TRY(exclusive_scan_i32_to_i64(ctx, counts, num_chunks * RADIX_BUCKETS, scanned, scratch, stream));
-        { KernelScope ks(ctx, KC_PART_SCATTER, stream); radix_scatter_kernel<<<blocks, PART_THREADS, 0, stream>>>(n, in, group_id, 8 * pass, num_chunks, scanned, out); }
+        { KernelScope ks(ctx, KC_PART_SCATTER, stream); launch_kernel(radix_scatter_kernel, blocks, PART_THREADS, 0, stream, n, in, group_id, 8 * pass, num_chunks, scanned, out); }
         RTMA_LAUNCH_CHECK(ctx);
         in = out;
     }
-    { KernelScope ks(ctx, KC_PART_COUNT, stream); part_count_kernel<<<blocks, PART_THREADS, 0, stream>>>(n, group_id, seed, M, num_chunks, counts, in); }
+    { KernelScope ks(ctx, KC_PART_COUNT, stream); launch_kernel(part_count_kernel, blocks, PART_THREADS, 0, stream, n, group_id, seed, M, num_chunks, counts, in); }
     RTMA_LAUNCH_CHECK(ctx);
     RTMA_TRY(exclusive_scan_i32_to_i64(ctx, counts, num_chunks * M, scanned, scratch, stream));
-    { KernelScope ks(ctx, KC_PART_SCATTER, stream); part_scatter_kernel<<<blocks, PART_THREADS, 0, stream>>>(n, group_id, seed, M, num_chunks, scanned, part_id,
+    { KernelScope ks(ctx, KC_PART_SCATTER, stream); launch_kernel(part_scatter_kernel, blocks, PART_THREADS, 0, stream, n, group_id, seed, M, num_chunks, scanned, part_id,
                                                              part_offsets, perm, local_id, in); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
@@ -272,6 +276,7 @@ int32_t static_fail(int32_t code, const char* fmt, ...) {
 // Exclusive scan of `cells` counts (cells + 1 outputs) by one block of 1024 threads.
 __global__ void __launch_bounds__(1024)
 part_scan_one_block_kernel(const int32_t* __restrict__ counts, int64_t cells, int64_t* __restrict__ scanned) {
+    wait_for_kernel_before();
     __shared__ int64_t warp_sums[32];
     __shared__ int64_t carry;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -344,9 +349,9 @@ extern "C" int32_t rtma_partition_static(int32_t device, int64_t n, const int32_
     int32_t* counts = reinterpret_cast<int32_t*>(g_partition_scratch_ptr[device]);
     int64_t* scanned = reinterpret_cast<int64_t*>(g_partition_scratch_ptr[device] + STATIC_COUNTS_BYTES);
     const unsigned blocks = (unsigned)ceil_div(num_chunks, PART_WARPS);
-    part_count_kernel<<<blocks, PART_THREADS, 0, stream>>>(n, group_id, seed, M, num_chunks, counts, nullptr);
-    part_scan_one_block_kernel<<<1, 1024, 0, stream>>>(counts, cells, scanned);
-    part_scatter_kernel<<<blocks, PART_THREADS, 0, stream>>>(n, group_id, seed, M, num_chunks, scanned, part_id,
+    launch_kernel(part_count_kernel, blocks, PART_THREADS, 0, stream, n, group_id, seed, M, num_chunks, counts, nullptr);
+    launch_kernel(part_scan_one_block_kernel, 1, 1024, 0, stream, counts, cells, scanned);
+    launch_kernel(part_scatter_kernel, blocks, PART_THREADS, 0, stream, n, group_id, seed, M, num_chunks, scanned, part_id,
                                                              part_offsets, perm, local_id, nullptr);
     e = cudaGetLastError();
     return e == cudaSuccess ? RTMA_OK : static_fail(RTMA_ERR_CUDA, "kernel launch: %s", cudaGetErrorString(e));

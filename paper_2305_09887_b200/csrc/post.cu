@@ -103,6 +103,7 @@ __device__ __forceinline__ void width_mask(int col, int d, uint32_t (&keep)[4]) 
 template <int NP, bool NORM>
 __global__ void __launch_bounds__(POST_THREADS)
 post_forward_kernel(const __grid_constant__ GroupDesc g, const PostArgs a) {
+    wait_for_kernel_before();
     constexpr int RB = NP == 1 ? 2 : 1;
     int k, r0;
     if (!locate_tile(g, POST_TILE_ROWS, blockIdx.x, &k, &r0)) return;
@@ -201,6 +202,7 @@ post_forward_kernel(const __grid_constant__ GroupDesc g, const PostArgs a) {
 template <int NP, bool NORM>
 __global__ void __launch_bounds__(POST_THREADS)
 post_backward_kernel(const __grid_constant__ GroupDesc g, const PostArgs a) {
+    wait_for_kernel_before();
     constexpr int RB = NP == 1 ? 2 : 1;
     __shared__ float red[POST_WARPS][2 * NP * 256 + 1];
     int k, r0;
@@ -324,6 +326,7 @@ post_backward_kernel(const __grid_constant__ GroupDesc g, const PostArgs a) {
 __global__ void __launch_bounds__(256)
 post_reduce_sgd_kernel(const __grid_constant__ GroupDesc g, const LayerShape ls, const float* __restrict__ partial,
                        const float lr, float* __restrict__ params, float* __restrict__ grads_record) {
+    wait_for_kernel_before();
     __shared__ float red[8][33];
     const int k = blockIdx.y;
     const int d = ls.d_out;
@@ -360,14 +363,14 @@ int64_t post_tiles(const GroupDesc& g) { return group_tiles(g, POST_TILE_ROWS); 
     do {                                                                                                      \
         const bool norm = (ls).gamma_offset >= 0;                                                             \
         if ((ls).d_out <= 256) {                                                                              \
-            if (norm) KERNEL<1, true><<<(unsigned)tiles, POST_THREADS, 0, s>>>(__VA_ARGS__);                  \
-            else KERNEL<1, false><<<(unsigned)tiles, POST_THREADS, 0, s>>>(__VA_ARGS__);                      \
+            if (norm) launch_kernel(KERNEL<1, true>, (unsigned)tiles, POST_THREADS, 0, s, __VA_ARGS__);                  \
+            else launch_kernel(KERNEL<1, false>, (unsigned)tiles, POST_THREADS, 0, s, __VA_ARGS__);                      \
         } else if ((ls).d_out <= 512) {                                                                       \
-            if (norm) KERNEL<2, true><<<(unsigned)tiles, POST_THREADS, 0, s>>>(__VA_ARGS__);                  \
-            else KERNEL<2, false><<<(unsigned)tiles, POST_THREADS, 0, s>>>(__VA_ARGS__);                      \
+            if (norm) launch_kernel(KERNEL<2, true>, (unsigned)tiles, POST_THREADS, 0, s, __VA_ARGS__);                  \
+            else launch_kernel(KERNEL<2, false>, (unsigned)tiles, POST_THREADS, 0, s, __VA_ARGS__);                      \
         } else {                                                                                              \
-            if (norm) KERNEL<4, true><<<(unsigned)tiles, POST_THREADS, 0, s>>>(__VA_ARGS__);                  \
-            else KERNEL<4, false><<<(unsigned)tiles, POST_THREADS, 0, s>>>(__VA_ARGS__);                      \
+            if (norm) launch_kernel(KERNEL<4, true>, (unsigned)tiles, POST_THREADS, 0, s, __VA_ARGS__);                  \
+            else launch_kernel(KERNEL<4, false>, (unsigned)tiles, POST_THREADS, 0, s, __VA_ARGS__);                      \
         }                                                                                                     \
     } while (0)
 
@@ -392,7 +395,7 @@ int32_t launch_post_backward(rtma_ctx* ctx, const GroupDesc& g, LayerShape ls, f
     RTMA_LAUNCH_CHECK(ctx);
     if (ls.gamma_offset >= 0 || ls.slope_offset >= 0) {
         dim3 grid((unsigned)ceil_div(2 * ls.d_out + 1, 32), (unsigned)g.num);
-        { KernelScope ks(ctx, KC_POST, s); post_reduce_sgd_kernel<<<grid, 256, 0, s>>>(g, ls, partial, lr, params, grads_record); }
+        { KernelScope ks(ctx, KC_POST, s); launch_kernel(post_reduce_sgd_kernel, grid, 256, 0, s, g, ls, partial, lr, params, grads_record); }
         RTMA_LAUNCH_CHECK(ctx);
     }
     return RTMA_OK;

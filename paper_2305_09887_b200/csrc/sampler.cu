@@ -33,6 +33,7 @@ __device__ __forceinline__ uint64_t mix_step(uint64_t x) {  // one step of the S
 __global__ void __launch_bounds__(256)
 sample_count_kernel(const int64_t* __restrict__ rowptr, int64_t n, int64_t frontier_size, const int32_t* __restrict__ frontier,
                     int32_t fanout, int32_t* __restrict__ counts, int32_t* __restrict__ member) {
+    wait_for_kernel_before();
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= frontier_size) return;
     const int32_t v = frontier[i];
@@ -116,6 +117,7 @@ __global__ void __launch_bounds__(256)
 sample_select_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, int64_t n, int64_t frontier_size,
                      const int32_t* __restrict__ frontier, int32_t fanout, double expected, uint64_t base,
                      const int64_t* __restrict__ block_rowptr, int32_t* __restrict__ block_col, int32_t* __restrict__ member) {
+    wait_for_kernel_before();
     __shared__ uint64_t cand_key[SEL_NODES][SEL_CAND];
     __shared__ int32_t cand_pos[SEL_NODES][SEL_CAND];
     const int lane = threadIdx.x & 31, sub = threadIdx.x / SEL_LANES, sl = threadIdx.x % SEL_LANES;
@@ -192,6 +194,7 @@ sample_select_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restri
 __global__ void __launch_bounds__(256)
 sample_emit_frontier_kernel(int64_t n, const int32_t* __restrict__ member, const int64_t* __restrict__ position,
                             int32_t* __restrict__ next_frontier, int64_t* __restrict__ next_size) {
+    wait_for_kernel_before();
     const int64_t v = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (v < n && member[v]) next_frontier[position[v]] = (int32_t)v;
     if (v == 0) *next_size = position[n];
@@ -200,6 +203,7 @@ sample_emit_frontier_kernel(int64_t n, const int32_t* __restrict__ member, const
 __global__ void __launch_bounds__(256)
 sample_relabel_kernel(const int64_t* __restrict__ block_rowptr, int64_t frontier_size, const int64_t* __restrict__ position,
                       int32_t* __restrict__ block_col) {
+    wait_for_kernel_before();
     const int64_t entries = block_rowptr[frontier_size];
     for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < entries; e += (int64_t)gridDim.x * 256)
         block_col[e] = (int32_t)position[block_col[e]];
@@ -232,7 +236,7 @@ extern "C" int32_t rtma_sample_hop(rtma_ctx* ctx, int64_t n, const int64_t* rowp
     RTMA_CUDA(ctx, cudaMemsetAsync(member, 0, sizeof(int32_t) * (n + 1), stream));
     if (frontier_size > 0) {
         KernelScope ks(ctx, KC_LINK, stream);
-        sample_count_kernel<<<(unsigned)ceil_div(frontier_size, 256), 256, 0, stream>>>(rowptr, n, frontier_size, frontier, fanout, counts, member);
+        launch_kernel(sample_count_kernel, (unsigned)ceil_div(frontier_size, 256), 256, 0, stream, rowptr, n, frontier_size, frontier, fanout, counts, member);
     }
     RTMA_LAUNCH_CHECK(ctx);
     RTMA_TRY(exclusive_scan_i32_to_i64(ctx, counts, frontier_size, block_rowptr, scratch, stream));
@@ -246,20 +250,20 @@ extern "C" int32_t rtma_sample_hop(rtma_ctx* ctx, int64_t n, const int64_t* rowp
         KernelScope ks(ctx, KC_LINK, stream);
         // candidates per row (see the kernel)
         const double expected = std::min((double)fanout + 6.0 * std::sqrt((double)fanout) + 16.0, 0.5 * ((double)fanout + SEL_CAND));
-        (fanout > SEL_RARE ? sample_select_kernel<true> : sample_select_kernel<false>)<<<(unsigned)ceil_div(frontier_size, SEL_NODES), 256, 0, stream>>>(
+        launch_kernel(fanout > SEL_RARE ? sample_select_kernel<true> : sample_select_kernel<false>, (unsigned)ceil_div(frontier_size, SEL_NODES), 256, 0, stream,
             rowptr, col, n, frontier_size, frontier, fanout, expected, base, block_rowptr, block_col, member);
     }
     RTMA_LAUNCH_CHECK(ctx);
     RTMA_TRY(exclusive_scan_i32_to_i64(ctx, member, n, position, scratch, stream));
     {
         KernelScope ks(ctx, KC_LINK, stream);
-        sample_emit_frontier_kernel<<<(unsigned)ceil_div(n > 0 ? n : 1, 256), 256, 0, stream>>>(n, member, position, next_frontier, next_size);
+        launch_kernel(sample_emit_frontier_kernel, (unsigned)ceil_div(n > 0 ? n : 1, 256), 256, 0, stream, n, member, position, next_frontier, next_size);
     }
     RTMA_LAUNCH_CHECK(ctx);
     if (frontier_size > 0) {
         const int64_t bound = frontier_size * (int64_t)(fanout < 4096 ? fanout : 4096);  // kept entries, roughly: sizes the grid only
         KernelScope ks(ctx, KC_LINK, stream);
-        sample_relabel_kernel<<<(unsigned)std::min<int64_t>(ceil_div(bound, 256), 148 * 32), 256, 0, stream>>>(block_rowptr, frontier_size,
+        launch_kernel(sample_relabel_kernel, (unsigned)std::min<int64_t>(ceil_div(bound, 256), 148 * 32), 256, 0, stream, block_rowptr, frontier_size,
                                                                                                         position, block_col);
     }
     RTMA_LAUNCH_CHECK(ctx);

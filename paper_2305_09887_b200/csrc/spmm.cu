@@ -33,6 +33,7 @@ constexpr int SPMM_ROWS_PER_WARP = 8;
 
 __global__ void __launch_bounds__(256)
 inv_degree_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict__ rowptr_out, float* __restrict__ inv_deg) {
+    wait_for_kernel_before();
     int k, r0;
     if (!locate_tile(g, 256, blockIdx.x, &k, &r0)) return;
     const int i = r0 + threadIdx.x;
@@ -45,6 +46,7 @@ inv_degree_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict
 // s[v] = (deg(v) + 1)^-1/2
 __global__ void __launch_bounds__(256)
 gcn_scale_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict__ rowptr_out, float* __restrict__ scale) {
+    wait_for_kernel_before();
     int k, r0;
     if (!locate_tile(g, 256, blockIdx.x, &k, &r0)) return;
     const int i = r0 + threadIdx.x;
@@ -56,6 +58,7 @@ gcn_scale_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict_
 __global__ void __launch_bounds__(256)
 to_planes_kernel(const __grid_constant__ GroupDesc g, const float* __restrict__ X, const int32_t* __restrict__ perm,
                  const int64_t n_total, const int d, const Planes out) {
+    wait_for_kernel_before();
     int k, r0;
     if (!locate_tile(g, 32, blockIdx.x, &k, &r0)) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -94,6 +97,7 @@ struct ClearList {
 // 2 M rows (2.3 ms; 1.9 ms on 5 M rows of two layers): the kernels write every row of a part before it is read.
 __global__ void __launch_bounds__(256)
 clear_gaps_kernel(const __grid_constant__ GroupDesc g, const __grid_constant__ ClearList list, int* __restrict__ counters, const int words) {
+    wait_for_kernel_before();
     if (blockIdx.x == 0 && blockIdx.y == 0)
         for (int i = threadIdx.x; i < words; i += 256) counters[i] = 0;
     if (!list.mat[blockIdx.y].hi) return;
@@ -109,6 +113,7 @@ clear_gaps_kernel(const __grid_constant__ GroupDesc g, const __grid_constant__ C
 
 __global__ void __launch_bounds__(256)
 from_planes_kernel(const Planes src, const int64_t first_row, const int64_t rows, const int d, float* __restrict__ dst) {
+    wait_for_kernel_before();
     const int64_t total = rows * d;
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < total; i += (int64_t)gridDim.x * 256) {
         const int64_t r = i / d;
@@ -133,6 +138,7 @@ __device__ __forceinline__ int64_t group_entries(const GroupDesc& g, const int64
 __global__ void __launch_bounds__(256)
 heavy_list_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict__ rowptr_out, const int64_t total_groups,
                   const int64_t heavy, int* __restrict__ count, int* __restrict__ list) {
+    wait_for_kernel_before();
     for (int64_t grp = (int64_t)blockIdx.x * 256 + threadIdx.x; grp < total_groups; grp += (int64_t)gridDim.x * 256)
         if (group_entries(g, rowptr_out, grp) >= heavy) list[atomicAdd(count, 1)] = (int)grp;
 }
@@ -145,6 +151,7 @@ constexpr int LOCAL_SPAN = 512;
 __global__ void __launch_bounds__(256)
 locality_probe_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict__ rowptr_out,
                       const int32_t* __restrict__ col_out, const int64_t total_rows, unsigned long long* __restrict__ near_total) {
+    wait_for_kernel_before();
     unsigned long long near = 0, total = 0;
     for (int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x; t * 8 < total_rows; t += (int64_t)gridDim.x * 256) {
         int k, i;
@@ -186,6 +193,7 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long x) {
 __global__ void __launch_bounds__(256)
 symmetry_check_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict__ rowptr_out,
                       const int32_t* __restrict__ col_out, unsigned long long* __restrict__ sums, int* __restrict__ flag) {
+    wait_for_kernel_before();
     unsigned long long fwd = 0, rev = 0;
     int k, r0;
     if (locate_tile(g, 256, blockIdx.x, &k, &r0)) {
@@ -427,6 +435,7 @@ __global__ void __launch_bounds__(SPMM_THREADS, NCH == 1 ? 2 : 1)
 spmm_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict__ rowptr_out,
             const int32_t* __restrict__ col_out, const float* __restrict__ inv_deg, const Planes src, const Planes out,
             const int d, const int64_t total_groups, const SpmmOrder order, int* __restrict__ ticket) {
+    wait_for_kernel_before();
     if (order.near_total && order.near_total[1] > 0 && 2 * order.near_total[0] >= order.near_total[1])
         spmm_rows<NCH, MODE, true>(g, rowptr_out, col_out, inv_deg, src, out, d, total_groups, order, ticket);
     else
@@ -643,6 +652,7 @@ spmm_narrow_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restric
                    const int32_t* __restrict__ col_out, const float* __restrict__ inv_deg, const Planes src,
                    const Planes out, const int d, const int64_t total_groups, const SpmmOrder order,
                    int* __restrict__ ticket) {
+    wait_for_kernel_before();
     if (order.near_total && order.near_total[1] > 0 && 2 * order.near_total[0] >= order.near_total[1])
         spmm_narrow_rows<LPR, MODE, true>(g, rowptr_out, col_out, inv_deg, src, out, d, total_groups, order, ticket);
     else
@@ -666,6 +676,7 @@ template <int MODE>
 __global__ void __launch_bounds__(TINY_TILE_ROWS, 5)
 spmm_tiny_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict__ rowptr_out,
                  const int32_t* __restrict__ col_out, const float* __restrict__ inv_deg, const Planes src, const Planes out, const int d) {
+    wait_for_kernel_before();
     int k, r0;
     if (!locate_tile(g, TINY_TILE_ROWS, blockIdx.x, &k, &r0)) return;
     const int n_p = g.rows[k], i = r0 + threadIdx.x, lane = threadIdx.x & 31;
@@ -778,7 +789,7 @@ int32_t dispatch_spmm(rtma_ctx* ctx, int kclass, const GroupDesc& g, const int64
         return launch_spmm_dense(ctx, kclass, g, rowptr_out, col_out, inv_deg, order, src, out, d, MODE == 1, s);
     if (d <= 8) {
         const int64_t tiles = group_tiles(g, TINY_TILE_ROWS);
-        { KernelScope ks(ctx, kclass, s); spmm_tiny_kernel<MODE><<<(unsigned)tiles, TINY_TILE_ROWS, 0, s>>>(g, rowptr_out, col_out, inv_deg, src, out, d); }
+        { KernelScope ks(ctx, kclass, s); launch_kernel(spmm_tiny_kernel<MODE>, (unsigned)tiles, TINY_TILE_ROWS, 0, s, g, rowptr_out, col_out, inv_deg, src, out, d); }
         RTMA_LAUNCH_CHECK(ctx);
         return RTMA_OK;
     }
@@ -788,13 +799,13 @@ int32_t dispatch_spmm(rtma_ctx* ctx, int kclass, const GroupDesc& g, const int64
 #define RTMA_SPMM(N)                                                                                      \
     do {                                                                                                  \
         KernelScope ks(ctx, kclass, s);                                                                   \
-        spmm_kernel<N, MODE><<<grid, SPMM_THREADS, 0, s>>>(g, rowptr_out, col_out, inv_deg, src, out, d,  \
+        launch_kernel(spmm_kernel<N, MODE>, grid, SPMM_THREADS, 0, s, g, rowptr_out, col_out, inv_deg, src, out, d,  \
                                                            groups, order, ticket);                        \
     } while (0)
     if (d <= 64) {
         KernelScope ks(ctx, kclass, s);
-        if (d <= 32) spmm_narrow_kernel<4, MODE><<<grid, SPMM_THREADS, 0, s>>>(g, rowptr_out, col_out, inv_deg, src, out, d, groups, order, ticket);
-        else spmm_narrow_kernel<8, MODE><<<grid, SPMM_THREADS, 0, s>>>(g, rowptr_out, col_out, inv_deg, src, out, d, groups, order, ticket);
+        if (d <= 32) launch_kernel(spmm_narrow_kernel<4, MODE>, grid, SPMM_THREADS, 0, s, g, rowptr_out, col_out, inv_deg, src, out, d, groups, order, ticket);
+        else launch_kernel(spmm_narrow_kernel<8, MODE>, grid, SPMM_THREADS, 0, s, g, rowptr_out, col_out, inv_deg, src, out, d, groups, order, ticket);
     } else if (d <= 256) RTMA_SPMM(1);
     else if (d <= 512) RTMA_SPMM(2);
     else if (d <= 1024) RTMA_SPMM(4);
@@ -812,7 +823,7 @@ int32_t launch_to_planes(rtma_ctx* ctx, const GroupDesc& g, const float* X, cons
                          Planes out, cudaStream_t s) {
     const int64_t tiles = group_tiles(g, 32);
     if (tiles == 0) return RTMA_OK;
-    { KernelScope ks(ctx, KC_TO_PLANES, s); to_planes_kernel<<<(unsigned)tiles, 256, 0, s>>>(g, X, perm, n_total, d, out); }
+    { KernelScope ks(ctx, KC_TO_PLANES, s); launch_kernel(to_planes_kernel, (unsigned)tiles, 256, 0, s, g, X, perm, n_total, d, out); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }
@@ -822,7 +833,7 @@ int32_t launch_clear_gaps(rtma_ctx* ctx, const GroupDesc& g, const Planes* mats,
     ClearList list{};
     for (int i = 0; i < count; ++i) list.mat[i] = mats[i];
     const dim3 grid((unsigned)std::max(1, (int)g.num), (unsigned)std::max(1, count));
-    { KernelScope ks(ctx, KC_TO_PLANES, s); clear_gaps_kernel<<<grid, 256, 0, s>>>(g, list, counters, words); }
+    { KernelScope ks(ctx, KC_TO_PLANES, s); launch_kernel(clear_gaps_kernel, grid, 256, 0, s, g, list, counters, words); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }
@@ -830,7 +841,7 @@ int32_t launch_clear_gaps(rtma_ctx* ctx, const GroupDesc& g, const Planes* mats,
 int32_t launch_from_planes(rtma_ctx* ctx, Planes src, int64_t first_row, int64_t rows, int d, float* dst, cudaStream_t s) {
     if (rows <= 0 || d <= 0) return RTMA_OK;
     const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(rows * d, 256), 148 * 16);
-    { KernelScope ks(ctx, KC_COPY, s); from_planes_kernel<<<grid, 256, 0, s>>>(src, first_row, rows, d, dst); }
+    { KernelScope ks(ctx, KC_COPY, s); launch_kernel(from_planes_kernel, grid, 256, 0, s, src, first_row, rows, d, dst); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }
@@ -839,7 +850,7 @@ int32_t launch_symmetry_check(rtma_ctx* ctx, const GroupDesc& g, const int64_t* 
                               unsigned long long* sums, cudaStream_t s) {
     const int64_t tiles = group_tiles(g, 256);
     if (tiles == 0) return RTMA_OK;
-    { KernelScope ks(ctx, KC_INV_DEGREE, s); symmetry_check_kernel<<<(unsigned)tiles, 256, 0, s>>>(g, rowptr_out, col_out, sums, ctx->error_word + 1); }
+    { KernelScope ks(ctx, KC_INV_DEGREE, s); launch_kernel(symmetry_check_kernel, (unsigned)tiles, 256, 0, s, g, rowptr_out, col_out, sums, ctx->error_word + 1); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }
@@ -847,7 +858,7 @@ int32_t launch_symmetry_check(rtma_ctx* ctx, const GroupDesc& g, const int64_t* 
 int32_t launch_inv_degree(rtma_ctx* ctx, const GroupDesc& g, const int64_t* rowptr_out, float* inv_deg, cudaStream_t s) {
     const int64_t tiles = group_tiles(g, 256);
     if (tiles == 0) return RTMA_OK;
-    { KernelScope ks(ctx, KC_INV_DEGREE, s); inv_degree_kernel<<<(unsigned)tiles, 256, 0, s>>>(g, rowptr_out, inv_deg); }
+    { KernelScope ks(ctx, KC_INV_DEGREE, s); launch_kernel(inv_degree_kernel, (unsigned)tiles, 256, 0, s, g, rowptr_out, inv_deg); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }
@@ -874,7 +885,7 @@ int32_t launch_spmm_gcn(rtma_ctx* ctx, const GroupDesc& g, const int64_t* rowptr
 int32_t launch_gcn_scale(rtma_ctx* ctx, const GroupDesc& g, const int64_t* rowptr_out, float* scale, cudaStream_t s) {
     const int64_t tiles = group_tiles(g, 256);
     if (tiles == 0) return RTMA_OK;
-    { KernelScope ks(ctx, KC_INV_DEGREE, s); gcn_scale_kernel<<<(unsigned)tiles, 256, 0, s>>>(g, rowptr_out, scale); }
+    { KernelScope ks(ctx, KC_INV_DEGREE, s); launch_kernel(gcn_scale_kernel, (unsigned)tiles, 256, 0, s, g, rowptr_out, scale); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }
@@ -890,10 +901,10 @@ int32_t launch_spmm_order(rtma_ctx* ctx, const GroupDesc& g, const int64_t* rowp
     // heavy = several times the average group, and enough entries to be worth the detour
     const int64_t heavy = std::max<int64_t>(128, 4 * ceil_div(entries, groups));
     const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(groups, 256), 148 * 4);
-    { KernelScope ks(ctx, KC_INV_DEGREE, s); heavy_list_kernel<<<grid, 256, 0, s>>>(g, rowptr_out, groups, heavy, count, list); }
+    { KernelScope ks(ctx, KC_INV_DEGREE, s); launch_kernel(heavy_list_kernel, grid, 256, 0, s, g, rowptr_out, groups, heavy, count, list); }
     RTMA_LAUNCH_CHECK(ctx);
     unsigned long long* near_total = reinterpret_cast<unsigned long long*>(count + 2);
-    { KernelScope ks(ctx, KC_INV_DEGREE, s); locality_probe_kernel<<<grid, 256, 0, s>>>(g, rowptr_out, col_out, group_tiles(g, 1), near_total); }
+    { KernelScope ks(ctx, KC_INV_DEGREE, s); launch_kernel(locality_probe_kernel, grid, 256, 0, s, g, rowptr_out, col_out, group_tiles(g, 1), near_total); }
     RTMA_LAUNCH_CHECK(ctx);
     *order = SpmmOrder{count, list, heavy, near_total, nullptr, 0, nullptr, nullptr, nullptr, nullptr, false};
     return RTMA_OK;

@@ -135,6 +135,7 @@ __device__ __forceinline__ uint32_t tile_blocks(const unsigned char* block_mask,
 // TRANSPOSED = false: A counts, out = (1 / deg v) * A src;  true: A = counts x 1 / deg u, out = A src
 template <bool TRANSPOSED>
 __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_constant__ DenseArgs a) {
+    wait_for_kernel_before();
     extern __shared__ uint8_t smem_raw[];
     __shared__ DenseBarriers pb;
     {   // nothing to do unless a part of this launch is aggregated here: leave before any set-up
@@ -505,6 +506,7 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
                     const int* __restrict__ dense, const unsigned char* __restrict__ left_cnt,
                     const int32_t* __restrict__ left_col, const Planes src, const Planes out, const int width,
                     const int64_t total_groups) {
+    wait_for_kernel_before();
     constexpr int S = 32 / LPR;            // rows side by side in a warp
     constexpr int NR = 2;                  // rows a lane works on at a time
     constexpr int EL = 2;                  // listed entries of each of them requested together (most rows have one or two)
@@ -675,6 +677,7 @@ dense_lists_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restric
                    const int32_t* __restrict__ col_out, int* __restrict__ dense,
                    unsigned long long* __restrict__ win_bits, unsigned char* __restrict__ block_mask,
                    unsigned char* __restrict__ left_cnt, int32_t* __restrict__ left_col) {
+    wait_for_kernel_before();
     int k, r0;
     if (!locate_tile(g, 256, blockIdx.x, &k, &r0)) return;
     const int i = r0 + threadIdx.x;
@@ -726,6 +729,7 @@ dense_lists_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restric
 __global__ void __launch_bounds__(256)
 dense_probe_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict__ rowptr_out,
                    const int32_t* __restrict__ col_out, const int64_t tiles, unsigned long long* __restrict__ counts) {
+    wait_for_kernel_before();
     for (int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x; t < tiles; t += (int64_t)gridDim.x * 256) {
         int k, i;
         if (!locate_tile(g, 64, t, &k, &i)) break;
@@ -764,6 +768,7 @@ dense_probe_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restric
 // and the sampled rows have at least 4 entries on average (below that, gathering is cheaper than a tile).
 __global__ void dense_decide_kernel(const __grid_constant__ GroupDesc g, const unsigned long long* __restrict__ counts,
                                     const int mode, int* __restrict__ dense) {
+    wait_for_kernel_before();
     const int k = threadIdx.x;
     if (k >= g.num) return;
     const int p = g.part[k];
@@ -778,9 +783,9 @@ int32_t launch_dense_probe(rtma_ctx* ctx, const GroupDesc& g, const int64_t* row
     const int64_t tiles = group_tiles(g, 64);
     if (tiles == 0) return RTMA_OK;
     const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(tiles, 256), 148 * 4);
-    { KernelScope ks(ctx, KC_INV_DEGREE, s); dense_probe_kernel<<<grid, 256, 0, s>>>(g, rowptr_out, col_out, tiles, counts); }
+    { KernelScope ks(ctx, KC_INV_DEGREE, s); launch_kernel(dense_probe_kernel, grid, 256, 0, s, g, rowptr_out, col_out, tiles, counts); }
     RTMA_LAUNCH_CHECK(ctx);
-    { KernelScope ks(ctx, KC_INV_DEGREE, s); dense_decide_kernel<<<1, RTMA_MAX_PARTS, 0, s>>>(g, counts, mode, dense); }
+    { KernelScope ks(ctx, KC_INV_DEGREE, s); launch_kernel(dense_decide_kernel, 1, RTMA_MAX_PARTS, 0, s, g, counts, mode, dense); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }
@@ -790,7 +795,7 @@ int32_t launch_dense_lists(rtma_ctx* ctx, const GroupDesc& g, const int64_t* row
                            int32_t* left_col, cudaStream_t s) {
     const int64_t tiles = group_tiles(g, 256);
     if (tiles == 0) return RTMA_OK;
-    { KernelScope ks(ctx, KC_INV_DEGREE, s); dense_lists_kernel<<<(unsigned)tiles, 256, 0, s>>>(g, rowptr_out, col_out, dense, win_bits, block_mask, left_cnt, left_col); }
+    { KernelScope ks(ctx, KC_INV_DEGREE, s); launch_kernel(dense_lists_kernel, (unsigned)tiles, 256, 0, s, g, rowptr_out, col_out, dense, win_bits, block_mask, left_cnt, left_col); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }
@@ -842,7 +847,7 @@ int32_t launch_spmm_dense(rtma_ctx* ctx, int kclass, const GroupDesc& g, const i
     {
         KernelScope ks(ctx, kclass, s);
 #define RTMA_OUTSIDE(T, L)                                                                                              \
-    spmm_outside_kernel<T, L><<<lgrid, 256, 0, s>>>(g, rowptr_out, col_out, inv_deg, dense, order.left_cnt, order.left_col, \
+    launch_kernel(spmm_outside_kernel<T, L>, lgrid, 256, 0, s, g, rowptr_out, col_out, inv_deg, dense, order.left_cnt, order.left_col, \
                                                     src, out, a.width, groups)
         if (a.width <= 64) {
             if (transposed) RTMA_OUTSIDE(true, 8);
@@ -858,8 +863,8 @@ int32_t launch_spmm_dense(rtma_ctx* ctx, int kclass, const GroupDesc& g, const i
     const size_t smem = a.stages * stage_bytes + fixed;
     {
         KernelScope ks(ctx, kclass, s);
-        if (transposed) spmm_dense_kernel<true><<<grid, DT_THREADS, smem, s>>>(a);
-        else spmm_dense_kernel<false><<<grid, DT_THREADS, smem, s>>>(a);
+        if (transposed) launch_kernel(spmm_dense_kernel<true>, grid, DT_THREADS, smem, s, a);
+        else launch_kernel(spmm_dense_kernel<false>, grid, DT_THREADS, smem, s, a);
     }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;

@@ -5,7 +5,7 @@ import pytest
 import torch
 
 import oracle
-from paper_2305_09887_b200 import inputs
+from paper_2305_09887_b200 import binding, inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -155,3 +155,30 @@ def test_gather_rows(util, shape, dtype):
     perm = rng.permutation(shape[0]).astype(np.int32)
     got = util.ctx().gather_rows(util.dev(src), util.dev(perm)).cpu().numpy()
     assert np.array_equal(got, src[perm])
+
+
+def test_calls_captured_in_a_graph():
+    # launches that overlap their predecessor's end keep their order in a captured graph: partition, row gather, averaging
+    c, n, M = binding.Context(0), 70_003, 5                         # one that has not trained: its calls need not wait for that
+    src = torch.arange(n, dtype=torch.int32, device="cuda")
+    start = torch.randn(M, 9_001, device="cuda")
+
+    def calls():
+        part = c.partition(n, None, 7, M)
+        rows = c.gather_rows(src, part[2])
+        params = start.clone()
+        c.aggregate(params)
+        c.aggregate_masked(params, [1, 0, 1, 1, 0])
+        return [*part, rows, params]
+
+    want = calls()                                                  # sizes the scratch, too
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got = calls()
+    for _ in range(3):
+        for t in got:
+            t.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(got, want))
