@@ -224,17 +224,18 @@ class Context:
         _need(col, torch.int32, "col", dev)
         _need(frontier, torch.int32, "frontier", dev)
         n, fs = int(rowptr.numel()) - 1, int(frontier.numel())
-        block_rowptr = torch.empty(fs + 1, dtype=torch.int64, device=dev)
+        sizes = torch.empty(fs + 2, dtype=torch.int64, device=dev)  # the block's offsets and, behind them, the next frontier's size
+        block_rowptr, next_size = sizes[:fs + 1], sizes[fs + 1:]
         cap = min(fs * int(fanout), int(col.numel())) if fs else 0
         block_col = torch.empty(max(cap, 1), dtype=torch.int32, device=dev)
         next_frontier = torch.empty(max(n, 1), dtype=torch.int32, device=dev)
-        next_size = torch.zeros(1, dtype=torch.int64, device=dev)
         st = self._lib.rtma_sample_hop(
             self._h, ctypes.c_int64(n), _ptr(rowptr), _ptr(col), ctypes.c_int64(fs), _ptr(frontier), ctypes.c_int32(fanout),
             ctypes.c_uint64(seed), ctypes.c_int32(hop), _ptr(block_rowptr), _ptr(block_col), _ptr(next_frontier),
             _ptr(next_size), ctypes.c_void_p(_stream_handle(stream)))
         self._check(st, "rtma_sample_hop")
-        return block_rowptr, block_col[:int(block_rowptr[-1].item())], next_frontier[:int(next_size.item())]
+        entries, nodes = sizes[fs:].tolist()  # one wait for both
+        return block_rowptr, block_col[:entries], next_frontier[:nodes]
 
     # ---- R1 -------------------------------------------------------------------------
     def partition(self, n: int, group_id, seed: int, M: int, stream=None, grouped: bool = False):

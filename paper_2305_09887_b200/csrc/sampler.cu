@@ -103,22 +103,26 @@ __device__ void select_bit_by_bit(const int32_t* __restrict__ col, int64_t n, in
 
 // Half a warp per frontier node (two nodes of 30 entries fill a warp's lanes).  The keys are uniform 64-bit numbers, so the
 // fanout-th smallest of deg lies near fanout / deg of their range: one pass over the row hashes every entry once and collects
-// those below a bound at which `expected` of them are expected, in row order, in shared memory; a candidate is kept when
+// those below a bound at which `tight` of them are expected, in row order, in shared memory; a candidate is kept when
 // fewer than `fanout` candidates are smaller.  Only kept entries' columns are read.  Bound by instruction issue (the hash,
-// 25 instructions per entry, and the ranking).  Finding the key bit by bit for every node hashed every entry 64 times:
-// three hops (fan-outs 15, 10, 5) from 8,192 of 800,000 nodes took 8.06 ms with the program around them and take 0.83 ms.
-// expected = fanout + 6 sqrt(fanout) + 16, but no more than half way between the fan-out and the candidates' room: too few
-// or too many candidates come once in 10^6 rows up to a fan-out of 35, in 20,000 at 50, in 1,000 at 64, in 60 at 80 and in 8 at
-// SEL_FANOUT; such rows, and all that are cut to larger fan-outs, are done bit by bit.
+// 25 instructions per entry, and the ranking, candidates squared), hence few candidates: tight = fanout + 2.7 sqrt(fanout) + 1,
+// which leaves one row in a hundred short; its half warp goes through the row once more with a bound for wide = fanout +
+// 6 sqrt(fanout) + 16.  Neither expects more than half way between the fan-out and the candidates' room: too few or too
+// many candidates at the wide bound come once in 10^6 rows up to a fan-out of 35, in 20,000 at 50, in 1,000 at 64, in 60 at 80
+// and in 8 at SEL_FANOUT; such rows, and all that are cut to larger fan-outs, are done bit by bit.
+// Bound and ranking look at the upper 32 bits of the keys; where these do not single out `fanout` candidates (equal ones at
+// the cut) the row is done bit by bit too.
+// Three hops (fan-outs 15, 10, 5) from 8,192 of 800,000 nodes, the whole call: with the wide bound alone and whole keys ranked
+// 848 us, with two waits for sizes a hop instead of one; now 584.
 constexpr int SEL_FANOUT = 96;  // largest fan-out for which candidates are collected
 constexpr int SEL_RARE = 35;    // largest fan-out at which a row without the right number of them is one in a million
 template <bool OFTEN>
 __global__ void __launch_bounds__(256)
 sample_select_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, int64_t n, int64_t frontier_size,
-                     const int32_t* __restrict__ frontier, int32_t fanout, double expected, uint64_t base,
+                     const int32_t* __restrict__ frontier, int32_t fanout, float tight, float wide, uint64_t base,
                      const int64_t* __restrict__ block_rowptr, int32_t* __restrict__ block_col, int32_t* __restrict__ member) {
     wait_for_kernel_before();
-    __shared__ uint64_t cand_key[SEL_NODES][SEL_CAND];
+    __shared__ __align__(16) uint32_t cand_key[SEL_NODES][SEL_CAND];
     __shared__ int32_t cand_pos[SEL_NODES][SEL_CAND];
     const int lane = threadIdx.x & 31, sub = threadIdx.x / SEL_LANES, sl = threadIdx.x % SEL_LANES;
     const int shift = lane & 16;                       // first lane of this node's half
@@ -141,40 +145,54 @@ sample_select_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restri
         }
     }
     // the others: candidates (both halves of the warp go through the longer row's rounds)
-    const double share = sel ? expected / (double)deg : 1.0;
-    const uint64_t bound = share >= 0.999 ? ~0ULL : (uint64_t)(share * 18446744073709551616.0);
-    const int64_t rounds = sel && fanout <= SEL_FANOUT && deg < (int64_t(1) << 31) ? (deg + SEL_LANES - 1) / SEL_LANES : 0;  // positions are 32-bit
-    const int64_t other = __shfl_xor_sync(0xffffffffu, rounds, 16);
-    const int64_t most = rounds > other ? rounds : other;
+    const bool collect = sel && fanout <= SEL_FANOUT && deg < (int64_t(1) << 31);  // positions are 32-bit
     int64_t count = 0;
-    for (int64_t t = 0; t < most; ++t) {
-        const int64_t q = t * SEL_LANES + sl;
-        const uint64_t key = mix_step(base ^ (vkey | (uint64_t)q));
-        const bool cand = sel && q < deg && key <= bound;
-        const unsigned votes = (__ballot_sync(0xffffffffu, cand) >> shift) & 0xFFFFu;
-        const int64_t at = count + __popc(votes & below);
-        if (cand && at < SEL_CAND) {
-            cand_key[sub][at] = key;
-            cand_pos[sub][at] = (int32_t)q;
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        const bool mine = collect && (attempt == 0 || count < fanout);
+        if (attempt == 1 && (!__any_sync(0xffffffffu, mine) || wide <= tight)) break;
+        const float share = (attempt == 0 ? tight : wide) / (float)deg;
+        const uint32_t bound = share >= 0.999f ? 0xFFFFFFFFu : (uint32_t)(share * 4294967296.f);
+        const int rounds = mine ? (int)((deg + SEL_LANES - 1) / SEL_LANES) : 0;
+        const int most = max(rounds, __shfl_xor_sync(0xffffffffu, rounds, 16));
+        if (mine) count = 0;
+        for (int t = 0; t < most; ++t) {
+            const uint32_t q = (uint32_t)t * SEL_LANES + sl;
+            const uint32_t key = (uint32_t)(mix_step(base ^ (vkey | (uint64_t)q)) >> 32);
+            const bool cand = mine && q < (uint32_t)deg && key <= bound;
+            const unsigned votes = (__ballot_sync(0xffffffffu, cand) >> shift) & 0xFFFFu;
+            const int64_t at = count + __popc(votes & below);
+            if (cand && at < SEL_CAND) {
+                cand_key[sub][at] = key;
+                cand_pos[sub][at] = (int32_t)q;
+            }
+            count += __popc(votes);
         }
-        count += __popc(votes);
+    }
+    bool ok = collect && count >= fanout && count <= SEL_CAND;
+    const int m = ok ? (int)count : 0;
+    if (sl < 3 && m + sl < (m + 3) / 4 * 4) cand_key[sub][m + sl] = 0xFFFFFFFFu;  // up to whole vectors: never smaller than a key
+    __syncwarp();
+    unsigned keep_mask = 0;  // bit t: the lane's candidate 16 t + sl is kept
+    int kept = 0;
+    for (int c0 = 0; c0 < m; c0 += SEL_LANES) {  // nothing crosses the halves
+        const int c = c0 + sl;
+        const uint32_t key = c < m ? cand_key[sub][c] : 0xFFFFFFFFu;
+        int rank = 0;  // candidates with a smaller key
+        for (int j = 0; j < m; j += 4) {
+            const uint4 other = *reinterpret_cast<const uint4*>(&cand_key[sub][j]);
+            rank += (other.x < key) + (other.y < key) + (other.z < key) + (other.w < key);
+        }
+        const bool keep = c < m && rank < fanout;
+        keep_mask |= keep ? 1u << (c0 / SEL_LANES) : 0u;
+        kept += __popc(__ballot_sync(0xFFFFu << shift, keep));
     }
     __syncwarp();
-    const bool ok = sel && count >= fanout && count <= SEL_CAND;
-    const int m = ok ? (int)count : 0;
-    const int m_most = max(m, __shfl_xor_sync(0xffffffffu, m, 16));
+    ok = ok && kept == fanout;  // more of them: candidates that share the upper half of the last kept key
+    const int m_write = ok ? m : 0, m_most = max(m_write, __shfl_xor_sync(0xffffffffu, m_write, 16));
     int64_t at = out;
     for (int c0 = 0; c0 < m_most; c0 += SEL_LANES) {
-        const int c = c0 + sl;
-        const uint64_t key = c < m ? cand_key[sub][c] : ~0ULL;
-        int rank = 0;  // candidates that come before this one: smaller keys, and equal keys earlier in the row
-        for (int j = 0; j < m; ++j) {
-            const uint64_t other_key = cand_key[sub][j];
-            rank += (other_key < key || (other_key == key && j < c)) ? 1 : 0;
-        }
-        __syncwarp();
-        bool keep = c < m && rank < fanout;
-        const int32_t u = keep ? col[begin + cand_pos[sub][c]] : 0;
+        bool keep = c0 < m_write && (keep_mask >> (c0 / SEL_LANES) & 1u);
+        const int32_t u = keep ? col[begin + cand_pos[sub][c0 + sl]] : 0;
         if (keep && !rtma_index_ok(u, n, 5)) keep = false;
         const unsigned votes = (__ballot_sync(0xffffffffu, keep) >> shift) & 0xFFFFu;
         if (keep) {
@@ -249,9 +267,10 @@ extern "C" int32_t rtma_sample_hop(rtma_ctx* ctx, int64_t n, const int64_t* rowp
         const uint64_t base = z ^ (z >> 31);
         KernelScope ks(ctx, KC_LINK, stream);
         // candidates per row (see the kernel)
-        const double expected = std::min((double)fanout + 6.0 * std::sqrt((double)fanout) + 16.0, 0.5 * ((double)fanout + SEL_CAND));
+        const double root = std::sqrt((double)fanout), half_way = 0.5 * ((double)fanout + SEL_CAND);
+        const float tight = (float)std::min(fanout + 2.7 * root + 1.0, half_way), wide = (float)std::min(fanout + 6.0 * root + 16.0, half_way);
         launch_kernel(fanout > SEL_RARE ? sample_select_kernel<true> : sample_select_kernel<false>, (unsigned)ceil_div(frontier_size, SEL_NODES), 256, 0, stream,
-            rowptr, col, n, frontier_size, frontier, fanout, expected, base, block_rowptr, block_col, member);
+            rowptr, col, n, frontier_size, frontier, fanout, tight, wide, base, block_rowptr, block_col, member);
     }
     RTMA_LAUNCH_CHECK(ctx);
     RTMA_TRY(exclusive_scan_i32_to_i64(ctx, member, n, position, scratch, stream));

@@ -60,3 +60,19 @@ def test_sampled_blocks_match_the_oracle(util, which):
         e = c.sample_hop(d_rp, d_col, torch.empty(0, dtype=torch.int32, device="cuda"), 4, 99, 0)
         assert e[0].cpu().tolist() == [0] and e[1].numel() == 0 and e[2].numel() == 0
     c.check()
+
+
+@pytest.mark.parametrize("fanout", [1, 5, 10, 35, 36, 64, 95, 96, 97])
+def test_rows_at_the_edges_of_the_selection(util, fanout):
+    # degrees around the fan-out, around the rounds of 16 entries and the room for 128 candidates; enough rows of each that
+    # some have too few candidates at the first bound and go through their row again
+    edges = sorted({0, 1, max(fanout - 1, 0), fanout, fanout + 1, fanout + 2, 2 * fanout + 1, 15, 16, 17, 31, 32, 33, 127, 128, 129, 300, 1_000})
+    rng = np.random.default_rng(fanout)
+    deg = rng.permutation(np.repeat(edges, 150))
+    n = deg.size
+    rp = np.concatenate([[0], np.cumsum(deg)]).astype(np.int64)
+    cp = rng.integers(0, n, size=int(rp[-1])).astype(np.int32)
+    frontier = np.arange(n - 1, dtype=np.int32)                     # the last warp has one node
+    got = util.ctx().sample_hop(util.dev(rp), util.dev(cp), util.dev(frontier), fanout, 2**40 + fanout, 2)
+    for a, b in zip(got, oracle.sample_hop(rp, cp, frontier, fanout, 2**40 + fanout, 2)):
+        assert np.array_equal(a.cpu().numpy(), b)
