@@ -54,6 +54,13 @@ __device__ __forceinline__ void add_pair(float& a0, float& a1, float b0, float b
         : "+f"(a0), "+f"(a1)
         : "f"(b0), "f"(b1));
 }
+// (a0, a1) += b * (c0, c1) as one instruction, each rounded once
+__device__ __forceinline__ void fma_pair(float& a0, float& a1, float b, float c0, float c1) {
+    asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %2};\n\tmov.b64 c, {%3, %4};\n\tfma.rn.f32x2 a, b, c, a;\n\t"
+        "mov.b64 {%0, %1}, a;\n\t}"
+        : "+f"(a0), "+f"(a1)
+        : "f"(b), "f"(c0), "f"(c1));
+}
 // (x0, x1) -> packed hi and lo words, bit for bit as in Pack8::to_planes_cvt: both remainders by one fused pair
 // operation (hi * -1 + x is exact)
 __device__ __forceinline__ void split_pair(float x0, float x1, uint32_t& h, uint32_t& l) {
