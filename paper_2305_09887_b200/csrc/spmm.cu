@@ -246,8 +246,8 @@ __device__ __forceinline__ void
 spmm_rows(const GroupDesc& g, const int64_t* __restrict__ rowptr_out,
           const int32_t* __restrict__ col_out, const float* __restrict__ inv_deg, const Planes src, const Planes out,
           const int d, const int64_t total_groups, const SpmmOrder order, int* __restrict__ ticket) {
-    // neighbours' rows a lane has in flight
-    constexpr int W = NCH == 1 ? 8 : 4;
+    // neighbours' rows a lane has in flight (spmm_blocks_per_sm)
+    constexpr int W = NCH == 1 && MODE != 2 ? 8 : 4;
     const int lane = threadIdx.x & 31;
     const uint32_t src_row_bytes = (uint32_t)src.ld * 2u;
     bool live[NCH];          // the lane's 8 columns of chunk c exist
@@ -430,8 +430,13 @@ spmm_rows(const GroupDesc& g, const int64_t* __restrict__ rowptr_out,
     }
 }
 
+// Blocks of eight warps per SM.  Rows up to 256 values: two with eight rows in flight per lane, or three with four, which took as
+// long forward (97 / 99 us for 200,000 rows, 618,000 entries) and longer backward (101 / 105), but less with self
+// loops (131 / 114).  Up to 512 values, four rows in flight: one 680, two 519 (500,000 rows, 1.9 M entries; backward 710 / 538).
+constexpr int spmm_blocks_per_sm(int nch, int mode) { return nch == 1 ? (mode == 2 ? 3 : 2) : nch == 2 ? 2 : 1; }
+
 template <int NCH, int MODE>
-__global__ void __launch_bounds__(SPMM_THREADS, NCH == 1 ? 2 : 1)
+__global__ void __launch_bounds__(SPMM_THREADS, spmm_blocks_per_sm(NCH, MODE))
 spmm_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict__ rowptr_out,
             const int32_t* __restrict__ col_out, const float* __restrict__ inv_deg, const Planes src, const Planes out,
             const int d, const int64_t total_groups, const SpmmOrder order, int* __restrict__ ticket) {
@@ -794,7 +799,7 @@ int32_t dispatch_spmm(rtma_ctx* ctx, int kclass, const GroupDesc& g, const int64
         return RTMA_OK;
     }
     const int sms = ctx->sm_count;
-    const int blocks_per_sm = d <= 256 ? 2 : 1;
+    const int blocks_per_sm = d <= 64 ? 2 : spmm_blocks_per_sm(d <= 256 ? 1 : d <= 512 ? 2 : 4, MODE);
     const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(groups, SPMM_THREADS / 32), (int64_t)sms * blocks_per_sm);
 #define RTMA_SPMM(N)                                                                                      \
     do {                                                                                                  \
