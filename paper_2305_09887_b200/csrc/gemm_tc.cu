@@ -11,7 +11,7 @@
 //                 layer) and dgrad ([dZ | Abar^T dZ] times [Ws^T; Wn^T], gated by the sign of H
 //                 and written as planes over H).  A tiles are K-major straight from the planes,
 //                 B from the repacked weights.
-//   wgrad kernel  D[128 x d_out] = A^T * dZ over a chunk of rows, A = H or Abar H.  Both
+//   wgrad kernel  D[128 x 64 n] = dZ^T * [H | Abar H] over a chunk of rows.  Both
 //                 operands are MN-major straight from the planes.  Rows between parts are
 //                 zero in every plane, so chunks need no masking.  The bias gradient (column
 //                 sums of dZ) is added up from the staged dZ tiles by the otherwise idle
@@ -579,20 +579,31 @@ struct WgradArgs {
     GroupDesc g;
     SplitPlan sp;
     CUtensorMap mapHh, mapHl, mapNh, mapNl, mapZh, mapZl;
-    int d_in, d_out, nsrc;
-    int jt_per_src;   // 128-wide tiles over d_in, per source
-    int n_atoms;      // 64-wide atoms over d_out (all column tiles together); a tile takes up to 4
-    int acc_cols;     // tensor-memory columns of one accumulator
+    int d_in, d_out;
+    int src_atoms;    // 64-wide atoms over d_in, per source
+    int total_atoms;  // of all sources
+    int col_atoms;    // of them a block takes (the last block of a chunk may have fewer)
+    int z_tiles;      // 128-wide tiles over d_out that a block takes: 1 or 2
     int tmem_cols, stages;
     int bk;           // rows (k) per pipeline stage: 64 or 32
     int single;       // 1: operands rounded to bf16 (hi planes only)
-    float* partial;   // [slot][(2 d_in + 1) x d_out]
+    CUtensorMap mapP; // partial as rows of d_out values, boxes of 32 x 32
+    float* partial;   // [slot][(nsrc d_in + 1)] rows, padded_ld(d_out) apart
+    int64_t ld_partial;
     int* error_word;
 };
 
-// A block accumulates TWO 128-wide tiles of the left operand (both sources of a two-matrix layer, or
-// two neighbouring tiles of one source) against the same staged dZ tile, each into its own
-// accumulator: the dZ tile, the larger operand, crosses the shared-memory fill path once for both.
+// The product is taken transposed: the gradient dZ is the operand whose columns are the accumulator's rows (one or two
+// tiles of 128 of them), the sources' columns, H's and behind them N's, are the accumulator's columns, as many atoms of 64
+// as the tensor memory and the stages have room for (wgrad_shape).  A few classes then cost one MMA with 256 columns where
+// they cost two with 64 or 128.  The partial sums leave through shared memory, 32 x 32 of them by a bulk-tensor store, in rows
+// padded to 16 bytes (stored by the threads, 16 bytes of 32 rows at a time, they took 4 us of an 18 us launch; stored down
+// their columns, a line per warp, 8 us more than that).  The thread that issues the MMAs is as easily the longest chain as the loads are, with one
+// plane per operand above all: its loop keeps descriptors as a constant plus an address and no division by the number of
+// stages (500,000 rows, 1,024 x 512 in bf16: 658 us, with this form and divisions 975, now 574).
+// us a launch before and after: the head of 47 classes on 200 k rows of 256 62 / 55, on 2 M 615 / 495, of two classes on 5 M
+// 1,390 / 1,152; 512 -> 256 on 200 k rows 145 / 130, on 2 M 1,400 / 1,272; 256 -> 256 on 5 M 1,910 / 1,840 (5.6 TB/s; 1,634
+// without the MMAs); 180 -> 90 on three parts of 10 k rows 18 / 13.
 __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_constant__ WgradArgs a) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ PipeBarriers pb;
@@ -605,54 +616,43 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
     const int v1 = min(n_p, v0 + a.sp.rows_per_split[k]);
     const int BK = a.bk;
     const int KB = (v1 - v0 + BK - 1) / BK;
-    const int total_a = a.nsrc * a.jt_per_src;                 // left-operand tiles of the layer
-    const int na_tiles = min(2, total_a - 2 * (int)blockIdx.x);  // of this block: 1 or 2
-    int src_of[2], j0_of[2];
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        const int at = min(2 * (int)blockIdx.x + t, total_a - 1);
-        src_of[t] = at / a.jt_per_src;
-        j0_of[t] = (at % a.jt_per_src) * TC_BM;
-    }
     const int d_in = a.d_in, d_out = a.d_out;
+    const int first_atom = (int)blockIdx.x * a.col_atoms;             // of the sources' columns
+    const int NA = min(a.col_atoms, a.total_atoms - first_atom);      // atoms of this block
+    const int cbase = (int)blockIdx.z * a.z_tiles * TC_BM;            // first output column
+    const int ccount = min(a.z_tiles * TC_BM, d_out - cbase);         // output columns of this block
+    const int ZA = (ccount + 63) / 64, z_tiles = (ccount + TC_BM - 1) / TC_BM;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int cbase = blockIdx.z * 256;                       // first output column of this tile
-    const int ccount = min(256, d_out - cbase);               // valid columns in it
-    float* P = a.partial + (int64_t)slot * (a.nsrc * d_in + 1) * d_out;
+    const int64_t bias_row = (int64_t)a.total_atoms / a.src_atoms * d_in;  // behind the sources' columns
+    const int64_t slot_row = (int64_t)slot * (bias_row + 1);
+    float* P = a.partial + slot_row * a.ld_partial + cbase;
 
     const bool bias_tile = blockIdx.x == 0;  // these blocks also produce the bias gradient of their columns
 
     if (KB == 0) {  // empty chunk: the gradient contribution is zero
         wait_for_kernel_before();
-        for (int t = 0; t < na_tiles; ++t)
-            for (int idx = threadIdx.x; idx < TC_BM * ccount; idx += TC_THREADS) {
-                const int j = j0_of[t] + idx / ccount;
-                if (j < d_in) P[(int64_t)(src_of[t] * d_in + j) * d_out + cbase + idx % ccount] = 0.f;
-            }
+        for (int idx = threadIdx.x; idx < 64 * NA * ccount; idx += TC_THREADS) {
+            const int at = first_atom + idx / ccount / 64, j = at % a.src_atoms * 64 + idx / ccount % 64;
+            if (j < d_in) P[((int64_t)(at / a.src_atoms) * d_in + j) * a.ld_partial + idx % ccount] = 0.f;
+        }
         if (bias_tile)
-            for (int c = threadIdx.x; c < ccount; c += TC_THREADS) P[(int64_t)a.nsrc * d_in * d_out + cbase + c] = 0.f;
+            for (int c = threadIdx.x; c < ccount; c += TC_THREADS) P[bias_row * a.ld_partial + c] = 0.f;
         return;
     }
 
     uint8_t* smem = align_1024(smem_raw);
-    const int stages = a.stages, NA = min(4, a.n_atoms - 4 * (int)blockIdx.z);
+    const int stages = a.stages;
     const uint32_t ATOM_BYTES = (uint32_t)BK * 128u;  // one 64-wide column of BK k-rows
-    const uint32_t a_tile_bytes = 2u * ATOM_BYTES;     // one plane of one left-operand tile
-    const uint32_t a_plane_bytes = 2u * a_tile_bytes;  // room for two tiles
-    const uint32_t b_plane_bytes = (uint32_t)NA * ATOM_BYTES;
     const bool single = a.single != 0;
     const uint32_t np = single ? 1u : 2u;  // planes staged per operand
-    const uint32_t stage_bytes = np * (a_plane_bytes + b_plane_bytes);
-    // 64-column halves of the left-operand tiles that hold columns of the matrix; the others are not loaded (what their part
-    // of shared memory holds only reaches accumulator rows that are not stored)
-    int halves[2];
-#pragma unroll
-    for (int t = 0; t < 2; ++t) halves[t] = t < na_tiles ? (j0_of[t] + 64 < d_in ? 2 : 1) : 0;
-    const uint32_t tx_bytes = np * ((uint32_t)(halves[0] + halves[1]) * ATOM_BYTES + b_plane_bytes);
-    auto a_hi = [&](int s) { return smem + (size_t)s * stage_bytes; };
-    auto a_lo = [&](int s) { return smem + (size_t)s * stage_bytes + a_plane_bytes; };
-    auto b_hi = [&](int s) { return smem + (size_t)s * stage_bytes + np * a_plane_bytes; };
-    auto b_lo = [&](int s) { return smem + (size_t)s * stage_bytes + np * a_plane_bytes + b_plane_bytes; };
+    const uint32_t z_bytes = (uint32_t)ZA * ATOM_BYTES, s_bytes = (uint32_t)NA * ATOM_BYTES;
+    const uint32_t stage_bytes = np * (z_bytes + s_bytes);  // no more than the launch counted on
+    // A stage: dZ, then the sources, hi before lo.  Where the last tile of dZ has one atom, the MMA reads whatever lies behind it
+    // as the other: that only reaches accumulator rows that are not stored.
+    auto z_hi = [&](int s) { return smem + (size_t)s * stage_bytes; };
+    auto z_lo = [&](int s) { return smem + (size_t)s * stage_bytes + z_bytes; };
+    auto s_hi = [&](int s) { return smem + (size_t)s * stage_bytes + np * z_bytes; };
+    auto s_lo = [&](int s) { return smem + (size_t)s * stage_bytes + np * z_bytes + s_bytes; };
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < stages; ++s) {
@@ -676,54 +676,57 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
     tc::tc_fence_after_sync();
     wait_for_kernel_before();
     const uint32_t tmem_base = pb.tmem_base;
+    const uint32_t acc_cols = 64u * (uint32_t)NA;  // accumulator columns of one tile of dZ
 
     if (warp == 0) {
         if (lane == 0) {
             const int row = (int)(a.g.row_ws[k] + v0);
-            for (int kb = 0; kb < KB; ++kb) {
-                const int s = kb % stages;
-                if (!wait_or_abort(&pb.empty[s], ((kb / stages) & 1) ^ 1, &pb, a.error_word)) break;
-                tc::mbar_arrive_expect_tx(&pb.full[s], tx_bytes);
-                for (int t = 0; t < na_tiles; ++t) {
-                    const CUtensorMap* mapAh = src_of[t] == 0 ? &a.mapHh : &a.mapNh;
-                    const CUtensorMap* mapAl = src_of[t] == 0 ? &a.mapHl : &a.mapNl;
-                    for (int h = 0; h < halves[t]; ++h) {
-                        tc::tma_load_2d(a_hi(s) + t * a_tile_bytes + h * ATOM_BYTES, mapAh, &pb.full[s], j0_of[t] + 64 * h, row + kb * BK);
-                        if (!single)
-                            tc::tma_load_2d(a_lo(s) + t * a_tile_bytes + h * ATOM_BYTES, mapAl, &pb.full[s], j0_of[t] + 64 * h, row + kb * BK);
-                    }
+            tc::RingAt at;
+            for (int kb = 0; kb < KB; ++kb, at.advance(stages)) {
+                const int s = at.s;
+                if (!wait_or_abort(&pb.empty[s], at.phase ^ 1u, &pb, a.error_word)) break;
+                tc::mbar_arrive_expect_tx(&pb.full[s], stage_bytes);
+                for (int t = 0; t < ZA; ++t) {
+                    tc::tma_load_2d(z_hi(s) + t * ATOM_BYTES, &a.mapZh, &pb.full[s], cbase + 64 * t, row + kb * BK);
+                    if (!single) tc::tma_load_2d(z_lo(s) + t * ATOM_BYTES, &a.mapZl, &pb.full[s], cbase + 64 * t, row + kb * BK);
                 }
                 for (int t = 0; t < NA; ++t) {
-                    tc::tma_load_2d(b_hi(s) + t * ATOM_BYTES, &a.mapZh, &pb.full[s], cbase + 64 * t, row + kb * BK);
-                    if (!single) tc::tma_load_2d(b_lo(s) + t * ATOM_BYTES, &a.mapZl, &pb.full[s], cbase + 64 * t, row + kb * BK);
+                    const bool second = first_atom + t >= a.src_atoms;
+                    const int x = 64 * (first_atom + t - (second ? a.src_atoms : 0));
+                    tc::tma_load_2d(s_hi(s) + t * ATOM_BYTES, second ? &a.mapNh : &a.mapHh, &pb.full[s], x, row + kb * BK);
+                    if (!single) tc::tma_load_2d(s_lo(s) + t * ATOM_BYTES, second ? &a.mapNl : &a.mapHl, &pb.full[s], x, row + kb * BK);
                 }
             }
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            const uint32_t idesc = tc::idesc_bf16(TC_BM, 64 * NA, true, true);
-            for (int kb = 0; kb < KB; ++kb) {
-                const int s = kb % stages;
-                if (!wait_or_abort(&pb.full[s], (kb / stages) & 1, &pb, a.error_word)) break;
+            // up to 256 columns per MMA.  One thread feeds the tensor core: descriptors are a constant plus an address.
+            const uint32_t idesc0 = tc::idesc_bf16(TC_BM, 64 * min(NA, 4), true, true), idesc1 = tc::idesc_bf16(TC_BM, 64 * max(NA - 4, 1), true, true);
+            const uint64_t desc = tc::smem_desc_sw128(0, ATOM_BYTES, 1024);
+            const uint32_t atom = ATOM_BYTES >> 4;  // addresses of descriptors are in units of 16 bytes
+            // the products of one 128-wide tile of dZ with one group of the sources' atoms
+            auto product = [&](uint32_t d_tmem, uint32_t zh, uint32_t zl, uint32_t sh, uint32_t sl, uint32_t idesc, uint32_t accumulate) {
+                if (single) {
+                    tc::mma_bf16(d_tmem, desc + zh, desc + sh, idesc, accumulate);
+                } else {
+                    tc::mma_bf16(d_tmem, desc + zh, desc + sl, idesc, accumulate);
+                    tc::mma_bf16(d_tmem, desc + zl, desc + sh, idesc, 1u);
+                    tc::mma_bf16(d_tmem, desc + zh, desc + sh, idesc, 1u);
+                }
+            };
+            tc::RingAt at;
+            for (int kb = 0; kb < KB; ++kb, at.advance(stages)) {
+                const int s = at.s;
+                if (!wait_or_abort(&pb.full[s], at.phase, &pb, a.error_word)) break;
                 tc::tc_fence_after_sync();
-                const uint32_t bh = tc::smem_u32(b_hi(s)), bl = tc::smem_u32(b_lo(s));
+                uint32_t zh = tc::smem_u32(z_hi(s)) >> 4, zl = tc::smem_u32(z_lo(s)) >> 4, sh = tc::smem_u32(s_hi(s)) >> 4, sl = tc::smem_u32(s_lo(s)) >> 4;
+#pragma unroll 2
                 for (int ks = 0; ks < BK / 16; ++ks) {
-                    const uint32_t off = ks * 2048;  // 16 k-rows of 128 bytes
-                    const uint64_t dbh = tc::smem_desc_sw128(bh + off, ATOM_BYTES, 1024);
-                    const uint64_t dbl = tc::smem_desc_sw128(bl + off, ATOM_BYTES, 1024);
-                    for (int t = 0; t < na_tiles; ++t) {
-                        const uint32_t d_tmem = tmem_base + (uint32_t)(t * a.acc_cols);
-                        const uint32_t ah = tc::smem_u32(a_hi(s) + t * a_tile_bytes), al = tc::smem_u32(a_lo(s) + t * a_tile_bytes);
-                        const uint64_t dah = tc::smem_desc_sw128(ah + off, ATOM_BYTES, 1024);
-                        if (single) {
-                            tc::mma_bf16(d_tmem, dah, dbh, idesc, (kb | ks) ? 1u : 0u);
-                        } else {
-                            const uint64_t dal = tc::smem_desc_sw128(al + off, ATOM_BYTES, 1024);
-                            tc::mma_bf16(d_tmem, dal, dbh, idesc, (kb | ks) ? 1u : 0u);
-                            tc::mma_bf16(d_tmem, dah, dbl, idesc, 1u);
-                            tc::mma_bf16(d_tmem, dah, dbh, idesc, 1u);
-                        }
-                    }
+                    const uint32_t accumulate = (kb | ks) ? 1u : 0u;
+                    product(tmem_base, zh, zl, sh, sl, idesc0, accumulate);
+                    if (z_tiles > 1) product(tmem_base + acc_cols, zh + 2 * atom, zl + 2 * atom, sh, sl, idesc0, accumulate);
+                    else if (NA > 4) product(tmem_base + 256u, zh, zl, sh + 4 * atom, sl + 4 * atom, idesc1, accumulate);
+                    zh += 128; zl += 128; sh += 128; sl += 128;  // 16 k-rows of 128 bytes
                 }
                 tc::mma_commit(&pb.empty[s]);
             }
@@ -743,15 +746,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
             for (int e = 0; e < 8; ++e) colsum[t][e] = 0.f;
         bool ok = true;
         if (bias_tile) {
-            for (int kb = 0; kb < KB && ok; ++kb) {
-                const int s = kb % stages;
-                ok = wait_or_abort(&pb.full[s], (kb / stages) & 1, &pb, a.error_word);
+            tc::RingAt at;
+            for (int kb = 0; kb < KB && ok; ++kb, at.advance(stages)) {
+                const int s = at.s;
+                ok = wait_or_abort(&pb.full[s], at.phase, &pb, a.error_word);
                 if (!ok) break;
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
-                    if (t < NA) {
-                        const uint4* bh = reinterpret_cast<const uint4*>(b_hi(s) + t * ATOM_BYTES);
-                        const uint4* bl = reinterpret_cast<const uint4*>(b_lo(s) + t * ATOM_BYTES);
+                    if (t < ZA) {
+                        const uint4* bh = reinterpret_cast<const uint4*>(z_hi(s) + t * ATOM_BYTES);
+                        const uint4* bl = reinterpret_cast<const uint4*>(z_lo(s) + t * ATOM_BYTES);
                         for (int i = 0; i < BK / 16; ++i) {
                             Pack8 p;
                             p.zero();
@@ -769,8 +773,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
         ok = *reinterpret_cast<volatile int*>(&pb.abort) == 0;
         tc::tc_fence_after_sync();
         if (ok && bias_tile) {
-            // every load has landed and every MMA has finished: stage 0 is free to hold the sums
-            float* red = reinterpret_cast<float*>(a_hi(0));  // [128 threads][32]
+            // every load has landed and every MMA has finished: the ring is free to hold the sums
+            float* red = reinterpret_cast<float*>(smem);  // [128 threads][32]
 #pragma unroll
             for (int t = 0; t < 4; ++t)
 #pragma unroll
@@ -780,46 +784,51 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
                 const int t = c >> 6, lc = (c & 63) >> 3, e = c & 7;
                 float sum = 0.f;
                 for (int h = 0; h < 16; ++h) sum += red[(h * 8 + (lc ^ (h & 7))) * 32 + t * 8 + e];  // fixed order
-                P[(int64_t)a.nsrc * d_in * d_out + cbase + c] = sum;
+                P[bias_row * a.ld_partial + c] = sum;
             }
         }
         if (ok) {
+            // A lane holds output column c of 32 source columns j: through a 32 x 32 slab (row j, 16-byte piece c / 4 at piece
+            // c / 4 ^ j % 8, as the map's swizzle has it; the ring is free, behind the column sums' 16 KB) and out as a box.
             const int q = warp & 3;
-            // Every thread stores its own row, four floats at a time; where rows do not start on 16-byte boundaries (90 columns,
-            // or an odd number of parameters) that would be single floats, 32 rows apart (23 us a launch on chunks of 256 rows, 18
-            // this way): then 32 x 32 blocks go through shared memory (the ring is free: behind the column sums' 16 KB, 33 floats
-            // a row) and a store writes 128 bytes of a row.  With aligned rows the detour costs more: 48.6 -> 52.3 us.
-            const bool vec_ok = (d_out % 4 == 0) && (reinterpret_cast<uintptr_t>(P) % 16 == 0);
-            float* slab = reinterpret_cast<float*>(a_hi(0) + 16384) + q * 32 * 33;
-            for (int t = 0; t < na_tiles; ++t) {
-                const int j0 = j0_of[t] + q * 32;
-                const int rows_here = min(32, d_in - j0);
-                if (rows_here <= 0) continue;
-                float* o = P + (int64_t)(src_of[t] * d_in + j0) * d_out + cbase + lane;
-                for (int c0 = 0; c0 < 64 * NA; c0 += 32) {
-                    float v[32];
-                    tc::tmem_load_32x32(tmem_base + (uint32_t)(t * a.acc_cols) + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);
-                    if (vec_ok) {
-                        if (lane < rows_here) {
-                            float* own = P + (int64_t)(src_of[t] * d_in + j0 + lane) * d_out + cbase + c0;
-#pragma unroll
-                            for (int jj = 0; jj < 32; jj += 4)
-                                if (c0 + jj < ccount) *reinterpret_cast<float4*>(own + jj) = make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]);
-                        }
+            uint8_t* slab[2] = {smem + 16384 + q * 8192, smem + 16384 + q * 8192 + 4096};
+            int n_out = 0;
+            for (int t = 0; t < z_tiles; ++t) {
+                const int c0 = t * TC_BM + q * 32;                 // the warp's first output column
+                if (c0 >= ccount) break;
+                const uint32_t acc = tmem_base + (uint32_t)t * acc_cols + ((uint32_t)(q * 32) << 16);
+#pragma unroll 1
+                for (int n = 0; n < 2 * NA; ++n) {
+                    const bool second = first_atom + n / 2 >= a.src_atoms;
+                    const int j0 = 64 * (first_atom + n / 2 - (second ? a.src_atoms : 0)) + 32 * (n & 1);  // first source column of the 32
+                    if (j0 >= d_in) continue;
+                    uint32_t raw[32];
+                    tc::tmem_load_issue(acc + 32u * (uint32_t)n, raw);
+                    tc::tmem_load_wait(raw);
+                    const int64_t row = slot_row + (second ? d_in : 0) + j0;
+                    if (j0 + 32 <= d_in) {
+                        uint8_t* out = slab[n_out++ & 1];
+                        if (lane == 0) tc::tma_store_wait_read_but_one();  // the box before the last has left the slab
                         __syncwarp();
-                        continue;
-                    }
-                    if (c0 >= ccount) break;
-                    __syncwarp();
 #pragma unroll
-                    for (int jj = 0; jj < 32; ++jj) slab[lane * 33 + jj] = v[jj];
-                    __syncwarp();
-                    if (c0 + lane < ccount) {
-#pragma unroll 8
-                        for (int r = 0; r < rows_here; ++r) o[(int64_t)r * d_out + c0] = slab[r * 33 + lane];
+                        for (int e = 0; e < 32; ++e)
+                            *reinterpret_cast<uint32_t*>(out + e * 128 + (((lane >> 2) ^ (e & 7)) << 4) + (lane & 3) * 4) = raw[e];
+                        tc::fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0) {
+                            tc::tma_store_2d(&a.mapP, out, cbase + c0, (int)row);
+                            tc::tma_store_commit();
+                        }
+                    } else if (c0 + lane < ccount) {  // the source's last columns: the rows behind them are not its
+                        float* o = a.partial + row * a.ld_partial + cbase + c0 + lane;
+#pragma unroll
+                        for (int e = 0; e < 32; ++e)
+                            if (j0 + e < d_in) o[(int64_t)e * a.ld_partial] = __uint_as_float(raw[e]);
                     }
+                    __syncwarp();
                 }
             }
+            if (lane == 0) tc::tma_store_wait_all();
         }
     }
     tc::tc_fence_before_sync();
@@ -913,6 +922,18 @@ bool make_tensor_map_bf16(CUtensorMap* out, const void* base, uint64_t rows, uin
     return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), gdim, gstride, box, estride,
               CU_TENSOR_MAP_INTERLEAVE_NONE, box_cols <= 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// fp32 rows in boxes of 32 x 32, 128-byte swizzle
+static bool make_tensor_map_f32(CUtensorMap* out, const float* base, uint64_t rows, uint64_t cols, uint64_t ld) {
+    EncodeTiledFn fn = encode_tiled();
+    if (!fn || rows == 0 || cols == 0) return false;
+    const cuuint64_t gdim[2] = {cols, rows};
+    const cuuint64_t gstride[1] = {ld * sizeof(float)};
+    const cuuint32_t box[2] = {32, 32};
+    const cuuint32_t estride[2] = {1, 1};
+    return fn(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // Column tile of the rows kernel for `d` columns: at most 256 wide, equal tiles, a multiple of 16; from 64 columns on a
@@ -1091,12 +1112,32 @@ int32_t launch_tc_dgrad(rtma_ctx* ctx, const GroupDesc& g, LayerShape ls, const 
     return launch_rows(ctx, a, rows_total, pairs, KC_GEMM_DGRAD, s);
 }
 
+// How a chunk of a layer's weight gradient is cut into blocks.  Two tiles of dZ leave tensor memory for four atoms of the sources,
+// one for eight; and three stages of 32 rows are to fit (16 atoms of one plane, 8 of two).
+struct WgradShape {
+    int z_tiles, z_atoms;        // of dZ, per block
+    int col_atoms, total_atoms;  // of the sources: per block, of all
+    int blocks_x, blocks_z;
+};
+static WgradShape wgrad_shape(const LayerShape& ls, bool single) {
+    WgradShape w;
+    const int all_z = (int)ceil_div(ls.d_out, 64);
+    w.z_tiles = all_z > 2 ? 2 : 1;
+    w.z_atoms = std::min(all_z, 2 * w.z_tiles);
+    w.total_atoms = ls.nsrc * (int)ceil_div(ls.d_in, 64);
+    const int most = std::min(8 / w.z_tiles, (single ? 16 : 8) - w.z_atoms);
+    w.blocks_x = (int)ceil_div(w.total_atoms, most);
+    w.col_atoms = (int)ceil_div(w.total_atoms, w.blocks_x);
+    w.blocks_z = (int)ceil_div(all_z, 2 * w.z_tiles);
+    return w;
+}
+
 WgradCost tc_wgrad_cost(const LayerShape& ls, bool single) {
-    const int64_t a_tiles = ls.nsrc * ceil_div(ls.d_in, TC_BM), atoms = ceil_div(ls.d_out, 64);
+    const WgradShape w = wgrad_shape(ls, single);
     WgradCost c;
-    c.blocks_per_slot = ceil_div(a_tiles, 2) * ceil_div(atoms, 4);
-    c.bytes_per_row = (single ? 1 : 2) * 128 * (std::min<int64_t>(a_tiles, 2) * (ls.d_in > 64 ? 2 : 1) + std::min<int64_t>(atoms, 4));
-    c.params = (int64_t)(ls.nsrc * ls.d_in + 1) * ls.d_out;
+    c.blocks_per_slot = (int64_t)w.blocks_x * w.blocks_z;
+    c.bytes_per_row = (single ? 1 : 2) * 128 * (w.z_atoms + w.col_atoms);
+    c.params = (int64_t)(ls.nsrc * ls.d_in + 1) * padded_ld(ls.d_out);
     return c;
 }
 
@@ -1109,25 +1150,27 @@ int32_t launch_tc_wgrad(rtma_ctx* ctx, const GroupDesc& g, const SplitPlan& sp, 
     const int slots = sp.split_begin[g.num];
     if (slots == 0) return RTMA_OK;
     if (slots > 65535) return rtma_fail(ctx, RTMA_ERR_UNSUPPORTED, "too many weight-gradient chunks (%d)", slots);
+    const WgradShape w = wgrad_shape(ls, single);
     WgradArgs a{};
     a.g = g;
     a.sp = sp;
     a.d_in = ls.d_in;
     a.d_out = ls.d_out;
-    a.nsrc = ls.nsrc;
-    a.jt_per_src = (int)ceil_div(ls.d_in, TC_BM);
-    a.n_atoms = (int)ceil_div(ls.d_out, 64);
-    const int tile_atoms = a.n_atoms < 4 ? a.n_atoms : 4;
-    a.acc_cols = 64 * tile_atoms;
-    a.tmem_cols = (int)tmem_columns_for(2 * a.acc_cols);  // two accumulators, at most 512 columns
+    a.src_atoms = w.total_atoms / ls.nsrc;
+    a.total_atoms = w.total_atoms;
+    a.col_atoms = w.col_atoms;
+    a.z_tiles = w.z_tiles;
+    a.tmem_cols = (int)tmem_columns_for(w.z_tiles * 64 * w.col_atoms);
     a.single = single ? 1 : 0;
-    // a stage = two left-operand tiles and the dZ tile, BK rows deep; 32-row stages where 64-row ones
-    // would leave fewer than three of them
-    const size_t stage64 = (single ? 1 : 2) * ((size_t)4 + (size_t)tile_atoms) * 64 * 128;
+    // 32-row stages where 64-row ones would leave fewer than three of them
+    const size_t stage64 = (single ? 1 : 2) * (size_t)(w.z_atoms + w.col_atoms) * 64 * 128;
     a.bk = SMEM_BUDGET / stage64 >= 3 ? 64 : 32;
     const size_t stage_bytes = stage64 * a.bk / 64;
     a.stages = stages_for(stage_bytes, MAX_STAGES);
     a.partial = partial;
+    a.ld_partial = padded_ld(ls.d_out);
+    if (!make_tensor_map_f32(&a.mapP, partial, (uint64_t)slots * (ls.nsrc * ls.d_in + 1), ls.d_out, a.ld_partial))
+        return rtma_fail(ctx, RTMA_ERR_CUDA, "cuTensorMapEncodeTiled refused the partial sums");
     a.error_word = ctx->error_word;
     // boxes of 64 columns x BK rows: one atom of a stage
     if (!plane_maps(&a.mapHh, &a.mapHl, H, rows_total, ls.d_in, 64, (uint32_t)a.bk) ||
@@ -1138,7 +1181,7 @@ int32_t launch_tc_wgrad(rtma_ctx* ctx, const GroupDesc& g, const SplitPlan& sp, 
         a.mapHh = a.mapNh;
         a.mapHl = a.mapNl;
     }
-    dim3 grid((unsigned)ceil_div(ls.nsrc * a.jt_per_src, 2), (unsigned)slots, (unsigned)ceil_div(a.n_atoms, 4));
+    const dim3 grid((unsigned)w.blocks_x, (unsigned)slots, (unsigned)w.blocks_z);
     { KernelScope ks(ctx, KC_GEMM_WGRAD, s); launch_kernel(tc_wgrad_kernel, grid, TC_THREADS, a.stages * stage_bytes + 1024, s, a); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;

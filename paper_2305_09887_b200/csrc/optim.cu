@@ -14,14 +14,15 @@ reduce_sgd_kernel(const __grid_constant__ GroupDesc g, const __grid_constant__ S
                   float* __restrict__ grads_record) {
     wait_for_kernel_before();
     const int k = blockIdx.y;
-    const int64_t stride = (int64_t)(ls.nsrc * ls.d_in + 1) * ls.d_out;  // the weight matrices and the bias row
-    const int64_t count = ls.has_bias ? stride : stride - ls.d_out;       // the bias row is last
+    const int64_t rows = (int64_t)ls.nsrc * ls.d_in;                      // the weight matrices; behind them the bias row
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (i >= count) return;
+    if (i >= (rows + (ls.has_bias ? 1 : 0)) * ls.d_out) return;
+    const int64_t ld = (ls.d_out + 3) / 4 * 4, stride = (rows + 1) * ld;  // of the partial sums
+    const int64_t at_partial = (int64_t)((uint32_t)i / (uint32_t)ls.d_out) * ld + (uint32_t)i % (uint32_t)ls.d_out;
     float gsum = 0.f;
     const int s_end = sp.split_begin[k + 1];
 #pragma unroll 8
-    for (int s = sp.split_begin[k]; s < s_end; ++s) gsum += __ldcs(partial + (int64_t)s * stride + i);  // eight loads in flight
+    for (int s = sp.split_begin[k]; s < s_end; ++s) gsum += __ldcs(partial + (int64_t)s * stride + at_partial);  // eight loads in flight
     const int64_t at = (int64_t)g.part[k] * ls.P + ls.param_offset + i;
     if (grads_record) grads_record[at] = gsum;
     params[at] -= lr * gsum;

@@ -123,7 +123,7 @@ ScratchPlan plan_scratch(const Model& m, bool head, bool record) {
         if (l < m.L - 1) per_row += 4 * planes_ld(m.dims[l + 1]);  // H^{l+1}, later overwritten by dZ^l
         if (l < m.L - 1 && m.post) per_row += 4 * planes_ld(m.dims[l + 1]) + sizeof(float2);  // Z^{l}, (mean, 1/std)
         if (l >= 1 && !(head && l == m.L - 1)) q_width = std::max(q_width, m.dims[l + 1]);
-        sp.max_layer_params = std::max(sp.max_layer_params, (size_t)(m.layer[l].nsrc * m.dims[l] + 1) * m.dims[l + 1]);
+        sp.max_layer_params = std::max(sp.max_layer_params, (size_t)(m.layer[l].nsrc * m.dims[l] + 1) * padded_ld(m.dims[l + 1]));
         if (head && l == m.L - 1) sp.max_layer_params = std::max(sp.max_layer_params, (size_t)(m.dims[l] + 1) * 2 * m.Cp);
         if (l < m.L - 1 && m.post) sp.post_width = std::max(sp.post_width, (size_t)m.dims[l + 1]);
         const TcLayerPlan lp = (head && l == m.L - 1) ? tc_plan_head(m.layer[l], m.Cp) : tc_plan_layer(m.layer[l]);
@@ -140,7 +140,7 @@ ScratchPlan plan_scratch(const Model& m, bool head, bool record) {
     sp.per_pair_bytes = 0;
     for (int k = 0; k < m.Kd; ++k) {
         sp.per_pair_bytes += 4 * planes_ld(m.ddims[k]) + 4 * planes_ld(m.ddims[k + 1]);
-        sp.max_decoder_params = std::max(sp.max_decoder_params, (size_t)(m.ddims[k] + 1) * m.ddims[k + 1]);
+        sp.max_decoder_params = std::max(sp.max_decoder_params, (size_t)(m.ddims[k] + 1) * padded_ld(m.ddims[k + 1]));
         sp.prep_bytes += sizeof(__nv_bfloat16) * tc_prep_elems(tc_plan_layer(m.dec[k]), true) + 4 * 256;
         if (k < m.Kd - 1) sp.post_width = std::max(sp.post_width, (size_t)m.ddims[k + 1]);
     }

@@ -258,7 +258,7 @@ struct WgradCost {
     int64_t params;           // partial sums a chunk leaves
 };
 WgradCost tc_wgrad_cost(const LayerShape& ls, bool single);
-// partial[slot][(nsrc d_in + 1) x d_out] = [H | N | 1]^T dZ ([N | 1]^T dZ for a one-matrix layer)
+// partial[slot][(nsrc d_in + 1) x d_out, rows padded_ld(d_out) apart] = [H | N | 1]^T dZ ([N | 1]^T dZ for a one-matrix layer)
 // over one chunk of rows.
 int32_t launch_tc_wgrad(rtma_ctx* ctx, const GroupDesc& g, const SplitPlan& sp, LayerShape ls, int64_t rows_total,
                         Planes H, Planes N, Planes dZ, float* partial, bool single, cudaStream_t s);

@@ -221,3 +221,25 @@ def test_parts_choose_for_themselves(util):
     w, got, want = w2, got2, want2
     auto, never = run(1), run(0)
     assert np.array_equal(auto, never)
+
+
+@pytest.mark.parametrize("n, degree", [(1_340, 3), (1_340, 8), (1_400, 11), (1_300, 60)])
+def test_entries_outside_the_windows(util, forced, tiny_workload, n, degree):
+    # two parts of about 670 rows, 5 tiles and a bit: rows without entries outside their window, with listed ones, with more than
+    # are listed, and two hubs with hundreds
+    g = inputs.uniform_graph(n, n * degree // 2, 31)
+    rows, cols = np.repeat(np.arange(n), np.diff(g.rowptr)), g.col.astype(np.int64)
+    rng = np.random.default_rng(32)
+    hubs = [(v, rng.permutation(n)[:size]) for v, size in ((5, 500), (n - 3, 320))]
+    u = np.concatenate([rows] + [np.full(x.size, v) for v, x in hubs] + [x for _, x in hubs])
+    v = np.concatenate([cols] + [x for _, x in hubs] + [np.full(x.size, w) for w, x in hubs])
+    key = np.unique((u * n + v)[u != v])
+    rowptr = np.zeros(n + 1, dtype=np.int32)
+    np.cumsum(np.bincount(key // n, minlength=n), out=rowptr[1:])
+    w = inputs.Workload(**{**tiny_workload.__dict__})
+    w.graph = inputs.Graph(n=n, rowptr=rowptr, col=(key % n).astype(np.int32))
+    w.M, w.dims = 2, (24, 72, 19)                                    # two atoms; one, of the head's narrow planes
+    w.X, w.y = inputs.normal_features(n, 24, 33), inputs.uniform_labels(n, 19, 34)
+    w.params0 = inputs.xavier_params(w.dims, 35)
+    got, want = util.check_one_step(w)
+    util.check_k_steps_and_average(w, got, want, 2)

@@ -342,3 +342,14 @@ def test_column_tiles_of_odd_multiples_of_32(util, dims, gemm_dtype, variant):
     w = _workload(1_000, 3_000, dims, 91)
     params0 = inputs.variant_params(variant, dims, 92)
     util.check_one_step(w, M=4, gemm_dtype=gemm_dtype, variant=variant, params0=params0, gradients_against_plain=gemm_dtype == 0)
+
+
+# the weight gradient's tiles: one and two tiles of output columns, the last with one atom of 64 or two; up to four atoms of the
+# sources' columns to an MMA and more (5 to 8), sources that end inside 32 columns, rows that are not a multiple of 16 bytes
+@pytest.mark.parametrize("dims, gemm_dtype", [
+    ((33, 448, 5), 0), ((200, 360, 3), 0), ((65, 96, 128, 47), 0), ((31, 64, 2), 0), ((32, 129, 33), 0), ((1, 65, 3, 7), 0), ((97, 257, 66), 0),
+    ((40, 512, 20), 1), ((300, 330, 45), 1), ((70, 90, 200), 1),
+])
+def test_weight_gradient_tiles(util, dims, gemm_dtype):
+    w = _workload(1_000, 3_000, dims, 17)
+    util.check_one_step(w, M=3, gemm_dtype=gemm_dtype, gradients_against_plain=gemm_dtype == 0)
