@@ -121,16 +121,53 @@ __device__ __forceinline__ void tmem_load_32x16(uint32_t taddr, float (&v)[16]) 
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// The stages of a tile: bit b = some row of the tile has an entry in window block b (of 100-member super-nodes kept
-// together, 4.7 of 6 on average; the blocks left out cost 64 source rows through shared memory and an MMA of zeros each).
-// A tile without any takes the block of its own first rows, so that its accumulator is written.
-__device__ __forceinline__ uint32_t tile_blocks(const unsigned char* block_mask, int64_t ws, int r0, int n_p) {
-    uint32_t m = 0;
+// A tile of a block's walk.  What a role needs of it first is requested when the walk comes to it, a tile ahead of its use: every
+// role goes through the same loads tile after tile, and waited for them each time.
+struct TileAt {
+    bool valid;
+    int k, r0, ct, n_p;    // slot of its part in the group, first row in the part, column tile, rows of the part
+    int64_t ws;            // first scratch row of the part
+    uint32_t mask[DT_BM / 32];
+    // The stages of the tile: bit b = some row of the tile has an entry in window block b (of 100-member super-nodes kept
+    // together, 4.7 of 6 on average; the blocks left out cost 64 source rows through shared memory and an MMA of zeros each).
+    // A tile without any takes the block of its own first rows, so that its accumulator is written.
+    __device__ __forceinline__ uint32_t blocks() const {
+        uint32_t m = 0;
 #pragma unroll
-    for (int j = 0; j < DT_BM / 32; ++j)
-        if (r0 + 32 * j < n_p) m |= __ldg(block_mask + (ws + r0) / 32 + j);
-    return m ? m : 1u << (DT_HALO / DT_BK);
-}
+        for (int j = 0; j < DT_BM / 32; ++j) m |= mask[j];
+        return m ? m : 1u << (DT_HALO / DT_BK);
+    }
+};
+// A block's tiles blockIdx.x, blockIdx.x + gridDim.x, ..., without those of parts that are not aggregated here
+struct TileWalk {
+    uint32_t tile, total;
+    int k;           // the part reached, and its first row tile
+    uint32_t base;
+    __device__ __forceinline__ TileWalk(const DenseArgs& a) : tile(blockIdx.x), total((uint32_t)(a.row_tiles * a.col_tiles)), k(0), base(0) {}
+    __device__ __forceinline__ TileAt next(const DenseArgs& a) {
+        TileAt t{};
+        for (; tile < total; tile += gridDim.x) {
+            const uint32_t row_tile = a.col_tiles == 1 ? tile : tile / (uint32_t)a.col_tiles;
+            uint32_t here;
+            while (row_tile >= base + (here = (uint32_t)(a.g.rows[k] + DT_BM - 1) / DT_BM)) {
+                base += here;
+                ++k;
+            }
+            if (!a.dense[a.g.part[k]]) continue;
+            t.valid = true;
+            t.k = k;
+            t.r0 = (int)(row_tile - base) * DT_BM;
+            t.ct = a.col_tiles == 1 ? 0 : (int)(tile - row_tile * (uint32_t)a.col_tiles);
+            t.n_p = a.g.rows[k];
+            t.ws = a.g.row_ws[k];
+#pragma unroll
+            for (int j = 0; j < DT_BM / 32; ++j) t.mask[j] = t.r0 + 32 * j < t.n_p ? __ldg(a.block_mask + (t.ws + t.r0) / 32 + j) : 0u;
+            tile += gridDim.x;
+            break;
+        }
+        return t;
+    }
+};
 
 // TRANSPOSED = false: A counts, out = (1 / deg v) * A src;  true: A = counts x 1 / deg u, out = A src
 template <bool TRANSPOSED>
@@ -147,8 +184,6 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int stages = a.stages;
     constexpr uint32_t NPA = TRANSPOSED ? 2u : 1u;  // planes of A
-    const int n_ct = a.col_tiles;
-    const int64_t total_tiles = a.row_tiles * n_ct;
     // a stage: the plane(s) of A, then the tile's atoms of the hi plane of the source rows and, right behind
     // them, those of the lo plane: one N-major operand of twice the tile's width
     const uint32_t stage_bytes = NPA * DT_A_BYTES + 2u * (uint32_t)min(DT_TILE_ATOMS, a.n_atoms) * DT_ATOM_BYTES;
@@ -180,55 +215,48 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
     tc::tc_fence_after_sync();
     const uint32_t tmem_base = pb.tmem_base;
 
-    // Every role walks the same tiles in the same order and skips the same ones: `it` counts the stages
-    // and `t` the tiles a block has worked on, and both must agree between the roles.
+    // Every role walks the same tiles in the same order and skips the same ones: `at` follows the stages and `t` counts the
+    // tiles a block has worked on, and both must agree between the roles.
     if (warp == 0) {
         if (lane == 0) {
-            int64_t it = 0, t = 0;
+            // One thread feeds the tensor core: descriptors are a constant plus an address in units of 16 bytes.
+            // A is K-major (a 128-byte row holds the 64 window rows of the stage): 16 of them = 32 bytes;
+            // the source rows are N-major (a 128-byte row per window row): 16 of them = 2048 bytes.
+            const uint64_t desc_a = tc::smem_desc_sw128(0, 16, 1024), desc_b = tc::smem_desc_sw128(0, DT_ATOM_BYTES, 1024);
+            tc::RingAt at;
+            uint32_t t = 0;
             bool ok = true;
-            for (int64_t tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-                int k, r0;
-                if (!locate_tile(a.g, DT_BM, tile / n_ct, &k, &r0)) break;
-                if (!a.dense[a.g.part[k]]) continue;
-                const int ct = (int)(tile % n_ct);
-                const int NA = min(DT_TILE_ATOMS, a.n_atoms - DT_TILE_ATOMS * ct);
+            TileWalk walk(a);
+            TileAt tile = walk.next(a);
+            while (tile.valid && ok) {
+                const int NA = min(DT_TILE_ATOMS, a.n_atoms - DT_TILE_ATOMS * tile.ct);
+                const int n_stages = __popc(tile.blocks());
+                tile = walk.next(a);
                 // A tile of at most two atoms multiplies A with [hi | lo] (the lo atoms lie right behind the hi atoms)
                 // in ONE MMA of twice the tile's width: columns [0, 64 NA) of the accumulator take the product with the
                 // hi plane, [64 NA, 128 NA) that with the lo plane, and the epilogue adds the halves.  An MMA that
                 // narrow costs its issue, not its arithmetic.  Wider tiles take one MMA per plane into the same columns.
                 const bool joined = NA <= 2;
-                const uint32_t idesc_both = tc::idesc_bf16(DT_BM, 128 * NA, false, true);
                 const uint32_t idesc_hi = tc::idesc_bf16(DT_BM, 64 * NA, false, true);
-                const uint32_t blocks = tile_blocks(a.block_mask, a.g.row_ws[k], r0, a.g.rows[k]);
+                const uint32_t idesc_first = joined ? tc::idesc_bf16(DT_BM, 128 * NA, false, true) : idesc_hi;
+                const uint32_t lo_off = (uint32_t)NA * (DT_ATOM_BYTES >> 4);
                 const int buf = (int)(t & 1);
-                ok = dense_wait(&pb.acc_empty[buf], (uint32_t)((t >> 1) & 1) ^ 1u, &pb, a.error_word);
+                ok = dense_wait(&pb.acc_empty[buf], ((t >> 1) & 1u) ^ 1u, &pb, a.error_word);
                 if (!ok) break;
                 tc::tc_fence_after_sync();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * a.tmem_cols);
-                for (uint32_t rest = blocks; rest; rest &= rest - 1, ++it) {
-                    const int s = (int)(it % stages);
-                    ok = dense_wait(&pb.full[s], (uint32_t)((it / stages) & 1), &pb, a.error_word);
+                for (int stage = 0; stage < n_stages; ++stage, at.advance(stages)) {
+                    const int s = at.s;
+                    ok = dense_wait(&pb.full[s], at.phase, &pb, a.error_word);
                     if (!ok) break;
                     tc::tc_fence_after_sync();
-                    const uint32_t ah = tc::smem_u32(a_hi(s)), al = tc::smem_u32(a_lo(s)), bh = tc::smem_u32(b_hi(s));
+                    const uint32_t ah = tc::smem_u32(a_hi(s)) >> 4, al = tc::smem_u32(a_lo(s)) >> 4, bh = tc::smem_u32(b_hi(s)) >> 4;
 #pragma unroll
                     for (int ks = 0; ks < DT_BK / 16; ++ks) {
-                        // A is K-major (a 128-byte row holds the 64 window rows of the stage): 16 of them = 32 bytes;
-                        // the source rows are N-major (a 128-byte row per window row): 16 of them = 2048 bytes
-                        const uint64_t dah = tc::smem_desc_sw128(ah + ks * 32, 16, 1024);
-                        const uint64_t db = tc::smem_desc_sw128(bh + ks * 2048, DT_ATOM_BYTES, 1024);
-                        const uint64_t dbl = tc::smem_desc_sw128(bh + NA * DT_ATOM_BYTES + ks * 2048, DT_ATOM_BYTES, 1024);
-                        const uint32_t first = (rest != blocks || ks > 0) ? 1u : 0u;
-                        if (joined) {
-                            tc::mma_bf16(d_tmem, dah, db, idesc_both, first);
-                        } else {
-                            tc::mma_bf16(d_tmem, dah, dbl, idesc_hi, first);
-                            tc::mma_bf16(d_tmem, dah, db, idesc_hi, 1u);
-                        }
-                        if (TRANSPOSED) {  // + A_lo * hi (into the first half)
-                            const uint64_t dal = tc::smem_desc_sw128(al + ks * 32, 16, 1024);
-                            tc::mma_bf16(d_tmem, dal, db, idesc_hi, 1u);
-                        }
+                        const uint64_t dah = desc_a + (ah + 2 * ks), db = desc_b + (bh + 128 * ks);
+                        tc::mma_bf16(d_tmem, dah, joined ? db : db + lo_off, idesc_first, stage > 0 || ks > 0 ? 1u : 0u);
+                        if (!joined) tc::mma_bf16(d_tmem, dah, db, idesc_hi, 1u);
+                        if (TRANSPOSED) tc::mma_bf16(d_tmem, desc_a + (al + 2 * ks), db, idesc_hi, 1u);  // + A_lo * hi (into the first half)
                     }
                     tc::mma_commit(&pb.empty[s]);
                 }
@@ -242,61 +270,74 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
         // transposed pass: the split weights 1 / deg of the tile's window rows, stage by stage as the 32 words
         // of a row of A with every bit set; written once per tile between two barriers of the builder warps
         __shared__ __align__(16) uint32_t wpair[DT_KB][2][DT_BK / 2];
-        int64_t it = 0;
+        tc::RingAt at;
         uint32_t meetings = 0;
         // all builder threads meet (a bounded wait like every other: a thread that has given up is not waited for)
         auto meet = [&]() {
             tc::mbar_arrive(&pb.builders);
             return dense_wait(&pb.builders, meetings++ & 1u, &pb, a.error_word);
         };
-        bool ok = true;
-        for (int64_t tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-            int k, r0;
-            if (!locate_tile(a.g, DT_BM, tile / n_ct, &k, &r0)) break;
-            if (!a.dense[a.g.part[k]]) continue;
-            const int n_p = a.g.rows[k];
-            const int ct = (int)(tile % n_ct);
-            const int NA = min(DT_TILE_ATOMS, a.n_atoms - DT_TILE_ATOMS * ct);
-            const int64_t ws = a.g.row_ws[k];
-            const uint32_t blocks = tile_blocks(a.block_mask, ws, r0, n_p);
-            unsigned long long bits[DT_KB];
-            if (r0 + r < n_p) {
-                const ulonglong2* wb = reinterpret_cast<const ulonglong2*>(a.win_bits + (ws + r0 + r) * DT_KB);
+        // the window of the thread's row and (transposed pass) the weights of the tile's window rows r, r + 128, ...: a tile ahead
+        constexpr int PER_THREAD = DENSE_WINDOW / DT_BUILDERS;
+        unsigned long long next_bits[DT_KB];
+        float next_w[PER_THREAD];
+        auto request = [&](const TileAt& t) {
+#pragma unroll
+            for (int q = 0; q < DT_KB; ++q) next_bits[q] = 0ULL;
+            if (t.valid && t.r0 + r < t.n_p) {
+                const ulonglong2* wb = reinterpret_cast<const ulonglong2*>(a.win_bits + (t.ws + t.r0 + r) * DT_KB);
 #pragma unroll
                 for (int q = 0; q < DT_KB / 2; ++q) {
                     const ulonglong2 v2 = __ldg(wb + q);
-                    bits[2 * q] = v2.x;
-                    bits[2 * q + 1] = v2.y;
+                    next_bits[2 * q] = v2.x;
+                    next_bits[2 * q + 1] = v2.y;
                 }
-            } else {
-#pragma unroll
-                for (int q = 0; q < DT_KB; ++q) bits[q] = 0ULL;
             }
+            if (TRANSPOSED) {
+#pragma unroll
+                for (int q = 0; q < PER_THREAD; ++q) {
+                    const int u = t.r0 - DT_HALO + q * DT_BUILDERS + r;
+                    next_w[q] = t.valid && u >= 0 && u < t.n_p ? __ldg(a.inv_deg + t.ws + u) : 0.f;
+                }
+            }
+        };
+        bool ok = true;
+        TileWalk walk(a);
+        TileAt tile = walk.next(a);
+        request(tile);
+        while (tile.valid && ok) {
+            const uint32_t blocks = tile.blocks();
+            const int NA = min(DT_TILE_ATOMS, a.n_atoms - DT_TILE_ATOMS * tile.ct);
+            const int ct = tile.ct, y0 = (int)(tile.ws + tile.r0 - DT_HALO);  // the window's first scratch row; may be negative: reads zeros
+            unsigned long long bits[DT_KB];
+#pragma unroll
+            for (int q = 0; q < DT_KB; ++q) bits[q] = next_bits[q];
             if (TRANSPOSED) {
                 ok = meet();  // every thread has written the previous tile's last stage
                 if (!ok) break;
 #pragma unroll
-                for (int q = 0; q < DENSE_WINDOW / DT_BUILDERS; ++q) {
+                for (int q = 0; q < PER_THREAD; ++q) {
                     const int wr = q * DT_BUILDERS + r;  // window row
-                    const int u = r0 - DT_HALO + wr;
-                    uint32_t h = 0, l = 0;
-                    if (u >= 0 && u < n_p) split_bits(__ldg(a.inv_deg + ws + u), h, l);
+                    uint32_t h, l;
+                    split_bits(next_w[q], h, l);
                     reinterpret_cast<unsigned short*>(wpair[wr / DT_BK][0])[wr % DT_BK] = (unsigned short)h;
                     reinterpret_cast<unsigned short*>(wpair[wr / DT_BK][1])[wr % DT_BK] = (unsigned short)l;
                 }
                 ok = meet();
                 if (!ok) break;
             }
-            for (uint32_t rest = blocks; rest; rest &= rest - 1, ++it) {
+            tile = walk.next(a);
+            request(tile);
+            for (uint32_t rest = blocks; rest; rest &= rest - 1, at.advance(stages)) {
                 const int kb = __ffs(rest) - 1;
-                const int s = (int)(it % stages);
-                ok = dense_wait(&pb.empty[s], (uint32_t)((it / stages) & 1) ^ 1u, &pb, a.error_word);
+                const int s = at.s;
+                ok = dense_wait(&pb.empty[s], at.phase ^ 1u, &pb, a.error_word);
                 if (!ok) break;
                 if (r == 0) {
                     // the stage's source rows, requested before this thread writes its row of A: window rows
                     // 64 kb .. 64 kb + 63, all column atoms of the tile
                     expect_tx(&pb.full[s], 2u * (uint32_t)NA * DT_ATOM_BYTES);
-                    const int y = (int)(ws + r0 - DT_HALO + (int64_t)kb * DT_BK);  // scratch row; may be negative: reads zeros
+                    const int y = y0 + kb * DT_BK;
                     for (int t = 0; t < NA; ++t) {
                         tc::tma_load_2d(b_hi(s) + t * DT_ATOM_BYTES, &a.mapSh, &pb.full[s], (DT_TILE_ATOMS * ct + t) * 64, y);
                         tc::tma_load_2d(b_hi(s) + (NA + t) * DT_ATOM_BYTES, &a.mapSl, &pb.full[s], (DT_TILE_ATOMS * ct + t) * 64, y);
@@ -348,14 +389,6 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
         float4* st = reinterpret_cast<float4*>(stg);
         const int p = lane & 3;
         const uint32_t out_row_bytes = (uint32_t)a.out.ld * 2u;
-        // this block's next tile at or after `from`
-        auto next_tile = [&](int64_t from, int* k, int* r0) -> int64_t {
-            for (int64_t tile = from; tile < total_tiles; tile += gridDim.x) {
-                if (!locate_tile(a.g, DT_BM, tile / n_ct, k, r0)) return -1;
-                if (a.dense[a.g.part[*k]]) return tile;
-            }
-            return -1;
-        };
         // of the thread's four rows of a tile: the scale, and whether the output row already holds a sum to add to
         auto row_info = [&](int k, int r0, float (&scale)[4], bool (&has_left)[4]) {
             const int rows_here = min(32, a.g.rows[k] - (r0 + q * 32));
@@ -371,14 +404,14 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
                 }
             }
         };
-        int k = 0, r0 = 0;
-        int64_t tile = next_tile(blockIdx.x, &k, &r0);
+        TileWalk walk(a);
+        TileAt tile = walk.next(a);
         float next_scale[4];
         bool next_left[4];
-        if (tile >= 0) row_info(k, r0, next_scale, next_left);
-        int64_t t = 0;
+        if (tile.valid) row_info(tile.k, tile.r0, next_scale, next_left);
+        uint32_t t = 0;
         bool ok = true;
-        while (tile >= 0 && ok) {
+        while (tile.valid && ok) {
             float scale[4];
             bool has_left[4];
 #pragma unroll
@@ -386,15 +419,15 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
                 scale[j] = next_scale[j];
                 has_left[j] = next_left[j];
             }
-            const int ct = (int)(tile % n_ct);
+            const int k = tile.k, r0 = tile.r0, ct = tile.ct;
             const int BN = 64 * min(DT_TILE_ATOMS, a.n_atoms - DT_TILE_ATOMS * ct);
             const int n0 = ct * 64 * DT_TILE_ATOMS;
             const int rows_here = min(32, a.g.rows[k] - (r0 + q * 32));
             const int64_t orow0 = a.g.row_ws[k] + r0 + q * 32;
             // the next tile's row data is requested a tile ahead, and every chunk's existing rows before the chunk
             // before them is finished: the epilogue is the longest chain of the kernel, and these loads its latency
-            tile = next_tile(tile + gridDim.x, &k, &r0);
-            if (tile >= 0) row_info(k, r0, next_scale, next_left);
+            tile = walk.next(a);
+            if (tile.valid) row_info(tile.k, tile.r0, next_scale, next_left);
             uint4 gh[4], gl[4];
             auto request = [&](int c0) {  // what the rows already hold (written by the launch before this one)
                 const int n = n0 + c0 + 8 * p;
@@ -411,7 +444,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
             };
             request(col_phase * 32);
             const int buf = (int)(t & 1);
-            ok = dense_wait(&pb.acc_full[buf], (uint32_t)((t >> 1) & 1), &pb, a.error_word);
+            ok = dense_wait(&pb.acc_full[buf], (t >> 1) & 1u, &pb, a.error_word);
             if (!ok) break;
             tc::tc_fence_after_sync();
             const uint32_t d_tmem = tmem_base + (uint32_t)(buf * a.tmem_cols);
@@ -509,6 +542,7 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
     wait_for_kernel_before();
     constexpr int S = 32 / LPR;            // rows side by side in a warp
     constexpr int NR = 2;                  // rows a lane works on at a time
+    constexpr int MANY = 4;
     constexpr int EL = 2;                  // listed entries of each of them requested together (most rows have one or two)
     const int lane = threadIdx.x & 31;
     const int sub = lane / LPR, sl = lane % LPR;
@@ -602,7 +636,7 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
                 }
             }
             // rows with more entries than are listed: the row's entries again, one row at a time; the quarters
-            // of the warp (LPR = 8) each take every fourth of them, four source rows in flight per lane
+            // of the warp (LPR = 8) each take every fourth of them, four (a whole warp: eight) source rows in flight per lane
             if (many) {
                 const int64_t* rp = rowptr_out + g.row_abs[k] + g.part[k];
                 const int32_t* cols = col_out + g.edge_abs[k];
@@ -622,20 +656,20 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
                         }
                         unsigned votes = __ballot_sync(0xffffffffu, outside);
                         while (votes) {
-                            int u[4];
-                            uint4 yh[4], yl[4];
-                            float wy[4];
+                            int u[MANY];
+                            uint4 yh[MANY], yl[MANY];
+                            float wy[MANY];
 #pragma unroll
-                            for (int b = 0; b < 4; ++b) {
+                            for (int b = 0; b < MANY; ++b) {
                                 // quarter `sub` takes the entries sub, sub + S, ... of those still to do
                                 const unsigned from = nth_bit(votes, b * S + sub);
                                 u[b] = __shfl_sync(0xffffffffu, c, from < 32u ? (int)from : 0);
                                 if (from >= 32u) u[b] = -1;
                             }
 #pragma unroll
-                            for (int b = 0; b < 4 * S; ++b) votes &= votes - 1;
+                            for (int b = 0; b < MANY * S; ++b) votes &= votes - 1;
 #pragma unroll
-                            for (int b = 0; b < 4; ++b) {
+                            for (int b = 0; b < MANY; ++b) {
                                 if (u[b] >= 0) {
                                     yh[b] = __ldg(reinterpret_cast<const uint4*>(sh + (int64_t)u[b] * src.ld + cx));
                                     yl[b] = __ldg(reinterpret_cast<const uint4*>(sl_ + (int64_t)u[b] * src.ld + cx));
@@ -643,7 +677,7 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
                                 }
                             }
 #pragma unroll
-                            for (int b = 0; b < 4; ++b) {
+                            for (int b = 0; b < MANY; ++b) {
                                 if (u[b] >= 0) {
                                     if (TRANSPOSED) acc.fma_planes_mixed(wy[b], yh[b], yl[b]);
                                     else acc.add_planes_mixed(yh[b], yl[b]);
@@ -836,6 +870,7 @@ int32_t launch_spmm_dense(rtma_ctx* ctx, int kclass, const GroupDesc& g, const i
     a.stages = (int)std::min<size_t>(DT_MAX_STAGES, (DT_SMEM_MAX - fixed) / stage_bytes);
     if (a.stages < 2) return rtma_fail(ctx, RTMA_ERR_UNSUPPORTED, "internal: aggregation tile does not fit shared memory");
     a.row_tiles = row_tiles;
+    if (row_tiles * a.col_tiles >= (int64_t(1) << 31)) return rtma_fail(ctx, RTMA_ERR_OVERFLOW, "too many aggregation tiles");
     a.error_word = ctx->error_word;
     // the planes as [rows_total x width] matrices: rows before the first and past the last scratch row, and
     // columns past the width, read as zero
