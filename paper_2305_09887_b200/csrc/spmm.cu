@@ -899,7 +899,7 @@ int64_t spmm_order_entries(const GroupDesc& g) { return group_tiles(g, SPMM_ROWS
 
 int32_t launch_spmm_order(rtma_ctx* ctx, const GroupDesc& g, const int64_t* rowptr_out, const int32_t* col_out,
                           int64_t entries, int* count, int* list, SpmmOrder* order, cudaStream_t s) {
-    *order = SpmmOrder{nullptr, nullptr, 0, nullptr, nullptr, 0, nullptr, nullptr, nullptr, nullptr, false};
+    *order = SpmmOrder{};
     const int64_t groups = group_tiles(g, SPMM_ROWS_PER_WARP);
     if (groups == 0) return RTMA_OK;
     if (groups >= (int64_t(1) << 30)) return rtma_fail(ctx, RTMA_ERR_OVERFLOW, "too many row groups");
@@ -911,6 +911,9 @@ int32_t launch_spmm_order(rtma_ctx* ctx, const GroupDesc& g, const int64_t* rowp
     unsigned long long* near_total = reinterpret_cast<unsigned long long*>(count + 2);
     { KernelScope ks(ctx, KC_INV_DEGREE, s); launch_kernel(locality_probe_kernel, grid, 256, 0, s, g, rowptr_out, col_out, group_tiles(g, 1), near_total); }
     RTMA_LAUNCH_CHECK(ctx);
-    *order = SpmmOrder{count, list, heavy, near_total, nullptr, 0, nullptr, nullptr, nullptr, nullptr, false};
+    order->heavy_count = count;
+    order->heavy_list = list;
+    order->heavy = heavy;
+    order->near_total = near_total;
     return RTMA_OK;
 }

@@ -49,6 +49,7 @@ constexpr int DT_MAX_STAGES = 6;
 constexpr int DT_TILE_ATOMS = 4;                 // 64-column atoms of a column tile
 constexpr int DT_LCAP = DENSE_LEFT_CAP;          // listed entries outside the window, per row
 constexpr unsigned char DT_OVERFLOW = 255;       // left_cnt of a row with more than that
+constexpr int DT_HUB = 64;                       // entries outside the window from which on a row is shared by a block
 constexpr int DT_SMEM_MAX = 225 * 1024;           // with the static part (under 2 KB) within the 227 KB a block may have
 static_assert(DT_BM == 128 && DENSE_WINDOW % DT_BK == 0 && DT_HALO % DT_BK == 0, "tile shape of the MMA and whole stages");
 
@@ -527,27 +528,122 @@ __device__ __forceinline__ unsigned nth_bit(unsigned m, int n) {
 
 // The entries outside the window of their row's tile, before the tiles run: for every row that has any,
 // out[row] = their sum (transposed pass: weighted by 1 / deg of the column), unscaled; the tile's epilogue adds
-// its product and the scale.  A warp takes 32 consecutive rows: their counts and listed columns with one load
+// its product and the scale.  Bound by the latency of chains of loads, so the rows are told apart, and rows that take long
+// begin first.  Blocks 0 .. hub_blocks - 1: a block per row of more than DT_HUB such entries, its warps taking every eighth piece of 32 of the row's
+// entries in the part's CSR, the sums added in a fixed order.  The next many_blocks: a warp per other row of more than
+// DT_LCAP.  The rest: a warp takes 32 consecutive rows with up to DT_LCAP, their counts and listed columns with one load
 // each; then the rows that have entries, several at a time, two source rows of each requested together (most
 // rows have one or two).  LPR lanes own a row (pieces of 8 values per lane): 32 for rows wider than 64 values,
-// two rows at a time per warp; 8 for narrower rows, eight at a time, two per quarter of the warp.  A row with more than DT_LCAP such entries is looked
-// up in the part's CSR again, 32 entries at a time, by the whole warp.
+// two rows at a time per warp; 8 for narrower rows, eight at a time, two per quarter of the warp.
+// In one kernel with the long rows looked up by the warp that met them: 610 us for 2 M rows of 256 values of which 27 % have such
+// entries (1.2 M entries; now 335), of 48 values 285 (now 180), 40,000 rows with hubs of 280 entries 105 (now 23).
 template <bool TRANSPOSED, int LPR>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(256, 3)
 spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict__ rowptr_out,
                     const int32_t* __restrict__ col_out, const float* __restrict__ inv_deg,
                     const int* __restrict__ dense, const unsigned char* __restrict__ left_cnt,
-                    const int32_t* __restrict__ left_col, const Planes src, const Planes out, const int width,
-                    const int64_t total_groups) {
+                    const int32_t* __restrict__ left_col, const int* __restrict__ long_count, const int32_t* __restrict__ long_rows,
+                    const int64_t long_room, const unsigned hub_blocks, const unsigned many_blocks, const Planes src, const Planes out,
+                    const int width, const int64_t total_groups) {
     wait_for_kernel_before();
     constexpr int S = 32 / LPR;            // rows side by side in a warp
     constexpr int NR = 2;                  // rows a lane works on at a time
-    constexpr int MANY = 4;
     constexpr int EL = 2;                  // listed entries of each of them requested together (most rows have one or two)
     const int lane = threadIdx.x & 31;
     const int sub = lane / LPR, sl = lane % LPR;
-    const int64_t warps = (int64_t)gridDim.x * 8;
-    for (int64_t grp = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); grp < total_groups; grp += warps) {
+    const int warp = threadIdx.x >> 5;
+    if (blockIdx.x < hub_blocks + many_blocks) {
+        // ---- rows whose entries are looked up again: hubs from the list's front, the others from its back ----
+        __shared__ __align__(16) float piece[8][LPR * 8];
+        const bool hub = blockIdx.x < hub_blocks;
+        const int n = long_count[hub ? 0 : 1];
+        const int first = hub ? (int)blockIdx.x : (int)(blockIdx.x - hub_blocks) * 8 + warp, step = hub ? (int)hub_blocks : (int)many_blocks * 8;
+        for (int item = first; item < n; item += step) {
+            const int64_t row = long_rows[hub ? (int64_t)item : long_room - 1 - item];
+            int k = 0;
+            while (k < g.num && !(row >= g.row_ws[k] && row < g.row_ws[k] + g.rows[k])) ++k;
+            if (k == g.num || !dense[g.part[k]]) continue;  // a part that has finished its steps, or was taken back
+            const int i = (int)(row - g.row_ws[k]), n_p = g.rows[k];
+            const int64_t ws = g.row_ws[k];
+            const int64_t* rp = rowptr_out + g.row_abs[k] + g.part[k];
+            const int32_t* cols = col_out + g.edge_abs[k];
+            const int w_begin = i / DT_BM * DT_BM - DT_HALO, w_end = w_begin + DENSE_WINDOW;
+            const int64_t e0 = rp[i], e1 = rp[i + 1];
+            for (int cb = 0; cb < width; cb += LPR * 8) {  // the same trip count for every lane: the shuffles below need the whole warp
+                const int c0 = cb + sl * 8;
+                const bool live = c0 < width;
+                const __nv_bfloat16* sh = src.hi + ws * src.ld + (live ? c0 : 0);  // lanes past the width read column 0 and store nothing
+                const __nv_bfloat16* sl_ = src.lo + ws * src.ld + (live ? c0 : 0);
+                Pack8 acc;
+                acc.zero();
+                for (int64_t eb = e0 + (hub ? warp * 32 : 0); eb < e1; eb += hub ? 8 * 32 : 32) {
+                    const int64_t e = eb + lane;
+                    bool outside = false;
+                    int c = 0;
+                    if (e < e1) {
+                        c = __ldg(cols + e);
+                        outside = rtma_index_ok(c, n_p, 5) && (c < w_begin || c >= w_end);
+                    }
+                    unsigned votes = __ballot_sync(0xffffffffu, outside);
+                    while (votes) {
+                        int u[4];
+                        uint4 yh[4], yl[4];
+                        float wy[4];
+#pragma unroll
+                        for (int b = 0; b < 4; ++b) {
+                            // quarter `sub` takes the entries sub, sub + S, ... of those still to do
+                            const unsigned from = nth_bit(votes, b * S + sub);
+                            u[b] = __shfl_sync(0xffffffffu, c, from < 32u ? (int)from : 0);
+                            if (from >= 32u) u[b] = -1;
+                        }
+#pragma unroll
+                        for (int b = 0; b < 4 * S; ++b) votes &= votes - 1;
+#pragma unroll
+                        for (int b = 0; b < 4; ++b) {
+                            if (u[b] >= 0) {
+                                yh[b] = __ldg(reinterpret_cast<const uint4*>(sh + (int64_t)u[b] * src.ld));
+                                yl[b] = __ldg(reinterpret_cast<const uint4*>(sl_ + (int64_t)u[b] * src.ld));
+                                if (TRANSPOSED) wy[b] = __ldg(inv_deg + ws + u[b]);
+                            }
+                        }
+#pragma unroll
+                        for (int b = 0; b < 4; ++b) {
+                            if (u[b] >= 0) {
+                                if (TRANSPOSED) acc.fma_planes_mixed(wy[b], yh[b], yl[b]);
+                                else acc.add_planes_mixed(yh[b], yl[b]);
+                            }
+                        }
+                    }
+                }
+                // the quarters' sums, added in a fixed order
+#pragma unroll
+                for (int step_ = S / 2; step_ > 0; step_ >>= 1)
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) acc.v[e] += __shfl_down_sync(0xffffffffu, acc.v[e], step_ * LPR);
+                if (hub) {  // and the warps'
+                    __syncthreads();
+                    if (sub == 0)
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) piece[warp][sl * 8 + e] = acc.v[e];
+                    __syncthreads();
+                    if (warp == 0 && sub == 0) {
+                        for (int w = 1; w < 8; ++w)
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) acc.v[e] += piece[w][sl * 8 + e];
+                    }
+                }
+                if (live && sub == 0 && (!hub || warp == 0)) {
+                    uint4 h, l;
+                    acc.to_planes_lean(h, l);
+                    *reinterpret_cast<uint4*>(out.hi + row * out.ld + c0) = h;
+                    *reinterpret_cast<uint4*>(out.lo + row * out.ld + c0) = l;
+                }
+            }
+        }
+        return;
+    }
+    const int64_t warps = (int64_t)(gridDim.x - hub_blocks - many_blocks) * 8;
+    for (int64_t grp = (int64_t)(blockIdx.x - hub_blocks - many_blocks) * 8 + warp; grp < total_groups; grp += warps) {
         int k, i0;
         if (!locate_tile(g, 32, grp, &k, &i0)) break;
         if (!dense[g.part[k]]) continue;
@@ -557,8 +653,7 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
         int4 my_cols = make_int4(0, 0, 0, 0);
         if (my_cnt > 0 && my_cnt <= DT_LCAP) my_cols = *reinterpret_cast<const int4*>(left_col + (ws + i0 + lane) * DT_LCAP);
         const unsigned listed = __ballot_sync(0xffffffffu, my_cnt > 0 && my_cnt <= DT_LCAP);
-        const unsigned many = __ballot_sync(0xffffffffu, my_cnt == DT_OVERFLOW);
-        if (!(listed | many)) continue;
+        if (!listed) continue;
         const __nv_bfloat16* sh = src.hi + ws * src.ld;
         const __nv_bfloat16* sl_ = src.lo + ws * src.ld;
         for (int cb = 0; cb < width; cb += LPR * 8) {  // the same trip count for every lane: the shuffles below need the whole warp
@@ -635,82 +730,20 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
                     }
                 }
             }
-            // rows with more entries than are listed: the row's entries again, one row at a time; the quarters
-            // of the warp (LPR = 8) each take every fourth of them, four (a whole warp: eight) source rows in flight per lane
-            if (many) {
-                const int64_t* rp = rowptr_out + g.row_abs[k] + g.part[k];
-                const int32_t* cols = col_out + g.edge_abs[k];
-                const int w_begin = i0 / DT_BM * DT_BM - DT_HALO, w_end = w_begin + DENSE_WINDOW;  // 32 divides the tile
-                for (unsigned rest = many; rest; rest &= rest - 1) {
-                    const int i = i0 + __ffs(rest) - 1;
-                    const int64_t e0 = rp[i], e1 = rp[i + 1];
-                    Pack8 acc;
-                    acc.zero();
-                    for (int64_t eb = e0; eb < e1; eb += 32) {
-                        const int64_t e = eb + lane;
-                        bool outside = false;
-                        int c = 0;
-                        if (e < e1) {
-                            c = __ldg(cols + e);
-                            outside = rtma_index_ok(c, n_p, 5) && (c < w_begin || c >= w_end);
-                        }
-                        unsigned votes = __ballot_sync(0xffffffffu, outside);
-                        while (votes) {
-                            int u[MANY];
-                            uint4 yh[MANY], yl[MANY];
-                            float wy[MANY];
-#pragma unroll
-                            for (int b = 0; b < MANY; ++b) {
-                                // quarter `sub` takes the entries sub, sub + S, ... of those still to do
-                                const unsigned from = nth_bit(votes, b * S + sub);
-                                u[b] = __shfl_sync(0xffffffffu, c, from < 32u ? (int)from : 0);
-                                if (from >= 32u) u[b] = -1;
-                            }
-#pragma unroll
-                            for (int b = 0; b < MANY * S; ++b) votes &= votes - 1;
-#pragma unroll
-                            for (int b = 0; b < MANY; ++b) {
-                                if (u[b] >= 0) {
-                                    yh[b] = __ldg(reinterpret_cast<const uint4*>(sh + (int64_t)u[b] * src.ld + cx));
-                                    yl[b] = __ldg(reinterpret_cast<const uint4*>(sl_ + (int64_t)u[b] * src.ld + cx));
-                                    if (TRANSPOSED) wy[b] = __ldg(inv_deg + ws + u[b]);
-                                }
-                            }
-#pragma unroll
-                            for (int b = 0; b < MANY; ++b) {
-                                if (u[b] >= 0) {
-                                    if (TRANSPOSED) acc.fma_planes_mixed(wy[b], yh[b], yl[b]);
-                                    else acc.add_planes_mixed(yh[b], yl[b]);
-                                }
-                            }
-                        }
-                    }
-                    // the quarters' sums, added in a fixed order
-#pragma unroll
-                    for (int step = S / 2; step > 0; step >>= 1)
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) acc.v[e] += __shfl_down_sync(0xffffffffu, acc.v[e], step * LPR);
-                    if (live && sub == 0) {
-                        uint4 h, l;
-                        acc.to_planes_lean(h, l);
-                        *reinterpret_cast<uint4*>(out.hi + (ws + i) * out.ld + c0) = h;
-                        *reinterpret_cast<uint4*>(out.lo + (ws + i) * out.ld + c0) = l;
-                    }
-                }
-            }
         }
     }
 }
 
 // Once per call, for every row of a part that takes the tiles: its window as DT_KB 64-bit masks, and the
 // entries outside the window in row order: up to DT_LCAP columns and their number, or DT_OVERFLOW when there
-// are more.  A row that repeats an entry inside its window takes its part back to the gather kernels
+// are more; such rows are listed too, hubs from the front of long_rows (long_count[0] of them), others from its back ([1]).  A row that repeats an entry inside its window takes its part back to the gather kernels
 // (dense[trainer] = 0): a bit cannot count.
 __global__ void __launch_bounds__(256)
 dense_lists_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict__ rowptr_out,
                    const int32_t* __restrict__ col_out, int* __restrict__ dense,
                    unsigned long long* __restrict__ win_bits, unsigned char* __restrict__ block_mask,
-                   unsigned char* __restrict__ left_cnt, int32_t* __restrict__ left_col) {
+                   unsigned char* __restrict__ left_cnt, int32_t* __restrict__ left_col, int* __restrict__ long_count,
+                   int32_t* __restrict__ long_rows, const int64_t long_room) {
     wait_for_kernel_before();
     int k, r0;
     if (!locate_tile(g, 256, blockIdx.x, &k, &r0)) return;
@@ -755,6 +788,8 @@ dense_lists_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restric
 #pragma unroll
     for (int q = 0; q < DT_KB; ++q) win_bits[row * DT_KB + q] = bits[q];
     left_cnt[row] = cnt <= DT_LCAP ? (unsigned char)cnt : DT_OVERFLOW;
+    if (cnt > DT_HUB) long_rows[atomicAdd(long_count, 1)] = (int32_t)row;  // the order does not matter
+    else if (cnt > DT_LCAP) long_rows[long_room - 1 - atomicAdd(long_count + 1, 1)] = (int32_t)row;
     if (repeated) dense[g.part[k]] = 0;
 }
 
@@ -826,10 +861,10 @@ int32_t launch_dense_probe(rtma_ctx* ctx, const GroupDesc& g, const int64_t* row
 
 int32_t launch_dense_lists(rtma_ctx* ctx, const GroupDesc& g, const int64_t* rowptr_out, const int32_t* col_out,
                            int* dense, unsigned long long* win_bits, unsigned char* block_mask, unsigned char* left_cnt,
-                           int32_t* left_col, cudaStream_t s) {
+                           int32_t* left_col, int* long_count, int32_t* long_rows, int64_t long_room, cudaStream_t s) {
     const int64_t tiles = group_tiles(g, 256);
     if (tiles == 0) return RTMA_OK;
-    { KernelScope ks(ctx, KC_INV_DEGREE, s); launch_kernel(dense_lists_kernel, (unsigned)tiles, 256, 0, s, g, rowptr_out, col_out, dense, win_bits, block_mask, left_cnt, left_col); }
+    { KernelScope ks(ctx, KC_INV_DEGREE, s); launch_kernel(dense_lists_kernel, (unsigned)tiles, 256, 0, s, g, rowptr_out, col_out, dense, win_bits, block_mask, left_cnt, left_col, long_count, long_rows, long_room); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }
@@ -877,13 +912,15 @@ int32_t launch_spmm_dense(rtma_ctx* ctx, int kclass, const GroupDesc& g, const i
     if (!make_tensor_map_bf16(&a.mapSh, src.hi, (uint64_t)rows_total, (uint64_t)a.width, (uint64_t)src.ld, 64, DT_BK) ||
         !make_tensor_map_bf16(&a.mapSl, src.lo, (uint64_t)rows_total, (uint64_t)a.width, (uint64_t)src.ld, 64, DT_BK))
         return rtma_fail(ctx, RTMA_ERR_CUDA, "cuTensorMapEncodeTiled refused the aggregation operands");
+    // how many rows of each kind there are only the device knows: a block per SM for the hubs, two for the other long rows
     const int64_t groups = group_tiles(g, 32);
-    const unsigned lgrid = (unsigned)std::min<int64_t>(ceil_div(groups, 8), (int64_t)ctx->sm_count * 8);
+    const unsigned hub_blocks = (unsigned)ctx->sm_count, many_blocks = 2u * (unsigned)ctx->sm_count;
+    const unsigned lgrid = hub_blocks + many_blocks + (unsigned)std::min<int64_t>(ceil_div(groups, 8), (int64_t)ctx->sm_count * 12);
     {
         KernelScope ks(ctx, kclass, s);
 #define RTMA_OUTSIDE(T, L)                                                                                              \
     launch_kernel(spmm_outside_kernel<T, L>, lgrid, 256, 0, s, g, rowptr_out, col_out, inv_deg, dense, order.left_cnt, order.left_col, \
-                                                    src, out, a.width, groups)
+                  order.long_count, order.long_rows, rows_total, hub_blocks, many_blocks, src, out, a.width, groups)
         if (a.width <= 64) {
             if (transposed) RTMA_OUTSIDE(true, 8);
             else RTMA_OUTSIDE(false, 8);

@@ -115,7 +115,7 @@ int64_t aligned_rows(int64_t n_p) { return ceil_div(n_p, GROUP_ROW_ALIGN) * GROU
 ScratchPlan plan_scratch(const Model& m, bool head, bool record) {
     ScratchPlan sp{};
     size_t per_row = sizeof(float);              // inv_deg
-    per_row += DENSE_WINDOW / 8 + sizeof(int32_t) * DENSE_LEFT_CAP + 1;  // tensor-core aggregation: window masks, entries outside
+    per_row += DENSE_WINDOW / 8 + sizeof(int32_t) * (DENSE_LEFT_CAP + 1) + 1;  // tensor-core aggregation: window masks, entries outside
     per_row += 4 * planes_ld(m.dims[0]);         // X as planes
     int q_width = 0;
     for (int l = 0; l < m.L; ++l) {
@@ -197,7 +197,7 @@ int plan_splits(const GroupDesc& g, int parts_in_flight, const WgradCost& cost, 
 size_t part_scratch_bytes(const Model& m, const ScratchPlan& sp, int64_t n_p, int64_t pairs) {
     const size_t rows = (size_t)aligned_rows(n_p);
     const size_t prows = (size_t)aligned_rows(pairs);
-    const size_t matrices = 8 * m.L + 8 * m.Kd + 24;  // every matrix start is rounded up to 256 bytes
+    const size_t matrices = 8 * m.L + 8 * m.Kd + 25;  // every matrix start is rounded up to 256 bytes
     const size_t decoder = sp.per_pair_bytes * prows + sizeof(float) * (64 * sp.max_decoder_params + (size_t)ceil_div(pairs, 32) + 256) +
                            sizeof(float) * ((size_t)ceil_div(pairs, 64) + 1) * (2 * sp.post_width + 1);
     return sp.per_row_bytes * rows + sizeof(float) * (64 * sp.max_layer_params + (size_t)ceil_div(n_p, 32) + 256) +
@@ -463,6 +463,8 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
             unsigned long long* win_bits = cur.take<unsigned long long>((size_t)rows * (DENSE_WINDOW / 64) + 2);
             int32_t* left_col = cur.take<int32_t>((size_t)rows * DENSE_LEFT_CAP + 4);
             unsigned char* left_cnt = cur.take<unsigned char>((size_t)rows + 16);
+            int32_t* long_rows = cur.take<int32_t>((size_t)rows);
+            int* long_count = ticket + 32;
             unsigned char* block_mask = cur.take<unsigned char>((size_t)rows / 32 + 1);
             float* post_partial = m.post ? cur.take<float>((size_t)post_tiles(g) * (2 * plan.post_width + 1) + 4) : nullptr;
             if (link && m.Kd > 1) dec_post_partial = cur.take<float>((size_t)post_tiles(gd) * (2 * plan.post_width + 1) + 4);
@@ -545,7 +547,7 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                 };
                 RTMA_TRY(read_flags());
                 if (any_dense) {  // the per-row masks and lists; a part with repeated entries is taken back: read again
-                    RTMA_TRY(launch_dense_lists(ctx, g, rowptr_out, col_out, dense_flags, win_bits, block_mask, left_cnt, left_col, s));
+                    RTMA_TRY(launch_dense_lists(ctx, g, rowptr_out, col_out, dense_flags, win_bits, block_mask, left_cnt, left_col, long_count, long_rows, rows, s));
                     RTMA_TRY(read_flags());
                 }
                 wave_order.all_dense = any_dense && all_dense;
@@ -554,6 +556,8 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                     wave_order.rows_total = rows;
                     wave_order.left_cnt = left_cnt;
                     wave_order.left_col = left_col;
+                    wave_order.long_count = long_count;
+                    wave_order.long_rows = long_rows;
                     wave_order.win_bits = win_bits;
                     wave_order.block_mask = block_mask;
                 }
@@ -575,7 +579,11 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                 bool all_run = true;
                 for (int k = 0; k < wave.num; ++k) all_run = all_run && steps[wave.part[k]] > step;
                 // the order was built for the whole wave; which parts go to the tensor cores is a matter of each part
-                const SpmmOrder order = all_run ? wave_order : SpmmOrder{nullptr, nullptr, 0, nullptr, wave_order.dense, wave_order.rows_total, wave_order.left_cnt, wave_order.left_col, wave_order.win_bits, wave_order.block_mask, wave_order.all_dense};
+                SpmmOrder order = wave_order;
+                if (!all_run) {
+                    order.heavy_count = nullptr;
+                    order.near_total = nullptr;
+                }
                 SplitPlan spl[RTMA_MAX_LAYERS];
                 if (all_run) {
                     g = wave;
