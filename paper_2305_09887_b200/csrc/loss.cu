@@ -255,8 +255,9 @@ softmax_xent_head_kernel(const __grid_constant__ GroupDesc g, const Planes Tself
 
 // The head form with 9 to 64 classes: LPR lanes own a row, eight columns each, so that the loads and stores of a warp cover
 // whole pieces of rows; the maximum and the sum go over the row's lanes.  With a thread per row every load touched 32
-// lines and every store half a sector: 52 us for 200,000 rows of 47 classes (115 MB), 41 us this way; bound by the
-// instructions of 47 exponentials a row.
+// lines and every store half a sector: 52 us for 200,000 rows of 47 classes (115 MB).  Bound by the instructions (issue slots 82 %
+// used at 41.5 us; 38 with the tile found by the warp, planes joined by mixed-precision adds and columns past the classes as
+// minus infinity instead of a test each time).  Several rows a thread, to wait for memory less often, took 52.
 template <int LPR>
 __global__ void __launch_bounds__(LOSS_TILE_ROWS * LPR)
 softmax_xent_head_lanes_kernel(const __grid_constant__ GroupDesc g, const Planes Tself, const Planes NT,
@@ -266,36 +267,43 @@ softmax_xent_head_lanes_kernel(const __grid_constant__ GroupDesc g, const Planes
     constexpr int WARPS = LOSS_TILE_ROWS * LPR / 32;
     __shared__ float warp_loss[WARPS];
     int k, r0;
-    if (!locate_tile(g, LOSS_TILE_ROWS, blockIdx.x, &k, &r0)) return;
+    if (!locate_tile_by_warp(g, LOSS_TILE_ROWS, blockIdx.x, &k, &r0)) return;
     const int n_p = g.rows[k];
     const int i = r0 + threadIdx.x / LPR, c0 = (threadIdx.x % LPR) * 8;
     const bool row_ok = i < n_p, live = row_ok && c0 < NT.ld;
     const int64_t r = g.row_ws[k] + i;
-    const float* bias = params + (int64_t)g.part[k] * P + bias_offset;
-    const int label = row_ok ? checked_label(yp[g.row_abs[k] + i], C) : 0;
+    const float* bias = params + (int64_t)g.part[k] * P + bias_offset + c0;
+    const int label = (row_ok ? checked_label(yp[g.row_abs[k] + i], C) : 0) - c0;  // as one of the lane's columns
+    const int columns = C - c0;                                                    // of the lane that exist: at most 8 count
     Pack8 x;
     x.zero();
     if (live) {
-        x.add_planes(*reinterpret_cast<const uint4*>(NT.hi + r * NT.ld + c0), *reinterpret_cast<const uint4*>(NT.lo + r * NT.ld + c0));
-        if (Tself.hi)
-            x.add_planes(*reinterpret_cast<const uint4*>(Tself.hi + r * Tself.ld + c0), *reinterpret_cast<const uint4*>(Tself.lo + r * Tself.ld + c0));
+        x.set_planes_mixed(*reinterpret_cast<const uint4*>(NT.hi + r * NT.ld + c0), *reinterpret_cast<const uint4*>(NT.lo + r * NT.ld + c0));
+        if (Tself.hi) {
+            Pack8 own;
+            own.set_planes_mixed(*reinterpret_cast<const uint4*>(Tself.hi + r * Tself.ld + c0), *reinterpret_cast<const uint4*>(Tself.lo + r * Tself.ld + c0));
+#pragma unroll
+            for (int e = 0; e < 8; ++e) x.v[e] += own.v[e];
+        }
     }
     float zmax = -INFINITY;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        if (c0 + e < C) {
-            x.v[e] += __ldg(bias + c0 + e);
-            zmax = fmaxf(zmax, x.v[e]);
-            if (scores.ptr && row_ok) scores.ptr[r * scores.ld + c0 + e] = x.v[e];
-        }
+    for (int e = 0; e < 8; ++e) {  // columns past the classes: no share in the maximum or the sum
+        x.v[e] = e < columns ? x.v[e] + __ldg(bias + e) : -INFINITY;
+        zmax = fmaxf(zmax, x.v[e]);
+    }
+    if (scores.ptr && row_ok) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            if (e < columns) scores.ptr[r * scores.ld + c0 + e] = x.v[e];
     }
 #pragma unroll
     for (int o = LPR / 2; o > 0; o >>= 1) zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
     float sum = 0.f, zl = 0.f;
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-        if (c0 + e == label) zl = x.v[e];
-        x.v[e] = c0 + e < C ? expf(x.v[e] - zmax) : 0.f;
+        if (e == label) zl = x.v[e];
+        x.v[e] = expf(x.v[e] - zmax);
         sum += x.v[e];
     }
 #pragma unroll
@@ -308,7 +316,7 @@ softmax_xent_head_lanes_kernel(const __grid_constant__ GroupDesc g, const Planes
         const float hot = 1.0f / (float)n_p;
 #pragma unroll
         for (int e = 0; e < 8; ++e)  // padding columns stay zero
-            x.v[e] = c0 + e < C ? x.v[e] * scale - (c0 + e == label ? hot : 0.f) : 0.f;
+            x.v[e] = e < columns ? x.v[e] * scale - (e == label ? hot : 0.f) : 0.f;
         uint4 h, l;
         x.to_planes_cvt(h, l);
         *reinterpret_cast<uint4*>(dZ.hi + r * dZ.ld + c0) = h;

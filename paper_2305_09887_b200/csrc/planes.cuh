@@ -104,6 +104,15 @@ struct Pack8 {
             v[2 * i + 1] = add_f32_bf16(add_f32_bf16(v[2 * i + 1], (unsigned short)(hw[i] >> 16)), (unsigned short)(lw[i] >> 16));
         }
     }
+    // v = hi + lo (exact)
+    __device__ __forceinline__ void set_planes_mixed(const uint4 h, const uint4 l) {
+        const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, lw[4] = {l.x, l.y, l.z, l.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            v[2 * i] = add_f32_bf16(__uint_as_float(lw[i] << 16), (unsigned short)(hw[i] & 0xFFFFu));
+            v[2 * i + 1] = add_f32_bf16(__uint_as_float(lw[i] & 0xFFFF0000u), (unsigned short)(hw[i] >> 16));
+        }
+    }
     // v += w * (hi + lo), hi + lo formed exactly by two mixed-precision adds
     __device__ __forceinline__ void fma_planes_mixed(const float w, const uint4 h, const uint4 l) {
         const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, lw[4] = {l.x, l.y, l.z, l.w};
