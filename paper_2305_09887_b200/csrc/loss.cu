@@ -18,7 +18,6 @@ namespace {
 __device__ __forceinline__ int checked_label(int label, int C) { return rtma_index_ok(label, C, 6) ? label : 0; }
 
 constexpr int LOSS_THREADS = 256;
-constexpr int LOSS_TILE_ROWS = 64;
 constexpr int LOSS_ROWS_PER_WARP = LOSS_TILE_ROWS / (LOSS_THREADS / 32);
 constexpr int LOSS_REG_CLASSES = 128;
 
@@ -382,21 +381,7 @@ __global__ void __launch_bounds__(256)
 loss_finalize_kernel(const __grid_constant__ GroupDesc g, const float* __restrict__ tile_loss,
                      float* __restrict__ loss_out, const int64_t loss_stride, const int64_t loss_col) {
     wait_for_kernel_before();
-    __shared__ float red[256];
-    const int k = blockIdx.x;
-    int64_t first = 0;
-    for (int q = 0; q < k; ++q) first += (g.rows[q] + LOSS_TILE_ROWS - 1) / LOSS_TILE_ROWS;
-    const int64_t count = (g.rows[k] + LOSS_TILE_ROWS - 1) / LOSS_TILE_ROWS;
-    float s = 0.f;
-    for (int64_t t = threadIdx.x; t < count; t += 256) s += tile_loss[first + t];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0)
-        loss_out[(int64_t)g.part[k] * loss_stride + loss_col] = g.rows[k] > 0 ? red[0] / (float)g.rows[k] : 0.f;
+    finalize_loss(g, blockIdx.x, tile_loss, loss_out, loss_stride, loss_col);
 }
 
 }  // namespace
@@ -420,8 +405,7 @@ int32_t launch_softmax_xent(rtma_ctx* ctx, const GroupDesc& g, Mat logits, int C
 }
 
 int32_t launch_softmax_xent_head(rtma_ctx* ctx, const GroupDesc& g, Planes Tself, Planes NT, const float* params, int64_t P,
-                                 int64_t bias_offset, int C, const int32_t* yp, Planes dZ, Mat scores, float* tile_loss,
-                                 float* loss_out, int64_t loss_stride, int64_t loss_col, cudaStream_t s) {
+                                 int64_t bias_offset, int C, const int32_t* yp, Planes dZ, Mat scores, float* tile_loss, cudaStream_t s) {
     if (C > 64) return rtma_fail(ctx, RTMA_ERR_UNSUPPORTED, "internal: head kernel with %d classes", C);
     const int64_t tiles = group_tiles(g, LOSS_TILE_ROWS);
     if (tiles > 0) {
@@ -435,7 +419,7 @@ int32_t launch_softmax_xent_head(rtma_ctx* ctx, const GroupDesc& g, Planes Tself
 #undef RTMA_HEAD
         RTMA_LAUNCH_CHECK(ctx);
     }
-    return launch_loss_finalize(ctx, g, tile_loss, loss_out, loss_stride, loss_col, s);
+    return RTMA_OK;
 }
 
 int32_t launch_loss_finalize(rtma_ctx* ctx, const GroupDesc& g, const float* tile_loss, float* loss_out,

@@ -32,9 +32,14 @@ reduce_sgd_kernel(const __grid_constant__ GroupDesc g, const __grid_constant__ S
 __global__ void __launch_bounds__(256)
 reduce_sgd_head_kernel(const __grid_constant__ GroupDesc g, const __grid_constant__ SplitPlan sp, const LayerShape ls,
                        const int cp, const float* __restrict__ partial, const float lr, float* __restrict__ params,
-                       float* __restrict__ grads_record) {
+                       float* __restrict__ grads_record, const float* __restrict__ tile_loss, float* __restrict__ loss_out,
+                       const int64_t loss_stride, const int64_t loss_col) {
     wait_for_kernel_before();
     const int k = blockIdx.y;
+    if (loss_out && blockIdx.x == gridDim.x - 1) {  // the last block of a part: its loss
+        finalize_loss(g, k, tile_loss, loss_out, loss_stride, loss_col);
+        return;
+    }
     const int64_t count = (int64_t)(ls.nsrc * ls.d_in + 1) * ls.d_out;  // the layer's parameters: weight matrices, bias
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= count) return;
@@ -158,11 +163,15 @@ int32_t launch_reduce_sgd(rtma_ctx* ctx, const GroupDesc& g, const SplitPlan& sp
 }
 
 int32_t launch_reduce_sgd_head(rtma_ctx* ctx, const GroupDesc& g, const SplitPlan& sp, LayerShape ls, int head_cp,
-                               const float* partial, float lr, float* params, float* grads_record, cudaStream_t s) {
+                               const float* partial, float lr, float* params, float* grads_record, const float* tile_loss,
+                               float* loss_out, int64_t loss_stride, int64_t loss_col, cudaStream_t s) {
     if (g.num == 0) return RTMA_OK;
     const int64_t count = (int64_t)(ls.nsrc * ls.d_in + 1) * ls.d_out;
-    dim3 grid((unsigned)ceil_div(count, 256), (unsigned)g.num);
-    { KernelScope ks(ctx, KC_REDUCE_SGD, s); launch_kernel(reduce_sgd_head_kernel, grid, 256, 0, s, g, sp, ls, head_cp, partial, lr, params, grads_record); }
+    dim3 grid((unsigned)ceil_div(count, 256) + (loss_out ? 1 : 0), (unsigned)g.num);
+    {
+        KernelScope ks(ctx, KC_REDUCE_SGD, s);
+        launch_kernel(reduce_sgd_head_kernel, grid, 256, 0, s, g, sp, ls, head_cp, partial, lr, params, grads_record, tile_loss, loss_out, loss_stride, loss_col);
+    }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }

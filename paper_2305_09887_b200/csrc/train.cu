@@ -661,7 +661,7 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                     const LayerShape& ll = m.layer[m.L - 1];
                     RTMA_TRY(launch_softmax_xent_head(ctx, g, m.gcn ? no_planes : Planes{T.hi, T.lo, T.ld}, NT, params, ll.P,
                                                       ll.param_offset + (int64_t)ll.nsrc * ll.d_in * ll.d_out, C, yp, dZlast,
-                                                      (tap && record) ? logits : no_mat, tile_loss, loss_out, loss_stride, step, s));
+                                                      (tap && record) ? logits : no_mat, tile_loss, s));
                     // Abar^T dZ into the second half of DQ: the weight gradient needs it even in a one-layer model
                     if (m.gcn) RTMA_TRY(launch_spmm_gcn(ctx, g, rowptr_out, col_out, inv_deg, dZlast, Qlast, C, true, order, ticket, s));
                     else RTMA_TRY(launch_spmm_transposed(ctx, g, rowptr_out, col_out, inv_deg, dZlast, Qlast, C, order, ticket, s));
@@ -736,7 +736,8 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                                 RTMA_TRY(launch_post_backward(ctx, g, m.layer[l - 1], params, Zl[l - 1], Hl[l], stats[l - 1], post_partial,
                                                               m.lr, tap ? taps->grads : nullptr, s));
                         }
-                        RTMA_TRY(launch_reduce_sgd_head(ctx, g, spl[l], m.layer[l], Cp, partial, m.lr, params, tap ? taps->grads : nullptr, s));
+                        RTMA_TRY(launch_reduce_sgd_head(ctx, g, spl[l], m.layer[l], Cp, partial, m.lr, params, tap ? taps->grads : nullptr, tile_loss,
+                                                        loss_out, loss_stride, step, s));
                         continue;
                     }
                     RTMA_TRY(launch_tc_wgrad(ctx, g, spl[l], m.layer[l], rows, Hl[l], Nl[l], dZ, partial, single_pass, s));

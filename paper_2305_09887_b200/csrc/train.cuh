@@ -68,6 +68,28 @@ __device__ __forceinline__ bool locate_tile_by_warp(const GroupDesc& g, int tile
 }
 #endif
 
+#ifdef __CUDACC__
+// loss_out[part of slot k * loss_stride + loss_col] = (sum of the part's tile sums) / rows of the part; the whole block of 256 threads
+constexpr int LOSS_TILE_ROWS = 64;
+__device__ __forceinline__ void finalize_loss(const GroupDesc& g, int k, const float* __restrict__ tile_loss, float* __restrict__ loss_out,
+                                              int64_t loss_stride, int64_t loss_col) {
+    __shared__ float red[256];
+    int64_t first = 0;
+    for (int q = 0; q < k; ++q) first += (g.rows[q] + LOSS_TILE_ROWS - 1) / LOSS_TILE_ROWS;
+    const int64_t count = (g.rows[k] + LOSS_TILE_ROWS - 1) / LOSS_TILE_ROWS;
+    float s = 0.f;
+    for (int64_t t = threadIdx.x; t < count; t += 256) s += tile_loss[first + t];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0)
+        loss_out[(int64_t)g.part[k] * loss_stride + loss_col] = g.rows[k] > 0 ? red[0] / (float)g.rows[k] : 0.f;
+}
+#endif
+
 // An fp32 scratch matrix addressed by the group's scratch rows.
 struct Mat {
     float* ptr;
@@ -198,10 +220,9 @@ int32_t launch_softmax_xent(rtma_ctx* ctx, const GroupDesc& g, Mat logits, int C
 
 // The head when the last layer's aggregate is taken after the product: scores = [Tself +] NT + b
 // (Tself.hi == NULL: one-matrix layer), at most 64 classes; dZ as above; scores.ptr != NULL records the
-// scores as fp32.
+// scores as fp32.  Leaves the tiles' loss sums: launch_reduce_sgd_head turns them into the parts' losses.
 int32_t launch_softmax_xent_head(rtma_ctx* ctx, const GroupDesc& g, Planes Tself, Planes NT, const float* params, int64_t P,
-                                 int64_t bias_offset, int C, const int32_t* yp, Planes dZ, Mat scores, float* tile_loss,
-                                 float* loss_out, int64_t loss_stride, int64_t loss_col, cudaStream_t s);
+                                 int64_t bias_offset, int C, const int32_t* yp, Planes dZ, Mat scores, float* tile_loss, cudaStream_t s);
 
 // ---- post.cu (Layer Normalization before the activation, PReLU) ------------------------------
 int64_t post_tiles(const GroupDesc& g);
@@ -236,9 +257,11 @@ int32_t launch_reduce_sgd(rtma_ctx* ctx, const GroupDesc& g, const SplitPlan& sp
                           float lr, float* params, float* grads_record, cudaStream_t s);
 // The same for the head form of the last layer: partial[slot] is [(d_in + 1) x 2 head_cp], the product of
 // [H | 1]^T with [dZ | Q]; columns c of the first block give dWs (and db in the last row), columns
-// head_cp + c give dWn (for a one-matrix layer dW, and the first block only gives db).
+// head_cp + c give dWn (for a one-matrix layer dW, and the first block only gives db).  And the parts' losses from the sums that
+// the loss kernel left (as launch_loss_finalize; a launch of its own was 3 us of 90 us of a small step).
 int32_t launch_reduce_sgd_head(rtma_ctx* ctx, const GroupDesc& g, const SplitPlan& sp, LayerShape ls, int head_cp,
-                               const float* partial, float lr, float* params, float* grads_record, cudaStream_t s);
+                               const float* partial, float lr, float* params, float* grads_record, const float* tile_loss,
+                               float* loss_out, int64_t loss_stride, int64_t loss_col, cudaStream_t s);
 int32_t launch_copy_rows(rtma_ctx* ctx, const float* src, int64_t ld_src, float* dst, int64_t ld_dst, int64_t rows,
                          int width, cudaStream_t s);
 
