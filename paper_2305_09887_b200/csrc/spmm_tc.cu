@@ -49,7 +49,8 @@ constexpr int DT_MAX_STAGES = 6;
 constexpr int DT_TILE_ATOMS = 4;                 // 64-column atoms of a column tile
 constexpr int DT_LCAP = DENSE_LEFT_CAP;          // listed entries outside the window, per row
 constexpr unsigned char DT_OVERFLOW = 255;       // left_cnt of a row with more than that
-constexpr int DT_HUB = 64;                       // entries outside the window from which on a row is shared by a block
+constexpr unsigned char DT_HUB_MARK = 254;       // and of one with more than DT_HUB
+constexpr int DT_HUB = 64;                       // entries outside the window up to which a row is not shared by a block
 constexpr int DT_SMEM_MAX = 225 * 1024;           // with the static part (under 2 KB) within the 227 KB a block may have
 static_assert(DT_BM == 128 && DENSE_WINDOW % DT_BK == 0 && DT_HALO % DT_BK == 0, "tile shape of the MMA and whole stages");
 
@@ -529,9 +530,10 @@ __device__ __forceinline__ unsigned nth_bit(unsigned m, int n) {
 // The entries outside the window of their row's tile, before the tiles run: for every row that has any,
 // out[row] = their sum (transposed pass: weighted by 1 / deg of the column), unscaled; the tile's epilogue adds
 // its product and the scale.  Bound by the latency of chains of loads, so the rows are told apart, and rows that take long
-// begin first.  Blocks 0 .. hub_blocks - 1: a block per row of more than DT_HUB such entries, its warps taking every eighth piece of 32 of the row's
-// entries in the part's CSR, the sums added in a fixed order.  The next many_blocks: a warp per other row of more than
-// DT_LCAP.  The rest: a warp takes 32 consecutive rows with up to DT_LCAP, their counts and listed columns with one load
+// begin first.  Blocks 0 .. hub_blocks - 1 take the rows of more than DT_HUB such entries, a block each: its warps take every eighth piece of 32
+// of the row's entries in the part's CSR, and the sums are added in a fixed order.  The next many_blocks take the other rows of more than
+// DT_LCAP, a warp each.  (Where the scratch has no word to spare per row, both take groups of 32 rows: 23 us for single rows, 45 for
+// groups in the last example below, 80 with the marks searched for instead of listed.)  The rest: a warp takes 32 consecutive rows with up to DT_LCAP, their counts and listed columns with one load
 // each; then the rows that have entries, several at a time, two source rows of each requested together (most
 // rows have one or two).  LPR lanes own a row (pieces of 8 values per lane): 32 for rows wider than 64 values,
 // two rows at a time per warp; 8 for narrower rows, eight at a time, two per quarter of the warp.
@@ -543,7 +545,7 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
                     const int32_t* __restrict__ col_out, const float* __restrict__ inv_deg,
                     const int* __restrict__ dense, const unsigned char* __restrict__ left_cnt,
                     const int32_t* __restrict__ left_col, const int* __restrict__ long_count, const int32_t* __restrict__ long_rows,
-                    const int64_t long_room, const unsigned hub_blocks, const unsigned many_blocks, const Planes src, const Planes out,
+                    const int64_t long_room, const int long_unit, const unsigned hub_blocks, const unsigned many_blocks, const Planes src, const Planes out,
                     const int width, const int64_t total_groups) {
     wait_for_kernel_before();
     constexpr int S = 32 / LPR;            // rows side by side in a warp
@@ -553,16 +555,14 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
     const int sub = lane / LPR, sl = lane % LPR;
     const int warp = threadIdx.x >> 5;
     if (blockIdx.x < hub_blocks + many_blocks) {
-        // ---- rows whose entries are looked up again: hubs from the list's front, the others from its back ----
+        // ---- rows whose entries are looked up again ----
         __shared__ __align__(16) float piece[8][LPR * 8];
         const bool hub = blockIdx.x < hub_blocks;
-        const int n = long_count[hub ? 0 : 1];
-        const int first = hub ? (int)blockIdx.x : (int)(blockIdx.x - hub_blocks) * 8 + warp, step = hub ? (int)hub_blocks : (int)many_blocks * 8;
-        for (int item = first; item < n; item += step) {
-            const int64_t row = long_rows[hub ? (int64_t)item : long_room - 1 - item];
+        // the sum of one row by this warp (a hub: of this warp's share, the block's first warp then adds the shares and stores)
+        auto do_row = [&](const int row) {
             int k = 0;
             while (k < g.num && !(row >= g.row_ws[k] && row < g.row_ws[k] + g.rows[k])) ++k;
-            if (k == g.num || !dense[g.part[k]]) continue;  // a part that has finished its steps, or was taken back
+            if (k == g.num || !dense[g.part[k]]) return;  // past a part's end, of a part that has finished its steps or was taken back
             const int i = (int)(row - g.row_ws[k]), n_p = g.rows[k];
             const int64_t ws = g.row_ws[k];
             const int64_t* rp = rowptr_out + g.row_abs[k] + g.part[k];
@@ -635,10 +635,19 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
                 if (live && sub == 0 && (!hub || warp == 0)) {
                     uint4 h, l;
                     acc.to_planes_lean(h, l);
-                    *reinterpret_cast<uint4*>(out.hi + row * out.ld + c0) = h;
-                    *reinterpret_cast<uint4*>(out.lo + row * out.ld + c0) = l;
+                    *reinterpret_cast<uint4*>(out.hi + (int64_t)row * out.ld + c0) = h;
+                    *reinterpret_cast<uint4*>(out.lo + (int64_t)row * out.ld + c0) = l;
                 }
             }
+        };
+        // single scratch rows or groups of 32 (all of one part), from the list's front (with a hub: a block each) or back (a warp each)
+        const int n = long_count[hub ? 0 : 1], step = hub ? (int)hub_blocks : (int)many_blocks * 8;
+#pragma unroll 1
+        for (int item = hub ? (int)blockIdx.x : (int)(blockIdx.x - hub_blocks) * 8 + warp; item < n; item += step) {
+            const int first = long_unit * long_rows[hub ? (int64_t)item : long_room - 1 - item];
+#pragma unroll 1
+            for (unsigned rest = long_unit == 1 ? 1u : __ballot_sync(0xffffffffu, left_cnt[first + lane] >= DT_HUB_MARK); rest; rest &= rest - 1)
+                do_row(first + __ffs(rest) - 1);
         }
         return;
     }
@@ -735,15 +744,15 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
 }
 
 // Once per call, for every row of a part that takes the tiles: its window as DT_KB 64-bit masks, and the
-// entries outside the window in row order: up to DT_LCAP columns and their number, or DT_OVERFLOW when there
-// are more; such rows are listed too, hubs from the front of long_rows (long_count[0] of them), others from its back ([1]).  A row that repeats an entry inside its window takes its part back to the gather kernels
+// entries outside the window in row order: up to DT_LCAP columns and their number, or DT_OVERFLOW or DT_HUB_MARK when there
+// are more; and such rows (long_unit 32: the groups of 32 with such rows) in long_rows, hubs from its front (long_count[0] of them), others from its back ([1]).  A row that repeats an entry inside its window takes its part back to the gather kernels
 // (dense[trainer] = 0): a bit cannot count.
 __global__ void __launch_bounds__(256)
 dense_lists_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict__ rowptr_out,
                    const int32_t* __restrict__ col_out, int* __restrict__ dense,
                    unsigned long long* __restrict__ win_bits, unsigned char* __restrict__ block_mask,
-                   unsigned char* __restrict__ left_cnt, int32_t* __restrict__ left_col, int* __restrict__ long_count,
-                   int32_t* __restrict__ long_rows, const int64_t long_room) {
+                   unsigned char* __restrict__ left_cnt, int32_t* __restrict__ left_col, int* __restrict__ long_count, int32_t* __restrict__ long_rows,
+                   const int64_t long_room, const int long_unit) {
     wait_for_kernel_before();
     int k, r0;
     if (!locate_tile(g, 256, blockIdx.x, &k, &r0)) return;
@@ -783,13 +792,18 @@ dense_lists_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restric
 #pragma unroll
     for (int q = 0; q < DT_KB; ++q) blocks |= bits[q] ? 1u << q : 0u;
     blocks = __reduce_or_sync(0xffffffffu, blocks);
+    const int most = __reduce_max_sync(0xffffffffu, cnt);
     if (!live) return;
-    if ((threadIdx.x & 31) == 0) block_mask[row / 32] = (unsigned char)blocks;  // parts start at multiples of 64 scratch rows
+    if ((threadIdx.x & 31) == 0) {  // parts start at multiples of 64 scratch rows
+        block_mask[row / 32] = (unsigned char)blocks;
+    }
+    // the order in the lists does not matter
+    const int longest = long_unit == 1 ? cnt : (threadIdx.x & 31) == 0 ? most : 0;
+    if (longest > DT_HUB) long_rows[atomicAdd(long_count, 1)] = (int32_t)(row / long_unit);
+    else if (longest > DT_LCAP) long_rows[long_room - 1 - atomicAdd(long_count + 1, 1)] = (int32_t)(row / long_unit);
 #pragma unroll
     for (int q = 0; q < DT_KB; ++q) win_bits[row * DT_KB + q] = bits[q];
-    left_cnt[row] = cnt <= DT_LCAP ? (unsigned char)cnt : DT_OVERFLOW;
-    if (cnt > DT_HUB) long_rows[atomicAdd(long_count, 1)] = (int32_t)row;  // the order does not matter
-    else if (cnt > DT_LCAP) long_rows[long_room - 1 - atomicAdd(long_count + 1, 1)] = (int32_t)row;
+    left_cnt[row] = cnt <= DT_LCAP ? (unsigned char)cnt : cnt <= DT_HUB ? DT_OVERFLOW : DT_HUB_MARK;
     if (repeated) dense[g.part[k]] = 0;
 }
 
@@ -861,10 +875,10 @@ int32_t launch_dense_probe(rtma_ctx* ctx, const GroupDesc& g, const int64_t* row
 
 int32_t launch_dense_lists(rtma_ctx* ctx, const GroupDesc& g, const int64_t* rowptr_out, const int32_t* col_out,
                            int* dense, unsigned long long* win_bits, unsigned char* block_mask, unsigned char* left_cnt,
-                           int32_t* left_col, int* long_count, int32_t* long_rows, int64_t long_room, cudaStream_t s) {
+                           int32_t* left_col, int* long_count, int32_t* long_rows, int64_t long_room, int long_unit, cudaStream_t s) {
     const int64_t tiles = group_tiles(g, 256);
     if (tiles == 0) return RTMA_OK;
-    { KernelScope ks(ctx, KC_INV_DEGREE, s); launch_kernel(dense_lists_kernel, (unsigned)tiles, 256, 0, s, g, rowptr_out, col_out, dense, win_bits, block_mask, left_cnt, left_col, long_count, long_rows, long_room); }
+    { KernelScope ks(ctx, KC_INV_DEGREE, s); launch_kernel(dense_lists_kernel, (unsigned)tiles, 256, 0, s, g, rowptr_out, col_out, dense, win_bits, block_mask, left_cnt, left_col, long_count, long_rows, long_room, long_unit); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }
@@ -920,7 +934,7 @@ int32_t launch_spmm_dense(rtma_ctx* ctx, int kclass, const GroupDesc& g, const i
         KernelScope ks(ctx, kclass, s);
 #define RTMA_OUTSIDE(T, L)                                                                                              \
     launch_kernel(spmm_outside_kernel<T, L>, lgrid, 256, 0, s, g, rowptr_out, col_out, inv_deg, dense, order.left_cnt, order.left_col, \
-                  order.long_count, order.long_rows, rows_total, hub_blocks, many_blocks, src, out, a.width, groups)
+                  order.long_count, order.long_rows, rows_total / order.long_unit, order.long_unit, hub_blocks, many_blocks, src, out, a.width, groups)
         if (a.width <= 64) {
             if (transposed) RTMA_OUTSIDE(true, 8);
             else RTMA_OUTSIDE(false, 8);

@@ -104,6 +104,7 @@ struct ScratchPlan {
     size_t per_row_bytes;     // planes, logits, 1/deg
     size_t max_layer_params;  // largest (2 d_in + 1) d_out
     size_t max_decoder_params;  // the same of the decoder's layers (link prediction)
+    size_t max_layer_partial, max_decoder_partial;  // the same with d_out rounded up, as a chunk's partial sums are stored
     size_t prep_bytes;        // repacked weights, per part
     int q_width;              // widest Abar^T dZ (widths of the layers above the first)
     size_t post_width;        // widest normalised / PReLU layer output (0: none)
@@ -115,7 +116,7 @@ int64_t aligned_rows(int64_t n_p) { return ceil_div(n_p, GROUP_ROW_ALIGN) * GROU
 ScratchPlan plan_scratch(const Model& m, bool head, bool record) {
     ScratchPlan sp{};
     size_t per_row = sizeof(float);              // inv_deg
-    per_row += DENSE_WINDOW / 8 + sizeof(int32_t) * (DENSE_LEFT_CAP + 1) + 1;  // tensor-core aggregation: window masks, entries outside
+    per_row += DENSE_WINDOW / 8 + sizeof(int32_t) * DENSE_LEFT_CAP + 1;  // tensor-core aggregation: window masks, entries outside
     per_row += 4 * planes_ld(m.dims[0]);         // X as planes
     int q_width = 0;
     for (int l = 0; l < m.L; ++l) {
@@ -123,8 +124,12 @@ ScratchPlan plan_scratch(const Model& m, bool head, bool record) {
         if (l < m.L - 1) per_row += 4 * planes_ld(m.dims[l + 1]);  // H^{l+1}, later overwritten by dZ^l
         if (l < m.L - 1 && m.post) per_row += 4 * planes_ld(m.dims[l + 1]) + sizeof(float2);  // Z^{l}, (mean, 1/std)
         if (l >= 1 && !(head && l == m.L - 1)) q_width = std::max(q_width, m.dims[l + 1]);
-        sp.max_layer_params = std::max(sp.max_layer_params, (size_t)(m.layer[l].nsrc * m.dims[l] + 1) * padded_ld(m.dims[l + 1]));
-        if (head && l == m.L - 1) sp.max_layer_params = std::max(sp.max_layer_params, (size_t)(m.dims[l] + 1) * 2 * m.Cp);
+        sp.max_layer_params = std::max(sp.max_layer_params, (size_t)(m.layer[l].nsrc * m.dims[l] + 1) * m.dims[l + 1]);
+        sp.max_layer_partial = std::max(sp.max_layer_partial, (size_t)(m.layer[l].nsrc * m.dims[l] + 1) * padded_ld(m.dims[l + 1]));
+        if (head && l == m.L - 1) {
+            sp.max_layer_params = std::max(sp.max_layer_params, (size_t)(m.dims[l] + 1) * 2 * m.Cp);
+            sp.max_layer_partial = std::max(sp.max_layer_partial, (size_t)(m.dims[l] + 1) * 2 * m.Cp);
+        }
         if (l < m.L - 1 && m.post) sp.post_width = std::max(sp.post_width, (size_t)m.dims[l + 1]);
         const TcLayerPlan lp = (head && l == m.L - 1) ? tc_plan_head(m.layer[l], m.Cp) : tc_plan_layer(m.layer[l]);
         sp.prep_bytes += sizeof(__nv_bfloat16) * tc_prep_elems(lp, l >= 1) + 4 * 256;
@@ -140,7 +145,8 @@ ScratchPlan plan_scratch(const Model& m, bool head, bool record) {
     sp.per_pair_bytes = 0;
     for (int k = 0; k < m.Kd; ++k) {
         sp.per_pair_bytes += 4 * planes_ld(m.ddims[k]) + 4 * planes_ld(m.ddims[k + 1]);
-        sp.max_decoder_params = std::max(sp.max_decoder_params, (size_t)(m.ddims[k] + 1) * padded_ld(m.ddims[k + 1]));
+        sp.max_decoder_params = std::max(sp.max_decoder_params, (size_t)(m.ddims[k] + 1) * m.ddims[k + 1]);
+        sp.max_decoder_partial = std::max(sp.max_decoder_partial, (size_t)(m.ddims[k] + 1) * padded_ld(m.ddims[k + 1]));
         sp.prep_bytes += sizeof(__nv_bfloat16) * tc_prep_elems(tc_plan_layer(m.dec[k]), true) + 4 * 256;
         if (k < m.Kd - 1) sp.post_width = std::max(sp.post_width, (size_t)m.ddims[k + 1]);
     }
@@ -154,7 +160,7 @@ ScratchPlan plan_scratch(const Model& m, bool head, bool record) {
 // moved by 1.3e-5 in five steps.  More than that where it is faster: a block (one per SM at a time) takes a fixed 4 us and then
 // stages its rows at about 41 bytes per ns, and every chunk adds a set of partial sums that is written and read back
 // (about 4,000 bytes per ns).  Small parts gain: 3 parts of 10,000 rows ran 30 blocks, 37 us a launch, now 120 of 256 rows.
-int splits_for(int64_t n_p, int parts_in_flight, const WgradCost& c) {
+int splits_for(int64_t n_p, int parts_in_flight, const WgradCost& c, int64_t cap) {
     constexpr int64_t SMS = 148;
     if (n_p <= 0) return 1;
     auto waves_of = [&](int64_t ns, int64_t* rows, int64_t* slots) {
@@ -169,12 +175,12 @@ int splits_for(int64_t n_p, int parts_in_flight, const WgradCost& c) {
             if (cost(ns) <= best * 1.03) return ns;
         return to;
     };
-    const int64_t fewest = least_within(1, std::min<int64_t>(64, std::max<int64_t>(1, ceil_div(n_p, 1024))), [&](int64_t ns) {
+    const int64_t fewest = least_within(1, std::min<int64_t>(cap, std::max<int64_t>(1, ceil_div(n_p, 1024))), [&](int64_t ns) {
         int64_t rows, slots;
         const int64_t waves = waves_of(ns, &rows, &slots);
         return (double)waves * (double)rows;
     });
-    const int64_t most = std::max(fewest, std::min<int64_t>(64, ceil_div(n_p, 128)));
+    const int64_t most = std::max(fewest, std::min<int64_t>(cap, ceil_div(n_p, 128)));
     return (int)least_within(fewest, most, [&](int64_t ns) {
         int64_t rows, slots;
         const int64_t waves = waves_of(ns, &rows, &slots);
@@ -182,11 +188,18 @@ int splits_for(int64_t n_p, int parts_in_flight, const WgradCost& c) {
     });
 }
 
-int plan_splits(const GroupDesc& g, int parts_in_flight, const WgradCost& cost, SplitPlan* sp) {
+// The chunks of a part that its share of the scratch has room for: it holds 64 sets of `params` values, a set takes `partial`, and
+// `others` words of other lists lie there too.
+int64_t most_splits(size_t params, size_t partial, size_t others) {
+    const size_t room = 64 * params > others ? 64 * params - others : 0;
+    return std::max<int64_t>(1, (int64_t)(room / std::max<size_t>(partial, 1)));
+}
+
+int plan_splits(const GroupDesc& g, int parts_in_flight, const WgradCost& cost, int64_t cap, SplitPlan* sp) {
     int slots = 0;
     for (int k = 0; k < g.num; ++k) {
         sp->split_begin[k] = slots;
-        const int nsplit = splits_for(g.rows[k], parts_in_flight, cost);
+        const int nsplit = splits_for(g.rows[k], parts_in_flight, cost, cap);
         sp->rows_per_split[k] = (int32_t)std::max<int64_t>(GROUP_ROW_ALIGN, aligned_rows(ceil_div(g.rows[k], nsplit)));
         slots += (int)std::max<int64_t>(1, ceil_div(g.rows[k], sp->rows_per_split[k]));
     }
@@ -197,7 +210,7 @@ int plan_splits(const GroupDesc& g, int parts_in_flight, const WgradCost& cost, 
 size_t part_scratch_bytes(const Model& m, const ScratchPlan& sp, int64_t n_p, int64_t pairs) {
     const size_t rows = (size_t)aligned_rows(n_p);
     const size_t prows = (size_t)aligned_rows(pairs);
-    const size_t matrices = 8 * m.L + 8 * m.Kd + 25;  // every matrix start is rounded up to 256 bytes
+    const size_t matrices = 8 * m.L + 8 * m.Kd + 24;  // every matrix start is rounded up to 256 bytes
     const size_t decoder = sp.per_pair_bytes * prows + sizeof(float) * (64 * sp.max_decoder_params + (size_t)ceil_div(pairs, 32) + 256) +
                            sizeof(float) * ((size_t)ceil_div(pairs, 64) + 1) * (2 * sp.post_width + 1);
     return sp.per_row_bytes * rows + sizeof(float) * (64 * sp.max_layer_params + (size_t)ceil_div(n_p, 32) + 256) +
@@ -366,13 +379,20 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
             // one chunking per layer: the number of blocks per chunk depends on the layer's shape
             SplitPlan wave_spl[RTMA_MAX_LAYERS];
             int slots = 0;
+            // The list of rows with many entries outside their tile's window takes a word per row where that costs the largest part at
+            // most a quarter of its chunks, else one per 32 rows (half of which the loss tiles leave of theirs).
+            size_t most_rows = 0;
+            for (int k = 0; k < g.num; ++k) most_rows = std::max(most_rows, (size_t)aligned_rows(g.rows[k]));
+            const int long_unit = 64 * plan.max_layer_params >= 48 * plan.max_layer_partial + most_rows + 64 ? 1 : 32;
+            const size_t long_lists = (long_unit == 1 ? most_rows : most_rows / 64) + 64;
             for (int l = 0; l < m.L; ++l) {
                 LayerShape shape = m.layer[l];
                 if (head && l == m.L - 1) {  // the head form's weight gradient: H^T [dZ | Q]
                     shape.nsrc = 1;
                     shape.d_out = 2 * m.Cp;
                 }
-                slots = std::max(slots, plan_splits(g, running, tc_wgrad_cost(shape, single_pass), &wave_spl[l]));
+                slots = std::max(slots, plan_splits(g, running, tc_wgrad_cost(shape, single_pass),
+                                                    most_splits(plan.max_layer_params, plan.max_layer_partial, long_lists), &wave_spl[l]));
             }
             int wave_steps = 0;
             for (int k = 0; k < g.num; ++k) wave_steps = std::max(wave_steps, steps[g.part[k]]);
@@ -443,14 +463,14 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                     const WgradCost c = tc_wgrad_cost(m.dec[k], single_pass);
                     if (c.blocks_per_slot * c.bytes_per_row > widest.blocks_per_slot * widest.bytes_per_row) widest = c;
                 }
-                const int dslots = plan_splits(gd, running, widest, &spd);
-                dec_partial = cur.take<float>((size_t)dslots * plan.max_decoder_params + 4);
+                const int dslots = plan_splits(gd, running, widest, most_splits(plan.max_decoder_params, plan.max_decoder_partial, 0), &spd);
+                dec_partial = cur.take<float>((size_t)dslots * plan.max_decoder_partial + 4);
                 dec_tile_loss = cur.take<float>((size_t)loss_tiles(gd) + 4);
             }
             // Abar^T dZ of the layer in hand; carved at the widest layer, addressed at each layer's own width
             __nv_bfloat16* q_hi = plan.q_width ? cur.take<__nv_bfloat16>((size_t)rows * planes_ld(plan.q_width) + 8) : nullptr;
             __nv_bfloat16* q_lo = plan.q_width ? cur.take<__nv_bfloat16>((size_t)rows * planes_ld(plan.q_width) + 8) : nullptr;
-            float* partial = cur.take<float>((size_t)slots * plan.max_layer_params + 4);
+            float* partial = cur.take<float>((size_t)slots * plan.max_layer_partial + 4);
             float* tile_loss = cur.take<float>((size_t)loss_tiles(g) + 4);
             const size_t counters_at = cur.used;  // from here to counters_end: zero on entry
             int* ticket = cur.take<int>(64);  // work counter of the aggregation kernels (zero between launches)
@@ -463,7 +483,7 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
             unsigned long long* win_bits = cur.take<unsigned long long>((size_t)rows * (DENSE_WINDOW / 64) + 2);
             int32_t* left_col = cur.take<int32_t>((size_t)rows * DENSE_LEFT_CAP + 4);
             unsigned char* left_cnt = cur.take<unsigned char>((size_t)rows + 16);
-            int32_t* long_rows = cur.take<int32_t>((size_t)rows);
+            int32_t* long_rows = cur.take<int32_t>((size_t)(rows / long_unit) + 1);
             int* long_count = ticket + 32;
             unsigned char* block_mask = cur.take<unsigned char>((size_t)rows / 32 + 1);
             float* post_partial = m.post ? cur.take<float>((size_t)post_tiles(g) * (2 * plan.post_width + 1) + 4) : nullptr;
@@ -547,7 +567,7 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                 };
                 RTMA_TRY(read_flags());
                 if (any_dense) {  // the per-row masks and lists; a part with repeated entries is taken back: read again
-                    RTMA_TRY(launch_dense_lists(ctx, g, rowptr_out, col_out, dense_flags, win_bits, block_mask, left_cnt, left_col, long_count, long_rows, rows, s));
+                    RTMA_TRY(launch_dense_lists(ctx, g, rowptr_out, col_out, dense_flags, win_bits, block_mask, left_cnt, left_col, long_count, long_rows, rows / long_unit, long_unit, s));
                     RTMA_TRY(read_flags());
                 }
                 wave_order.all_dense = any_dense && all_dense;
@@ -558,6 +578,7 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                     wave_order.left_col = left_col;
                     wave_order.long_count = long_count;
                     wave_order.long_rows = long_rows;
+                    wave_order.long_unit = long_unit;
                     wave_order.win_bits = win_bits;
                     wave_order.block_mask = block_mask;
                 }

@@ -223,10 +223,11 @@ def test_parts_choose_for_themselves(util):
     assert np.array_equal(auto, never)
 
 
-@pytest.mark.parametrize("n, degree", [(1_340, 3), (1_340, 8), (1_400, 11), (1_300, 60)])
-def test_entries_outside_the_windows(util, forced, tiny_workload, n, degree):
+@pytest.mark.parametrize("n, degree, dims", [(1_340, 3, (24, 72, 19)), (1_340, 8, (24, 72, 19)), (1_400, 11, (24, 300, 19)), (1_300, 60, (24, 72, 19)),
+                                             (24_000, 7, (16, 16, 5))])
+def test_entries_outside_the_windows(util, forced, tiny_workload, n, degree, dims):
     # two parts of about 670 rows, 5 tiles and a bit: rows without entries outside their window, with listed ones, with more than
-    # are listed, and two hubs with hundreds
+    # are listed, and two hubs with hundreds.  The last: parts so large beside their weights that long rows are listed by groups of 32
     g = inputs.uniform_graph(n, n * degree // 2, 31)
     rows, cols = np.repeat(np.arange(n), np.diff(g.rowptr)), g.col.astype(np.int64)
     rng = np.random.default_rng(32)
@@ -238,8 +239,8 @@ def test_entries_outside_the_windows(util, forced, tiny_workload, n, degree):
     np.cumsum(np.bincount(key // n, minlength=n), out=rowptr[1:])
     w = inputs.Workload(**{**tiny_workload.__dict__})
     w.graph = inputs.Graph(n=n, rowptr=rowptr, col=(key % n).astype(np.int32))
-    w.M, w.dims = 2, (24, 72, 19)                                    # two atoms; one, of the head's narrow planes
-    w.X, w.y = inputs.normal_features(n, 24, 33), inputs.uniform_labels(n, 19, 34)
+    w.M, w.dims = 2, dims
+    w.X, w.y = inputs.normal_features(n, dims[0], 33), inputs.uniform_labels(n, dims[-1], 34)
     w.params0 = inputs.xavier_params(w.dims, 35)
     got, want = util.check_one_step(w)
     util.check_k_steps_and_average(w, got, want, 2)
