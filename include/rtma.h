@@ -371,6 +371,13 @@ const char* rtma_kernel_class_name(int32_t cls);
  * The paper has no counterpart.                                                             */
 int32_t rtma_selftest_wait_timeout(rtma_ctx* ctx, void* stream);
 
+/* Self-test of the planning of the weight gradients, on the host alone: into how many chunks of
+ * rows the gradient of every layer is cut for a part of n_p rows, one of `parts` that run at the
+ * same time (chunks [md->L]); with a decoder (dd not NULL) chunks[md->L] is that of its layers for
+ * n_p pairs.  The paper has no counterpart.                                                  */
+int32_t rtma_selftest_chunks(const rtma_model_desc* md, const rtma_decoder_desc* dd, int64_t n_p,
+                             int32_t parts, int32_t* chunks);
+
 /* ---- the whole path on HOST buffers (Sec. 3: partition, Algorithm 2, Algorithm 1) --------
  * Every pointer here is a HOST pointer (pageable or pinned).  Copies the graph (CSR as for
  * rtma_build_induced_csr), group_id_h (NULL = RandomTMA), features X_h [n][dims[0]], labels

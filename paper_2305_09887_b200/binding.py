@@ -25,7 +25,7 @@ EXPORTS = (
     "rtma_kernel_class_name", "rtma_check", "rtma_partition_static", "rtma_partition_static_error",
     "rtma_local_steps_var", "rtma_aggregate_masked", "rtma_selftest_wait_timeout", "rtma_link_param_count",
     "rtma_link_steps", "rtma_set_workspace_limit", "rtma_local_steps_gathered", "rtma_bounds_checked", "rtma_sample_hop",
-    "rtma_set_dense_aggregation",
+    "rtma_set_dense_aggregation", "rtma_selftest_chunks",
 )
 KERNEL_CLASSES = 21
 
@@ -102,6 +102,18 @@ def link_param_count(dims, ddims, variant=(0, 0, 0)) -> int:
 
 def param_count(dims, variant=(0, 0, 0)) -> int:
     return int(load_library().rtma_param_count(ctypes.byref(model_desc(dims, variant=variant))))
+
+
+def selftest_chunks(dims, n_p: int, parts: int = 1, ddims=None, gemm_dtype: int = 0, variant=(0, 0, 0)):
+    """Into how many chunks of rows every layer's weight gradient is cut for a part of n_p rows, one of `parts` that run at
+    the same time; with ddims the last number is the decoder's, for n_p pairs."""
+    chunks = (ctypes.c_int32 * (MAX_LAYERS + 1))()
+    dd = ctypes.byref(decoder_desc(ddims)) if ddims else None
+    st = load_library().rtma_selftest_chunks(ctypes.byref(model_desc(dims, 0.0, gemm_dtype, variant)), dd, ctypes.c_int64(n_p),
+                                             ctypes.c_int32(parts), chunks)
+    if st != 0:
+        raise RtmaError(f"rtma_selftest_chunks failed ({st})")
+    return list(chunks)[:len(dims) - 1 + (1 if ddims else 0)]
 
 
 def _ptr(t):

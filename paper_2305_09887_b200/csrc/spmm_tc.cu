@@ -532,8 +532,8 @@ __device__ __forceinline__ unsigned nth_bit(unsigned m, int n) {
 // its product and the scale.  Bound by the latency of chains of loads, so the rows are told apart, and rows that take long
 // begin first.  Blocks 0 .. hub_blocks - 1 take the rows of more than DT_HUB such entries, a block each: its warps take every eighth piece of 32
 // of the row's entries in the part's CSR, and the sums are added in a fixed order.  The next many_blocks take the other rows of more than
-// DT_LCAP, a warp each.  (Where the scratch has no word to spare per row, both take groups of 32 rows: 23 us for single rows, 45 for
-// groups in the last example below, 80 with the marks searched for instead of listed.)  The rest: a warp takes 32 consecutive rows with up to DT_LCAP, their counts and listed columns with one load
+// DT_LCAP, a warp each.  Where the scratch had no room to list them all (long_room), both kinds of blocks look for the marks in left_cnt,
+// 32 rows at a time.  The rest: a warp takes 32 consecutive rows with up to DT_LCAP, their counts and listed columns with one load
 // each; then the rows that have entries, several at a time, two source rows of each requested together (most
 // rows have one or two).  LPR lanes own a row (pieces of 8 values per lane): 32 for rows wider than 64 values,
 // two rows at a time per warp; 8 for narrower rows, eight at a time, two per quarter of the warp.
@@ -545,7 +545,7 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
                     const int32_t* __restrict__ col_out, const float* __restrict__ inv_deg,
                     const int* __restrict__ dense, const unsigned char* __restrict__ left_cnt,
                     const int32_t* __restrict__ left_col, const int* __restrict__ long_count, const int32_t* __restrict__ long_rows,
-                    const int64_t long_room, const int long_unit, const unsigned hub_blocks, const unsigned many_blocks, const Planes src, const Planes out,
+                    const int64_t long_room, const unsigned hub_blocks, const unsigned many_blocks, const Planes src, const Planes out,
                     const int width, const int64_t total_groups) {
     wait_for_kernel_before();
     constexpr int S = 32 / LPR;            // rows side by side in a warp
@@ -640,14 +640,25 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
                 }
             }
         };
-        // single scratch rows or groups of 32 (all of one part), from the list's front (with a hub: a block each) or back (a warp each)
-        const int n = long_count[hub ? 0 : 1], step = hub ? (int)hub_blocks : (int)many_blocks * 8;
+        // scratch rows from the list's front (hubs) or back; of an incomplete list nothing counts but the numbers
+        const int n_hub = long_count[0], n_many = long_count[1];
+        const bool listed = (int64_t)n_hub + n_many <= long_room;
+        const int n = hub ? n_hub : n_many;
+        const int64_t items = n == 0 ? 0 : listed ? n : total_groups, step = hub ? (int64_t)hub_blocks : (int64_t)many_blocks * 8;
 #pragma unroll 1
-        for (int item = hub ? (int)blockIdx.x : (int)(blockIdx.x - hub_blocks) * 8 + warp; item < n; item += step) {
-            const int first = long_unit * long_rows[hub ? (int64_t)item : long_room - 1 - item];
+        for (int64_t item = hub ? (int64_t)blockIdx.x : (int64_t)(blockIdx.x - hub_blocks) * 8 + warp; item < items; item += step) {
+            int first;
+            unsigned rest = 1u;
+            if (listed) {
+                first = long_rows[hub ? item : long_room - 1 - item];
+            } else {
+                int k, i0;
+                if (!locate_tile(g, 32, item, &k, &i0)) break;
+                first = (int)g.row_ws[k] + i0;
+                rest = __ballot_sync(0xffffffffu, dense[g.part[k]] && i0 + lane < g.rows[k] && left_cnt[first + lane] == (hub ? DT_HUB_MARK : DT_OVERFLOW));
+            }
 #pragma unroll 1
-            for (unsigned rest = long_unit == 1 ? 1u : __ballot_sync(0xffffffffu, left_cnt[first + lane] >= DT_HUB_MARK); rest; rest &= rest - 1)
-                do_row(first + __ffs(rest) - 1);
+            for (; rest; rest &= rest - 1) do_row(first + __ffs(rest) - 1);
         }
         return;
     }
@@ -745,14 +756,15 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
 
 // Once per call, for every row of a part that takes the tiles: its window as DT_KB 64-bit masks, and the
 // entries outside the window in row order: up to DT_LCAP columns and their number, or DT_OVERFLOW or DT_HUB_MARK when there
-// are more; and such rows (long_unit 32: the groups of 32 with such rows) in long_rows, hubs from its front (long_count[0] of them), others from its back ([1]).  A row that repeats an entry inside its window takes its part back to the gather kernels
-// (dense[trainer] = 0): a bit cannot count.
+// are more; and such rows in long_rows, hubs from its front (long_count[0] of them), others from its back ([1]), as far as its long_room
+// words reach: the list is complete if the two numbers together are no larger.  A row that repeats an entry inside its window takes its
+// part back to the gather kernels (dense[trainer] = 0): a bit cannot count.
 __global__ void __launch_bounds__(256)
 dense_lists_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict__ rowptr_out,
                    const int32_t* __restrict__ col_out, int* __restrict__ dense,
                    unsigned long long* __restrict__ win_bits, unsigned char* __restrict__ block_mask,
                    unsigned char* __restrict__ left_cnt, int32_t* __restrict__ left_col, int* __restrict__ long_count, int32_t* __restrict__ long_rows,
-                   const int64_t long_room, const int long_unit) {
+                   const int64_t long_room) {
     wait_for_kernel_before();
     int k, r0;
     if (!locate_tile(g, 256, blockIdx.x, &k, &r0)) return;
@@ -792,15 +804,13 @@ dense_lists_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restric
 #pragma unroll
     for (int q = 0; q < DT_KB; ++q) blocks |= bits[q] ? 1u << q : 0u;
     blocks = __reduce_or_sync(0xffffffffu, blocks);
-    const int most = __reduce_max_sync(0xffffffffu, cnt);
     if (!live) return;
-    if ((threadIdx.x & 31) == 0) {  // parts start at multiples of 64 scratch rows
-        block_mask[row / 32] = (unsigned char)blocks;
+    if ((threadIdx.x & 31) == 0) block_mask[row / 32] = (unsigned char)blocks;  // parts start at multiples of 64 scratch rows
+    if (cnt > DT_LCAP) {  // the order in the list does not matter
+        const bool hub = cnt > DT_HUB;
+        const int64_t at = atomicAdd(long_count + (hub ? 0 : 1), 1);
+        if (at < long_room) long_rows[hub ? at : long_room - 1 - at] = (int32_t)row;
     }
-    // the order in the lists does not matter
-    const int longest = long_unit == 1 ? cnt : (threadIdx.x & 31) == 0 ? most : 0;
-    if (longest > DT_HUB) long_rows[atomicAdd(long_count, 1)] = (int32_t)(row / long_unit);
-    else if (longest > DT_LCAP) long_rows[long_room - 1 - atomicAdd(long_count + 1, 1)] = (int32_t)(row / long_unit);
 #pragma unroll
     for (int q = 0; q < DT_KB; ++q) win_bits[row * DT_KB + q] = bits[q];
     left_cnt[row] = cnt <= DT_LCAP ? (unsigned char)cnt : cnt <= DT_HUB ? DT_OVERFLOW : DT_HUB_MARK;
@@ -875,10 +885,10 @@ int32_t launch_dense_probe(rtma_ctx* ctx, const GroupDesc& g, const int64_t* row
 
 int32_t launch_dense_lists(rtma_ctx* ctx, const GroupDesc& g, const int64_t* rowptr_out, const int32_t* col_out,
                            int* dense, unsigned long long* win_bits, unsigned char* block_mask, unsigned char* left_cnt,
-                           int32_t* left_col, int* long_count, int32_t* long_rows, int64_t long_room, int long_unit, cudaStream_t s) {
+                           int32_t* left_col, int* long_count, int32_t* long_rows, int64_t long_room, cudaStream_t s) {
     const int64_t tiles = group_tiles(g, 256);
     if (tiles == 0) return RTMA_OK;
-    { KernelScope ks(ctx, KC_INV_DEGREE, s); launch_kernel(dense_lists_kernel, (unsigned)tiles, 256, 0, s, g, rowptr_out, col_out, dense, win_bits, block_mask, left_cnt, left_col, long_count, long_rows, long_room, long_unit); }
+    { KernelScope ks(ctx, KC_INV_DEGREE, s); launch_kernel(dense_lists_kernel, (unsigned)tiles, 256, 0, s, g, rowptr_out, col_out, dense, win_bits, block_mask, left_cnt, left_col, long_count, long_rows, long_room); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }
@@ -934,7 +944,7 @@ int32_t launch_spmm_dense(rtma_ctx* ctx, int kclass, const GroupDesc& g, const i
         KernelScope ks(ctx, kclass, s);
 #define RTMA_OUTSIDE(T, L)                                                                                              \
     launch_kernel(spmm_outside_kernel<T, L>, lgrid, 256, 0, s, g, rowptr_out, col_out, inv_deg, dense, order.left_cnt, order.left_col, \
-                  order.long_count, order.long_rows, rows_total / order.long_unit, order.long_unit, hub_blocks, many_blocks, src, out, a.width, groups)
+                  order.long_count, order.long_rows, order.long_room, hub_blocks, many_blocks, src, out, a.width, groups)
         if (a.width <= 64) {
             if (transposed) RTMA_OUTSIDE(true, 8);
             else RTMA_OUTSIDE(false, 8);

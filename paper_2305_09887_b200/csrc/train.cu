@@ -99,6 +99,21 @@ int32_t parse_model(rtma_ctx* ctx, const rtma_model_desc* md, Model* m) {
     return RTMA_OK;
 }
 
+int32_t parse_decoder(rtma_ctx* ctx, const rtma_model_desc* md, const rtma_decoder_desc* dd, Model* m) {
+    if (!dd || dd->Kd < 1 || dd->Kd > RTMA_MAX_LAYERS) return rtma_fail(ctx, RTMA_ERR_INVALID_ARG, "decoder layers outside [1,%d]", RTMA_MAX_LAYERS);
+    if (dd->ddims[0] != md->dims[md->L] || dd->ddims[dd->Kd] != 1)
+        return rtma_fail(ctx, RTMA_ERR_INVALID_ARG, "decoder widths must start at the embedding width %d and end at 1", md->dims[md->L]);
+    for (int k = 0; k <= dd->Kd; ++k) {
+        if (dd->ddims[k] < 1) return rtma_fail(ctx, RTMA_ERR_INVALID_ARG, "ddims[%d]=%d", k, dd->ddims[k]);
+        m->ddims[k] = dd->ddims[k];
+    }
+    m->Kd = dd->Kd;
+    m->P = layout_decoder(dd, m->P, m->dec);
+    for (int l = 0; l < m->L; ++l) m->layer[l].P = m->P;
+    for (int k = 0; k < m->Kd; ++k) m->dec[k].P = m->P;
+    return RTMA_OK;
+}
+
 // Scratch one part of n_p rows needs.
 struct ScratchPlan {
     size_t per_row_bytes;     // planes, logits, 1/deg
@@ -188,12 +203,8 @@ int splits_for(int64_t n_p, int parts_in_flight, const WgradCost& c, int64_t cap
     });
 }
 
-// The chunks of a part that its share of the scratch has room for: it holds 64 sets of `params` values, a set takes `partial`, and
-// `others` words of other lists lie there too.
-int64_t most_splits(size_t params, size_t partial, size_t others) {
-    const size_t room = 64 * params > others ? 64 * params - others : 0;
-    return std::max<int64_t>(1, (int64_t)(room / std::max<size_t>(partial, 1)));
-}
+// The chunks of a part that its share of the scratch has room for: it holds 64 sets of `params` values, a set takes `partial`.
+int64_t most_splits(size_t params, size_t partial) { return std::max<int64_t>(1, (int64_t)(64 * params / std::max<size_t>(partial, 1))); }
 
 int plan_splits(const GroupDesc& g, int parts_in_flight, const WgradCost& cost, int64_t cap, SplitPlan* sp) {
     int slots = 0;
@@ -205,6 +216,32 @@ int plan_splits(const GroupDesc& g, int parts_in_flight, const WgradCost& cost, 
     }
     sp->split_begin[g.num] = slots;
     return slots;
+}
+
+// The chunks of every layer of the network for the parts of g.  One chunking per layer: the number of blocks per chunk depends on the
+// layer's shape.  Returns the largest number of chunks.
+int plan_layers(const Model& m, const ScratchPlan& plan, bool head, bool single, const GroupDesc& g, int parts_in_flight, SplitPlan* spl) {
+    int slots = 0;
+    for (int l = 0; l < m.L; ++l) {
+        LayerShape shape = m.layer[l];
+        if (head && l == m.L - 1) {  // the head form's weight gradient: H^T [dZ | Q]
+            shape.nsrc = 1;
+            shape.d_out = 2 * m.Cp;
+        }
+        slots = std::max(slots, plan_splits(g, parts_in_flight, tc_wgrad_cost(shape, single),
+                                            most_splits(plan.max_layer_params, plan.max_layer_partial), &spl[l]));
+    }
+    return slots;
+}
+
+// The same for the decoder: one chunking for all its layers, that of the costliest.
+int plan_decoder(const Model& m, const ScratchPlan& plan, bool single, const GroupDesc& gd, int parts_in_flight, SplitPlan* spd) {
+    WgradCost widest{};
+    for (int k = 0; k < m.Kd; ++k) {
+        const WgradCost c = tc_wgrad_cost(m.dec[k], single);
+        if (c.blocks_per_slot * c.bytes_per_row > widest.blocks_per_slot * widest.bytes_per_row) widest = c;
+    }
+    return plan_splits(gd, parts_in_flight, widest, most_splits(plan.max_decoder_params, plan.max_decoder_partial), spd);
 }
 
 size_t part_scratch_bytes(const Model& m, const ScratchPlan& sp, int64_t n_p, int64_t pairs) {
@@ -227,6 +264,23 @@ extern "C" int64_t rtma_param_count(const rtma_model_desc* md) {
     return layout_model(md, nullptr);
 }
 
+extern "C" int32_t rtma_selftest_chunks(const rtma_model_desc* md, const rtma_decoder_desc* dd, int64_t n_p, int32_t parts, int32_t* chunks) {
+    if (!md || n_p < 0 || n_p >= (int64_t(1) << 31) || parts < 1 || !chunks) return RTMA_ERR_INVALID_ARG;
+    Model m;
+    RTMA_TRY(parse_model(nullptr, md, &m));
+    if (dd) RTMA_TRY(parse_decoder(nullptr, md, dd, &m));
+    const bool head = m.head && !dd;
+    const ScratchPlan plan = plan_scratch(m, head, false);
+    GroupDesc g{};
+    g.num = 1;
+    g.rows[0] = (int32_t)n_p;
+    SplitPlan spl[RTMA_MAX_LAYERS];
+    plan_layers(m, plan, head, md->gemm_dtype == 1, g, parts, spl);
+    for (int l = 0; l < m.L; ++l) chunks[l] = spl[l].split_begin[1];
+    if (dd) chunks[m.L] = plan_decoder(m, plan, md->gemm_dtype == 1, g, parts, &spl[0]);
+    return RTMA_OK;
+}
+
 namespace {
 
 // The training loop behind rtma_local_steps, rtma_local_steps_var (link == NULL: softmax
@@ -241,18 +295,7 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
     Model m;
     RTMA_TRY(parse_model(ctx, md, &m));
     if (link) {
-        const rtma_decoder_desc* dd = link->dd;
-        if (!dd || dd->Kd < 1 || dd->Kd > RTMA_MAX_LAYERS) return rtma_fail(ctx, RTMA_ERR_INVALID_ARG, "decoder layers outside [1,%d]", RTMA_MAX_LAYERS);
-        if (dd->ddims[0] != md->dims[md->L] || dd->ddims[dd->Kd] != 1)
-            return rtma_fail(ctx, RTMA_ERR_INVALID_ARG, "decoder widths must start at the embedding width %d and end at 1", md->dims[md->L]);
-        for (int k = 0; k <= dd->Kd; ++k) {
-            if (dd->ddims[k] < 1) return rtma_fail(ctx, RTMA_ERR_INVALID_ARG, "ddims[%d]=%d", k, dd->ddims[k]);
-            m.ddims[k] = dd->ddims[k];
-        }
-        m.Kd = dd->Kd;
-        m.P = layout_decoder(dd, m.P, m.dec);
-        for (int l = 0; l < m.L; ++l) m.layer[l].P = m.P;
-        for (int k = 0; k < m.Kd; ++k) m.dec[k].P = m.P;
+        RTMA_TRY(parse_decoder(ctx, md, link->dd, &m));
         if (!link->pair_offsets) return rtma_fail(ctx, RTMA_ERR_INVALID_ARG, "rtma_link_steps: null pair offsets");
         for (int p = 0; p < M && M <= RTMA_MAX_PARTS; ++p)
             if (link->pair_offsets[p + 1] < link->pair_offsets[p] || link->pair_offsets[p + 1] - link->pair_offsets[p] >= (int64_t(1) << 31))
@@ -314,25 +357,30 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
     const bool head = m.head && !link;
     const bool record = taps && taps->acts;     // the verification record wants Abar H of every layer and the scores
     const ScratchPlan plan = plan_scratch(m, head, record);
-    size_t want_share = 0, min_share = 0;
+    const bool tiles = ctx->dense_mode != 0 && !m.gcn;  // parts may be aggregated on the tensor cores
+    size_t want_share = 0, min_share = 0, list_share = 0;
     for (size_t gi = 0; gi < G; ++gi) {
-        size_t sum = 0;
+        size_t sum = 0, rows = 0;
         for (int p : group_parts[gi]) {
             const size_t b = part_scratch_bytes(m, plan, part_offsets[p + 1] - part_offsets[p],
                                                 link ? link->pair_offsets[p + 1] - link->pair_offsets[p] : 0);
             sum += b;
+            rows += (size_t)aligned_rows(part_offsets[p + 1] - part_offsets[p]);
             min_share = std::max(min_share, b);
         }
         want_share = std::max(want_share, sum);
+        list_share = std::max(list_share, sum + (tiles ? sizeof(int32_t) * rows + 256 : 0));
     }
     want_share = ArenaCursor::granule(want_share);
     min_share = ArenaCursor::granule(min_share);
+    list_share = ArenaCursor::granule(list_share);
     const size_t cap = ctx->arena_limit ? ctx->arena_limit : ~size_t(0);
     if (std::min(ctx->arena_bytes, cap) < want_share * G) {
         size_t free_b = 0, total_b = 0;
         RTMA_CUDA(ctx, cudaMemGetInfo(&free_b, &total_b));
         const size_t reachable = std::min(cap, ctx->arena_bytes + (size_t)((double)free_b * 0.9));
-        size_t target = std::min(want_share * G, reachable);
+        // an arena that has to grow gets a word per row on top, for the list of long rows below, which does with less
+        size_t target = std::min(list_share * G, reachable);
         if (target < min_share * G)
             return rtma_fail(ctx, RTMA_ERR_WORKSPACE,
                              "need %zu bytes of scratch per stream for the largest part (%zu streams), %zu reachable; use fewer distinct streams",
@@ -376,24 +424,8 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                 bytes += b;
                 ++at;
             }
-            // one chunking per layer: the number of blocks per chunk depends on the layer's shape
             SplitPlan wave_spl[RTMA_MAX_LAYERS];
-            int slots = 0;
-            // The list of rows with many entries outside their tile's window takes a word per row where that costs the largest part at
-            // most a quarter of its chunks, else one per 32 rows (half of which the loss tiles leave of theirs).
-            size_t most_rows = 0;
-            for (int k = 0; k < g.num; ++k) most_rows = std::max(most_rows, (size_t)aligned_rows(g.rows[k]));
-            const int long_unit = 64 * plan.max_layer_params >= 48 * plan.max_layer_partial + most_rows + 64 ? 1 : 32;
-            const size_t long_lists = (long_unit == 1 ? most_rows : most_rows / 64) + 64;
-            for (int l = 0; l < m.L; ++l) {
-                LayerShape shape = m.layer[l];
-                if (head && l == m.L - 1) {  // the head form's weight gradient: H^T [dZ | Q]
-                    shape.nsrc = 1;
-                    shape.d_out = 2 * m.Cp;
-                }
-                slots = std::max(slots, plan_splits(g, running, tc_wgrad_cost(shape, single_pass),
-                                                    most_splits(plan.max_layer_params, plan.max_layer_partial, long_lists), &wave_spl[l]));
-            }
+            const int slots = plan_layers(m, plan, head, single_pass, g, running, wave_spl);
             int wave_steps = 0;
             for (int k = 0; k < g.num; ++k) wave_steps = std::max(wave_steps, steps[g.part[k]]);
 
@@ -458,12 +490,7 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                     El[k] = take_pair_planes(m.ddims[k]);
                     ZDl[k] = take_pair_planes(m.ddims[k + 1]);
                 }
-                WgradCost widest{};  // one chunking for all decoder layers: that of the costliest
-                for (int k = 0; k < m.Kd; ++k) {
-                    const WgradCost c = tc_wgrad_cost(m.dec[k], single_pass);
-                    if (c.blocks_per_slot * c.bytes_per_row > widest.blocks_per_slot * widest.bytes_per_row) widest = c;
-                }
-                const int dslots = plan_splits(gd, running, widest, most_splits(plan.max_decoder_params, plan.max_decoder_partial, 0), &spd);
+                const int dslots = plan_decoder(m, plan, single_pass, gd, running, &spd);
                 dec_partial = cur.take<float>((size_t)dslots * plan.max_decoder_partial + 4);
                 dec_tile_loss = cur.take<float>((size_t)loss_tiles(gd) + 4);
             }
@@ -483,8 +510,6 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
             unsigned long long* win_bits = cur.take<unsigned long long>((size_t)rows * (DENSE_WINDOW / 64) + 2);
             int32_t* left_col = cur.take<int32_t>((size_t)rows * DENSE_LEFT_CAP + 4);
             unsigned char* left_cnt = cur.take<unsigned char>((size_t)rows + 16);
-            int32_t* long_rows = cur.take<int32_t>((size_t)(rows / long_unit) + 1);
-            int* long_count = ticket + 32;
             unsigned char* block_mask = cur.take<unsigned char>((size_t)rows / 32 + 1);
             float* post_partial = m.post ? cur.take<float>((size_t)post_tiles(g) * (2 * plan.post_width + 1) + 4) : nullptr;
             if (link && m.Kd > 1) dec_post_partial = cur.take<float>((size_t)post_tiles(gd) * (2 * plan.post_width + 1) + 4);
@@ -512,6 +537,12 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
             }
             if (cur.used > share)
                 return rtma_fail(ctx, RTMA_ERR_WORKSPACE, "internal: wave needs %zu bytes, share is %zu", cur.used, share);
+            // What is left of the share lists the rows with many entries outside their tile's window: how far it reaches changes the time
+            // of their pass and nothing else (paid for with chunks of the weight gradient, the list took that from 459 us to 13,700 for
+            // 1 M rows of an 8-8-2 network, and some calls did not fit).
+            const int64_t long_room = tiles ? std::min<int64_t>(rows, (int64_t)((share - cur.used) / 256 * (256 / sizeof(int32_t)))) : 0;
+            int32_t* long_rows = cur.take<int32_t>((size_t)long_room);
+            int* long_count = ticket + 32;
             if (rows == 0) continue;
 
             // the rows between the parts of every matrix that a tile may read past a part's end
@@ -548,7 +579,7 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
             for (int k = 0; k < g.num; ++k) wave_entries += edge_offsets[g.part[k] + 1] - edge_offsets[g.part[k]];
             SpmmOrder wave_order;
             RTMA_TRY(launch_spmm_order(ctx, g, rowptr_out, col_out, wave_entries, ticket + 16, heavy_list, &wave_order, s));
-            if (ctx->dense_mode != 0 && !m.gcn && tc_available()) {
+            if (tiles) {
                 // Which parts take the tensor-core tiles is decided on the device; the host waits for the answer
                 // (the only synchronisation of the call), so that a wave without such parts launches nothing for them.
                 RTMA_TRY(launch_dense_probe(ctx, g, rowptr_out, col_out, ctx->dense_mode, dense_counts, dense_flags, s));
@@ -567,7 +598,7 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                 };
                 RTMA_TRY(read_flags());
                 if (any_dense) {  // the per-row masks and lists; a part with repeated entries is taken back: read again
-                    RTMA_TRY(launch_dense_lists(ctx, g, rowptr_out, col_out, dense_flags, win_bits, block_mask, left_cnt, left_col, long_count, long_rows, rows / long_unit, long_unit, s));
+                    RTMA_TRY(launch_dense_lists(ctx, g, rowptr_out, col_out, dense_flags, win_bits, block_mask, left_cnt, left_col, long_count, long_rows, long_room, s));
                     RTMA_TRY(read_flags());
                 }
                 wave_order.all_dense = any_dense && all_dense;
@@ -578,7 +609,7 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                     wave_order.left_col = left_col;
                     wave_order.long_count = long_count;
                     wave_order.long_rows = long_rows;
-                    wave_order.long_unit = long_unit;
+                    wave_order.long_room = long_room;
                     wave_order.win_bits = win_bits;
                     wave_order.block_mask = block_mask;
                 }

@@ -149,9 +149,9 @@ struct SpmmOrder {
     const unsigned char* left_cnt;  // device, per scratch row of such a part: its entries outside the tile's window
                                     // (254, 255: more than DENSE_LEFT_CAP), and their columns [row][DENSE_LEFT_CAP]
     const int32_t* left_col;
-    const int* long_count;     // device: rows of more, listed in long_rows: [0] hubs from its front, [1] the others from its back;
-    const int32_t* long_rows;  // scratch row / long_unit (1, or 32: groups of rows)
-    int long_unit;
+    const int* long_count;     // device: the rows of more: [0] hubs, listed in long_rows from its front, [1] the others, from its back;
+    const int32_t* long_rows;  // where both together are more than long_room nothing is listed
+    int64_t long_room;
     const unsigned long long* win_bits;  // device, per scratch row of such a part: its window as DENSE_WINDOW bits
     const unsigned char* block_mask;     // device, per 32 scratch rows of such a part: bit b = one of them has an entry in
                                          // its window's 64-row block b
@@ -189,11 +189,11 @@ int32_t launch_dense_probe(rtma_ctx* ctx, const GroupDesc& g, const int64_t* row
 // Once per call, after launch_dense_probe, for every row of the flagged parts: the window as a bit mask and the
 // entries outside it.  win_bits: DENSE_WINDOW / 64 words per scratch row (16-byte aligned); left_cnt: one byte
 // per scratch row; left_col: DENSE_LEFT_CAP ints per scratch row (16-byte aligned); block_mask: one byte per 32
-// scratch rows.  long_rows: long_room = scratch rows / long_unit ints; long_count: two ints, zero on entry.  Clears the flag of a
+// scratch rows.  long_rows: long_room ints, any number; long_count: two ints, zero on entry.  Clears the flag of a
 // part in which a row repeats an entry inside its window.
 int32_t launch_dense_lists(rtma_ctx* ctx, const GroupDesc& g, const int64_t* rowptr_out, const int32_t* col_out,
                            int* dense, unsigned long long* win_bits, unsigned char* block_mask, unsigned char* left_cnt,
-                           int32_t* left_col, int* long_count, int32_t* long_rows, int64_t long_room, int long_unit, cudaStream_t s);
+                           int32_t* left_col, int* long_count, int32_t* long_rows, int64_t long_room, cudaStream_t s);
 // The parts of g flagged in order.dense: out = Abar src (transposed: Abar^T src on a symmetric part), window
 // entries by tensor-core tiles, the others summed into the output rows beforehand by a gather pass.  Other
 // parts are left alone.

@@ -227,7 +227,7 @@ def test_parts_choose_for_themselves(util):
                                              (24_000, 7, (16, 16, 5))])
 def test_entries_outside_the_windows(util, forced, tiny_workload, n, degree, dims):
     # two parts of about 670 rows, 5 tiles and a bit: rows without entries outside their window, with listed ones, with more than
-    # are listed, and two hubs with hundreds.  The last: parts so large beside their weights that long rows are listed by groups of 32
+    # are listed, and two hubs with hundreds.  The last: large parts of a network with few weights
     g = inputs.uniform_graph(n, n * degree // 2, 31)
     rows, cols = np.repeat(np.arange(n), np.diff(g.rowptr)), g.col.astype(np.int64)
     rng = np.random.default_rng(32)
