@@ -609,8 +609,8 @@ struct WgradArgs {
     int tmem_cols, stages;
     int bk;           // rows (k) per pipeline stage: 64 or 32
     int single;       // 1: operands rounded to bf16 (hi planes only)
-    CUtensorMap mapP; // partial as rows of d_out values, boxes of 32 x 32
-    float* partial;   // [slot][(nsrc d_in + 1)] rows, padded_ld(d_out) apart
+    CUtensorMap mapP; // partial as rows of d_out values, boxes of 32 x 32; used where its rows start at multiples of 16 bytes
+    float* partial;   // [slot][(nsrc d_in + 1)] rows, ld_partial apart
     int64_t ld_partial;
     int* error_word;
 };
@@ -619,8 +619,8 @@ struct WgradArgs {
 // tiles of 128 of them), the sources' columns, H's and behind them N's, are the accumulator's columns, as many atoms of 64
 // as the tensor memory and the stages have room for (wgrad_shape).  A few classes then cost one MMA with 256 columns where
 // they cost two with 64 or 128.  The partial sums leave through shared memory, 32 x 32 of them by a bulk-tensor store, in rows
-// padded to 16 bytes (stored by the threads, 16 bytes of 32 rows at a time, they took 4 us of an 18 us launch; stored down
-// their columns, a line per warp, 8 us more than that).  The thread that issues the MMAs is as easily the longest chain as the loads are, with one
+// padded to 16 bytes where the scratch holds that (stored by the threads, 16 bytes of 32 rows at a time, they took 4 us of an 18 us launch;
+// stored down their columns, a line per warp, 8 us more than that: so they are where it does not, in chunks of thousands of rows).  The thread that issues the MMAs is as easily the longest chain as the loads are, with one
 // plane per operand above all: its loop keeps descriptors as a constant plus an address and no division by the number of
 // stages (500,000 rows, 1,024 x 512 in bf16: 658 us, with this form and divisions 975, now 574).
 // us a launch before and after: the head of 47 classes on 200 k rows of 256 62 / 55, on 2 M 615 / 495, of two classes on 5 M
@@ -813,6 +813,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
             // A lane holds output column c of 32 source columns j: through a 32 x 32 slab (row j, 16-byte piece c / 4 at piece
             // c / 4 ^ j % 8, as the map's swizzle has it; the ring is free, behind the column sums' 16 KB) and out as a box.
             const int q = warp & 3;
+            const bool boxes = a.ld_partial % 4 == 0;
             uint8_t* slab[2] = {smem + 16384 + q * 8192, smem + 16384 + q * 8192 + 4096};
             int n_out = 0;
             for (int t = 0; t < z_tiles; ++t) {
@@ -828,7 +829,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
                     tc::tmem_load_issue(acc + 32u * (uint32_t)n, raw);
                     tc::tmem_load_wait(raw);
                     const int64_t row = slot_row + (second ? d_in : 0) + j0;
-                    if (j0 + 32 <= d_in) {
+                    if (boxes && j0 + 32 <= d_in) {
                         uint8_t* out = slab[n_out++ & 1];
                         if (lane == 0) tc::tma_store_wait_read_but_one();  // the box before the last has left the slab
                         __syncwarp();
@@ -841,7 +842,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
                             tc::tma_store_2d(&a.mapP, out, cbase + c0, (int)row);
                             tc::tma_store_commit();
                         }
-                    } else if (c0 + lane < ccount) {  // the source's last columns: the rows behind them are not its
+                    } else if (c0 + lane < ccount) {  // the source's last columns (the rows behind them are not its), or rows at any address
                         float* o = a.partial + row * a.ld_partial + cbase + c0 + lane;
 #pragma unroll
                         for (int e = 0; e < 32; ++e)
@@ -1160,12 +1161,12 @@ WgradCost tc_wgrad_cost(const LayerShape& ls, bool single) {
     WgradCost c;
     c.blocks_per_slot = (int64_t)w.blocks_x * w.blocks_z;
     c.bytes_per_row = (single ? 1 : 2) * 128 * (w.z_atoms + w.col_atoms);
-    c.params = (int64_t)(ls.nsrc * ls.d_in + 1) * padded_ld(ls.d_out);
+    c.params = (int64_t)(ls.nsrc * ls.d_in + 1) * ls.d_out;
     return c;
 }
 
 int32_t launch_tc_wgrad(rtma_ctx* ctx, const GroupDesc& g, const SplitPlan& sp, LayerShape ls, int64_t rows_total,
-                        Planes H, Planes N, Planes dZ, float* partial, bool single, cudaStream_t s) {
+                        Planes H, Planes N, Planes dZ, float* partial, int64_t ld_partial, bool single, cudaStream_t s) {
     if (!ctx->wgrad_configured) {
         RTMA_TRY(set_smem_limit(ctx, reinterpret_cast<const void*>(tc_wgrad_kernel)));
         ctx->wgrad_configured = true;
@@ -1191,8 +1192,8 @@ int32_t launch_tc_wgrad(rtma_ctx* ctx, const GroupDesc& g, const SplitPlan& sp, 
     const size_t stage_bytes = stage64 * a.bk / 64;
     a.stages = stages_for(stage_bytes, MAX_STAGES);
     a.partial = partial;
-    a.ld_partial = padded_ld(ls.d_out);
-    if (!make_tensor_map_f32(&a.mapP, partial, (uint64_t)slots * (ls.nsrc * ls.d_in + 1), ls.d_out, a.ld_partial))
+    a.ld_partial = ld_partial;
+    if (ld_partial % 4 == 0 && !make_tensor_map_f32(&a.mapP, partial, (uint64_t)slots * (ls.nsrc * ls.d_in + 1), ls.d_out, a.ld_partial))
         return rtma_fail(ctx, RTMA_ERR_CUDA, "cuTensorMapEncodeTiled refused the partial sums");
     a.error_word = ctx->error_word;
     // boxes of 64 columns x BK rows: one atom of a stage

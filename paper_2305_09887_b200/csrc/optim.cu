@@ -10,14 +10,14 @@ namespace {
 
 __global__ void __launch_bounds__(256)
 reduce_sgd_kernel(const __grid_constant__ GroupDesc g, const __grid_constant__ SplitPlan sp, const LayerShape ls,
-                  const float* __restrict__ partial, const float lr, float* __restrict__ params,
+                  const float* __restrict__ partial, const int64_t ld, const float lr, float* __restrict__ params,
                   float* __restrict__ grads_record) {
     wait_for_kernel_before();
     const int k = blockIdx.y;
     const int64_t rows = (int64_t)ls.nsrc * ls.d_in;                      // the weight matrices; behind them the bias row
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= (rows + (ls.has_bias ? 1 : 0)) * ls.d_out) return;
-    const int64_t ld = (ls.d_out + 3) / 4 * 4, stride = (rows + 1) * ld;  // of the partial sums
+    const int64_t stride = (rows + 1) * ld;                               // of the partial sums, whose rows lie ld apart
     const int64_t at_partial = (int64_t)((uint32_t)i / (uint32_t)ls.d_out) * ld + (uint32_t)i % (uint32_t)ls.d_out;
     float gsum = 0.f;
     const int s_end = sp.split_begin[k + 1];
@@ -153,11 +153,11 @@ int32_t aggregate_impl(rtma_ctx* ctx, float* params, const float* grads, float l
 }  // namespace
 
 int32_t launch_reduce_sgd(rtma_ctx* ctx, const GroupDesc& g, const SplitPlan& sp, LayerShape ls, const float* partial,
-                          float lr, float* params, float* grads_record, cudaStream_t s) {
+                          int64_t ld_partial, float lr, float* params, float* grads_record, cudaStream_t s) {
     if (g.num == 0) return RTMA_OK;
     const int64_t count = (int64_t)(ls.nsrc * ls.d_in + 1) * ls.d_out;
     dim3 grid((unsigned)ceil_div(count, 256), (unsigned)g.num);
-    { KernelScope ks(ctx, KC_REDUCE_SGD, s); launch_kernel(reduce_sgd_kernel, grid, 256, 0, s, g, sp, ls, partial, lr, params, grads_record); }
+    { KernelScope ks(ctx, KC_REDUCE_SGD, s); launch_kernel(reduce_sgd_kernel, grid, 256, 0, s, g, sp, ls, partial, ld_partial, lr, params, grads_record); }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;
 }

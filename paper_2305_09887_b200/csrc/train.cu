@@ -119,7 +119,6 @@ struct ScratchPlan {
     size_t per_row_bytes;     // planes, logits, 1/deg
     size_t max_layer_params;  // largest (2 d_in + 1) d_out
     size_t max_decoder_params;  // the same of the decoder's layers (link prediction)
-    size_t max_layer_partial, max_decoder_partial;  // the same with d_out rounded up, as a chunk's partial sums are stored
     size_t prep_bytes;        // repacked weights, per part
     int q_width;              // widest Abar^T dZ (widths of the layers above the first)
     size_t post_width;        // widest normalised / PReLU layer output (0: none)
@@ -140,11 +139,7 @@ ScratchPlan plan_scratch(const Model& m, bool head, bool record) {
         if (l < m.L - 1 && m.post) per_row += 4 * planes_ld(m.dims[l + 1]) + sizeof(float2);  // Z^{l}, (mean, 1/std)
         if (l >= 1 && !(head && l == m.L - 1)) q_width = std::max(q_width, m.dims[l + 1]);
         sp.max_layer_params = std::max(sp.max_layer_params, (size_t)(m.layer[l].nsrc * m.dims[l] + 1) * m.dims[l + 1]);
-        sp.max_layer_partial = std::max(sp.max_layer_partial, (size_t)(m.layer[l].nsrc * m.dims[l] + 1) * padded_ld(m.dims[l + 1]));
-        if (head && l == m.L - 1) {
-            sp.max_layer_params = std::max(sp.max_layer_params, (size_t)(m.dims[l] + 1) * 2 * m.Cp);
-            sp.max_layer_partial = std::max(sp.max_layer_partial, (size_t)(m.dims[l] + 1) * 2 * m.Cp);
-        }
+        if (head && l == m.L - 1) sp.max_layer_params = std::max(sp.max_layer_params, (size_t)(m.dims[l] + 1) * 2 * m.Cp);
         if (l < m.L - 1 && m.post) sp.post_width = std::max(sp.post_width, (size_t)m.dims[l + 1]);
         const TcLayerPlan lp = (head && l == m.L - 1) ? tc_plan_head(m.layer[l], m.Cp) : tc_plan_layer(m.layer[l]);
         sp.prep_bytes += sizeof(__nv_bfloat16) * tc_prep_elems(lp, l >= 1) + 4 * 256;
@@ -161,7 +156,6 @@ ScratchPlan plan_scratch(const Model& m, bool head, bool record) {
     for (int k = 0; k < m.Kd; ++k) {
         sp.per_pair_bytes += 4 * planes_ld(m.ddims[k]) + 4 * planes_ld(m.ddims[k + 1]);
         sp.max_decoder_params = std::max(sp.max_decoder_params, (size_t)(m.ddims[k] + 1) * m.ddims[k + 1]);
-        sp.max_decoder_partial = std::max(sp.max_decoder_partial, (size_t)(m.ddims[k] + 1) * padded_ld(m.ddims[k + 1]));
         sp.prep_bytes += sizeof(__nv_bfloat16) * tc_prep_elems(tc_plan_layer(m.dec[k]), true) + 4 * 256;
         if (k < m.Kd - 1) sp.post_width = std::max(sp.post_width, (size_t)m.ddims[k + 1]);
     }
@@ -169,13 +163,15 @@ ScratchPlan plan_scratch(const Model& m, bool head, bool record) {
     return sp;
 }
 
+constexpr int MOST_SPLITS = 64;  // chunks a part may have; its share of the scratch holds the partial sums of as many
+
 // Row chunks of the weight gradient, every part taken for as large as this one.
 // At least `fewest`, the chunks (of 1024 rows or more) at which (waves of blocks) x (rows per chunk) is within 3 % of its
 // least: the tensor cores truncate when they accumulate, and with chunks 2.5 times as long the parameters of 5 M rows
 // moved by 1.3e-5 in five steps.  More than that where it is faster: a block (one per SM at a time) takes a fixed 4 us and then
 // stages its rows at about 41 bytes per ns, and every chunk adds a set of partial sums that is written and read back
 // (about 4,000 bytes per ns).  Small parts gain: 3 parts of 10,000 rows ran 30 blocks, 37 us a launch, now 120 of 256 rows.
-int splits_for(int64_t n_p, int parts_in_flight, const WgradCost& c, int64_t cap) {
+int splits_for(int64_t n_p, int parts_in_flight, const WgradCost& c) {
     constexpr int64_t SMS = 148;
     if (n_p <= 0) return 1;
     auto waves_of = [&](int64_t ns, int64_t* rows, int64_t* slots) {
@@ -190,12 +186,12 @@ int splits_for(int64_t n_p, int parts_in_flight, const WgradCost& c, int64_t cap
             if (cost(ns) <= best * 1.03) return ns;
         return to;
     };
-    const int64_t fewest = least_within(1, std::min<int64_t>(cap, std::max<int64_t>(1, ceil_div(n_p, 1024))), [&](int64_t ns) {
+    const int64_t fewest = least_within(1, std::min<int64_t>(MOST_SPLITS, std::max<int64_t>(1, ceil_div(n_p, 1024))), [&](int64_t ns) {
         int64_t rows, slots;
         const int64_t waves = waves_of(ns, &rows, &slots);
         return (double)waves * (double)rows;
     });
-    const int64_t most = std::max(fewest, std::min<int64_t>(cap, ceil_div(n_p, 128)));
+    const int64_t most = std::max(fewest, std::min<int64_t>(MOST_SPLITS, ceil_div(n_p, 128)));
     return (int)least_within(fewest, most, [&](int64_t ns) {
         int64_t rows, slots;
         const int64_t waves = waves_of(ns, &rows, &slots);
@@ -203,14 +199,11 @@ int splits_for(int64_t n_p, int parts_in_flight, const WgradCost& c, int64_t cap
     });
 }
 
-// The chunks of a part that its share of the scratch has room for: it holds 64 sets of `params` values, a set takes `partial`.
-int64_t most_splits(size_t params, size_t partial) { return std::max<int64_t>(1, (int64_t)(64 * params / std::max<size_t>(partial, 1))); }
-
-int plan_splits(const GroupDesc& g, int parts_in_flight, const WgradCost& cost, int64_t cap, SplitPlan* sp) {
+int plan_splits(const GroupDesc& g, int parts_in_flight, const WgradCost& cost, SplitPlan* sp) {
     int slots = 0;
     for (int k = 0; k < g.num; ++k) {
         sp->split_begin[k] = slots;
-        const int nsplit = splits_for(g.rows[k], parts_in_flight, cost, cap);
+        const int nsplit = splits_for(g.rows[k], parts_in_flight, cost);
         sp->rows_per_split[k] = (int32_t)std::max<int64_t>(GROUP_ROW_ALIGN, aligned_rows(ceil_div(g.rows[k], nsplit)));
         slots += (int)std::max<int64_t>(1, ceil_div(g.rows[k], sp->rows_per_split[k]));
     }
@@ -218,39 +211,51 @@ int plan_splits(const GroupDesc& g, int parts_in_flight, const WgradCost& cost, 
     return slots;
 }
 
+// How the partial sums of `slots` chunks lie: values between rows in *ld, the result is the words they take.  Rows start at
+// multiples of 16 bytes (the kernel then stores boxes) where `room` words hold that, and follow one another otherwise: padding is
+// not paid for with chunks (a decoder of one layer had a quarter of them: 131,072 pairs of 256 values, 80 us a launch instead of 35).
+size_t partial_words(const LayerShape& ls, int slots, size_t room, int64_t* ld) {
+    const size_t rows = (size_t)slots * (size_t)(ls.nsrc * ls.d_in + 1);
+    *ld = rows * (size_t)padded_ld(ls.d_out) <= room ? padded_ld(ls.d_out) : ls.d_out;
+    return rows * (size_t)*ld;
+}
+
 // The chunks of every layer of the network for the parts of g.  One chunking per layer: the number of blocks per chunk depends on the
-// layer's shape.  Returns the largest number of chunks.
-int plan_layers(const Model& m, const ScratchPlan& plan, bool head, bool single, const GroupDesc& g, int parts_in_flight, SplitPlan* spl) {
-    int slots = 0;
+// layer's shape.  Returns the words that the partial sums of a layer take at most.
+size_t plan_layers(const Model& m, const ScratchPlan& plan, bool head, bool single, const GroupDesc& g, int parts_in_flight, SplitPlan* spl, int64_t* ld) {
+    size_t words = 0;
     for (int l = 0; l < m.L; ++l) {
         LayerShape shape = m.layer[l];
         if (head && l == m.L - 1) {  // the head form's weight gradient: H^T [dZ | Q]
             shape.nsrc = 1;
             shape.d_out = 2 * m.Cp;
         }
-        slots = std::max(slots, plan_splits(g, parts_in_flight, tc_wgrad_cost(shape, single),
-                                            most_splits(plan.max_layer_params, plan.max_layer_partial), &spl[l]));
+        const int slots = plan_splits(g, parts_in_flight, tc_wgrad_cost(shape, single), &spl[l]);
+        words = std::max(words, partial_words(shape, slots, (size_t)g.num * MOST_SPLITS * plan.max_layer_params, &ld[l]));
     }
-    return slots;
+    return words;
 }
 
 // The same for the decoder: one chunking for all its layers, that of the costliest.
-int plan_decoder(const Model& m, const ScratchPlan& plan, bool single, const GroupDesc& gd, int parts_in_flight, SplitPlan* spd) {
+size_t plan_decoder(const Model& m, const ScratchPlan& plan, bool single, const GroupDesc& gd, int parts_in_flight, SplitPlan* spd, int64_t* ld) {
     WgradCost widest{};
     for (int k = 0; k < m.Kd; ++k) {
         const WgradCost c = tc_wgrad_cost(m.dec[k], single);
         if (c.blocks_per_slot * c.bytes_per_row > widest.blocks_per_slot * widest.bytes_per_row) widest = c;
     }
-    return plan_splits(gd, parts_in_flight, widest, most_splits(plan.max_decoder_params, plan.max_decoder_partial), spd);
+    const int slots = plan_splits(gd, parts_in_flight, widest, spd);
+    size_t words = 0;
+    for (int k = 0; k < m.Kd; ++k) words = std::max(words, partial_words(m.dec[k], slots, (size_t)gd.num * MOST_SPLITS * plan.max_decoder_params, &ld[k]));
+    return words;
 }
 
 size_t part_scratch_bytes(const Model& m, const ScratchPlan& sp, int64_t n_p, int64_t pairs) {
     const size_t rows = (size_t)aligned_rows(n_p);
     const size_t prows = (size_t)aligned_rows(pairs);
     const size_t matrices = 8 * m.L + 8 * m.Kd + 24;  // every matrix start is rounded up to 256 bytes
-    const size_t decoder = sp.per_pair_bytes * prows + sizeof(float) * (64 * sp.max_decoder_params + (size_t)ceil_div(pairs, 32) + 256) +
+    const size_t decoder = sp.per_pair_bytes * prows + sizeof(float) * (MOST_SPLITS * sp.max_decoder_params + (size_t)ceil_div(pairs, 32) + 256) +
                            sizeof(float) * ((size_t)ceil_div(pairs, 64) + 1) * (2 * sp.post_width + 1);
-    return sp.per_row_bytes * rows + sizeof(float) * (64 * sp.max_layer_params + (size_t)ceil_div(n_p, 32) + 256) +
+    return sp.per_row_bytes * rows + sizeof(float) * (MOST_SPLITS * sp.max_layer_params + (size_t)ceil_div(n_p, 32) + 256) +
            (m.Kd ? decoder : 0) + rows / 32 +
            sizeof(int) * ((size_t)ceil_div(n_p, 8) + 64 + 7 * RTMA_MAX_PARTS) +  // processing order of the aggregation kernels, per-part flags
            sizeof(float) * ((size_t)ceil_div(n_p, 64) + 1) * (2 * sp.post_width + 1) +  // per-tile sums of d gamma, d beta, d a
@@ -275,9 +280,13 @@ extern "C" int32_t rtma_selftest_chunks(const rtma_model_desc* md, const rtma_de
     g.num = 1;
     g.rows[0] = (int32_t)n_p;
     SplitPlan spl[RTMA_MAX_LAYERS];
-    plan_layers(m, plan, head, md->gemm_dtype == 1, g, parts, spl);
+    int64_t ld[RTMA_MAX_LAYERS];
+    plan_layers(m, plan, head, md->gemm_dtype == 1, g, parts, spl, ld);
     for (int l = 0; l < m.L; ++l) chunks[l] = spl[l].split_begin[1];
-    if (dd) chunks[m.L] = plan_decoder(m, plan, md->gemm_dtype == 1, g, parts, &spl[0]);
+    if (dd) {
+        plan_decoder(m, plan, md->gemm_dtype == 1, g, parts, &spl[0], ld);
+        chunks[m.L] = spl[0].split_begin[1];
+    }
     return RTMA_OK;
 }
 
@@ -425,7 +434,8 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                 ++at;
             }
             SplitPlan wave_spl[RTMA_MAX_LAYERS];
-            const int slots = plan_layers(m, plan, head, single_pass, g, running, wave_spl);
+            int64_t ld_partial[RTMA_MAX_LAYERS], ld_dec_partial[RTMA_MAX_LAYERS];
+            const size_t partial_size = plan_layers(m, plan, head, single_pass, g, running, wave_spl, ld_partial);
             int wave_steps = 0;
             for (int k = 0; k < g.num; ++k) wave_steps = std::max(wave_steps, steps[g.part[k]]);
 
@@ -490,14 +500,13 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                     El[k] = take_pair_planes(m.ddims[k]);
                     ZDl[k] = take_pair_planes(m.ddims[k + 1]);
                 }
-                const int dslots = plan_decoder(m, plan, single_pass, gd, running, &spd);
-                dec_partial = cur.take<float>((size_t)dslots * plan.max_decoder_partial + 4);
+                dec_partial = cur.take<float>(plan_decoder(m, plan, single_pass, gd, running, &spd, ld_dec_partial) + 4);
                 dec_tile_loss = cur.take<float>((size_t)loss_tiles(gd) + 4);
             }
             // Abar^T dZ of the layer in hand; carved at the widest layer, addressed at each layer's own width
             __nv_bfloat16* q_hi = plan.q_width ? cur.take<__nv_bfloat16>((size_t)rows * planes_ld(plan.q_width) + 8) : nullptr;
             __nv_bfloat16* q_lo = plan.q_width ? cur.take<__nv_bfloat16>((size_t)rows * planes_ld(plan.q_width) + 8) : nullptr;
-            float* partial = cur.take<float>((size_t)slots * plan.max_layer_partial + 4);
+            float* partial = cur.take<float>(partial_size + 4);
             float* tile_loss = cur.take<float>((size_t)loss_tiles(g) + 4);
             const size_t counters_at = cur.used;  // from here to counters_end: zero on entry
             int* ticket = cur.take<int>(64);  // work counter of the aggregation kernels (zero between launches)
@@ -736,11 +745,11 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                     RTMA_TRY(launch_loss_finalize(ctx, gd, dec_tile_loss, loss_out, loss_stride, step, s));
                     // decoder backward + SGD
                     for (int k = m.Kd - 1; k >= 0 && prows > 0; --k) {
-                        RTMA_TRY(launch_tc_wgrad(ctx, gd, spd, m.dec[k], prows, El[k], El[k], ZDl[k], dec_partial, single_pass, s));
+                        RTMA_TRY(launch_tc_wgrad(ctx, gd, spd, m.dec[k], prows, El[k], El[k], ZDl[k], dec_partial, ld_dec_partial[k], single_pass, s));
                         // d e^k = d Z^k Theta^k^T, written over e^k
                         RTMA_TRY(launch_tc_dgrad(ctx, gd, m.dec[k], dtcp[k], prows, ZDl[k], ZDl[k], DBd_hi[k], DBd_lo[k], El[k], false,
                                                  single_pass, s));
-                        RTMA_TRY(launch_reduce_sgd(ctx, gd, spd, m.dec[k], dec_partial, m.lr, params, grads_rec, s));
+                        RTMA_TRY(launch_reduce_sgd(ctx, gd, spd, m.dec[k], dec_partial, ld_dec_partial[k], m.lr, params, grads_rec, s));
                         if (k > 0)
                             RTMA_TRY(launch_post_backward(ctx, gd, m.dec[k - 1], params, ZDl[k - 1], El[k], nullptr, dec_post_partial,
                                                           m.lr, grads_rec, s));
@@ -777,7 +786,7 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                         LayerShape ws = m.layer[l];
                         ws.nsrc = 1;
                         ws.d_out = 2 * Cp;
-                        RTMA_TRY(launch_tc_wgrad(ctx, g, spl[l], ws, rows, Hl[l], Hl[l], DQ, partial, single_pass, s));
+                        RTMA_TRY(launch_tc_wgrad(ctx, g, spl[l], ws, rows, Hl[l], Hl[l], DQ, partial, ld_partial[l], single_pass, s));
                         if (l > 0) {
                             if (!single_pass && dgrad_narrow_applies(m.layer[l]))
                                 RTMA_TRY(launch_dgrad_narrow(ctx, g, m.layer[l], params, dZlast, Qlast, Hl[l], !m.post, s));
@@ -792,7 +801,7 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                                                         loss_out, loss_stride, step, s));
                         continue;
                     }
-                    RTMA_TRY(launch_tc_wgrad(ctx, g, spl[l], m.layer[l], rows, Hl[l], Nl[l], dZ, partial, single_pass, s));
+                    RTMA_TRY(launch_tc_wgrad(ctx, g, spl[l], m.layer[l], rows, Hl[l], Nl[l], dZ, partial, ld_partial[l], single_pass, s));
                     if (l > 0) {
                         // dH^l = dZ Ws^T + Abar^T (dZ Wn^T) = [dZ | Abar^T dZ] [Ws^T ; Wn^T]: aggregate first,
                         // at the layer's output width, then one product whose epilogue applies the ReLU
@@ -805,7 +814,7 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                             RTMA_TRY(launch_post_backward(ctx, g, m.layer[l - 1], params, Zl[l - 1], Hl[l], stats[l - 1], post_partial,
                                                           m.lr, tap ? taps->grads : nullptr, s));
                     }
-                    RTMA_TRY(launch_reduce_sgd(ctx, g, spl[l], m.layer[l], partial, m.lr, params, tap ? taps->grads : nullptr, s));
+                    RTMA_TRY(launch_reduce_sgd(ctx, g, spl[l], m.layer[l], partial, ld_partial[l], m.lr, params, tap ? taps->grads : nullptr, s));
                 }
             }
         }

@@ -255,7 +255,7 @@ int32_t launch_dgrad_narrow(rtma_ctx* ctx, const GroupDesc& g, LayerShape ls, co
 // ---- optim.cu -------------------------------------------------------------------------
 // grad = sum of the part's chunk slots; params -= lr * grad; optionally records grad.
 int32_t launch_reduce_sgd(rtma_ctx* ctx, const GroupDesc& g, const SplitPlan& sp, LayerShape ls, const float* partial,
-                          float lr, float* params, float* grads_record, cudaStream_t s);
+                          int64_t ld_partial, float lr, float* params, float* grads_record, cudaStream_t s);
 // The same for the head form of the last layer: partial[slot] is [(d_in + 1) x 2 head_cp], the product of
 // [H | 1]^T with [dZ | Q]; columns c of the first block give dWs (and db in the last row), columns
 // head_cp + c give dWn (for a one-matrix layer dW, and the first block only gives db).  And the parts' losses from the sums that
@@ -309,7 +309,7 @@ struct WgradCost {
     int64_t params;           // partial sums a chunk leaves
 };
 WgradCost tc_wgrad_cost(const LayerShape& ls, bool single);
-// partial[slot][(nsrc d_in + 1) x d_out, rows padded_ld(d_out) apart] = [H | N | 1]^T dZ ([N | 1]^T dZ for a one-matrix layer)
+// partial[slot][(nsrc d_in + 1) x d_out, rows ld_partial apart] = [H | N | 1]^T dZ ([N | 1]^T dZ for a one-matrix layer)
 // over one chunk of rows.
 int32_t launch_tc_wgrad(rtma_ctx* ctx, const GroupDesc& g, const SplitPlan& sp, LayerShape ls, int64_t rows_total,
-                        Planes H, Planes N, Planes dZ, float* partial, bool single, cudaStream_t s);
+                        Planes H, Planes N, Planes dZ, float* partial, int64_t ld_partial, bool single, cudaStream_t s);

@@ -53,3 +53,12 @@ def _check(dims, n, parts=1, ddims=None, gemm_dtype=0, variant=(0, 0, 0)):
 def test_chunks_of_networks_that_are_small_beside_their_part(dims, n, variant):
     _check(dims, n, 1, variant=variant)
     _check(dims, n // 5, 5, variant=variant)
+
+
+# widths that are no multiple of four: the rows of the partial sums are padded, the scratch counts them unpadded
+@pytest.mark.parametrize("dims, n, ddims", [((16, 16, 5), 1_000_000, None), ((16, 16, 5), 4_000_000, None), ((32, 32, 7), 5_000_000, None), ((64, 90, 3), 1_000_000, None),
+                                            ((10, 33, 3), 200_000, None), ((8, 5), 1_000_000, None), ((64, 256, 256), 131_072, (256, 1)), ((64, 128, 128), 1_000_000, (128, 1)),
+                                            ((64, 64, 30), 500_000, (30, 7, 1))])
+def test_chunks_of_widths_whose_partial_sums_are_padded(dims, n, ddims):
+    _check(dims, n, 1, ddims)
+    _check(dims, n // 3, 3, ddims)

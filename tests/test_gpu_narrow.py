@@ -91,3 +91,21 @@ def test_long_rows_listed_or_searched_for_give_the_same_bits(util):
     want, _ = oracle.local_steps_variant((0, 0, 0), dims, 0.1, rowptr, (key % n).astype(np.int32), w.X.astype(np.float64), w.y,
                                          w.params0.astype(np.float64), 3)
     assert util.rel_err(searched, want) <= util.TOL_PARAM
+
+
+@pytest.mark.parametrize("dims, M", [((10, 33, 3), 1), ((10, 70, 33), 2), ((20, 5), 1)])
+def test_as_many_chunks_as_a_part_may_have_of_an_odd_width(util, dims, M):
+    # the padded rows of the partial sums do not fit then: they follow one another, at addresses that no bulk-tensor store can take
+    n = 140_000
+    sums = [(c * (2 * a + 1), b) for c, a, b in zip(binding.selftest_chunks(dims, n // M, M), dims[:-1], dims[1:])]
+    assert max(rows * -(-b // 4) * 4 for rows, b in sums) > 64 * max((2 * a + 1) * b for a, b in zip(dims[:-1], dims[1:]))
+    w = _workload(n, 3, dims, (0, 0, 0), M)
+    got, want = util.check_one_step(w)
+    util.check_k_steps_and_average(w, got, want, 2)
+
+
+def test_linear_decoder_on_many_pairs(util):
+    import test_gpu_link as tl
+    w = _workload(30_000, 8, (24, 40, 40), (0, 0, 0))
+    assert binding.selftest_chunks(w.dims, 131_072, ddims=(40, 1))[-1] == 64
+    tl._check_link(util, w, (0, 1, 1), (40, 1), per_part=65_536, K=2)
