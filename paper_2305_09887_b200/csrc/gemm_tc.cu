@@ -1160,6 +1160,7 @@ WgradCost tc_wgrad_cost(const LayerShape& ls, bool single) {
     const WgradShape w = wgrad_shape(ls, single);
     WgradCost c;
     c.blocks_per_slot = (int64_t)w.blocks_x * w.blocks_z;
+    c.plain_blocks_per_slot = ceil_div(ls.nsrc * ceil_div(ls.d_in, 128), 2) * ceil_div(ls.d_out, 256);
     c.bytes_per_row = (single ? 1 : 2) * 128 * (w.z_atoms + w.col_atoms);
     c.params = (int64_t)(ls.nsrc * ls.d_in + 1) * ls.d_out;
     return c;

@@ -167,17 +167,18 @@ constexpr int MOST_SPLITS = 64;  // chunks a part may have; its share of the scr
 
 // Row chunks of the weight gradient, every part taken for as large as this one.
 // At least `fewest`, the chunks (of 1024 rows or more) at which (waves of blocks) x (rows per chunk) is within 3 % of its
-// least: the tensor cores truncate when they accumulate, and with chunks 2.5 times as long the parameters of 5 M rows
-// moved by 1.3e-5 in five steps.  More than that where it is faster: a block (one per SM at a time) takes a fixed 4 us and then
+// least, counted in blocks of 256 x 256 sums whatever the kernel's blocks are: the tensor cores truncate when they accumulate, and with
+// chunks 2.5 times as long the parameters of 5 M rows moved by 1.3e-5 in five steps.  (Counted in the kernel's own blocks, up to 512
+// columns wide, 16 parts of 13,800 rows of 512 -> 64 took 3 chunks each instead of 9.)  More than that where it is faster: a block (one per SM at a time) takes a fixed 4 us and then
 // stages its rows at about 41 bytes per ns, and every chunk adds a set of partial sums that is written and read back
 // (about 4,000 bytes per ns).  Small parts gain: 3 parts of 10,000 rows ran 30 blocks, 37 us a launch, now 120 of 256 rows.
 int splits_for(int64_t n_p, int parts_in_flight, const WgradCost& c) {
     constexpr int64_t SMS = 148;
     if (n_p <= 0) return 1;
-    auto waves_of = [&](int64_t ns, int64_t* rows, int64_t* slots) {
+    auto waves_of = [&](int64_t ns, int64_t blocks_per_slot, int64_t* rows, int64_t* slots) {
         *rows = aligned_rows(ceil_div(n_p, ns));
         *slots = (int64_t)parts_in_flight * ceil_div(n_p, *rows);
-        return ceil_div(*slots * c.blocks_per_slot, SMS);
+        return ceil_div(*slots * blocks_per_slot, SMS);
     };
     auto least_within = [&](int64_t from, int64_t to, auto cost) {
         double best = cost(from);
@@ -188,13 +189,13 @@ int splits_for(int64_t n_p, int parts_in_flight, const WgradCost& c) {
     };
     const int64_t fewest = least_within(1, std::min<int64_t>(MOST_SPLITS, std::max<int64_t>(1, ceil_div(n_p, 1024))), [&](int64_t ns) {
         int64_t rows, slots;
-        const int64_t waves = waves_of(ns, &rows, &slots);
+        const int64_t waves = waves_of(ns, c.plain_blocks_per_slot, &rows, &slots);
         return (double)waves * (double)rows;
     });
     const int64_t most = std::max(fewest, std::min<int64_t>(MOST_SPLITS, ceil_div(n_p, 128)));
     return (int)least_within(fewest, most, [&](int64_t ns) {
         int64_t rows, slots;
-        const int64_t waves = waves_of(ns, &rows, &slots);
+        const int64_t waves = waves_of(ns, c.blocks_per_slot, &rows, &slots);
         return (double)waves * (4000.0 + (double)rows * c.bytes_per_row / 41.0) + (double)slots * (double)c.params * 2.0 * sizeof(float) / 4000.0;
     });
 }

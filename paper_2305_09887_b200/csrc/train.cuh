@@ -304,9 +304,10 @@ int32_t launch_tc_dgrad(rtma_ctx* ctx, const GroupDesc& g, LayerShape ls, const 
                         bool single, cudaStream_t s);
 // What a chunk of rows costs launch_tc_wgrad for a layer of this shape.
 struct WgradCost {
-    int64_t blocks_per_slot;  // blocks started per chunk
-    int64_t bytes_per_row;    // that one of them stages
-    int64_t params;           // partial sums a chunk leaves
+    int64_t blocks_per_slot;        // blocks started per chunk
+    int64_t plain_blocks_per_slot;  // and if each took 256 x 256 sums
+    int64_t bytes_per_row;          // that one of them stages
+    int64_t params;                 // partial sums a chunk leaves
 };
 WgradCost tc_wgrad_cost(const LayerShape& ls, bool single);
 // partial[slot][(nsrc d_in + 1) x d_out, rows ld_partial apart] = [H | N | 1]^T dZ ([N | 1]^T dZ for a one-matrix layer)

@@ -62,3 +62,13 @@ def test_chunks_of_networks_that_are_small_beside_their_part(dims, n, variant):
 def test_chunks_of_widths_whose_partial_sums_are_padded(dims, n, ddims):
     _check(dims, n, 1, ddims)
     _check(dims, n // 3, 3, ddims)
+
+
+# layers whose sources are wider than what a block takes: however a chunk is cut into blocks, it is no longer for it
+@pytest.mark.parametrize("dims, n, parts", [((512, 64), 13_800, 16), ((512, 128), 9_700, 16), ((512, 96), 57_600, 16), ((512, 128), 10_072, 23), ((1024, 128), 3_152, 23),
+                                            ((512, 90), 7_991, 64), ((512, 512), 62_500, 8), ((128, 256, 256), 25_000, 8)])
+@pytest.mark.parametrize("gemm_dtype", [0, 1])
+def test_chunks_of_wide_layers(dims, n, parts, gemm_dtype):
+    got = binding.selftest_chunks(dims, n, parts, gemm_dtype=gemm_dtype)
+    for chunks, a, b in zip(got, dims[:-1], dims[1:]):
+        assert chunks >= _fewest(n, parts, _blocks(2, a, b)), (a, b, got)
