@@ -4,16 +4,20 @@
 // split planes.  With two classes that is four multiply-adds per output: the tensor cores would
 // spend their time on zero padding (K = 2 x 2 padded to 2 x 64), while this kernel only streams
 // the gate in and the gradient out.  It was bound by instructions and by the loads that a warp had in flight:
-// with the coefficients two to a word (instead of a 16-byte piece per plane, eight values for two), eight rows
+// with the coefficients two to a word (instead of a 16-byte piece per plane, eight values for two), up to eight rows
 // in flight instead of four, multiply-adds two at a time and the gate as a mask on the packed planes, 5 M rows of 256
-// columns and two classes take 1,285 us instead of 1,560 (6.2 TB/s).
+// columns and two classes take 1,285 us instead of 1,560 (6.2 TB/s), three 1,372 instead of 1,500, four 1,929 instead of 2,530.
 #include "train.cuh"
 
 namespace {
 
 constexpr int DN_THREADS = 256;
 constexpr int DN_TILE_ROWS = 512;  // rows of one part handled by a block: 64 per warp
-constexpr int DN_BATCH = 8;        // rows a warp has in flight
+// Rows a warp has in flight: as many as the weights (eight registers a product) leave room for at two blocks per SM.  5 M rows of 256
+// columns, us: six products with 4 rows 1,458, 5 rows 1,372, 8 rows 2,315 (they spill; alone on an SM 1,637); eight products with 3
+// rows 1,929, 4 rows 1,909 (they spill), 8 rows 3,320.  With one load per plane for the two words of a row: before, 4 rows 1,513.
+template <int PRODUCTS>
+constexpr int DN_ROWS = PRODUCTS <= 4 ? 8 : PRODUCTS <= 6 ? 5 : 3;
 
 // The c-th of the values whose planes lie two to a word
 template <int N>
@@ -22,12 +26,21 @@ __device__ __forceinline__ float half_of(const uint32_t (&hi)[N], const uint32_t
                  : __uint_as_float(hi[c / 2] << 16) + __uint_as_float(lo[c / 2] << 16);
 }
 
+// A row's first values, two to a word, with one load
+__device__ __forceinline__ void load_words(const __nv_bfloat16* p, uint32_t (&w)[1]) { w[0] = *reinterpret_cast<const uint32_t*>(p); }
+__device__ __forceinline__ void load_words(const __nv_bfloat16* p, uint32_t (&w)[2]) {
+    const uint2 v = *reinterpret_cast<const uint2*>(p);
+    w[0] = v.x;
+    w[1] = v.y;
+}
+
 // NSRC weight matrices (2: Ws and Wn; 1: W alone, multiplying Q), C classes: NSRC * C products per output
 template <int NSRC, int C>
 __global__ void __launch_bounds__(DN_THREADS, 2)
 dgrad_narrow_kernel(const __grid_constant__ GroupDesc g, const LayerShape ls, const float* __restrict__ params,
                     const Planes dZ, const Planes Q, const Planes H, const int gate) {
     wait_for_kernel_before();
+    constexpr int BATCH = DN_ROWS<NSRC * C>;
     int k, r0;
     if (!locate_tile(g, DN_TILE_ROWS, blockIdx.x, &k, &r0)) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -46,27 +59,24 @@ dgrad_narrow_kernel(const __grid_constant__ GroupDesc g, const LayerShape ls, co
 #pragma unroll
                 for (int c = 0; c < C; ++c)
                     w[m * C + c][e] = c0 + e < d_in ? __ldg(W + (int64_t)(m * d_in + c0 + e) * C + c) : 0.f;
-        for (int q0 = q_begin; q0 < q_end; q0 += DN_BATCH) {
+        for (int q0 = q_begin; q0 < q_end; q0 += BATCH) {
             // the rows' coefficients: dZ for the first weight matrix, Q for the second (or only) one; two to a word
             constexpr int CW = (C + 1) / 2;
-            uint32_t zh[DN_BATCH][CW], zl[DN_BATCH][CW], qh[DN_BATCH][CW], ql[DN_BATCH][CW];
-            uint4 gw[DN_BATCH];
+            uint32_t zh[BATCH][CW], zl[BATCH][CW], qh[BATCH][CW], ql[BATCH][CW];
+            uint4 gw[BATCH];
 #pragma unroll
-            for (int b = 0; b < DN_BATCH; ++b) {
+            for (int b = 0; b < BATCH; ++b) {
                 const int64_t r = g.row_ws[k] + r0 + min(q0 + b, q_end - 1);
-#pragma unroll
-                for (int c = 0; c < CW; ++c) {
-                    if (NSRC == 2) {
-                        zh[b][c] = reinterpret_cast<const uint32_t*>(dZ.hi + r * dZ.ld)[c];
-                        zl[b][c] = reinterpret_cast<const uint32_t*>(dZ.lo + r * dZ.ld)[c];
-                    }
-                    qh[b][c] = reinterpret_cast<const uint32_t*>(Q.hi + r * Q.ld)[c];
-                    ql[b][c] = reinterpret_cast<const uint32_t*>(Q.lo + r * Q.ld)[c];
+                if (NSRC == 2) {
+                    load_words(dZ.hi + r * dZ.ld, zh[b]);
+                    load_words(dZ.lo + r * dZ.ld, zl[b]);
                 }
+                load_words(Q.hi + r * Q.ld, qh[b]);
+                load_words(Q.lo + r * Q.ld, ql[b]);
                 gw[b] = gate ? *reinterpret_cast<const uint4*>(H.hi + r * H.ld + c0) : make_uint4(0u, 0u, 0u, 0u);
             }
 #pragma unroll
-            for (int b = 0; b < DN_BATCH; ++b) {
+            for (int b = 0; b < BATCH; ++b) {
                 if (q0 + b >= q_end) break;
                 const int64_t r = g.row_ws[k] + r0 + q0 + b;
                 Pack8 x;

@@ -353,3 +353,12 @@ def test_column_tiles_of_odd_multiples_of_32(util, dims, gemm_dtype, variant):
 def test_weight_gradient_tiles(util, dims, gemm_dtype):
     w = _workload(1_000, 3_000, dims, 17)
     util.check_one_step(w, M=3, gemm_dtype=gemm_dtype, gradients_against_plain=gemm_dtype == 0)
+
+
+# the input gradient of one to four classes: five, three or eight rows at a time of a warp's 64, parts whose last rows are fewer
+@pytest.mark.parametrize("dims, variant", [((24, 72, 3), (0, 0, 0)), ((24, 300, 4), (0, 0, 0)), ((24, 72, 4), (0, 1, 1)), ((24, 40, 3), (1, 0, 0)), ((24, 72, 1), (0, 0, 0)),
+                                           ((24, 264, 2), (1, 1, 0))])
+def test_input_gradient_of_a_few_classes(util, dims, variant):
+    for n in (1_541, 1_550):
+        w = _workload(n, 3 * n, dims, 19)
+        util.check_one_step(w, M=3, variant=variant, params0=inputs.variant_params(variant, dims, 20))
