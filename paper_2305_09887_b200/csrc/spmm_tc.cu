@@ -51,6 +51,7 @@ constexpr int DT_LCAP = DENSE_LEFT_CAP;          // listed entries outside the w
 constexpr unsigned char DT_OVERFLOW = 255;       // left_cnt of a row with more than that
 constexpr unsigned char DT_HUB_MARK = 254;       // and of one with more than DT_HUB
 constexpr int DT_HUB = 64;                       // entries outside the window up to which a row is not shared by a block
+constexpr int DT_HUBS_PER_BLOCK = 24;            // rows of more that a block takes one after another; more of them: a warp each
 constexpr int DT_SMEM_MAX = 225 * 1024;           // with the static part (under 2 KB) within the 227 KB a block may have
 static_assert(DT_BM == 128 && DENSE_WINDOW % DT_BK == 0 && DT_HALO % DT_BK == 0, "tile shape of the MMA and whole stages");
 
@@ -530,23 +531,24 @@ __device__ __forceinline__ unsigned nth_bit(unsigned m, int n) {
 // The entries outside the window of their row's tile, before the tiles run: for every row that has any,
 // out[row] = their sum (transposed pass: weighted by 1 / deg of the column), unscaled; the tile's epilogue adds
 // its product and the scale.  Bound by the latency of chains of loads, so the rows are told apart, and rows that take long
-// begin first.  Blocks 0 .. hub_blocks - 1 take the rows of more than DT_HUB such entries, a block each: its warps take every eighth piece of 32
-// of the row's entries in the part's CSR, and the sums are added in a fixed order.  The next many_blocks take the other rows of more than
-// DT_LCAP, a warp each.  Where the scratch had no room to list them all (long_room), both kinds of blocks look for the marks in left_cnt,
-// 32 rows at a time.  The rest: a warp takes 32 consecutive rows with up to DT_LCAP, their counts and listed columns with one load
+// begin first.  Blocks 0 .. hub_blocks - 1 take the rows of more than DT_HUB such entries, a block each: its warps take every eighth piece of
+// 32 of the row's entries in the part's CSR, and the sums are added in a fixed order.  The next many_blocks take the other rows of more than
+// DT_LCAP, a warp each.  The rest: a warp takes 32 consecutive rows with up to DT_LCAP, their counts and listed columns with one load
 // each; then the rows that have entries, several at a time, two source rows of each requested together (most
 // rows have one or two).  LPR lanes own a row (pieces of 8 values per lane): 32 for rows wider than 64 values,
 // two rows at a time per warp; 8 for narrower rows, eight at a time, two per quarter of the warp.
 // In one kernel with the long rows looked up by the warp that met them: 610 us for 2 M rows of 256 values of which 27 % have such
 // entries (1.2 M entries; now 335), of 48 values 285 (now 180), 40,000 rows with hubs of 280 entries 105 (now 23).
-template <bool TRANSPOSED, int LPR>
+// MANY: all blocks but those of the hubs take long rows (the last ones behind them their listed rows), and the hubs if no block takes them, a
+// warp each, with the sums in the same order; and where the scratch had no room to list the long rows, 32 rows at a time are looked
+// through for their marks.  launch_spmm_dense says when.
+template <bool TRANSPOSED, int LPR, bool MANY>
 __global__ void __launch_bounds__(256, 3)
 spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restrict__ rowptr_out,
                     const int32_t* __restrict__ col_out, const float* __restrict__ inv_deg,
                     const int* __restrict__ dense, const unsigned char* __restrict__ left_cnt,
-                    const int32_t* __restrict__ left_col, const int* __restrict__ long_count, const int32_t* __restrict__ long_rows,
-                    const int64_t long_room, const unsigned hub_blocks, const unsigned many_blocks, const Planes src, const Planes out,
-                    const int width, const int64_t total_groups) {
+                    const int32_t* __restrict__ left_col, const LongRows long_rows, const unsigned hub_blocks, const unsigned many_blocks,
+                    const Planes src, const Planes out, const int width, const int64_t total_groups) {
     wait_for_kernel_before();
     constexpr int S = 32 / LPR;            // rows side by side in a warp
     constexpr int NR = 2;                  // rows a lane works on at a time
@@ -554,12 +556,16 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
     const int lane = threadIdx.x & 31;
     const int sub = lane / LPR, sl = lane % LPR;
     const int warp = threadIdx.x >> 5;
-    if (blockIdx.x < hub_blocks + many_blocks) {
-        // ---- rows whose entries are looked up again ----
+    if (MANY || blockIdx.x < hub_blocks + many_blocks) {
+        // ---- the rows whose entries are looked up again ----
+        // A hub block takes hubs; the warps of the other blocks take the other long rows, and the hubs if there are no hub blocks
+        const bool hub_block = blockIdx.x < hub_blocks, hub_by_warp = MANY && hub_blocks == 0;
+        const int mine_hub = hub_block || hub_by_warp ? long_rows.hubs : 0, mine_many = hub_block ? 0 : long_rows.many;
         __shared__ __align__(16) float piece[8][LPR * 8];
-        const bool hub = blockIdx.x < hub_blocks;
-        // the sum of one row by this warp (a hub: of this warp's share, the block's first warp then adds the shares and stores)
-        auto do_row = [&](const int row) {
+        // the sum of one row by this warp (a hub in a hub block: of this warp's share, the block's first warp then adds the shares and
+        // stores; a hub elsewhere: share by share)
+        auto do_row = [&](const int row, const bool marked_hub) {
+            const bool hub = MANY ? marked_hub : hub_block;
             int k = 0;
             while (k < g.num && !(row >= g.row_ws[k] && row < g.row_ws[k] + g.rows[k])) ++k;
             if (k == g.num || !dense[g.part[k]]) return;  // past a part's end, of a part that has finished its steps or was taken back
@@ -575,52 +581,62 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
                 const __nv_bfloat16* sh = src.hi + ws * src.ld + (live ? c0 : 0);  // lanes past the width read column 0 and store nothing
                 const __nv_bfloat16* sl_ = src.lo + ws * src.ld + (live ? c0 : 0);
                 Pack8 acc;
-                acc.zero();
-                for (int64_t eb = e0 + (hub ? warp * 32 : 0); eb < e1; eb += hub ? 8 * 32 : 32) {
-                    const int64_t e = eb + lane;
-                    bool outside = false;
-                    int c = 0;
-                    if (e < e1) {
-                        c = __ldg(cols + e);
-                        outside = rtma_index_ok(c, n_p, 5) && (c < w_begin || c >= w_end);
+                for (int share = 0; share < (MANY && hub && !hub_block ? 8 : 1); ++share) {
+                    const int64_t eb0 = e0 + (hub ? (hub_block ? warp : share) * 32 : 0);
+                    if (share > 0 && eb0 >= e1) break;  // acc holds the sum of the shares before
+                    acc.zero();
+                    for (int64_t eb = eb0; eb < e1; eb += hub ? 8 * 32 : 32) {
+                        const int64_t e = eb + lane;
+                        bool outside = false;
+                        int c = 0;
+                        if (e < e1) {
+                            c = __ldg(cols + e);
+                            outside = rtma_index_ok(c, n_p, 5) && (c < w_begin || c >= w_end);
+                        }
+                        unsigned votes = __ballot_sync(0xffffffffu, outside);
+                        while (votes) {
+                            int u[4];
+                            uint4 yh[4], yl[4];
+                            float wy[4];
+#pragma unroll
+                            for (int b = 0; b < 4; ++b) {
+                                // quarter `sub` takes the entries sub, sub + S, ... of those still to do
+                                const unsigned from = nth_bit(votes, b * S + sub);
+                                u[b] = __shfl_sync(0xffffffffu, c, from < 32u ? (int)from : 0);
+                                if (from >= 32u) u[b] = -1;
+                            }
+#pragma unroll
+                            for (int b = 0; b < 4 * S; ++b) votes &= votes - 1;
+#pragma unroll
+                            for (int b = 0; b < 4; ++b) {
+                                if (u[b] >= 0) {
+                                    yh[b] = __ldg(reinterpret_cast<const uint4*>(sh + (int64_t)u[b] * src.ld));
+                                    yl[b] = __ldg(reinterpret_cast<const uint4*>(sl_ + (int64_t)u[b] * src.ld));
+                                    if (TRANSPOSED) wy[b] = __ldg(inv_deg + ws + u[b]);
+                                }
+                            }
+#pragma unroll
+                            for (int b = 0; b < 4; ++b) {
+                                if (u[b] >= 0) {
+                                    if (TRANSPOSED) acc.fma_planes_mixed(wy[b], yh[b], yl[b]);
+                                    else acc.add_planes_mixed(yh[b], yl[b]);
+                                }
+                            }
+                        }
                     }
-                    unsigned votes = __ballot_sync(0xffffffffu, outside);
-                    while (votes) {
-                        int u[4];
-                        uint4 yh[4], yl[4];
-                        float wy[4];
+                    // the quarters' sums, added in a fixed order
 #pragma unroll
-                        for (int b = 0; b < 4; ++b) {
-                            // quarter `sub` takes the entries sub, sub + S, ... of those still to do
-                            const unsigned from = nth_bit(votes, b * S + sub);
-                            u[b] = __shfl_sync(0xffffffffu, c, from < 32u ? (int)from : 0);
-                            if (from >= 32u) u[b] = -1;
-                        }
+                    for (int step_ = S / 2; step_ > 0; step_ >>= 1)
 #pragma unroll
-                        for (int b = 0; b < 4 * S; ++b) votes &= votes - 1;
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) {
-                            if (u[b] >= 0) {
-                                yh[b] = __ldg(reinterpret_cast<const uint4*>(sh + (int64_t)u[b] * src.ld));
-                                yl[b] = __ldg(reinterpret_cast<const uint4*>(sl_ + (int64_t)u[b] * src.ld));
-                                if (TRANSPOSED) wy[b] = __ldg(inv_deg + ws + u[b]);
-                            }
-                        }
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) {
-                            if (u[b] >= 0) {
-                                if (TRANSPOSED) acc.fma_planes_mixed(wy[b], yh[b], yl[b]);
-                                else acc.add_planes_mixed(yh[b], yl[b]);
-                            }
+                        for (int e = 0; e < 8; ++e) acc.v[e] += __shfl_down_sync(0xffffffffu, acc.v[e], step_ * LPR);
+                    if (MANY && hub && !hub_block && sub == 0) {  // the shares' sums, added as a block adds them
+                        for (int e = 0; e < 8; ++e) {
+                            float& sum = piece[warp][sl * 8 + e];
+                            sum = acc.v[e] = share == 0 ? acc.v[e] : sum + acc.v[e];
                         }
                     }
                 }
-                // the quarters' sums, added in a fixed order
-#pragma unroll
-                for (int step_ = S / 2; step_ > 0; step_ >>= 1)
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) acc.v[e] += __shfl_down_sync(0xffffffffu, acc.v[e], step_ * LPR);
-                if (hub) {  // and the warps'
+                if (hub_block) {  // and the warps'
                     __syncthreads();
                     if (sub == 0)
 #pragma unroll
@@ -632,7 +648,7 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
                             for (int e = 0; e < 8; ++e) acc.v[e] += piece[w][sl * 8 + e];
                     }
                 }
-                if (live && sub == 0 && (!hub || warp == 0)) {
+                if (live && sub == 0 && (!hub_block || warp == 0)) {
                     uint4 h, l;
                     acc.to_planes_lean(h, l);
                     *reinterpret_cast<uint4*>(out.hi + (int64_t)row * out.ld + c0) = h;
@@ -640,27 +656,32 @@ spmm_outside_kernel(const __grid_constant__ GroupDesc g, const int64_t* __restri
                 }
             }
         };
-        // scratch rows from the list's front (hubs) or back; of an incomplete list nothing counts but the numbers
-        const int n_hub = long_count[0], n_many = long_count[1];
-        const bool listed = (int64_t)n_hub + n_many <= long_room;
-        const int n = hub ? n_hub : n_many;
-        const int64_t items = n == 0 ? 0 : listed ? n : total_groups, step = hub ? (int64_t)hub_blocks : (int64_t)many_blocks * 8;
+        // scratch rows from the list's front (hubs) or back, or 32 rows and their marks
+        const bool listed = !MANY || long_rows.listed;
+        const int takers = (int)(MANY ? gridDim.x - hub_blocks : many_blocks);  // blocks whose warps take rows
+        const int items = listed ? mine_hub + mine_many : (int)total_groups, step = hub_block ? (int)hub_blocks : takers * 8;
 #pragma unroll 1
-        for (int64_t item = hub ? (int64_t)blockIdx.x : (int64_t)(blockIdx.x - hub_blocks) * 8 + warp; item < items; item += step) {
+        for (int item = hub_block ? (int)blockIdx.x : (int)(blockIdx.x - hub_blocks) * 8 + warp; item < items; item += step) {
             int first;
-            unsigned rest = 1u;
+            unsigned rest = 1u, hubs;
             if (listed) {
-                first = long_rows[hub ? item : long_room - 1 - item];
+                hubs = item < mine_hub ? 1u : 0u;
+                first = long_rows.list[hubs ? (int64_t)item : long_rows.room - 1 - (item - mine_hub)];
             } else {
                 int k, i0;
                 if (!locate_tile(g, 32, item, &k, &i0)) break;
                 first = (int)g.row_ws[k] + i0;
-                rest = __ballot_sync(0xffffffffu, dense[g.part[k]] && i0 + lane < g.rows[k] && left_cnt[first + lane] == (hub ? DT_HUB_MARK : DT_OVERFLOW));
+                const int mark = dense[g.part[k]] && i0 + lane < g.rows[k] ? (int)left_cnt[first + lane] : 0;
+                hubs = __ballot_sync(0xffffffffu, mark == DT_HUB_MARK && mine_hub > 0);
+                rest = __ballot_sync(0xffffffffu, mark == DT_OVERFLOW && mine_many > 0) | hubs;
             }
 #pragma unroll 1
-            for (; rest; rest &= rest - 1) do_row(first + __ffs(rest) - 1);
+            for (; rest; rest &= rest - 1) {
+                const int at = __ffs(rest) - 1;
+                do_row(first + at, hubs >> at & 1u);
+            }
         }
-        return;
+        if (blockIdx.x < hub_blocks + many_blocks) return;
     }
     const int64_t warps = (int64_t)(gridDim.x - hub_blocks - many_blocks) * 8;
     for (int64_t grp = (int64_t)(blockIdx.x - hub_blocks - many_blocks) * 8 + warp; grp < total_groups; grp += warps) {
@@ -936,22 +957,32 @@ int32_t launch_spmm_dense(rtma_ctx* ctx, int kclass, const GroupDesc& g, const i
     if (!make_tensor_map_bf16(&a.mapSh, src.hi, (uint64_t)rows_total, (uint64_t)a.width, (uint64_t)src.ld, 64, DT_BK) ||
         !make_tensor_map_bf16(&a.mapSl, src.lo, (uint64_t)rows_total, (uint64_t)a.width, (uint64_t)src.ld, 64, DT_BK))
         return rtma_fail(ctx, RTMA_ERR_CUDA, "cuTensorMapEncodeTiled refused the aggregation operands");
-    // how many rows of each kind there are only the device knows: a block per SM for the hubs, two for the other long rows
+    // A block per SM for the hubs, two for the other long rows.  100,000 rows, us a forward pass of 48 / 256 columns.  Hubs by warps from 24 a
+    // block on: 2,000 hubs of 280 entries by blocks 82 / 126, by warps 91 / 141; 4,000 102 / 194 and 109 / 185; 8,300 185 / 362 and 155 / 277; 100,000
+    // of 70 entries 830 / 1,440 and 229 / 366.  All blocks for the other long rows where these are most of the rows and give the warps of
+    // many_blocks more than 28 each: 98,000 of 10 entries 79 / 110 by many_blocks, 74 / 103 by all; 56,000 of 100,000 52 / 69 and 53 / 71 (740,000 of 2 M:
+    // 3 to 5 % slower by all); 36,000 of 40,000 with 100 hubs 35 / 46 and 40 / 53.
     const int64_t groups = group_tiles(g, 32);
-    const unsigned hub_blocks = (unsigned)ctx->sm_count, many_blocks = 2u * (unsigned)ctx->sm_count;
-    const unsigned lgrid = hub_blocks + many_blocks + (unsigned)std::min<int64_t>(ceil_div(groups, 8), (int64_t)ctx->sm_count * 12);
+    const LongRows& lr = order.long_rows;
+    const unsigned sms = (unsigned)ctx->sm_count;
+    const bool hubs_by_warp = lr.hubs > DT_HUBS_PER_BLOCK * (int)sms, many = !lr.listed || hubs_by_warp || (lr.hubs <= 4 * (int)sms && 2 * (int64_t)lr.many > rows_total && lr.many > 28 * 16 * (int)sms);
+    const unsigned hub_blocks = hubs_by_warp || lr.hubs == 0 ? 0u : sms, many_blocks = lr.many > 0 || hubs_by_warp ? 2u * sms : 0u;
+    const unsigned lgrid = hub_blocks + many_blocks + (unsigned)std::min<int64_t>(ceil_div(groups, 8), (int64_t)sms * 12);
     {
         KernelScope ks(ctx, kclass, s);
-#define RTMA_OUTSIDE(T, L)                                                                                              \
-    launch_kernel(spmm_outside_kernel<T, L>, lgrid, 256, 0, s, g, rowptr_out, col_out, inv_deg, dense, order.left_cnt, order.left_col, \
-                  order.long_count, order.long_rows, order.long_room, hub_blocks, many_blocks, src, out, a.width, groups)
-        if (a.width <= 64) {
-            if (transposed) RTMA_OUTSIDE(true, 8);
-            else RTMA_OUTSIDE(false, 8);
-        } else {
-            if (transposed) RTMA_OUTSIDE(true, 32);
-            else RTMA_OUTSIDE(false, 32);
-        }
+#define RTMA_OUTSIDE(T, L, MANY)                                                                                              \
+    launch_kernel(spmm_outside_kernel<T, L, MANY>, lgrid, 256, 0, s, g, rowptr_out, col_out, inv_deg, dense, order.left_cnt, order.left_col, \
+                  lr, hub_blocks, many_blocks, src, out, a.width, groups)
+#define RTMA_OUTSIDE_BY_WIDTH(T, MANY)                  \
+    do {                                                \
+        if (a.width <= 64) RTMA_OUTSIDE(T, 8, MANY);    \
+        else RTMA_OUTSIDE(T, 32, MANY);                 \
+    } while (0)
+        if (transposed && many) RTMA_OUTSIDE_BY_WIDTH(true, true);
+        else if (transposed) RTMA_OUTSIDE_BY_WIDTH(true, false);
+        else if (many) RTMA_OUTSIDE_BY_WIDTH(false, true);
+        else RTMA_OUTSIDE_BY_WIDTH(false, false);
+#undef RTMA_OUTSIDE_BY_WIDTH
 #undef RTMA_OUTSIDE
     }
     RTMA_LAUNCH_CHECK(ctx);

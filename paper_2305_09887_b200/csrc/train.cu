@@ -512,8 +512,9 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
             const size_t counters_at = cur.used;  // from here to counters_end: zero on entry
             int* ticket = cur.take<int>(64);  // work counter of the aggregation kernels (zero between launches)
             unsigned long long* dense_counts = cur.take<unsigned long long>(3 * RTMA_MAX_PARTS);
-            int* dense_flags = cur.take<int>(RTMA_MAX_PARTS);  // per trainer: aggregated on the tensor cores
-            unsigned long long* sym_sums = cur.take<unsigned long long>(4);
+            int* dense_flags = cur.take<int>(RTMA_MAX_PARTS + 10);  // per trainer: aggregated on the tensor cores
+            int* long_count = dense_flags + RTMA_MAX_PARTS;         // 2: rows with many entries outside their tile's window
+            unsigned long long* sym_sums = reinterpret_cast<unsigned long long*>(long_count + 2);  // 4
             const size_t counters_end = cur.used;
             int* heavy_list = cur.take<int>((size_t)spmm_order_entries(g) + 4);
             // entries outside the window of a row's tile, for the parts aggregated on the tensor cores
@@ -552,7 +553,6 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
             // 1 M rows of an 8-8-2 network, and some calls did not fit).
             const int64_t long_room = tiles ? std::min<int64_t>(rows, (int64_t)((share - cur.used) / 256 * (256 / sizeof(int32_t)))) : 0;
             int32_t* long_rows = cur.take<int32_t>((size_t)long_room);
-            int* long_count = ticket + 32;
             if (rows == 0) continue;
 
             // the rows between the parts of every matrix that a tile may read past a part's end
@@ -596,7 +596,7 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                 int* flags_host = static_cast<int*>(ctx->pinned);
                 bool any_dense = false, all_dense = true;
                 auto read_flags = [&]() -> int32_t {
-                    RTMA_CUDA(ctx, cudaMemcpyAsync(flags_host, dense_flags, sizeof(int) * RTMA_MAX_PARTS, cudaMemcpyDeviceToHost, s));
+                    RTMA_CUDA(ctx, cudaMemcpyAsync(flags_host, dense_flags, sizeof(int) * (RTMA_MAX_PARTS + 2), cudaMemcpyDeviceToHost, s));
                     RTMA_CUDA(ctx, cudaStreamSynchronize(s));
                     any_dense = false;
                     all_dense = true;
@@ -617,9 +617,8 @@ int32_t train_impl(rtma_ctx* ctx, const rtma_model_desc* md, int32_t M, const in
                     wave_order.rows_total = rows;
                     wave_order.left_cnt = left_cnt;
                     wave_order.left_col = left_col;
-                    wave_order.long_count = long_count;
-                    wave_order.long_rows = long_rows;
-                    wave_order.long_room = long_room;
+                    const int hubs = flags_host[RTMA_MAX_PARTS], many = flags_host[RTMA_MAX_PARTS + 1];
+                    wave_order.long_rows = LongRows{hubs, many, (int64_t)hubs + many <= long_room, long_rows, long_room};
                     wave_order.win_bits = win_bits;
                     wave_order.block_mask = block_mask;
                 }

@@ -137,6 +137,14 @@ int32_t launch_symmetry_check(rtma_ctx* ctx, const GroupDesc& g, const int64_t* 
                               unsigned long long* sums, cudaStream_t s);
 // Processing order of the aggregation kernels' row groups (8 consecutive rows): the groups with at
 // least `heavy` entries, listed once per call, go first.  A zeroed SpmmOrder means plain row order.
+// Rows with many entries outside their tile's window, once per wave: numbers of them, known to the host, and a list of their scratch
+// rows if all have room in it: hubs from its front, the others from its back.
+struct LongRows {
+    int hubs, many;
+    bool listed;
+    const int32_t* list;  // device
+    int64_t room;
+};
 struct SpmmOrder {
     const int* heavy_count;  // device: number of listed groups
     const int* heavy_list;   // device: their indices
@@ -149,9 +157,7 @@ struct SpmmOrder {
     const unsigned char* left_cnt;  // device, per scratch row of such a part: its entries outside the tile's window
                                     // (254, 255: more than DENSE_LEFT_CAP), and their columns [row][DENSE_LEFT_CAP]
     const int32_t* left_col;
-    const int* long_count;     // device: the rows of more: [0] hubs, listed in long_rows from its front, [1] the others, from its back;
-    const int32_t* long_rows;  // where both together are more than long_room nothing is listed
-    int64_t long_room;
+    LongRows long_rows;      // and the rows of more
     const unsigned long long* win_bits;  // device, per scratch row of such a part: its window as DENSE_WINDOW bits
     const unsigned char* block_mask;     // device, per 32 scratch rows of such a part: bit b = one of them has an entry in
                                          // its window's 64-row block b

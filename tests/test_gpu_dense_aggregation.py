@@ -244,3 +244,71 @@ def test_entries_outside_the_windows(util, forced, tiny_workload, n, degree, dim
     w.params0 = inputs.xavier_params(w.dims, 35)
     got, want = util.check_one_step(w)
     util.check_k_steps_and_average(w, got, want, 2)
+
+
+def _hub_parts(n, M, outside, seed):
+    """M parts of n rows in clusters of 100 that are nearly complete, every row with about `outside` entries all over its part."""
+    parts = []
+    for p in range(M):
+        rng = np.random.default_rng(seed + p)
+        u = np.repeat(np.arange(n), 90)
+        u2 = np.repeat(np.arange(n), outside // 2)
+        v = np.concatenate([u // 100 * 100 + rng.integers(0, 100, u.size), rng.integers(0, n, u2.size)])
+        u = np.concatenate([u, u2])
+        key = np.unique(np.concatenate([u * n + v, v * n + u])[np.concatenate([u != v, u != v])])
+        rowptr = np.zeros(n + 1, dtype=np.int64)
+        np.cumsum(np.bincount(key // n, minlength=n), out=rowptr[1:])
+        parts.append((rowptr, (key % n).astype(np.int32)))
+    return parts
+
+
+# rows with more than 64 entries outside their window: a block each where there are fewer than 24 for every SM, a warp each where there
+# are more, with the same sums: two parts of 2,200 such rows together and one of them by itself
+def test_few_and_many_hubs_are_summed_alike(util, forced):
+    import oracle
+    n, M, dims, K = 2_200, 2, (24, 72, 40, 19), 2
+    parts = _hub_parts(n, M, 110, 51)
+    X, y = inputs.normal_features(M * n, dims[0], 52), inputs.uniform_labels(M * n, dims[-1], 53)
+    params0 = inputs.xavier_params(dims, 54)
+    edges = np.cumsum([0] + [c.size for _, c in parts]).tolist()
+    rowptr, col = util.dev(np.concatenate([r for r, _ in parts])), util.dev(np.concatenate([c for _, c in parts]))
+    for rp, cp in parts:  # nearly every row is a hub: of its entries more than 64 lie outside its tile's window
+        tile = np.repeat(np.arange(n), np.diff(rp)) // 128 * 128
+        outside = np.add.reduceat((cp < tile - 128) | (cp >= tile + 256), rp[:-1])
+        assert 3_552 // 2 < (outside > 64).sum() <= 3_552
+
+    def run(steps):
+        params = util.dev(np.tile(params0, (M, 1)))
+        forced.local_steps(dims, 0.1, M, [0, n, 2 * n], edges, rowptr, col, util.dev(X), util.dev(y), params, steps)
+        forced.check()
+        return params.cpu().numpy()
+
+    both = run([K, K])
+    assert np.array_equal(both[0], run([K, 0])[0]) and np.array_equal(both[1], run([0, K])[1])
+    for p, (rp, cp) in enumerate(parts):
+        want, _ = oracle.local_steps_variant((0, 0, 0), dims, 0.1, rp, cp, X[p * n:(p + 1) * n].astype(np.float64), y[p * n:(p + 1) * n],
+                                             params0.astype(np.float64), K)
+        assert util.rel_err(both[p], want) <= util.TOL_PARAM
+
+
+# parts of which every row is one cost 2.3 times on the tensor cores what gathering costs there (5.7 times while all such rows belonged to
+# one block per SM)
+def test_parts_full_of_hubs_are_not_left_to_a_few_blocks(util):
+    from paper_2305_09887_b200 import binding
+    n, dims = 50_000, (16, 48, 48, 47)
+    (rowptr, col), = _hub_parts(n, 1, 74, 61)
+    rowptr, col, edges = util.dev(rowptr), util.dev(col), int(rowptr[-1])
+    X, y = torch.randn(n, dims[0], device="cuda"), torch.zeros(n, dtype=torch.int32, device="cuda")
+    c, times = binding.Context(0), []
+    c.profile(True)
+    for mode in (0, 2):
+        c.set_dense_aggregation(mode)
+        best = 1e9
+        for _ in range(4):
+            params = util.dev(inputs.xavier_params(dims, 62)[None])
+            c.local_steps(dims, 0.1, 1, [0, n], [0, edges], rowptr, col, X, y, params, 2)
+            times_now = c.profile_read()
+            best = min(best, times_now["spmm_forward"][0] + times_now["spmm_backward"][0])
+        times.append(best)
+    c.close()
+    assert times[1] <= 3.5 * times[0], times

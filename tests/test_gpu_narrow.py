@@ -55,9 +55,9 @@ def test_a_call_on_a_large_part_fits_the_scratch_it_asks_for(util, monkeypatch, 
 
 
 def test_long_rows_listed_or_searched_for_give_the_same_bits(util):
-    # tensor-core tiles forced on a graph without neighbourhoods: nearly all of 70,000 rows have more entries outside their windows than
+    # tensor-core tiles forced on a graph without neighbourhoods: nearly all of 72,000 rows have more entries outside their windows than
     # are listed, two of them hundreds.  A context that has no room to list such rows, one that has, and one whose arena a call grew
-    n, dims = 70_000, (16, 16, 5)
+    n, dims = 72_000, (16, 16, 5)
     w = _workload(n, 9, dims, (0, 0, 0))
     g = w.graph
     rng = np.random.default_rng(47)
