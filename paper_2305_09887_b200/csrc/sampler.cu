@@ -150,6 +150,7 @@ sample_select_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restri
     for (int attempt = 0; attempt < 2; ++attempt) {
         const bool mine = collect && (attempt == 0 || count < fanout);
         if (attempt == 1 && (!__any_sync(0xffffffffu, mine) || wide <= tight)) break;
+        __syncwarp();  // the second attempt overwrites what other lanes wrote in the first
         const float share = (attempt == 0 ? tight : wide) / (float)deg;
         const uint32_t bound = share >= 0.999f ? 0xFFFFFFFFu : (uint32_t)(share * 4294967296.f);
         const int rounds = mine ? (int)((deg + SEL_LANES - 1) / SEL_LANES) : 0;
