@@ -173,7 +173,8 @@ struct TileWalk {
 };
 
 // TRANSPOSED = false: A counts, out = (1 / deg v) * A src;  true: A = counts x 1 / deg u, out = A src
-template <bool TRANSPOSED>
+// AHEAD: the rows' windows and weights are requested a tile ahead
+template <bool TRANSPOSED, bool AHEAD>
 __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_constant__ DenseArgs a) {
     wait_for_kernel_before();
     extern __shared__ uint8_t smem_raw[];
@@ -280,7 +281,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
             tc::mbar_arrive(&pb.builders);
             return dense_wait(&pb.builders, meetings++ & 1u, &pb, a.error_word);
         };
-        // the window of the thread's row and (transposed pass) the weights of the tile's window rows r, r + 128, ...: a tile ahead
+        // the window of the thread's row and (transposed pass) the weights of the tile's window rows r, r + 128, ...
         constexpr int PER_THREAD = DENSE_WINDOW / DT_BUILDERS;
         unsigned long long next_bits[DT_KB];
         float next_w[PER_THREAD];
@@ -307,8 +308,9 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
         bool ok = true;
         TileWalk walk(a);
         TileAt tile = walk.next(a);
-        request(tile);
+        if (AHEAD) request(tile);
         while (tile.valid && ok) {
+            if (!AHEAD) request(tile);
             const uint32_t blocks = tile.blocks();
             const int NA = min(DT_TILE_ATOMS, a.n_atoms - DT_TILE_ATOMS * tile.ct);
             const int ct = tile.ct, y0 = (int)(tile.ws + tile.r0 - DT_HALO);  // the window's first scratch row; may be negative: reads zeros
@@ -329,8 +331,10 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
                 ok = meet();
                 if (!ok) break;
             }
-            tile = walk.next(a);
-            request(tile);
+            if (AHEAD) {
+                tile = walk.next(a);
+                request(tile);
+            }
             for (uint32_t rest = blocks; rest; rest &= rest - 1, at.advance(stages)) {
                 const int kb = __ffs(rest) - 1;
                 const int s = at.s;
@@ -383,6 +387,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
                 tc::fence_proxy_async_smem();  // the tensor core reads what this thread has just written
                 tc::mbar_arrive(&pb.full[s]);
             }
+            if (!AHEAD) tile = walk.next(a);
         }
     } else {
         const int ew = warp - (1 + DT_BUILDERS / 32);  // 0..7
@@ -392,10 +397,21 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
         float4* st = reinterpret_cast<float4*>(stg);
         const int p = lane & 3;
         const uint32_t out_row_bytes = (uint32_t)a.out.ld * 2u;
-        // of the thread's four rows of a tile: the scale, and whether the output row already holds a sum to add to
-        auto row_info = [&](int k, int r0, float (&scale)[4], bool (&has_left)[4]) {
+        TileWalk walk(a);
+        TileAt tile = walk.next(a);
+        uint32_t t = 0;
+        bool ok = true;
+        while (tile.valid && ok) {
+            const int k = tile.k, r0 = tile.r0, ct = tile.ct;
+            const int BN = 64 * min(DT_TILE_ATOMS, a.n_atoms - DT_TILE_ATOMS * ct);
+            const int n0 = ct * 64 * DT_TILE_ATOMS;
             const int rows_here = min(32, a.g.rows[k] - (r0 + q * 32));
             const int64_t orow0 = a.g.row_ws[k] + r0 + q * 32;
+            // of the thread's four rows: the scale, and whether the output row already holds a sum to add to.  (Not a tile ahead: 13 warps leave
+            // a thread 128 registers, the loop below needs them, and spilled forward it took 1,290 us instead of 1,100 for 256 columns of 2 M
+            // rows, 560 instead of 484 for 64; 1,170 and 550 with two divisions a stage and nothing ahead but this.)
+            float scale[4];
+            bool has_left[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int row = j * 8 + (lane >> 2);
@@ -406,31 +422,8 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
                     has_left[j] = a.left_cnt[orow0 + row] != 0;
                 }
             }
-        };
-        TileWalk walk(a);
-        TileAt tile = walk.next(a);
-        float next_scale[4];
-        bool next_left[4];
-        if (tile.valid) row_info(tile.k, tile.r0, next_scale, next_left);
-        uint32_t t = 0;
-        bool ok = true;
-        while (tile.valid && ok) {
-            float scale[4];
-            bool has_left[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                scale[j] = next_scale[j];
-                has_left[j] = next_left[j];
-            }
-            const int k = tile.k, r0 = tile.r0, ct = tile.ct;
-            const int BN = 64 * min(DT_TILE_ATOMS, a.n_atoms - DT_TILE_ATOMS * ct);
-            const int n0 = ct * 64 * DT_TILE_ATOMS;
-            const int rows_here = min(32, a.g.rows[k] - (r0 + q * 32));
-            const int64_t orow0 = a.g.row_ws[k] + r0 + q * 32;
-            // the next tile's row data is requested a tile ahead, and every chunk's existing rows before the chunk
-            // before them is finished: the epilogue is the longest chain of the kernel, and these loads its latency
-            tile = walk.next(a);
-            if (tile.valid) row_info(tile.k, tile.r0, next_scale, next_left);
+            // every chunk's existing rows are requested before the chunk before them is finished: the epilogue is the longest chain of the
+            // kernel, and these loads its latency
             uint4 gh[4], gl[4];
             auto request = [&](int c0) {  // what the rows already hold (written by the launch before this one)
                 const int n = n0 + c0 + 8 * p;
@@ -507,6 +500,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) spmm_dense_kernel(const __grid_
             tc::tc_fence_before_sync();
             tc::mbar_arrive(&pb.acc_empty[buf]);
             ++t;
+            tile = walk.next(a);
         }
     }
     tc::tc_fence_before_sync();
@@ -924,10 +918,9 @@ int32_t launch_spmm_dense(rtma_ctx* ctx, int kclass, const GroupDesc& g, const i
     const int64_t row_tiles = group_tiles(g, DT_BM);
     if (row_tiles == 0) return RTMA_OK;
     if (!ctx->dense_configured) {
-        RTMA_CUDA(ctx, cudaFuncSetAttribute(reinterpret_cast<const void*>(spmm_dense_kernel<false>),
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize, DT_SMEM_MAX));
-        RTMA_CUDA(ctx, cudaFuncSetAttribute(reinterpret_cast<const void*>(spmm_dense_kernel<true>),
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize, DT_SMEM_MAX));
+        for (const void* kernel : {reinterpret_cast<const void*>(spmm_dense_kernel<false, true>), reinterpret_cast<const void*>(spmm_dense_kernel<true, true>),
+                                   reinterpret_cast<const void*>(spmm_dense_kernel<true, false>)})
+            RTMA_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DT_SMEM_MAX));
         ctx->dense_configured = true;
     }
     DenseArgs a{};
@@ -990,8 +983,11 @@ int32_t launch_spmm_dense(rtma_ctx* ctx, int kclass, const GroupDesc& g, const i
     const size_t smem = a.stages * stage_bytes + fixed;
     {
         KernelScope ks(ctx, kclass, s);
-        if (transposed) launch_kernel(spmm_dense_kernel<true>, grid, DT_THREADS, smem, s, a);
-        else launch_kernel(spmm_dense_kernel<false>, grid, DT_THREADS, smem, s, a);
+        // transposed with several column tiles: 2 M rows of 512 values 3,460 us with the windows a tile ahead, 3,330 without; of 64 and 128
+        // values on 300,000 rows 97 / 136 and 102 / 139
+        if (!transposed) launch_kernel(spmm_dense_kernel<false, true>, grid, DT_THREADS, smem, s, a);
+        else if (a.col_tiles == 1) launch_kernel(spmm_dense_kernel<true, true>, grid, DT_THREADS, smem, s, a);
+        else launch_kernel(spmm_dense_kernel<true, false>, grid, DT_THREADS, smem, s, a);
     }
     RTMA_LAUNCH_CHECK(ctx);
     return RTMA_OK;

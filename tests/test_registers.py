@@ -18,3 +18,8 @@ def spills(source, tmp_path):
 def test_input_gradient_of_a_few_classes_does_not_spill(tmp_path):
     got = {k: v for k, v in spills("dgrad_narrow.cu", tmp_path).items() if "dgrad_narrow_kernel" in k}
     assert len(got) == 8 and not any(got.values()), got
+
+
+def test_window_tiles_keep_their_epilogue_in_registers(tmp_path):
+    got = {k: v for k, v in spills("spmm_tc.cu", tmp_path).items() if "spmm_dense_kernel" in k}
+    assert len(got) == 3 and all(v <= 8 for v in got.values()), got
