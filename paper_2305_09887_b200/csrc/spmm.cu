@@ -271,7 +271,6 @@ spmm_rows(const GroupDesc& g, const int64_t* __restrict__ rowptr_out,
     if (lane + 32 >= g.num) first_hi = INT_MAX;
     const int n_heavy = order.heavy_count ? *order.heavy_count : 0;
     const int last_ticket = n_heavy + (int)total_groups;
-    const int64_t heavy = order.heavy_count ? order.heavy : INT64_MAX;
 
     constexpr bool by_block = BY_BLOCK;
     __shared__ int block_ticket;
@@ -317,7 +316,7 @@ spmm_rows(const GroupDesc& g, const int64_t* __restrict__ rowptr_out,
     const float my_w = (MODE != 1 && lane < nrows) ? inv_deg[ws + i0 + lane] : 1.f;
     const int64_t e_begin = __shfl_sync(0xffffffffu, my_off, 0);
     const int64_t e_end = __shfl_sync(0xffffffffu, my_off, nrows);
-    if (!listed && e_end - e_begin >= heavy) continue;  // done as a listed group
+    if (!listed && n_heavy > 0 && e_end - e_begin >= order.heavy) continue;  // done as a listed group
     // the offsets relative to the group's first entry (a part has fewer than 2^31 entries: checked by the caller)
     const int my_rel = (int)(my_off - e_begin);
     const int n_entries = (int)(e_end - e_begin);
@@ -329,48 +328,10 @@ spmm_rows(const GroupDesc& g, const int64_t* __restrict__ rowptr_out,
     int cur = 0;                                          // row (relative to i0) the accumulators belong to
     int next_rel = __shfl_sync(0xffffffffu, my_rel, 1);  // first entry past row `cur`
 
-    // the lane's columns of the group's first output row; the rows are finished in order
-    char* out_hi[NCH];
-    char* out_lo[NCH];
-    const char* self_hi[NCH];
-    const char* self_lo[NCH];
+    // the lane's first columns of the group's next output row; the rows are finished in order.  A live lane's further columns lie 512
+    // bytes apart, the lo plane at the planes' distance: one pointer, as the registers are for the rows in flight.
+    char* out_at = reinterpret_cast<char*>(out.hi + (ws + i0) * out.ld) + lane * 16;
     const uint32_t out_row_bytes = (uint32_t)out.ld * 2u;
-#pragma unroll
-    for (int c = 0; c < NCH; ++c) {
-        out_hi[c] = reinterpret_cast<char*>(out.hi + (ws + i0) * out.ld) + col_bytes[c];
-        out_lo[c] = reinterpret_cast<char*>(out.lo + (ws + i0) * out.ld) + col_bytes[c];
-        if (MODE == 2) {
-            self_hi[c] = reinterpret_cast<const char*>(src.hi + (ws + i0) * src.ld) + col_bytes[c];
-            self_lo[c] = reinterpret_cast<const char*>(src.lo + (ws + i0) * src.ld) + col_bytes[c];
-        }
-    }
-    // finishes row `row` (= the next row in order): scale, store, clear
-    auto flush = [&](int row) {
-        const float w = MODE == 1 ? 1.f : __shfl_sync(0xffffffffu, my_w, row);
-#pragma unroll
-        for (int c = 0; c < NCH; ++c) {
-            if (live[c]) {
-                if (MODE == 2)  // the self loop
-                    acc[c].fma_planes_mixed(w, *reinterpret_cast<const uint4*>(self_hi[c]), *reinterpret_cast<const uint4*>(self_lo[c]));
-                if (MODE != 1) {
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) acc[c].v[e] *= w;
-                }
-                uint4 h, l;
-                acc[c].to_planes_lean(h, l);
-                *reinterpret_cast<uint4*>(out_hi[c]) = h;
-                *reinterpret_cast<uint4*>(out_lo[c]) = l;
-            }
-            acc[c].zero();
-            out_hi[c] += out_row_bytes;
-            out_lo[c] += out_row_bytes;
-            if (MODE == 2) {
-                self_hi[c] += src_row_bytes;
-                self_lo[c] += src_row_bytes;
-            }
-        }
-    };
-
     // the lane's columns of the part's first source row
     const char* base_hi[NCH];
     const char* base_lo[NCH];
@@ -379,6 +340,29 @@ spmm_rows(const GroupDesc& g, const int64_t* __restrict__ rowptr_out,
         base_hi[c] = reinterpret_cast<const char*>(src.hi + ws * src.ld) + col_bytes[c];
         base_lo[c] = reinterpret_cast<const char*>(src.lo + ws * src.ld) + col_bytes[c];
     }
+    // finishes row `row` (= the next row in order): scale, store, clear
+    auto flush = [&](int row) {
+        const float w = MODE == 1 ? 1.f : __shfl_sync(0xffffffffu, my_w, row);
+#pragma unroll
+        for (int c = 0; c < NCH; ++c) {
+            if (live[c]) {
+                if (MODE == 2) {  // the self loop
+                    const uint64_t at = (uint64_t)(uint32_t)(i0 + row) * src_row_bytes;
+                    acc[c].fma_planes_mixed(w, *reinterpret_cast<const uint4*>(base_hi[c] + at), *reinterpret_cast<const uint4*>(base_lo[c] + at));
+                }
+                if (MODE != 1) {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) acc[c].v[e] *= w;
+                }
+                uint4 h, l;
+                acc[c].to_planes_lean(h, l);
+                *reinterpret_cast<uint4*>(out_at + c * 512) = h;
+                *reinterpret_cast<uint4*>(out_at + (reinterpret_cast<char*>(out.lo) - reinterpret_cast<char*>(out.hi)) + c * 512) = l;
+            }
+            acc[c].zero();
+        }
+        out_at += out_row_bytes;
+    };
 
     for (int p0 = 0; p0 < n_entries; p0 += 32) {   // pieces of 32 entries
         const int cnt = min(32, n_entries - p0);
@@ -432,7 +416,10 @@ spmm_rows(const GroupDesc& g, const int64_t* __restrict__ rowptr_out,
 
 // Blocks of eight warps per SM.  Rows up to 256 values: two with eight rows in flight per lane, or three with four, which took as
 // long forward (97 / 99 us for 200,000 rows, 618,000 entries) and longer backward (101 / 105), but less with self
-// loops (131 / 114).  Up to 512 values, four rows in flight: one 680, two 519 (500,000 rows, 1.9 M entries; backward 710 / 538).
+// loops (131 / 114).  Up to 512 values, four rows in flight: one 680, two 519 (500,000 rows, 1.9 M entries; backward 710 / 538); with
+// self loops one 1,265, two 922 (200,000 rows and 618,000 entries 359 / 238, of 300 values 310 / 194; 30,000 rows of 400 values, where the
+// longest row decides, 68 / 69).  With pointers per plane and chunk to the lane's columns of the output and of the row itself those with self
+// loops spilled: 930, 244, 200 and 70.
 constexpr int spmm_blocks_per_sm(int nch, int mode) { return nch == 1 ? (mode == 2 ? 3 : 2) : nch == 2 ? 2 : 1; }
 
 template <int NCH, int MODE>

@@ -23,3 +23,8 @@ def test_input_gradient_of_a_few_classes_does_not_spill(tmp_path):
 def test_window_tiles_keep_their_epilogue_in_registers(tmp_path):
     got = {k: v for k, v in spills("spmm_tc.cu", tmp_path).items() if "spmm_dense_kernel" in k}
     assert len(got) == 3 and all(v <= 8 for v in got.values()), got
+
+
+def test_gathers_with_self_loops_keep_their_rows_in_registers(tmp_path):
+    got = {k: v for k, v in spills("spmm.cu", tmp_path).items() if "spmm_kernelILi2ELi2E" in k}  # 257 to 512 values
+    assert len(got) == 1 and not any(got.values()), got
